@@ -30,6 +30,10 @@ constexpr double kDropFP64 = 1e32, kDropFF = 1e16, kDropFP32 = 1e16;
 constexpr double kDropCapFF = 1e60, kDropCapFP32 = 1e30;
 constexpr long long kSmemVecBytes = 160 * 1024;   // dynamic smem of the border solves
 constexpr int kThreads = 256;     // threads per CTA of the dense kernels
+// FP64 factors on the tensor cores (k_dz.cu): digits per entry, and the row
+// exponent that marks a row holding a NaN or an infinity
+constexpr int kDzQ = 8;
+constexpr int kDzNotFinite = 1 << 20;
 
 // One dense lower-triangular "partial Cholesky" problem: an a x a matrix
 // (column-major, leading dimension lda, element offset base) whose first p
@@ -240,6 +244,12 @@ struct ahlp_problem {
   long long stage_slots = 0;
   int *tc_joff = nullptr;            // [maxTp][N + 1]
   std::vector<long long> tc_jobs;    // [maxTp]
+  // FP64 factors on the tensor cores: each panel tile of the current step as
+  // eight FP16 digit planes, one exponent per row, and the CUtensorMaps of the
+  // A and B operand copies
+  __half *dz_stage = nullptr;
+  int *dz_exp = nullptr;
+  unsigned char dz_map[2][128] = {};
   void *tc_tmap = nullptr;           // [N] CUtensorMap
   bool tc_ready = false;
   // float-float factors on the tensor cores: each panel tile as six FP16
@@ -368,9 +378,12 @@ cudaError_t launch_dscale(ahlp_problem *p);   // dscale = x / (z + fac_rho_x x)
 cudaError_t launch_form(ahlp_problem *p, double delta);
 // prof (nullable): a handle whose kernel-class timer records the launches
 // (kt_mark); classes 0 diagonal tiles, 1 panels, 2 trailing updates
+// with dz (a handle set up by dz_setup) the trailing updates run on the tensor
+// cores (k_dz.cu), else on the FP64 pipe
 cudaError_t launch_pchol(double *buf, const BlkInfo *info, const std::vector<BlkInfo> &h,
                          const double *diag0, double tol, int *status, cudaStream_t s,
-                         ahlp_problem *prof = nullptr, double drop = 0.0);
+                         ahlp_problem *prof = nullptr, double drop = 0.0,
+                         ahlp_problem *dz = nullptr);
 // float-float (hi = aug32, lo): diagonal tiles and panels in FP64 arithmetic,
 // trailing updates in double-float; then hi + lo is expanded into out (the
 // FP64 factor buffer, elems entries), which the Schur assembly and the solves use
@@ -458,6 +471,12 @@ cudaError_t launch_update_tc(ahlp_problem *p, int k, cudaStream_t s);
 // the same for float-float factors: FP16 digit staging and job offsets
 bool oz_setup(ahlp_problem *p);
 cudaError_t launch_update_oz(ahlp_problem *p, int k, cudaStream_t s);
+
+// the same for FP64 factors: eight-digit staging, job offsets, tensor maps
+bool dz_setup(ahlp_problem *p);
+cudaError_t launch_update_dz(ahlp_problem *p, int k, cudaStream_t s);
+// update jobs of every step (called by the three set-ups)
+void jobs_setup(ahlp_problem *p);
 
 // ---- kernel-class timer (option profile_kernels) -----------------------------
 // kt_mark records an event on s that ends the previous mark's interval and

@@ -1481,7 +1481,7 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
   }
   else
     ck(launch_pchol(p->aug, p->blk, p->h_blk, p->diag0, p->fac_pivot_tol, p->status, s, prof,
-                    drop ? kDropFP64 : 0.0),
+                    drop ? kDropFP64 : 0.0, p->maxT > 1 && dz_setup(p) ? p : nullptr),
        "pchol");
   ck(launch_tinv(p), "diagonal tile inverses");
   ck(cudaEventRecord(p->ev[2], s), "event");

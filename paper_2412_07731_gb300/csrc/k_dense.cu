@@ -150,10 +150,82 @@ __global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(T *buf, const Blk
   }
 }
 
+// One 64 x 64 FP64 panel tile as eight FP16 digit planes for the tensor-core
+// update (k_dz.cu): row r's exponent E_r is one more than its largest entry's,
+// v = round(x 2^(63 - E_r)) is a 64-bit integer below 2^62, and the bytes of
+// v + 0x8080...80 less 128 are its balanced digits, most significant first.
+// Plane p of the K slice of columns 16 sl .. 16 sl + 15 is a 64 x 16 K-major
+// operand of 8-row x 16-byte core matrices, 2 KB at ((8 sl + p) * slots +
+// slot): entry (r, c) at (r/8)*128 + ((c%16)/8)*64 + (r%8)*8 + c%8.  Rows past
+// the matrix and columns past the pivots are zero.  Thread (row r = tid / 4,
+// slice tid % 4); x(r, c) returns the entry.  A row holding a NaN or an
+// infinity gets the exponent kDzNotFinite and no digits.
+template <typename F>
+__device__ __forceinline__ void dz_stage_tile(F x, int nri, int npiv, __half *stage, int *dexp,
+                                              long long slots, long long slot) {
+  const int r = threadIdx.x >> 2, sl = threadIdx.x & 3, c0 = sl * 16;
+  const bool row = r < nri;
+  int mx = 0;   // largest biased exponent
+#pragma unroll
+  for (int j = 0; j < 16; ++j)
+    if (row && c0 + j < npiv)
+      mx = max(mx, (__double2hiint(x(r, c0 + j)) >> 20) & 0x7ff);
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+  const bool fin = mx < 0x7ff;
+  const int E = mx - 1021;   // |x| < 2^(E - 1)
+  if (sl == 0) dexp[slot * NB + r] = fin ? E : kDzNotFinite;
+  __half *st = stage + ((long long)(sl * kDzQ) * slots + slot) * 1024 + (r >> 3) * 128 + (r & 7) * 8;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {   // 8 columns: one 16-byte run per plane
+    uint32_t lo[8], hi[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int c = c0 + h * 8 + j;
+      unsigned long long v = 0;
+      if (row && fin && c < npiv) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(x(r, c));
+        const int be = (int)(b >> 52) & 0x7ff;
+        unsigned long long m = b & 0xfffffffffffffull;
+        if (be) m |= 1ull << 52;
+        // x = m 2^(max(be, 1) - 1075), so v = m 2^(max(be, 1) - 1012 - E)
+        const int sh = max(be, 1) - 1012 - E;   // at most 9
+        if (sh >= 0) m <<= sh;
+        else if (sh > -64) m = (m + (1ull << (-sh - 1))) >> -sh;
+        else m = 0;
+        v = (b >> 63) ? 0ull - m : m;
+      }
+      v += 0x8080808080808080ull;
+      lo[j] = (uint32_t)v;
+      hi[j] = (uint32_t)(v >> 32);
+    }
+#pragma unroll
+    for (int p = 0; p < kDzQ; ++p) {
+      const int byte = 3 - (p & 3);
+      const uint32_t sel = (uint32_t)(byte | ((byte + 4) << 4));   // that byte of both words
+      uint32_t w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t a = p < 4 ? hi[2 * q] : lo[2 * q], b = p < 4 ? hi[2 * q + 1] : lo[2 * q + 1];
+        // halves 1024 + byte, less 1152
+        const uint32_t y = __byte_perm(__byte_perm(a, b, sel), 0x64646464u, 0x4140);
+        const __half2 f = __hsub2(*reinterpret_cast<const __half2 *>(&y),
+                                  __floats2half2_rn(1152.0f, 1152.0f));
+        w[q] = *reinterpret_cast<const uint32_t *>(&f);
+      }
+      *reinterpret_cast<uint4 *>(st + (long long)p * slots * 1024 + h * 64) =
+          make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+}
+
 // panel tiles below the diagonal tile: X = A_Ik L_kk^-T on the pivot columns,
-// and the non-pivot (Schur) columns of the tile updated with the new X.
+// and the non-pivot (Schur) columns of the tile updated with the new X.  With
+// stage (FP64 factors, tensor-core update) the tile's digits are written too.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkInfo *blk, int k) {
+__global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkInfo *blk, int k,
+                                                              __half *stage, int *dexp,
+                                                              long long slots) {
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const int I = k + 1 + blockIdx.x;
@@ -188,6 +260,11 @@ __global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkI
   for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
     const int r = i % NB, c = i / NB;
     if (r < nri && c < nr) gx[(long long)c * bi.lda + r] = X[r][c];
+  }
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (stage)
+      dz_stage_tile([&](int r, int c) { return X[r][c]; }, nri, npiv, stage, dexp, slots,
+                    bi.soff + I);
   }
 }
 
@@ -1683,7 +1760,7 @@ template <typename T>
 cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkInfo> &h,
                     const double *diag0, double tol, int *status, cudaStream_t s,
                     ahlp_problem *tc = nullptr, ahlp_problem *prof = nullptr,
-                    double drop = 0.0) {
+                    double drop = 0.0, ahlp_problem *dz = nullptr) {
   int nblk = (int)h.size();
   if (nblk == 0) return cudaSuccess;
   int maxTp = 0;
@@ -1712,7 +1789,9 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
         count_launch(), pchol_trsm_kernel<T><<<dim3((unsigned)maxPanel, nblk), kThreads,
-                                               trsm_smem<T>(), s>>>(buf, info, k);
+                                               trsm_smem<T>(), s>>>(
+                            buf, info, k, dz ? dz->dz_stage : nullptr,
+                            dz ? dz->dz_exp : nullptr, dz ? dz->stage_slots : 0);
     }
     if (prof) kt_mark(prof, 2, s);
     if (maxTrail > 0) {
@@ -1724,9 +1803,13 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
           count_launch(), pchol_update_f32_kernel<<<dim3((unsigned)maxTrail, nblk),
                                                     kUpdF32Threads, 0, s>>>(buf, info, k);
         }
-      } else
+      } else if (dz) {
+        cudaError_t e = launch_update_dz(dz, k, s);
+        if (e != cudaSuccess) return e;
+      } else {
         count_launch(), pchol_update_kernel<T><<<dim3((unsigned)maxTrail, nblk), kThreads, 0, s>>>(
                             buf, info, k);
+      }
     }
     if (prof) kt_mark(prof, 3, s);
     cudaError_t e = cudaGetLastError();
@@ -1810,8 +1893,8 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
 
 cudaError_t launch_pchol(double *buf, const BlkInfo *info, const std::vector<BlkInfo> &h,
                          const double *diag0, double tol, int *status, cudaStream_t s,
-                         ahlp_problem *prof, double drop) {
-  return pchol_t<double>(buf, nullptr, info, h, diag0, tol, status, s, nullptr, prof, drop);
+                         ahlp_problem *prof, double drop, ahlp_problem *dz) {
+  return pchol_t<double>(buf, nullptr, info, h, diag0, tol, status, s, nullptr, prof, drop, dz);
 }
 
 cudaError_t launch_pchol_f32(float *buf, float *tinv, const BlkInfo *info,

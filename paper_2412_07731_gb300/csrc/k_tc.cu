@@ -36,6 +36,7 @@
 #include <new>
 
 #include "ahlp_internal.h"
+#include "tcgen05.h"
 
 namespace ahlp {
 
@@ -47,68 +48,6 @@ constexpr uint32_t kTileBytes = NB * NB * 4;            // one staged 64x64 FP32
 constexpr uint32_t kSmemA = 2 * kTileBytes;             // 128 rows x 64 k
 constexpr uint32_t kSmemB = kTileBytes;                 // 64 rows x 64 k
 constexpr uint32_t kSmemBytes = 2 * kSmemA + 2 * kSmemB + 1024;   // hi/lo of A and B + alignment
-constexpr unsigned long long kWaitNs = 1000000000ull;   // 1 s
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ unsigned long long globaltimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// bounded wait for phase `parity` of the barrier; false when it ran out
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  const unsigned long long t0 = globaltimer();
-  while (!mbar_try(bar, parity))
-    if (globaltimer() - t0 > kWaitNs) return false;
-  return true;
-}
-
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes,
-                                         uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-          "r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-
-// Shared-memory matrix descriptor of a K-major operand without swizzling:
-// 8-row x 16-byte core matrices, LBO = byte distance between core matrices
-// adjacent in K, SBO = byte distance between adjacent 8-row groups.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;   // descriptor version of the tcgen05 family
-  return d;                 // base offset 0, absolute LBO, no swizzle
-}
-
 // Instruction descriptor of kind::tf32: FP32 accumulator, TF32 A and B, both
 // K-major, M = 128, N = 64.
 constexpr uint32_t kIdescTf32 = (1u << 4)                    // D format F32
@@ -125,19 +64,6 @@ __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
       "l"(adesc), "l"(bdesc), "r"(kIdescTf32), "r"(accumulate)
       : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::
-                   "r"(bar)
-               : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
 // 32 lanes x 32 bits, 32 consecutive columns: register j <- column col + j of
@@ -157,46 +83,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-}
-
-// One update job of step k: block b, the row tile pair (I0, I0 + 1) (the
-// second one only when has_i1) and the column tile J.  The jobs of a step are
-// numbered block after block (joff: prefix over the blocks); inside a block
-// with t trailing tiles, row pair R holds min(2R + 2, t) jobs, so the jobs
-// before it number R(R + 1).
-struct Job {
-  int b, I0, J;
-  bool has_i1;
-};
-
-__device__ __forceinline__ Job decode_job(const int *joff, int nblk, int k, const BlkInfo *blk,
-                                          int q, const int4 *jt) {
-  if (jt) {   // tile-sparse: the kept jobs of this step, in the dense order
-    const int4 v = jt[q];
-    Job j;
-    j.b = v.x;
-    j.I0 = v.y;
-    j.J = v.z;
-    j.has_i1 = v.w != 0;
-    return j;
-  }
-  int lo = 0, hi = nblk;   // joff[lo] <= q < joff[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (joff[mid] <= q) lo = mid;
-    else hi = mid;
-  }
-  const int t = blk[lo].T - k - 1;
-  const long long local = q - joff[lo];
-  long long R = (long long)((sqrt(4.0 * (double)local + 1.0) - 1.0) * 0.5);
-  while (R * (R + 1) > local) --R;
-  while ((R + 1) * (R + 2) <= local) ++R;
-  Job j;
-  j.b = lo;
-  j.I0 = k + 1 + 2 * (int)R;
-  j.J = k + 1 + (int)(local - R * (R + 1));
-  j.has_i1 = 2 * R + 1 < t;
-  return j;
 }
 
 struct TcArgs {
@@ -1051,11 +937,6 @@ long long tc_jobs_of(int t) {
   return n;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                                  const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                  const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 // Tile-sparse jobs of the tensor-core trailing updates (host only).  A
 // tile-level symbolic factorisation of each block's augmented matrix: tile
 // (I, J) of L is nonzero if the formed matrix has entries there or if some
@@ -1117,9 +998,27 @@ long long tile_sparse_jobs(int nblk, const int *T, const int *Tp,
   return (long long)tab.size();
 }
 
-// job offsets per step, over the blocks (shared by both tensor-core updates)
+}  // namespace
+
+EncodeTiledFn tensor_map_encoder() {
+  void *fn = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
+                                       &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess || !fn) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return reinterpret_cast<EncodeTiledFn>(fn);
+}
+
+// job offsets per step, over the blocks (shared by the tensor-core updates)
 void jobs_setup(ahlp_problem *p) {
   if (p->tc_joff) return;
+  int dev = 0, sms = 0;
+  ck(cudaGetDevice(&dev), "device");
+  ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+  p->num_sms = std::max(sms, 1);
   const int N = (int)p->h_blk.size();
   const int maxTp = p->maxTp;
   std::vector<int> joff((size_t)std::max(maxTp, 1) * (N + 1), 0);
@@ -1160,22 +1059,13 @@ void jobs_setup(ahlp_problem *p) {
     p->tc_jtab = static_cast<int4 *>(dupload_bytes(p, tab.data(), tab.size() * sizeof(int4)));
 }
 
-}  // namespace
-
 // Staging slots, per-step job offsets and the per-block tensor maps of the
 // tensor-core update (FP32 factors).  Returns false (nothing changed) when
 // the driver offers no tensor-map encoder.
 bool tc_setup(ahlp_problem *p) {
   if (p->tc_ready) return true;
-  void *fn = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                       &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess || !fn) {
-    cudaGetLastError();
-    return false;
-  }
-  auto encode = reinterpret_cast<EncodeTiledFn>(fn);
+  const EncodeTiledFn encode = tensor_map_encoder();
+  if (!encode) return false;
   const int N = (int)p->h_blk.size();
   std::vector<CUtensorMap> maps(std::max(N, 1));
   for (int b = 0; b < N; ++b) {
@@ -1200,12 +1090,6 @@ bool tc_setup(ahlp_problem *p) {
   ck(cudaFuncSetAttribute(pchol_update_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)kTc2Smem),
      "tensor-core update shared memory");
-  {
-    int dev = 0, sms = 0;
-    ck(cudaGetDevice(&dev), "device");
-    ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    p->num_sms = std::max(sms, 1);
-  }
   p->tc_ready = true;
   return true;
 }
@@ -1228,15 +1112,8 @@ cudaError_t launch_update_tc(ahlp_problem *p, int k, cudaStream_t s) {
 // FP16 digit staging and job offsets of the float-float tensor-core update
 bool oz_setup(ahlp_problem *p) {
   if (p->oz_ready) return true;
-  void *fn = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                       &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess || !fn) {
-    cudaGetLastError();
-    return false;
-  }
-  auto encode = reinterpret_cast<EncodeTiledFn>(fn);
+  const EncodeTiledFn encode = tensor_map_encoder();
+  if (!encode) return false;
   const int N = (int)p->h_blk.size();
   std::vector<CUtensorMap> maps(std::max(2 * N, 1));
   for (int w = 0; w < 2; ++w)
@@ -1264,12 +1141,6 @@ bool oz_setup(ahlp_problem *p) {
   ck(cudaFuncSetAttribute(pchol_update_oz2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)kOz2Smem),
      "float-float tensor-core update shared memory");
-  {
-    int dev = 0, sms = 0;
-    ck(cudaGetDevice(&dev), "device");
-    ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    p->num_sms = std::max(sms, 1);
-  }
   p->oz_ready = true;
   return true;
 }
