@@ -107,40 +107,126 @@ __global__ void dscale_kernel(const double *x, const double *z, double *d, doubl
 // --------------------------------------------------------------------------
 // partial Cholesky, step k: diagonal tile
 // --------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(T *buf, const BlkInfo *blk, int k,
-                                                               const double *diag0, double tol,
-                                                               int *status, double drop) {
+// The FP64 pipe issues one warp instruction per 64 clocks and partition, so the
+// tile is bound by its chain of dependent FP64 operations (64 pivots) and by
+// the number of FP64 warp instructions, not by bandwidth.  Four 16-column
+// panels; a panel is factored in registers by four warps, one per partition:
+// every warp holds its own copy of the 16 x 16 diagonal block and 16 rows
+// below it (lane = row and column parity, eight entries each), so no column
+// waits for another warp, and a pivot costs one reciprocal square root (a
+// single third-order step from the FP32 one), a scaling and an update.  Then
+// all eight warps apply the panel to the lower triangle right of it, lanes
+// packed over the triangle.  28 us per 64 x 64 tile on one CTA (124 us with a
+// barrier, a square root and a division per column).
+// 1 / sqrt(p) of a positive finite p: y0 = rsqrtf of the mantissa (p scaled
+// by an even power of two into [1, 4)), then Householder's third-order
+// iteration y = y0 + y0 e (1/2 + 3/8 e), e = 1 - m y0^2, whose error is ~e^3.
+__device__ __forceinline__ double rsqrt_f64(double p) {
+  const int hi = __double2hiint(p);
+  const int ex = hi >> 20;
+  if (ex == 0 || ex >= 0x7ff) return rsqrt(p);   // subnormal or infinite
+  const int k = (ex - 1023) >> 1;
+  const double m = __hiloint2double(hi - (k << 21), __double2loint(p));   // [1, 4)
+  // FP32 value of m from its bits (truncated)
+  const int mh = __double2hiint(m);
+  const float f = __int_as_float(((mh - 0x38000000) << 3) | (int)((unsigned)__double2loint(m) >> 29));
+  const double y0 = (double)rsqrtf(f);
+  const double e = fma(-m * y0, y0, 1.0);
+  const double y = fma(y0 * e, fma(0.375, e, 0.5), y0);
+  return __hiloint2double(__double2hiint(y) - (k << 20), __double2loint(y));
+}
+
+constexpr int kPW = 16;   // panel width
+
+__global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(double *buf, const BlkInfo *blk,
+                                                               int k, const double *diag0,
+                                                               double tol, int *status,
+                                                               double drop) {
   const BlkInfo bi = blk[blockIdx.x];
   if (k >= bi.Tp) return;
-  __shared__ T t[NB][NB + 1];
-  __shared__ T s_inv;
+  __shared__ double t[NB][NB + 1];
   const int r0 = k * NB;
   const int nr = min(NB, bi.a - r0);
   const int npiv = min(NB, bi.p - r0);
-  T *g = buf + bi.base + (long long)r0 * bi.lda + r0;
+  double *g = buf + bi.base + (long long)r0 * bi.lda + r0;
   for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
     const int r = i % NB, c = i / NB;
-    t[r][c] = (r < nr && c < nr && r >= c) ? g[(long long)c * bi.lda + r] : T(0);
+    t[r][c] = (r < nr && c < nr && r >= c) ? g[(long long)c * bi.lda + r] : 0.0;
   }
   __syncthreads();
-  for (int c = 0; c < npiv; ++c) {
-    if (threadIdx.x == 0) {
-      double piv = (double)t[c][c];
-      pivot_fix(piv, diag0[bi.d0off + r0 + c], tol, status, bi.tag + (int)blockIdx.x, r0 + c,
-                drop, sizeof(T) == 4 ? kDropCapFP32 : 1e300);
-      const T l = (T)sqrt(piv);
-      t[c][c] = l;
-      s_inv = T(1) / l;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rr = lane & 15, hc = lane >> 4;   // row of 16, column parity
+  for (int c0 = 0; c0 < npiv; c0 += kPW) {
+    if (warp < 4) {
+      const int row = warp * 16 + rr;       // this warp's own rows
+      const bool own = warp * 16 > c0;      // below the diagonal block
+      double d[8], o[8];                    // columns c0 + 2j + hc
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        d[j] = t[c0 + rr][c0 + 2 * j + hc];
+        o[j] = own ? t[row][c0 + 2 * j + hc] : 0.0;
+      }
+      const double dref = c0 + rr < npiv ? diag0[bi.d0off + r0 + c0 + rr] : 0.0;
+#pragma unroll
+      for (int u = 0; u < kPW; ++u) {
+        if (c0 + u < npiv) {   // uniform over the CTA
+          const int src = (u & 1) * 16;
+          double piv = __shfl_sync(0xffffffffu, d[u >> 1], src + u);
+          const double orig = __shfl_sync(0xffffffffu, dref, u);
+          const double v = __shfl_sync(0xffffffffu, d[u >> 1], src + rr);
+          const double vo = __shfl_sync(0xffffffffu, o[u >> 1], src + rr);
+          // the safeguard of pivot_fix, reported by one lane
+          const double lim = tol * orig;
+          if (!(piv == piv) || !(piv > lim) || !(piv > 0.0)) {
+            if (threadIdx.x == 0)
+              pivot_fix(piv, orig, tol, status, bi.tag + (int)blockIdx.x, r0 + c0 + u, drop);
+            piv = drop > 0.0 ? fmin(drop * fmax(orig, 1.0), 1e300) : lim > 0.0 ? lim : 1.0;
+          }
+          const double inv = rsqrt_f64(piv);
+          double lcc = piv * inv;
+          lcc = fma(fma(-lcc, lcc, piv), 0.5 * inv, lcc);
+          const double ld = rr == u ? lcc : v * inv;
+          const double lo = vo * inv;
+          if (hc == (u & 1)) {
+            d[u >> 1] = ld;
+            o[u >> 1] = lo;
+          }
+#pragma unroll
+          for (int j = u >> 1; j < 8; ++j) {   // columns q = 2j + hc > u
+            const double lq = __shfl_sync(0xffffffffu, ld, 2 * j + hc);
+            if (2 * j + hc > u) {
+              d[j] = fma(-ld, lq, d[j]);
+              o[j] = fma(-lo, lq, o[j]);
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int q = 2 * j + hc;
+        if (warp == 0 && q <= rr) t[c0 + rr][c0 + q] = d[j];
+        if (own) t[row][c0 + q] = o[j];
+      }
     }
     __syncthreads();
-    const T inv = s_inv;
-    for (int r = c + 1 + threadIdx.x; r < nr; r += blockDim.x) t[r][c] *= inv;
-    __syncthreads();
-    const int m = nr - c - 1;
-    for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-      const int rr = idx % m, ss = idx / m;
-      if (rr >= ss) t[c + 1 + rr][c + 1 + ss] -= t[c + 1 + rr][c] * t[c + 1 + ss][c];
+    // rank-16 update of the lower triangle right of the panel
+    const int q0 = c0 + kPW, cend = min(q0, npiv);
+    if (q0 < nr) {
+      const int w = nr - q0, ne = w * (w + 1) / 2;
+      for (int idx = threadIdx.x; idx < ne; idx += blockDim.x) {
+        int ri = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+        while (ri * (ri + 1) / 2 > idx) --ri;
+        while ((ri + 1) * (ri + 2) / 2 <= idx) ++ri;
+        const int r = q0 + ri, q = q0 + idx - ri * (ri + 1) / 2;
+        double s0 = t[r][q], s1 = 0.0;
+        int c = c0;
+        for (; c + 1 < cend; c += 2) {
+          s0 = fma(-t[r][c], t[q][c], s0);
+          s1 = fma(-t[r][c + 1], t[q][c + 1], s1);
+        }
+        if (c < cend) s0 = fma(-t[r][c], t[q][c], s0);
+        t[r][q] = s0 + s1;
+      }
     }
     __syncthreads();
   }
@@ -233,6 +319,7 @@ __global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkI
   extern __shared__ __align__(16) unsigned char trsm_raw[];   // two (NB x NB+1) tiles
   T(*L)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(trsm_raw);
   T(*X)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(trsm_raw + sizeof(T) * NB * (NB + 1));
+  __shared__ T rinv[NB];
   const int r0 = k * NB;
   const int nr = min(NB, bi.a - r0);
   const int npiv = min(NB, bi.p - r0);
@@ -246,8 +333,13 @@ __global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkI
     X[r][c] = (r < nri && c < nr) ? gx[(long long)c * bi.lda + r] : T(0);
   }
   __syncthreads();
+  // one reciprocal per column (a division by every thread at every column took
+  // two thirds of this kernel: FP64 divisions are ~20 instructions of a pipe
+  // with two lanes per clock)
+  if (threadIdx.x < npiv) rinv[threadIdx.x] = T(1) / L[threadIdx.x][threadIdx.x];
+  __syncthreads();
   for (int c = 0; c < npiv; ++c) {
-    const T inv = T(1) / L[c][c];
+    const T inv = rinv[c];
     for (int r = threadIdx.x; r < nri; r += blockDim.x) X[r][c] *= inv;
     __syncthreads();
     const int ns = nr - c - 1;
@@ -287,8 +379,6 @@ __global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkI
 // above it, so its sequential depth is 16 rows rather than 64.
 // --------------------------------------------------------------------------
 constexpr int kPotrf32Threads = 256;
-constexpr int kPW = 16;   // panel width
-
 __global__ void __launch_bounds__(kPotrf32Threads) pchol_potrf_f32_kernel(
     float *buf, float *tinv, const BlkInfo *blk, int k, const double *diag0, float tol,
     int *status, float drop) {
@@ -1343,35 +1433,42 @@ __device__ void wait_ready(const int *f, int *err) {
   }
 }
 
-// Inverted diagonal tiles, one CTA (one thread per column) per pivot tile.
-// Column j of X = L_kk^-1 by forward substitution against e_j.  The
-// non-pivot rows of a block's last pivot tile keep the factor entries, so
-// the solves stage one 64x64 tile that covers their whole diagonal step.
-template <typename T>
-__global__ void __launch_bounds__(NB) tinv_kernel(const T *__restrict__ buf, T *__restrict__ tinv,
-                                                  const BlkInfo *__restrict__ blk,
-                                                  const int *__restrict__ sched) {
-  extern __shared__ __align__(16) unsigned char tinv_raw[];   // tinv_smem<T>() bytes
-  T(*Ls)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(tinv_raw);
-  T(*Xs)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(tinv_raw + sizeof(T) * NB * (NB + 1));
-  T *rinv = reinterpret_cast<T *>(tinv_raw + 2 * sizeof(T) * NB * (NB + 1));
+// Inverted diagonal tiles of FP64 factors, one CTA per pivot tile.  The
+// non-pivot rows of a block's last pivot tile keep the factor entries, so the
+// solves stage one 64x64 tile that covers their whole diagonal step.  By 16x16
+// blocks: the diagonal blocks by substitution (a warp each, lane = column),
+// then block rows 1..3 in turn, X_ij = -X_ii sum_{k=j}^{i-1} L_ik X_kj, all
+// threads on the entries; the FP64 pipe (two lanes per clock) bounds it.  All
+// tiles of 32 blocks (1130 tiles): 326 -> 150 us against one thread per column.
+constexpr size_t kTinvSmem = (2 * NB * (NB + 1) + 16 * NB + NB) * sizeof(double);
+
+__global__ void __launch_bounds__(kThreads) tinv_kernel(const double *__restrict__ buf,
+                                                        double *__restrict__ tinv,
+                                                        const BlkInfo *__restrict__ blk,
+                                                        const int *__restrict__ sched) {
+  extern __shared__ __align__(16) unsigned char tinv_raw[];   // kTinvSmem bytes
+  double(*Ls)[NB + 1] = reinterpret_cast<double(*)[NB + 1]>(tinv_raw);
+  double(*Xs)[NB + 1] = Ls + NB;
+  double *Tm = reinterpret_cast<double *>(Xs + NB);   // [16][wc]
+  double *rinv = Tm + 16 * NB;
   const int b = sched[2 * blockIdx.x], k = sched[2 * blockIdx.x + 1];
   const BlkInfo bi = blk[b];
-  const T *__restrict__ L = buf + bi.base;
+  const double *__restrict__ L = buf + bi.base;
   const int r0 = k * NB, nr = min(NB, bi.a - r0), npiv = min(NB, bi.p - r0);
   for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
     const int r = i % NB, c = i / NB;
-    Ls[r][c] = (r < nr && c < npiv && r >= c) ? L[(long long)(r0 + c) * bi.lda + r0 + r] : T(0);
-    Xs[r][c] = T(0);
+    Ls[r][c] = (r < nr && c < npiv && r >= c) ? L[(long long)(r0 + c) * bi.lda + r0 + r] : 0.0;
+    Xs[r][c] = 0.0;
   }
   __syncthreads();
-  if (threadIdx.x < npiv) rinv[threadIdx.x] = T(1) / Ls[threadIdx.x][threadIdx.x];
+  if (threadIdx.x < npiv) rinv[threadIdx.x] = 1.0 / Ls[threadIdx.x][threadIdx.x];
   __syncthreads();
-  const int j = threadIdx.x;
-  if (j < npiv) {
-    for (int i = j; i < npiv; ++i) {
-      T s0 = (i == j) ? T(1) : T(0), s1 = T(0);
-      int q = j;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < 4 && lane < 16) {
+    const int b0 = w * 16, j = b0 + lane, e = min(b0 + 16, npiv);
+    for (int i = b0; i < e; ++i) {   // rows above the column's diagonal come out zero
+      double s0 = i == j ? 1.0 : 0.0, s1 = 0.0;
+      int q = b0;
       for (; q + 1 < i; q += 2) {
         s0 = fma(-Ls[i][q], Xs[q][j], s0);
         s1 = fma(-Ls[i][q + 1], Xs[q + 1][j], s1);
@@ -1381,7 +1478,27 @@ __global__ void __launch_bounds__(NB) tinv_kernel(const T *__restrict__ buf, T *
     }
   }
   __syncthreads();
-  T *__restrict__ out = tinv + bi.ioff + (long long)k * NB * NB;
+  for (int i0 = 16; i0 < npiv; i0 += 16) {
+    const int wc = i0;   // columns 0 .. i0 - 1 of this block row
+    for (int e = threadIdx.x; e < 16 * wc; e += blockDim.x) {
+      const int r = e / wc, c = e - r * wc;
+      double s0 = 0.0, s1 = 0.0;
+      for (int q = c & ~15; q < i0; q += 2) {
+        s0 = fma(Ls[i0 + r][q], Xs[q][c], s0);
+        s1 = fma(Ls[i0 + r][q + 1], Xs[q + 1][c], s1);
+      }
+      Tm[r * wc + c] = s0 + s1;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < 16 * wc; e += blockDim.x) {
+      const int r = e / wc, c = e - r * wc;
+      double s = 0.0;
+      for (int q = 0; q <= r; ++q) s = fma(Xs[i0 + r][i0 + q], Tm[q * wc + c], s);
+      if (i0 + r < npiv) Xs[i0 + r][c] = -s;
+    }
+    __syncthreads();
+  }
+  double *__restrict__ out = tinv + bi.ioff + (long long)k * NB * NB;
   for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
     const int r = i % NB, c = i / NB;
     out[i] = r < npiv ? Xs[r][c] : Ls[r][c];
@@ -1752,11 +1869,6 @@ constexpr size_t trsm_smem() {
 }
 
 template <typename T>
-constexpr size_t tinv_smem() {
-  return (2 * NB * (NB + 1) + NB) * sizeof(T);
-}
-
-template <typename T>
 cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkInfo> &h,
                     const double *diag0, double tol, int *status, cudaStream_t s,
                     ahlp_problem *tc = nullptr, ahlp_problem *prof = nullptr,
@@ -1784,8 +1896,8 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
                             buf, tinv, info, k, tc ? tc->pstage : nullptr);
     } else {
       if (prof) kt_mark(prof, 0, s);
-      count_launch(), pchol_potrf_kernel<T><<<nblk, kThreads, 0, s>>>(buf, info, k, diag0, tol,
-                                                                      status, drop);
+      count_launch(), pchol_potrf_kernel<<<nblk, kThreads, 0, s>>>(buf, info, k, diag0, tol,
+                                                                   status, drop);
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
         count_launch(), pchol_trsm_kernel<T><<<dim3((unsigned)maxPanel, nblk), kThreads,
@@ -1950,15 +2062,14 @@ cudaError_t launch_tinv(ahlp_problem *p) {
   // FP32 factors write their inverse tiles in pchol_potrf_f32_kernel; FP64 and
   // float-float factors (through their FP64 copy) get them here
   if (p->trsv_nb == 0 || p->fac_prec == kPrecFP32) return cudaSuccess;
-  count_launch(), tinv_kernel<double><<<p->trsv_nb, NB, tinv_smem<double>(), p->stream>>>(
+  count_launch(), tinv_kernel<<<p->trsv_nb, kThreads, kTinvSmem, p->stream>>>(
       p->aug, p->tinv, p->blk, p->trsv_bsched);
   return cudaGetLastError();
 }
 
 cudaError_t set_dense_smem_limits(int bytes) {
-  cudaError_t e = cudaFuncSetAttribute(tinv_kernel<double>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)tinv_smem<double>());
+  cudaError_t e = cudaFuncSetAttribute(tinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kTinvSmem);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(trsv_fwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)trsv_smem<float>());
