@@ -28,7 +28,7 @@ constexpr double kFFPivotTol = 1e-12;     // smallest clamp threshold for float-
 // storage words
 constexpr double kDropFP64 = 1e32, kDropFF = 1e16, kDropFP32 = 1e16;
 constexpr double kDropCapFF = 1e60, kDropCapFP32 = 1e30;
-constexpr long long kSmemVecBytes = 160 * 1024;   // dynamic smem of the border solves
+constexpr long long kSmemVecBytes = 160 * 1024;   // limit of the border order, 8 bytes each
 constexpr int kThreads = 256;     // threads per CTA of the dense kernels
 // FP64 factors on the tensor cores (k_dz.cu): digits per entry, and the row
 // exponent that marks a row holding a NaN or an infinity
@@ -317,6 +317,12 @@ struct ahlp_problem {
   ahlp::BlkInfo *bx_info = nullptr, *bp_info = nullptr;
   ahlp::BlkInfo h_bx{}, h_bp{};
   double *border_diag0 = nullptr;
+  // the border solves: W = L^-1 of the whole border factor (x_0 and y_g parts),
+  // row-major and column-major (ld Bld), from its inverted diagonal tiles
+  ahlp::BlkInfo *bw_info = nullptr;
+  int *bw_sched = nullptr;
+  double *border_tinv = nullptr, *border_wr = nullptr, *border_wc = nullptr;
+  double *border_t = nullptr;        // [B] J W b
 
   // ---- vectors ------------------------------------------------------------
   double *x = nullptr, *z = nullptr, *dscale = nullptr;   // current point, d = x/z
@@ -401,10 +407,9 @@ cudaError_t launch_pchol_f32(float *buf, float *tinv, const BlkInfo *info,
                              const std::vector<BlkInfo> &h, const double *diag0, double tol,
                              int *status, cudaStream_t s, ahlp_problem *tc = nullptr,
                              ahlp_problem *prof = nullptr, double drop = 0.0);
-// forward / backward solves with one partial factor per CTA (the border
-// factors; vectors FP64, held in shared memory)
-cudaError_t launch_ptri(const double *buf, const BlkInfo *info, int nblk, int amax, double *vec,
-                        bool forward, cudaStream_t s);
+// inverted 64 x 64 diagonal tiles of an FP64 factor: (problem, tile) jobs of sched
+cudaError_t launch_tile_inverses(const double *buf, double *tinv, const BlkInfo *info,
+                                 const int *sched, int njobs, cudaStream_t s);
 // inverted diagonal tiles of the current block factors (p->tinv / tinv32)
 cudaError_t launch_tinv(ahlp_problem *p);
 // forward / backward wavefront solves with all block factors (p->vec, in the

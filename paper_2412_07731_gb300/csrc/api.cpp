@@ -21,7 +21,7 @@
 using namespace ahlp;
 
 namespace ahlp {
-cudaError_t set_dense_smem_limits(int bytes);
+cudaError_t set_dense_smem_limits();
 cudaError_t set_schur_smem_limits(int bytes);
 cudaError_t set_bcr_smem_limits(int lmax);
 }
@@ -1268,6 +1268,18 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     p->bx_info = dupload(p, std::vector<BlkInfo>(1, p->h_bx));
     p->bp_info = dupload(p, std::vector<BlkInfo>(1, p->h_bp));
     p->border_diag0 = dalloc<double>(p, p->B);
+    if (p->B > 0) {
+      const int T = (p->B + NB - 1) / NB;
+      p->bw_info = dupload(p, std::vector<BlkInfo>(
+                                  1, BlkInfo{0, 0, 0, p->Bld, p->B, p->B, T, T, 0, 0, 0, 0}));
+      std::vector<int> sched;
+      for (int k = 0; k < T; ++k) sched.insert(sched.end(), {0, k});
+      p->bw_sched = dupload(p, sched);
+      p->border_tinv = dalloc<double>(p, (long long)T * NB * NB);
+      p->border_wr = dalloc<double>(p, (long long)p->Bld * p->B);
+      p->border_wc = dalloc<double>(p, (long long)p->Bld * p->B);
+      p->border_t = dalloc<double>(p, p->B);
+    }
     p->x = dalloc<double>(p, p->n);
     p->z = dalloc<double>(p, p->n);
     p->dscale = dalloc<double>(p, p->n);
@@ -1291,7 +1303,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     p->status = dalloc<int>(p, 8);
     ck(cudaMallocHost(&p->h_scal, 512 * sizeof(double)), "cudaMallocHost");
     for (auto &e : p->ev) ck(cudaEventCreate(&e), "cudaEventCreate");
-    ck(set_dense_smem_limits((int)kSmemVecBytes), "smem limit");
+    ck(set_dense_smem_limits(), "smem limit");
     ck(set_schur_smem_limits(128 * 128 * 8), "smem limit");
     ck(cudaDeviceSynchronize(), "create sync");
   } catch (const Fail &f) {

@@ -260,82 +260,97 @@ __global__ void __launch_bounds__(kBcrThreads) bcr_z_kernel(BArgs A) {
   }
 }
 
-// forward solve of one level, in place on the link part of u (one warp per
-// row group, one CTA per pair): u_j = Linv_j (r_j - earlier-level terms)
-__global__ void __launch_bounds__(kBcrThreads) bcr_fwd_kernel(BArgs A, double *u) {
+// The two solve kernels work on a few thousand multiply-adds per pair, so they
+// are bound by latency: a thread that walks a dot product alone pays the load
+// and the FP64 latency of every term in turn (13.5 us per level with a thread
+// per row).  Eight lanes share a row instead, each taking every eighth entry of
+// every term; the terms' loads are independent of each other and run ahead of
+// the multiply-adds, and a row ends in three shuffles.
+constexpr int kBcrLanes = 8;
+constexpr int kBcrSolveThreads = 256;   // 32 rows at a time
+
+__device__ __forceinline__ double bcr_lanes_sum(double v) {
+#pragma unroll
+  for (int o = kBcrLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// s += sum_q G[q] z[q], q = lane, lane + 8, ... < k
+__device__ __forceinline__ void bcr_dot(const double *__restrict__ G, const double *z, int k,
+                                        int stride, int q0, double &s) {
+#pragma unroll 4
+  for (int q = q0; q < k; q += kBcrLanes) s = fma(G[(long long)q * stride], z[q], s);
+}
+
+// forward solve of one level, in place on the link part of u, one CTA per
+// pair: u_j = Linv_j (r_j - earlier-level terms)
+__global__ void __launch_bounds__(kBcrSolveThreads) bcr_fwd_kernel(BArgs A, double *u) {
   const int j = A.order[blockIdx.x];
   int lv, jb, je;
   pair_info(A, j, lv, jb, je);
   const int lj = A.l[j], lm = A.lmax;
+  const long long off = A.link_off[j];
   __shared__ double r[96];
-  const int tid = threadIdx.x;
-  for (int i = tid; i < lj; i += blockDim.x) {
-    double v = u[A.link_off[j] + i];
-    for (int w = 0; w < lv; ++w) {
-      const int ml = j - (1 << w), mr = j + (1 << w);
-      if (ml >= jb) {
-        const double *G = A.GR + (long long)ml * lm * lm;
-        const int k = A.l[ml];
-        const double *z = u + A.link_off[ml];
-        for (int q = 0; q < k; ++q) v = fma(-G[q + (long long)i * k], z[q], v);
-      }
-      if (mr < je) {
-        const double *G = A.GL + (long long)mr * lm * lm;
-        const int k = A.l[mr];
-        const double *z = u + A.link_off[mr];
-        for (int q = 0; q < k; ++q) v = fma(-G[q + (long long)i * k], z[q], v);
+  const int lane = threadIdx.x & (kBcrLanes - 1), row0 = threadIdx.x / kBcrLanes;
+  constexpr int rows = kBcrSolveThreads / kBcrLanes;
+  for (int i0 = 0; i0 < lj; i0 += rows) {
+    const int i = i0 + row0;
+    double s = 0.0;
+    if (i < lj) {
+      for (int w = 0; w < lv; ++w) {
+        const int ml = j - (1 << w), mr = j + (1 << w);
+        const int kl = ml >= jb ? A.l[ml] : 0, kr = mr < je ? A.l[mr] : 0;
+        const long long ol = ml >= jb ? A.link_off[ml] : 0, orr = mr < je ? A.link_off[mr] : 0;
+        bcr_dot(A.GR + (long long)ml * lm * lm + (long long)i * kl, u + ol, kl, 1, lane, s);
+        bcr_dot(A.GL + (long long)mr * lm * lm + (long long)i * kr, u + orr, kr, 1, lane, s);
       }
     }
-    r[i] = v;
+    s = bcr_lanes_sum(s);
+    if (lane == 0 && i < lj) r[i] = u[off + i] - s;
   }
   __syncthreads();
   const double *Li = A.Linv + A.td_off[j];
-  for (int i = tid; i < lj; i += blockDim.x) {
-    double a0 = 0.0, a1 = 0.0;
-    int q = 0;
-    for (; q + 1 <= i; q += 2) {
-      a0 = fma(Li[i + q * lj], r[q], a0);
-      a1 = fma(Li[i + (q + 1) * lj], r[q + 1], a1);
-    }
-    if (q <= i) a0 = fma(Li[i + q * lj], r[q], a0);
-    u[A.link_off[j] + i] = a0 + a1;
+  for (int i0 = 0; i0 < lj; i0 += rows) {
+    const int i = i0 + row0;
+    double s = 0.0;
+    if (i < lj) bcr_dot(Li + i, r, i + 1, lj, lane, s);
+    s = bcr_lanes_sum(s);
+    if (lane == 0 && i < lj) u[off + i] = s;
   }
 }
 
 // backward solve of one level: x_j = Linv_j' (u_j - GL_j x_a - GR_j x_b)
-__global__ void __launch_bounds__(kBcrThreads) bcr_bwd_kernel(BArgs A, double *u) {
+__global__ void __launch_bounds__(kBcrSolveThreads) bcr_bwd_kernel(BArgs A, double *u) {
   const int j = A.order[blockIdx.x];
   int lv, jb, je;
   pair_info(A, j, lv, jb, je);
   const int lj = A.l[j], lm = A.lmax;
+  const long long off = A.link_off[j];
   __shared__ double r[96];
-  const int tid = threadIdx.x;
+  const int lane = threadIdx.x & (kBcrLanes - 1), row0 = threadIdx.x / kBcrLanes;
+  constexpr int rows = kBcrSolveThreads / kBcrLanes;
   const int a = j - (1 << lv), b = j + (1 << lv);
-  for (int i = tid; i < lj; i += blockDim.x) {
-    double v = u[A.link_off[j] + i];
-    if (a >= jb) {
-      const double *G = A.GL + (long long)j * lm * lm;   // l_j x l_a
-      const double *x = u + A.link_off[a];
-      for (int q = 0; q < A.l[a]; ++q) v = fma(-G[i + (long long)q * lj], x[q], v);
+  const int ka = a >= jb ? A.l[a] : 0, kb = b < je ? A.l[b] : 0;
+  const long long oa = a >= jb ? A.link_off[a] : 0, ob = b < je ? A.link_off[b] : 0;
+  for (int i0 = 0; i0 < lj; i0 += rows) {
+    const int i = i0 + row0;
+    double s = 0.0;
+    if (i < lj) {
+      bcr_dot(A.GL + (long long)j * lm * lm + i, u + oa, ka, lj, lane, s);   // l_j x l_a
+      bcr_dot(A.GR + (long long)j * lm * lm + i, u + ob, kb, lj, lane, s);   // l_j x l_b
     }
-    if (b < je) {
-      const double *G = A.GR + (long long)j * lm * lm;   // l_j x l_b
-      const double *x = u + A.link_off[b];
-      for (int q = 0; q < A.l[b]; ++q) v = fma(-G[i + (long long)q * lj], x[q], v);
-    }
-    r[i] = v;
+    s = bcr_lanes_sum(s);
+    if (lane == 0 && i < lj) r[i] = u[off + i] - s;
   }
   __syncthreads();
   const double *Li = A.Linv + A.td_off[j];
-  for (int i = tid; i < lj; i += blockDim.x) {
-    double a0 = 0.0, a1 = 0.0;
-    int q = i;
-    for (; q + 1 < lj; q += 2) {
-      a0 = fma(Li[q + i * lj], r[q], a0);
-      a1 = fma(Li[q + 1 + i * lj], r[q + 1], a1);
-    }
-    if (q < lj) a0 = fma(Li[q + i * lj], r[q], a0);
-    u[A.link_off[j] + i] = a0 + a1;
+  for (int i0 = 0; i0 < lj; i0 += rows) {
+    const int i = i0 + row0;
+    double s = 0.0;
+    // entries i .. lj - 1 of column i
+    if (i < lj) bcr_dot(Li + (long long)i * lj + i, r + i, lj - i, 1, lane, s);
+    s = bcr_lanes_sum(s);
+    if (lane == 0 && i < lj) u[off + i] = s;
   }
 }
 
@@ -390,9 +405,9 @@ cudaError_t launch_bcr_solve(ahlp_problem *p, double *u, bool forward) {
     BArgs A = bargs(p);
     A.order = p->bcr_order + p->bcr_loff[v];
     if (forward)
-      count_launch(), bcr_fwd_kernel<<<n, kBcrThreads, 0, s>>>(A, u);
+      count_launch(), bcr_fwd_kernel<<<n, kBcrSolveThreads, 0, s>>>(A, u);
     else
-      count_launch(), bcr_bwd_kernel<<<n, kBcrThreads, 0, s>>>(A, u);
+      count_launch(), bcr_bwd_kernel<<<n, kBcrSolveThreads, 0, s>>>(A, u);
   }
   return cudaGetLastError();
 }

@@ -1246,143 +1246,6 @@ __global__ void __launch_bounds__(kUpdFFThreads) pchol_update_ff8_kernel(float *
 }
 
 // --------------------------------------------------------------------------
-// solves with the partial factor (one CTA per problem, vector in smem)
-// forward : v <- [L11 0; L21 I]^-1 v
-// backward: v_top <- L11^-T (v_top - L21' v_bottom), v_bottom unchanged
-// The arithmetic runs in the factor's precision; the vector in global memory
-// is FP64 either way.  Per 64-column step the diagonal tile and its
-// reciprocal pivots are staged in shared memory (the sequential part runs
-// there), and the panel below it is streamed with eight independent loads
-// per thread in flight so the step is bandwidth-, not latency-bound.
-// --------------------------------------------------------------------------
-constexpr int kSolveThreads = 1024;
-
-template <typename T>
-__device__ __forceinline__ void stage_diag_tile(const T *L, long long lda, int c0, int nr,
-                                                int npiv, T (*dt)[NB + 1], T *dinv) {
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
-    const int r = i % NB, c = i / NB;
-    if (r < nr && c < npiv) dt[r][c] = L[(long long)(c0 + c) * lda + c0 + r];
-  }
-  for (int c = threadIdx.x; c < npiv; c += blockDim.x)
-    dinv[c] = T(1) / L[(long long)(c0 + c) * lda + c0 + c];
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kSolveThreads) ptri_fwd_kernel(const T *__restrict__ buf,
-                                                                 const BlkInfo *blk,
-                                                                 double *vec) {
-  extern __shared__ __align__(16) unsigned char vraw[];
-  __shared__ T dt[NB][NB + 1];   // diagonal tile, dt[r][c]
-  __shared__ T dinv[NB];
-  T *v = reinterpret_cast<T *>(vraw);
-  const BlkInfo bi = blk[blockIdx.x];
-  double *gv = vec + bi.voff;
-  const T *__restrict__ L = buf + bi.base;
-  const int a = bi.a;
-  const long long lda = bi.lda;
-  for (int i = threadIdx.x; i < a; i += blockDim.x) v[i] = (T)gv[i];
-  for (int kt = 0; kt < bi.Tp; ++kt) {
-    const int c0 = kt * NB;
-    const int npiv = min(NB, bi.p - c0);
-    const int rend = min(c0 + NB, a);
-    const int nr = rend - c0;
-    stage_diag_tile(L, lda, c0, nr, npiv, dt, dinv);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
-      for (int c = 0; c < npiv; ++c) {
-        const T vc = v[c0 + c] * dinv[c];
-        __syncwarp();
-        if (lane == 0) v[c0 + c] = vc;
-        for (int r = c + 1 + lane; r < nr; r += 32) v[c0 + r] -= dt[r][c] * vc;
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    const T *__restrict__ P = L + (long long)c0 * lda;   // panel columns c0..c0+npiv
-    for (int r = rend + threadIdx.x; r < a; r += blockDim.x) {
-      T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
-      int c = 0;
-      for (; c + 8 <= npiv; c += 8) {
-        const T l0 = P[(long long)(c + 0) * lda + r], l1 = P[(long long)(c + 1) * lda + r];
-        const T l2 = P[(long long)(c + 2) * lda + r], l3 = P[(long long)(c + 3) * lda + r];
-        const T l4 = P[(long long)(c + 4) * lda + r], l5 = P[(long long)(c + 5) * lda + r];
-        const T l6 = P[(long long)(c + 6) * lda + r], l7 = P[(long long)(c + 7) * lda + r];
-        s0 = fma(l0, v[c0 + c + 0], s0);
-        s1 = fma(l1, v[c0 + c + 1], s1);
-        s2 = fma(l2, v[c0 + c + 2], s2);
-        s3 = fma(l3, v[c0 + c + 3], s3);
-        s0 = fma(l4, v[c0 + c + 4], s0);
-        s1 = fma(l5, v[c0 + c + 5], s1);
-        s2 = fma(l6, v[c0 + c + 6], s2);
-        s3 = fma(l7, v[c0 + c + 7], s3);
-      }
-      for (; c < npiv; ++c) s0 = fma(P[(long long)c * lda + r], v[c0 + c], s0);
-      v[r] -= (s0 + s1) + (s2 + s3);
-    }
-    __syncthreads();
-  }
-  for (int i = threadIdx.x; i < a; i += blockDim.x) gv[i] = (double)v[i];
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kSolveThreads) ptri_bwd_kernel(const T *__restrict__ buf,
-                                                                 const BlkInfo *blk,
-                                                                 double *vec) {
-  extern __shared__ __align__(16) unsigned char vraw[];
-  __shared__ T dt[NB][NB + 1];   // diagonal tile, dt[r][c]
-  __shared__ T dinv[NB];
-  T *v = reinterpret_cast<T *>(vraw);
-  const BlkInfo bi = blk[blockIdx.x];
-  double *gv = vec + bi.voff;
-  const T *__restrict__ L = buf + bi.base;
-  const int a = bi.a;
-  const long long lda = bi.lda;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  for (int i = threadIdx.x; i < a; i += blockDim.x) v[i] = (T)gv[i];
-  __syncthreads();
-  for (int kt = bi.Tp - 1; kt >= 0; --kt) {
-    const int c0 = kt * NB;
-    const int npiv = min(NB, bi.p - c0);
-    const int rend = min(c0 + NB, a);
-    const int nr = rend - c0;
-    stage_diag_tile(L, lda, c0, nr, npiv, dt, dinv);
-    // v[c] -= L(rend:a, c)' v(rend:a): one warp per column, lanes over rows
-    for (int cc = warp; cc < npiv; cc += nwarp) {
-      const T *__restrict__ col = L + (long long)(c0 + cc) * lda;
-      T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
-      int r = rend + lane;
-      for (; r + 96 < a; r += 128) {
-        const T l0 = col[r], l1 = col[r + 32], l2 = col[r + 64], l3 = col[r + 96];
-        s0 = fma(l0, v[r], s0);
-        s1 = fma(l1, v[r + 32], s1);
-        s2 = fma(l2, v[r + 64], s2);
-        s3 = fma(l3, v[r + 96], s3);
-      }
-      for (; r < a; r += 32) s0 = fma(col[r], v[r], s0);
-      T s = (s0 + s1) + (s2 + s3);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      if (lane == 0) v[c0 + cc] -= s;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      for (int c = npiv - 1; c >= 0; --c) {
-        T s = T(0);
-        for (int r = c + 1 + lane; r < nr; r += 32) s = fma(dt[r][c], v[c0 + r], s);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) v[c0 + c] = (v[c0 + c] - s) * dinv[c];
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-  }
-  for (int i = threadIdx.x; i < a; i += blockDim.x) gv[i] = (double)v[i];
-}
-
-// --------------------------------------------------------------------------
 // Wavefront solves with the block partial factors: one CTA per (block, 64-row
 // tile), so every block's factor is streamed by many SMs at once.
 //
@@ -2016,17 +1879,6 @@ cudaError_t launch_pchol_f32(float *buf, float *tinv, const BlkInfo *info,
   return pchol_t<float>(buf, tinv, info, h, diag0, tol, status, s, tc, prof, drop);
 }
 
-cudaError_t launch_ptri(const double *buf, const BlkInfo *info, int nblk, int amax, double *vec,
-                        bool forward, cudaStream_t s) {
-  if (nblk == 0 || amax == 0) return cudaSuccess;
-  size_t sm = (size_t)amax * sizeof(double);
-  if (forward)
-    count_launch(), ptri_fwd_kernel<double><<<nblk, kSolveThreads, sm, s>>>(buf, info, vec);
-  else
-    count_launch(), ptri_bwd_kernel<double><<<nblk, kSolveThreads, sm, s>>>(buf, info, vec);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_trsv(ahlp_problem *p, bool forward) {
   const int njobs = forward ? p->trsv_nf : p->trsv_nb;
   if (njobs == 0) return cudaSuccess;
@@ -2067,7 +1919,14 @@ cudaError_t launch_tinv(ahlp_problem *p) {
   return cudaGetLastError();
 }
 
-cudaError_t set_dense_smem_limits(int bytes) {
+cudaError_t launch_tile_inverses(const double *buf, double *tinv, const BlkInfo *info,
+                                 const int *sched, int njobs, cudaStream_t s) {
+  if (njobs > 0)
+    count_launch(), tinv_kernel<<<njobs, kThreads, kTinvSmem, s>>>(buf, tinv, info, sched);
+  return cudaGetLastError();
+}
+
+cudaError_t set_dense_smem_limits() {
   cudaError_t e = cudaFuncSetAttribute(tinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kTinvSmem);
   if (e != cudaSuccess) return e;
@@ -2093,11 +1952,6 @@ cudaError_t set_dense_smem_limits(int bytes) {
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)trsm_smem<double>());
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(ptri_fwd_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(ptri_bwd_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           bytes);
   return e;
 }
 

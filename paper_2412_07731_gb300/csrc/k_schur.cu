@@ -817,31 +817,136 @@ __global__ void __launch_bounds__(kChainSolveThreads) chain_solve_kernel(CArgs A
   }
 }
 
-// border rhs: sB -= Z' uT      (one warp per border row, lanes over link rows)
-__global__ void border_rhs_kernel(const double *Z, int B, int nl, double *svec) {
-  const int rb = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (rb >= B) return;
-  const double *zc = Z + (long long)rb * nl;
-  double acc = 0.0;
-  for (int q = lane; q < nl; q += 32) acc = fma(zc[q], svec[q], acc);
+// The border solves.  With L the factor of the border (x_0 pivots first, then
+// y_g) and J = diag(-I, I), the border system's solution is L^-T J L^-1 b.
+// Substitution is a chain of 64-column steps on one SM (35 + 71 us per solve
+// of order 100, 126 + 223 us of order 601); the explicit W = L^-1, formed once
+// per factor, makes a solve two matrix-vector products over many SMs.  W's
+// rows are independent of each other: row r solves w L = e_r' from its own
+// 64-column tile leftwards, tile j as v = e_r' - (w L)_j over the columns
+// already done, w_j = v X_jj with the inverted diagonal tile X_jj.  A CTA takes
+// two rows, so the columns of L it streams serve both.
+constexpr int kBinvThreads = 256;
+
+__global__ void __launch_bounds__(kBinvThreads) border_inv_kernel(const double *__restrict__ L,
+                                                                  const double *__restrict__ X,
+                                                                  int B, int ld, double *Wr,
+                                                                  double *Wc) {
+  __shared__ double xs[NB][NB + 1];   // xs[c][q] = X_jj(q, c)
+  __shared__ double v[2][NB];
+  const int r0 = 2 * blockIdx.x, r1 = min(r0 + 1, B - 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double *w0 = Wr + (long long)r0 * ld, *w1 = Wr + (long long)r1 * ld;
+  const int ti = r0 / NB;
+  for (int j = ti; j >= 0; --j) {
+    const int c0 = j * NB;
+    for (int i = threadIdx.x; i < NB * NB; i += kBinvThreads)
+      xs[i / NB][i % NB] = X[(long long)j * NB * NB + i];
+    for (int c = warp; c < NB; c += kBinvThreads / 32) {
+      double s0 = 0.0, s1 = 0.0;
+      if (c0 + c < B && j < ti) {
+        const double *col = L + (long long)(c0 + c) * ld;
+        for (int q = c0 + NB + lane; q <= r1; q += 32) {   // row r0 is zero at q = r1
+          const double l = col[q];
+          s0 = fma(w0[q], l, s0);
+          s1 = fma(w1[q], l, s1);
+        }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if (lane == 0) svec[nl + rb] -= acc;
+        for (int o = 16; o > 0; o >>= 1) {
+          s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        }
+      }
+      if (lane == 0) {
+        v[0][c] = (c0 + c == r0 ? 1.0 : 0.0) - s0;
+        v[1][c] = (c0 + c == r1 ? 1.0 : 0.0) - s1;
+      }
+    }
+    __syncthreads();
+    // thread (row a, column c, half h of the sum over q >= c)
+    const int a = threadIdx.x >> 7, c = (threadIdx.x >> 1) & (NB - 1), h = threadIdx.x & 1;
+    double s = 0.0;
+    for (int q = c + h; q < NB; q += 2) s = fma(v[a][q], xs[c][q], s);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if (h == 0 && c0 + c < B) {
+      (a ? w1 : w0)[c0 + c] = s;
+      Wc[(long long)(c0 + c) * ld + (a ? r1 : r0)] = s;
+    }
+    __syncthreads();
+  }
 }
 
-// uT -= Z sB      (one thread per link row)
-__global__ void link_back_kernel(const double *Z, int B, int nl, double *svec) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nl) return;
-  double acc = 0.0;
-  for (int rb = 0; rb < B; ++rb) acc = fma(Z[(long long)rb * nl + q], svec[nl + rb], acc);
-  svec[q] -= acc;
+// border rhs: sB -= Z' uT, one CTA per border row over its column's link rows
+__global__ void __launch_bounds__(128) border_rhs_kernel(const double *__restrict__ Z, int nl,
+                                                         const int *zlo, const int *zhi,
+                                                         double *svec) {
+  __shared__ double part[4];
+  const int rb = blockIdx.x;
+  const double *zc = Z + (long long)rb * nl;
+  const int q1 = zhi[rb];
+  double s0 = 0.0, s1 = 0.0;
+  int q = zlo[rb] + threadIdx.x;
+#pragma unroll 4
+  for (; q + 128 < q1; q += 256) {
+    s0 = fma(zc[q], svec[q], s0);
+    s1 = fma(zc[q + 128], svec[q + 128], s1);
+  }
+  if (q < q1) s0 = fma(zc[q], svec[q], s0);
+  double acc = s0 + s1;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) svec[nl + rb] -= (part[0] + part[1]) + (part[2] + part[3]);
 }
 
-__global__ void scale_kernel(double *v, double a, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] *= a;
+// t = J W b (fwd, W's rows) or x = W' t (columns), one warp per entry
+__global__ void __launch_bounds__(256) border_w_kernel(const double *__restrict__ W, int B, int ld,
+                                                       int n0, const double *__restrict__ in,
+                                                       double *out, int fwd) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= B) return;
+  const double *w = W + (long long)i * ld;
+  const int q1 = fwd ? i + 1 : B;
+  double s0 = 0.0, s1 = 0.0;
+  int q = (fwd ? 0 : i) + lane;
+#pragma unroll 4
+  for (; q + 32 < q1; q += 64) {
+    s0 = fma(w[q], in[q], s0);
+    s1 = fma(w[q + 32], in[q + 32], s1);
+  }
+  if (q < q1) s0 = fma(w[q], in[q], s0);
+  double s = s0 + s1;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[i] = fwd && i < n0 ? -s : s;
+}
+
+// uT -= Z sB: a CTA takes 32 link rows, 16 threads per row share the border
+// columns (one thread per row walked all of them: 28 us at 100, 156 us at 601)
+__global__ void __launch_bounds__(512) link_back_kernel(const double *__restrict__ Z, int B,
+                                                        int nl, double *svec) {
+  __shared__ double part[16][32];
+  const int rr = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int q = blockIdx.x * 32 + rr;
+  double s0 = 0.0, s1 = 0.0;
+  if (q < nl) {
+    int rb = g;
+#pragma unroll 4
+    for (; rb + 16 < B; rb += 32) {
+      s0 = fma(Z[(long long)rb * nl + q], svec[nl + rb], s0);
+      s1 = fma(Z[(long long)(rb + 16) * nl + q], svec[nl + rb + 16], s1);
+    }
+    if (rb < B) s0 = fma(Z[(long long)rb * nl + q], svec[nl + rb], s0);
+  }
+  part[g][rr] = s0 + s1;
+  __syncthreads();
+  if (g == 0 && q < nl) {
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) s += part[i][rr];
+    svec[q] -= s;
+  }
 }
 
 __global__ void gather_schur_kernel(const BlkInfo *blk, const SchurBlk *sb, const int *kmap,
@@ -979,6 +1084,11 @@ cudaError_t launch_schur_factor(ahlp_problem *p) {
                                    p->status, s);
       if (e != cudaSuccess) return e;
     }
+    const int T = (p->B + NB - 1) / NB;
+    cudaError_t e = launch_tile_inverses(p->border, p->border_tinv, p->bw_info, p->bw_sched, T, s);
+    if (e != cudaSuccess) return e;
+    count_launch(), border_inv_kernel<<<(p->B + 1) / 2, kBinvThreads, 0, s>>>(
+        p->border, p->border_tinv, p->B, p->Bld, p->border_wr, p->border_wc);
   }
   return cudaGetLastError();
 }
@@ -1025,24 +1135,17 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
       }
     }
     if (p->B > 0) {
-      if (p->nl > 0) count_launch(), border_rhs_kernel<<<nb((long long)p->B * 32, 256), 256, 0, s>>>(p->Et, p->B, p->nl, p->svec);
+      if (p->nl > 0)
+        count_launch(), border_rhs_kernel<<<p->B, 128, 0, s>>>(p->Et, p->nl, p->zlo, p->zhi,
+                                                               p->svec);
       double *sb = p->svec + p->nl;
-      if (p->n0 > 0) {
-        e = launch_ptri(p->border, p->bx_info, 1, p->B, sb, true, s);
-        if (e != cudaSuccess) return e;
-        count_launch(), scale_kernel<<<nb(p->n0, 256), 256, 0, s>>>(sb, -1.0, p->n0);
-      }
-      if (p->mg > 0) {
-        e = launch_ptri(p->border, p->bp_info, 1, p->B, sb, true, s);
-        if (e != cudaSuccess) return e;
-        e = launch_ptri(p->border, p->bp_info, 1, p->B, sb, false, s);
-        if (e != cudaSuccess) return e;
-      }
-      if (p->n0 > 0) {
-        e = launch_ptri(p->border, p->bx_info, 1, p->B, sb, false, s);
-        if (e != cudaSuccess) return e;
-      }
-      if (p->nl > 0) count_launch(), link_back_kernel<<<nb(p->nl, 128), 128, 0, s>>>(p->Et, p->B, p->nl, p->svec);
+      count_launch(), border_w_kernel<<<nb(p->B, 8), 256, 0, s>>>(p->border_wr, p->B, p->Bld,
+                                                                  p->n0, sb, p->border_t, 1);
+      count_launch(), border_w_kernel<<<nb(p->B, 8), 256, 0, s>>>(p->border_wc, p->B, p->Bld,
+                                                                  p->n0, p->border_t, sb, 0);
+      if (p->nl > 0)
+        count_launch(), link_back_kernel<<<nb(p->nl, 32), 512, 0, s>>>(p->Et, p->B, p->nl,
+                                                                       p->svec);
     }
     if (p->nl > 0 && lmax > 0 && p->nchain_seg > 0) {
       if (p->fac_bcr) {
