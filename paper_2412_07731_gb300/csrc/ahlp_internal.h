@@ -336,6 +336,7 @@ struct ahlp_problem {
   double *cor[3] = {nullptr, nullptr, nullptr};            // refinement correction
   double *ipmv[19] = {};      // IPM work vectors (the last three: a batch's balanced rhs)
   double *red_part = nullptr; // reduction partials
+  int *red_cnt = nullptr;     // arrivals at the reductions' last CTAs (0 between launches)
   double *mdot_part = nullptr;  // multi-dot partials [kMaxKrylov+1][304]
   double *gm_V = nullptr, *gm_Z = nullptr;   // Krylov bases, allocated on first use
   double *gm_coef = nullptr;    // device coefficients for multi-axpy
@@ -348,7 +349,9 @@ struct ahlp_problem {
   // flag per tile, then the forward and backward ticket counters
   int *trsv_fsched = nullptr, *trsv_bsched = nullptr;   // [2 * jobs]
   int *trsv_flag_off = nullptr;   // [N] first flag of each block
-  int *trsv_flags = nullptr;      // [trsv_nflags + 2]
+  // ready flags of the forward, then of the backward solve, and the two tickets
+  // (all zeroed by the first kernel of a solve)
+  int *trsv_flags = nullptr;      // [2 trsv_nflags + 2]
   int *trsv_err = nullptr;        // set when a wait timed out
   int trsv_nf = 0, trsv_nb = 0, trsv_nflags = 0;
   int tiny_pivots = 0;
@@ -412,9 +415,10 @@ cudaError_t launch_tile_inverses(const double *buf, double *tinv, const BlkInfo 
                                  const int *sched, int njobs, cudaStream_t s);
 // inverted diagonal tiles of the current block factors (p->tinv / tinv32)
 cudaError_t launch_tinv(ahlp_problem *p);
-// forward / backward wavefront solves with all block factors (p->vec, in the
-// precision of the current factor); wait timeouts set p->trsv_err
-cudaError_t launch_trsv(ahlp_problem *p, bool forward);
+// forward wavefront solve of rhs (ordered like y) with all block factors into
+// p->vec, or the backward one from p->vec and the Schur solution p->svec, which
+// also writes dy; wait timeouts set p->trsv_err
+cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double *dy);
 cudaError_t launch_schur_assemble(ahlp_problem *p, double delta, double rho);
 cudaError_t launch_schur_factor(ahlp_problem *p);
 // cyclic reduction of the link chain: factor (T_j, Linv_j, GL_j, GR_j, and Z
@@ -422,14 +426,27 @@ cudaError_t launch_schur_factor(ahlp_problem *p);
 cudaError_t launch_bcr_factor(ahlp_problem *p);
 cudaError_t launch_bcr_solve(ahlp_problem *p, double *u, bool forward);
 cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
-                         const double *r_c, double *dx, double *dy, double *dz, bool adjoint);
+                         const double *r_c, double *dx, double *dy, double *dz, bool adjoint,
+                         double *wx = nullptr, double *wc = nullptr);
 cudaError_t launch_residual(ahlp_problem *p, const double *r_d, const double *r_p,
                             const double *r_c, const double *dx, const double *dy,
                             const double *dz, double *e_d, double *e_p, double *e_c,
                             bool adjoint);
 
 // ---- vector utilities ------------------------------------------------------
-enum RedOp { RED_DOT = 0, RED_MAXABS = 1, RED_MINSTEP = 2, RED_MIN = 3, RED_SUM = 4 };
+enum RedOp { RED_DOT = 0, RED_MAXABS = 1, RED_MINSTEP = 2, RED_MIN = 3, RED_SUM = 4, RED_STEP = 5 };
+// one reduction of a set: out <- reduce(op, a, b [, c, d, s1, s2]) over len entries
+struct RedOne {
+  int op;
+  const double *a, *b;
+  long long len;
+  double *out;
+  const double *c = nullptr, *d = nullptr;
+  double s1 = 0.0, s2 = 0.0;
+};
+constexpr int kRedSetMax = 12;   // reductions per launch
+constexpr int kMdotParts = 608;  // CTAs of a multi-dot, at most
+cudaError_t launch_reduce_set(ahlp_problem *p, const RedOne *ops, int n);
 // out <- reduce(op, a, b) over len entries, deterministic order; out is a
 // device scalar.
 cudaError_t launch_reduce(ahlp_problem *p, int op, const double *a, const double *b,
@@ -448,15 +465,21 @@ constexpr int kMaxKrylov = 64;   // cap on GMRES iterations per solve
 // out[i] = <V_i, w>, i < k (V_i = V + i*ld), deterministic
 cudaError_t launch_mdot(ahlp_problem *p, const double *V, long long ld, int k, const double *w,
                         long long len, double *out);
-// w += sum_i coef[i] V_i   (coef in device memory)
-// w += sign * sum_i coef[i] V_i (coef on the device, fixed order over i)
-cudaError_t launch_maxpy(const double *V, long long ld, int k, const double *coef, double *w,
-                         long long len, cudaStream_t s, double sign = 1.0);
-// w *= 1 / sqrt(*nrm2) when *nrm2 > 0, nrm2 a device scalar
-cudaError_t launch_scale_inv_norm(double *w, long long len, const double *nrm2, cudaStream_t s);
-// o = J v (Newton matrix of Sec. 2.3) or J' v
-cudaError_t launch_jmul(ahlp_problem *p, const double *vx, const double *vy, const double *vz,
-                        double *ox, double *oy, double *oz, bool adjoint);
+// w += sign * sum_i coef[i] V_i (coef on the device, fixed order over i); with
+// nrm2 also nrm2[0] = <w, w> and nrm2[1] = 1 / |w| (1 when <w, w> is not positive)
+cudaError_t launch_maxpy(ahlp_problem *p, const double *V, long long ld, int k, const double *coef,
+                         double *w, long long len, double sign = 1.0, double *nrm2 = nullptr);
+// the same for w in three pieces of lengths n0, n1 and len - n0 - n1
+cudaError_t launch_maxpy3(ahlp_problem *p, const double *V, long long ld, int k,
+                          const double *coef, double *w0, long long n0, double *w1, long long n1,
+                          double *w2, long long len, double sign = 1.0, double *nrm2 = nullptr);
+// y = a x, the factor on the device when da is not null
+cudaError_t launch_scale(double *y, const double *x, const double *da, double a, long long len,
+                         cudaStream_t s);
+// dx, dz of a direction from dy (and the right-hand side's f, r_c); with wx, wc
+// also the first and third parts of J (dx, dy, dz) (adjoint: J')
+cudaError_t launch_finish(ahlp_problem *p, const double *dy, const double *rc, double *dx,
+                          double *dz, bool adjoint, double *wx, double *wc);
 cudaError_t launch_mul(double *y, const double *a, const double *b, double scale, long long n,
                        cudaStream_t s);   // y = scale * a .* b
 // centrality corrector right-hand side: rc2 = rc + t, where v = (x + ap dx) .* (z + ad dz)
@@ -464,9 +487,9 @@ cudaError_t launch_mul(double *y, const double *a, const double *b, double scale
 cudaError_t launch_centrality_rc(double *rc2, const double *rc, const double *x,
                                  const double *dx, double ap, const double *z, const double *dz,
                                  double ad, double lo, double hi, long long n, cudaStream_t s);
-cudaError_t launch_step_dot(const double *x, const double *dx, double ap, const double *z,
-                            const double *dz, double ad, long long n, double *part,
-                            double *out, cudaStream_t s);  // (x+ap dx)'(z+ad dz)
+cudaError_t launch_step_dot(ahlp_problem *p, const double *x, const double *dx, double ap,
+                            const double *z, const double *dz, double ad, long long n,
+                            double *out);  // (x+ap dx)'(z+ad dz)
 
 // ---- tensor-core trailing update (k_tc.cu) -----------------------------------
 // staging, job offsets and tensor maps for the FP32 factors (needs aug32);

@@ -1152,7 +1152,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
       if (!fs.empty()) p->trsv_fsched = dupload(p, fs);
       if (!bs.empty()) p->trsv_bsched = dupload(p, bs);
       if (N > 0) p->trsv_flag_off = dupload(p, foff);
-      p->trsv_flags = dalloc<int>(p, nflags + 2);
+      p->trsv_flags = dalloc<int>(p, 2 * nflags + 2);
       p->trsv_err = dalloc<int>(p, 1);
       ck(cudaMemset(p->trsv_err, 0, sizeof(int)), "memset");
     }
@@ -1292,13 +1292,17 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     p->rhat = dalloc<double>(p, p->m);
     const long long mx = std::max(p->n, p->m);
     for (auto &s : p->stg) s = dalloc<double>(p, mx);
-    for (auto &s : p->res) s = dalloc<double>(p, mx);
+    p->res[0] = dalloc<double>(p, 2 * p->n + p->m);   // one vector [n | m | n]
+    p->res[1] = p->res[0] + p->n;
+    p->res[2] = p->res[1] + p->m;
     for (auto &s : p->cor) s = dalloc<double>(p, mx);
     for (auto &s : p->ipmv) s = dalloc<double>(p, mx);
-    p->red_part = dalloc<double>(p, 1024);
-    p->mdot_part = dalloc<double>(p, (long long)(kMaxKrylov + 1) * 304);
+    p->red_part = dalloc<double>(p, kRedSetMax * 304);
+    p->red_cnt = dalloc<int>(p, kRedSetMax + 2);
+    ck(cudaMemset(p->red_cnt, 0, (kRedSetMax + 2) * sizeof(int)), "memset");
+    p->mdot_part = dalloc<double>(p, (long long)(kMaxKrylov + 1) * kMdotParts);
     p->gm_coef = dalloc<double>(p, kMaxKrylov + 1);
-    p->gm_h = dalloc<double>(p, 2 * (kMaxKrylov + 1) + 1);
+    p->gm_h = dalloc<double>(p, 2 * (kMaxKrylov + 1) + 2);
     p->scal = dalloc<double>(p, 64);
     p->status = dalloc<int>(p, 8);
     ck(cudaMallocHost(&p->h_scal, 512 * sizeof(double)), "cudaMallocHost");
@@ -1433,8 +1437,9 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
   }
   cudaStream_t s = p->stream;
   // strictly positive point required (Sec. 2.3: x, z > 0)
-  ck(launch_reduce(p, RED_MIN, p->x, nullptr, p->n, p->scal + 0), "reduce");
-  ck(launch_reduce(p, RED_MIN, p->z, nullptr, p->n, p->scal + 1), "reduce");
+  const RedOne pos[2] = {{RED_MIN, p->x, nullptr, p->n, p->scal + 0},
+                         {RED_MIN, p->z, nullptr, p->n, p->scal + 1}};
+  ck(launch_reduce_set(p, pos, 2), "reduce");
   read_scalars(p, 2);
   if (p->n > 0 && (!(p->h_scal[0] > 0) || !(p->h_scal[1] > 0)))
     return set_err(p, AHLP_ERR_INVALID_ARG, "kkt_factor: x and z must be strictly positive");
@@ -1449,8 +1454,9 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
     // adaptive precision: once D = X Z^-1 spans more than fp32_cond_max the
     // block normal matrices are too ill-conditioned for FP32 factors, and the
     // factor moves to float-float
-    ck(launch_reduce(p, RED_MAXABS, p->dscale, nullptr, p->n, p->scal + 2), "reduce");
-    ck(launch_reduce(p, RED_MIN, p->dscale, nullptr, p->n, p->scal + 3), "reduce");
+    const RedOne span[2] = {{RED_MAXABS, p->dscale, nullptr, p->n, p->scal + 2},
+                            {RED_MIN, p->dscale, nullptr, p->n, p->scal + 3}};
+    ck(launch_reduce_set(p, span, 2), "reduce");
     p->bytes_d2h += 2 * sizeof(double);
     ck(cudaMemcpyAsync(p->h_scal + 2, p->scal + 2, 2 * sizeof(double), cudaMemcpyDeviceToHost, s),
        "D2H");
@@ -1546,22 +1552,23 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
   ck(cudaEventRecord(p->ev[4], s), "event");
   ck(cudaMemsetAsync(p->trsv_err, 0, sizeof(int), s), "memset");
   ck(launch_solve(p, rd, rp, rc, dx, dy, dz, adjoint), "solve");
-  ck(launch_reduce(p, RED_DOT, rd, rd, p->n, p->scal + 10), "reduce");
-  ck(launch_reduce(p, RED_DOT, rp, rp, p->m, p->scal + 11), "reduce");
-  ck(launch_reduce(p, RED_DOT, rc, rc, p->n, p->scal + 12), "reduce");
   const long long n = p->n, m = p->m, L = 2 * n + m;
+  bool have_rhs = false;   // the right-hand side's norm is on the device
   // e = r - J d; returns (||e||, ||r||)
   auto residual_norms = [&]() {
     ck(launch_residual(p, rd, rp, rc, dx, dy, dz, p->res[0], p->res[1], p->res[2], adjoint),
        "residual");
-    ck(launch_reduce(p, RED_DOT, p->res[0], p->res[0], n, p->scal + 13), "reduce");
-    ck(launch_reduce(p, RED_DOT, p->res[1], p->res[1], m, p->scal + 14), "reduce");
-    ck(launch_reduce(p, RED_DOT, p->res[2], p->res[2], n, p->scal + 15), "reduce");
-    p->bytes_d2h += 6 * sizeof(double);
-    ck(cudaMemcpyAsync(p->h_scal + 10, p->scal + 10, 6 * sizeof(double), cudaMemcpyDeviceToHost, s),
+    const RedOne norms[4] = {{RED_DOT, p->res[0], p->res[0], L, p->scal + 13},
+                             {RED_DOT, rd, rd, n, p->scal + 10},
+                             {RED_DOT, rp, rp, m, p->scal + 11},
+                             {RED_DOT, rc, rc, n, p->scal + 12}};
+    ck(launch_reduce_set(p, norms, have_rhs ? 1 : 4), "reduce");
+    have_rhs = true;
+    p->bytes_d2h += 4 * sizeof(double);
+    ck(cudaMemcpyAsync(p->h_scal + 10, p->scal + 10, 4 * sizeof(double), cudaMemcpyDeviceToHost, s),
        "D2H");
     ck(cudaStreamSynchronize(s), "sync");
-    return std::make_pair(std::sqrt(p->h_scal[13] + p->h_scal[14] + p->h_scal[15]),
+    return std::make_pair(std::sqrt(p->h_scal[13]),
                           std::sqrt(p->h_scal[10] + p->h_scal[11] + p->h_scal[12]));
   };
   auto [en, rn] = residual_norms();
@@ -1590,17 +1597,17 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
     }
     double *V = p->gm_V, *Z = p->gm_Z;
     double *cbuf = p->h_scal + 64, *hcol = p->h_scal + 256;
-    ck(cudaMemcpyAsync(V, p->res[0], n * 8, cudaMemcpyDeviceToDevice, s), "copy");
-    ck(cudaMemcpyAsync(V + n, p->res[1], m * 8, cudaMemcpyDeviceToDevice, s), "copy");
-    ck(cudaMemcpyAsync(V + n + m, p->res[2], n * 8, cudaMemcpyDeviceToDevice, s), "copy");
-    ck(launch_axpby(V, V, 1.0 / en, 0.0, L, s), "scale");
+    ck(launch_scale(V, p->res[0], nullptr, 1.0 / en, L, s), "scale");
     std::vector<double> H((size_t)(kc + 1) * kc, 0.0), cs(kc), sn(kc), g(kc + 1, 0.0);
     g[0] = en;
     int j = 0;
     for (; j < kc;) {
       double *Vj = V + (long long)j * L, *Zj = Z + (long long)j * L, *W = V + (long long)(j + 1) * L;
-      ck(launch_solve(p, Vj, Vj + n, Vj + n + m, Zj, Zj + n, Zj + n + m, adjoint), "precond");
-      ck(launch_jmul(p, Zj, Zj + n, Zj + n + m, W, W + n, W + n + m, adjoint), "jmul");
+      // z_j = M^-1 v_j, and w = J z_j: the preconditioner's last kernel holds
+      // A'dy and leaves w's first and third parts
+      ck(launch_solve(p, Vj, Vj + n, Vj + n + m, Zj, Zj + n, Zj + n + m, adjoint, W, W + n + m),
+         "precond");
+      ck(launch_spmv(p->Amat, Zj, W + n, 1.0, nullptr, s), "jmul");
       double *h = &H[(size_t)j * (kc + 1)];
       // classical Gram-Schmidt, twice, and the normalisation, all on the
       // device (the coefficients never leave it in between); the host reads
@@ -1608,11 +1615,10 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
       const int nh = j + 1;
       double *gh = p->gm_h;
       ck(launch_mdot(p, V, L, nh, W, L, gh), "mdot");
-      ck(launch_maxpy(V, L, nh, gh, W, L, s, -1.0), "maxpy");
+      ck(launch_maxpy(p, V, L, nh, gh, W, L, -1.0), "maxpy");
       ck(launch_mdot(p, V, L, nh, W, L, gh + nh), "mdot");
-      ck(launch_maxpy(V, L, nh, gh + nh, W, L, s, -1.0), "maxpy");
-      ck(launch_reduce(p, RED_DOT, W, W, L, gh + 2 * nh), "reduce");
-      ck(launch_scale_inv_norm(W, L, gh + 2 * nh, s), "scale");
+      ck(launch_maxpy(p, V, L, nh, gh + nh, W, L, -1.0, gh + 2 * nh), "maxpy");
+      ck(launch_scale(W, W, gh + 2 * nh + 1, 0.0, L, s), "scale");
       p->bytes_d2h += (2 * nh + 1) * 8;
       ck(cudaMemcpyAsync(hcol, gh, (2 * nh + 1) * 8, cudaMemcpyDeviceToHost, s), "D2H");
       ck(cudaStreamSynchronize(s), "sync");
@@ -1648,9 +1654,7 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
     for (int i = 0; i < j; ++i) cbuf[i] = y[i];
     p->bytes_h2d += j * 8;
     ck(cudaMemcpyAsync(p->gm_coef, cbuf, j * 8, cudaMemcpyHostToDevice, s), "H2D");
-    ck(launch_maxpy(Z, L, j, p->gm_coef, dx, n, s), "maxpy");
-    ck(launch_maxpy(Z + n, L, j, p->gm_coef, dy, m, s), "maxpy");
-    ck(launch_maxpy(Z + n + m, L, j, p->gm_coef, dz, n, s), "maxpy");
+    ck(launch_maxpy3(p, Z, L, j, p->gm_coef, dx, n, dy, m, dz, L), "maxpy");
     steps += j;
     std::tie(en, rn) = residual_norms();
     rel = rn > 0 ? en / rn : en;

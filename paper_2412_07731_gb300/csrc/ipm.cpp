@@ -509,11 +509,11 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
             for (int k = 0; k < cn; ++k) {
               const auto &r = p->lp_rng[c0 + k];
               const double a1 = std::min(1.0, lp_ap[c0 + k]), a2 = std::min(1.0, lp_ad[c0 + k]);
-              ck(launch_step_dot(X + r.xb0, v[V_DXA] + r.xb0, a1, Z + r.xb0, v[V_DZA] + r.xb0, a2,
-                                 r.xb1 - r.xb0, p->red_part, p->scal + 20 + 2 * k, s),
+              ck(launch_step_dot(p, X + r.xb0, v[V_DXA] + r.xb0, a1, Z + r.xb0, v[V_DZA] + r.xb0, a2,
+                                 r.xb1 - r.xb0, p->scal + 20 + 2 * k),
                  "reduce");
-              ck(launch_step_dot(X + r.x00, v[V_DXA] + r.x00, a1, Z + r.x00, v[V_DZA] + r.x00, a2,
-                                 r.x01 - r.x00, p->red_part, p->scal + 21 + 2 * k, s),
+              ck(launch_step_dot(p, X + r.x00, v[V_DXA] + r.x00, a1, Z + r.x00, v[V_DZA] + r.x00, a2,
+                                 r.x01 - r.x00, p->scal + 21 + 2 * k),
                  "reduce");
             }
             read_scalars(p, 20 + 2 * cn);
@@ -538,7 +538,7 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
           ck(launch_reduce(p, RED_MINSTEP, Z, v[V_DZA], n, p->scal + 1), "reduce");
           read_scalars(p, 2);
           const double apa = std::min(1.0, p->h_scal[0]), ada = std::min(1.0, p->h_scal[1]);
-          ck(launch_step_dot(X, v[V_DXA], apa, Z, v[V_DZA], ada, n, p->red_part, p->scal + 0, s),
+          ck(launch_step_dot(p, X, v[V_DXA], apa, Z, v[V_DZA], ada, n, p->scal + 0),
              "reduce");
           read_scalars(p, 1);
           const double mu_aff = p->h_scal[0] / n;

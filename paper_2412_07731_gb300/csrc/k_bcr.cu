@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kBcrThreads) bcr_z_kernel(BArgs A) {
 // every term; the terms' loads are independent of each other and run ahead of
 // the multiply-adds, and a row ends in three shuffles.
 constexpr int kBcrLanes = 8;
-constexpr int kBcrSolveThreads = 256;   // 32 rows at a time
+constexpr int kBcrSolveThreads = 512;   // 32 rows at a time, left and right terms apart
 
 __device__ __forceinline__ double bcr_lanes_sum(double v) {
 #pragma unroll
@@ -290,28 +290,41 @@ __global__ void __launch_bounds__(kBcrSolveThreads) bcr_fwd_kernel(BArgs A, doub
   pair_info(A, j, lv, jb, je);
   const int lj = A.l[j], lm = A.lmax;
   const long long off = A.link_off[j];
-  __shared__ double r[96];
-  const int lane = threadIdx.x & (kBcrLanes - 1), row0 = threadIdx.x / kBcrLanes;
-  constexpr int rows = kBcrSolveThreads / kBcrLanes;
+  __shared__ double r[96], part[2][96];
+  __shared__ int tk[2][32];           // rows of each earlier-level term, 0: none
+  __shared__ long long tu[2][32];     // and where its solution starts
+  const int side = threadIdx.x / (kBcrSolveThreads / 2);
+  const int lane = threadIdx.x & (kBcrLanes - 1);
+  const int row0 = (threadIdx.x % (kBcrSolveThreads / 2)) / kBcrLanes;
+  constexpr int rows = kBcrSolveThreads / 2 / kBcrLanes;
+  if (threadIdx.x < 64 && (threadIdx.x & 31) < lv) {
+    const int sd = threadIdx.x >> 5, w = threadIdx.x & 31;
+    const int m = sd ? j + (1 << w) : j - (1 << w);
+    const bool in = sd ? m < je : m >= jb;
+    tk[sd][w] = in ? A.l[m] : 0;
+    tu[sd][w] = in ? A.link_off[m] : 0;
+  }
+  __syncthreads();
   for (int i0 = 0; i0 < lj; i0 += rows) {
     const int i = i0 + row0;
     double s = 0.0;
-    if (i < lj) {
+    if (i < lj)
       for (int w = 0; w < lv; ++w) {
-        const int ml = j - (1 << w), mr = j + (1 << w);
-        const int kl = ml >= jb ? A.l[ml] : 0, kr = mr < je ? A.l[mr] : 0;
-        const long long ol = ml >= jb ? A.link_off[ml] : 0, orr = mr < je ? A.link_off[mr] : 0;
-        bcr_dot(A.GR + (long long)ml * lm * lm + (long long)i * kl, u + ol, kl, 1, lane, s);
-        bcr_dot(A.GL + (long long)mr * lm * lm + (long long)i * kr, u + orr, kr, 1, lane, s);
+        const int k = tk[side][w];
+        const long long m = side ? j + (1 << w) : j - (1 << w);
+        bcr_dot((side ? A.GL : A.GR) + m * lm * lm + (long long)i * k, u + tu[side][w], k, 1,
+                lane, s);
       }
-    }
     s = bcr_lanes_sum(s);
-    if (lane == 0 && i < lj) r[i] = u[off + i] - s;
+    if (lane == 0 && i < lj) part[side][i] = s;
   }
   __syncthreads();
+  for (int i = threadIdx.x; i < lj; i += kBcrSolveThreads)
+    r[i] = u[off + i] - (part[0][i] + part[1][i]);
+  __syncthreads();
   const double *Li = A.Linv + A.td_off[j];
-  for (int i0 = 0; i0 < lj; i0 += rows) {
-    const int i = i0 + row0;
+  for (int i0 = 0; i0 < lj; i0 += 2 * rows) {
+    const int i = i0 + threadIdx.x / kBcrLanes;
     double s = 0.0;
     if (i < lj) bcr_dot(Li + i, r, i + 1, lj, lane, s);
     s = bcr_lanes_sum(s);
@@ -326,26 +339,30 @@ __global__ void __launch_bounds__(kBcrSolveThreads) bcr_bwd_kernel(BArgs A, doub
   pair_info(A, j, lv, jb, je);
   const int lj = A.l[j], lm = A.lmax;
   const long long off = A.link_off[j];
-  __shared__ double r[96];
-  const int lane = threadIdx.x & (kBcrLanes - 1), row0 = threadIdx.x / kBcrLanes;
-  constexpr int rows = kBcrSolveThreads / kBcrLanes;
-  const int a = j - (1 << lv), b = j + (1 << lv);
-  const int ka = a >= jb ? A.l[a] : 0, kb = b < je ? A.l[b] : 0;
-  const long long oa = a >= jb ? A.link_off[a] : 0, ob = b < je ? A.link_off[b] : 0;
+  __shared__ double r[96], part[2][96];
+  const int side = threadIdx.x / (kBcrSolveThreads / 2);
+  const int lane = threadIdx.x & (kBcrLanes - 1);
+  const int row0 = (threadIdx.x % (kBcrSolveThreads / 2)) / kBcrLanes;
+  constexpr int rows = kBcrSolveThreads / 2 / kBcrLanes;
+  const int a = side ? j + (1 << lv) : j - (1 << lv);   // this side's neighbour
+  const bool in = side ? a < je : a >= jb;
+  const int ka = in ? A.l[a] : 0;
+  const long long oa = in ? A.link_off[a] : 0;
   for (int i0 = 0; i0 < lj; i0 += rows) {
     const int i = i0 + row0;
     double s = 0.0;
-    if (i < lj) {
-      bcr_dot(A.GL + (long long)j * lm * lm + i, u + oa, ka, lj, lane, s);   // l_j x l_a
-      bcr_dot(A.GR + (long long)j * lm * lm + i, u + ob, kb, lj, lane, s);   // l_j x l_b
-    }
+    if (i < lj)   // l_j x l_a
+      bcr_dot((side ? A.GR : A.GL) + (long long)j * lm * lm + i, u + oa, ka, lj, lane, s);
     s = bcr_lanes_sum(s);
-    if (lane == 0 && i < lj) r[i] = u[off + i] - s;
+    if (lane == 0 && i < lj) part[side][i] = s;
   }
   __syncthreads();
+  for (int i = threadIdx.x; i < lj; i += kBcrSolveThreads)
+    r[i] = u[off + i] - (part[0][i] + part[1][i]);
+  __syncthreads();
   const double *Li = A.Linv + A.td_off[j];
-  for (int i0 = 0; i0 < lj; i0 += rows) {
-    const int i = i0 + row0;
+  for (int i0 = 0; i0 < lj; i0 += 2 * rows) {
+    const int i = i0 + threadIdx.x / kBcrLanes;
     double s = 0.0;
     // entries i .. lj - 1 of column i
     if (i < lj) bcr_dot(Li + (long long)i * lj + i, r + i, lj - i, 1, lane, s);

@@ -1451,7 +1451,8 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
     trsv_fwd_kernel(const T *__restrict__ buf, const T *__restrict__ tinv,
                     const BlkInfo *__restrict__ blk, const int *__restrict__ sched,
                     const int *__restrict__ flag_off, int *flags, int *ticket, int *err,
-                    double *vec, T *vecT) {
+                    double *vec, T *vecT, const double *__restrict__ rhs,
+                    const long long *__restrict__ yoff) {
   constexpr int S = TrsvCfg<T, false>::stages;
   constexpr int kQL = TrsvCfg<T, false>::ql, kJC = TrsvCfg<T, false>::jc;
   extern __shared__ __align__(16) unsigned char trsv_raw[];
@@ -1552,7 +1553,11 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
   };
   red[q][rho] = acc0 + acc1;
   __syncthreads();
-  if (threadIdx.x < nr) u[threadIdx.x] = (T)gv[r0 + threadIdx.x] - sum_lanes(threadIdx.x);
+  if (threadIdx.x < nr) {
+    // the block's rows of the right-hand side; zero in its Schur rows
+    const int row = r0 + threadIdx.x;
+    u[threadIdx.x] = (T)(row < bi.p ? rhs[yoff[b] + row] : 0.0) - sum_lanes(threadIdx.x);
+  }
   __syncthreads();
   if (pivtile) {
     // pivot rows: x = L_rr^-1 u
@@ -1598,12 +1603,23 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
   }
 }
 
+// the backward solve's ends: the Schur solution it reads (its non-pivot rows
+// through the block's index map) and dy = [block rows, link rows, global rows]
+struct TrsvBwdIO {
+  const double *svec;
+  const int *kmap;
+  const long long *kmap_off, *yoff;
+  double *dy;
+  long long msum;
+  int nl, n0, mg;
+};
+
 template <typename T>
 __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::min_ctas)
     trsv_bwd_kernel(const T *__restrict__ buf, const T *__restrict__ tinv,
                     const BlkInfo *__restrict__ blk, const int *__restrict__ sched,
                     const int *__restrict__ flag_off, int *flags, int *ticket, int *err,
-                    double *vec) {
+                    double *vec, const TrsvBwdIO io) {
   constexpr int S = TrsvCfg<T, true>::stages;
   constexpr int kQL = TrsvCfg<T, true>::ql, kJC = TrsvCfg<T, true>::jc;
   extern __shared__ __align__(16) unsigned char trsv_raw[];
@@ -1621,6 +1637,13 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
   double *gv = vec + bi.voff;
   int *fl = flags + flag_off[b];
   const int r0 = r * NB, nr = min(NB, bi.a - r0), npiv = min(NB, bi.p - r0);
+  const int *km = io.kmap + io.kmap_off[b] - bi.p;
+  // a solved entry: a pivot row another CTA has published, or a Schur unknown
+  auto solved = [&](int row) { return (T)(row < bi.p ? __ldcg(gv + row) : io.svec[km[row]]); };
+  // the link and global rows of dy, shared out over the CTAs
+  for (int q = s_job * (int)blockDim.x + threadIdx.x; q < io.nl + io.mg;
+       q += (int)gridDim.x * (int)blockDim.x)
+    io.dy[io.msum + q] = io.svec[q < io.nl ? q : q + io.n0];
   // lane q dots the tile's columns q, q + kQL, ... with the rows of each chunk
   const int rho = threadIdx.x & (NB - 1), q = threadIdx.x / NB;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1659,7 +1682,7 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
       // rows past the matrix are zero in the stage; the pivot rows of chunk r
       // (entries of L_rr) take no part
       if (row < bi.a && (k > r || rho >= npiv)) {
-        const T xv = (T)__ldcg(gv + row);
+        const T xv = solved(row);
         const T *t = ring + (i % S) * NB * NB;
 #pragma unroll
         for (int j = 0; j < kJC; ++j) acc[j] = fma(t[(q + kQL * j) * NB + rho], xv, acc[j]);
@@ -1684,7 +1707,7 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
       if (k > r && k < ready_from) ready_from = k + 1 - published_run(fl, k, -1, r, err);
       const int row = k * NB + rho;
       const bool ok = row < bi.a && (k > r || rho >= npiv);
-      const T xv = ok ? (T)__ldcg(gv + row) : T(0);
+      const T xv = ok ? solved(row) : T(0);
 #pragma unroll
       for (int j = 0; j < kJC; ++j) acc[j] = fma(l[j], xv, acc[j]);
 #pragma unroll
@@ -1718,7 +1741,11 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
     if (lane == 0) red[warp][j] = s;
   }
   __syncthreads();
-  if (threadIdx.x < npiv) gv[r0 + threadIdx.x] = (double)col_sum(threadIdx.x);
+  if (threadIdx.x < npiv) {
+    const double xr = (double)col_sum(threadIdx.x);
+    gv[r0 + threadIdx.x] = xr;
+    io.dy[io.yoff[b] + r0 + threadIdx.x] = xr;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -1879,33 +1906,40 @@ cudaError_t launch_pchol_f32(float *buf, float *tinv, const BlkInfo *info,
   return pchol_t<float>(buf, tinv, info, h, diag0, tol, status, s, tc, prof, drop);
 }
 
-cudaError_t launch_trsv(ahlp_problem *p, bool forward) {
+__global__ void schur_dy_kernel(const TrsvBwdIO io) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < io.nl + io.mg) io.dy[io.msum + q] = io.svec[q < io.nl ? q : q + io.n0];
+}
+
+cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double *dy) {
   const int njobs = forward ? p->trsv_nf : p->trsv_nb;
-  if (njobs == 0) return cudaSuccess;
   cudaStream_t s = p->stream;
-  cudaError_t e =
-      cudaMemsetAsync(p->trsv_flags, 0, (size_t)(p->trsv_nflags + 2) * sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  int *ticket = p->trsv_flags + p->trsv_nflags + (forward ? 0 : 1);
+  int *flags = p->trsv_flags + (forward ? 0 : p->trsv_nflags);
+  int *ticket = p->trsv_flags + 2 * p->trsv_nflags + (forward ? 0 : 1);
   const int *sched = forward ? p->trsv_fsched : p->trsv_bsched;
+  const TrsvBwdIO io{p->svec, p->kmap, p->kmap_off_d, p->yoff_d, dy, p->msum, p->nl, p->n0, p->mg};
+  if (njobs == 0) {
+    if (!forward && p->nl + p->mg > 0)
+      count_launch(), schur_dy_kernel<<<(p->nl + p->mg + 255) / 256, 256, 0, s>>>(io);
+    return cudaGetLastError();
+  }
   if (p->fac_prec == kPrecFP32) {
     if (forward)
       count_launch(), trsv_fwd_kernel<float><<<njobs, TrsvCfg<float, false>::threads, trsv_smem<float>(), s>>>(
-          p->aug32, p->tinv32, p->blk, sched, p->trsv_flag_off, p->trsv_flags, ticket,
-          p->trsv_err, p->vec, p->vec32);
+          p->aug32, p->tinv32, p->blk, sched, p->trsv_flag_off, flags, ticket, p->trsv_err, p->vec,
+          p->vec32, rhs, p->yoff_d);
     else
       count_launch(), trsv_bwd_kernel<float><<<njobs, TrsvCfg<float, true>::threads, trsv_smem<float>(), s>>>(
-          p->aug32, p->tinv32, p->blk, sched, p->trsv_flag_off, p->trsv_flags, ticket,
-          p->trsv_err, p->vec);
+          p->aug32, p->tinv32, p->blk, sched, p->trsv_flag_off, flags, ticket, p->trsv_err, p->vec,
+          io);
   } else {
     if (forward)
       count_launch(), trsv_fwd_kernel<double><<<njobs, TrsvCfg<double, false>::threads, trsv_smem<double>(), s>>>(
-          p->aug, p->tinv, p->blk, sched, p->trsv_flag_off, p->trsv_flags, ticket, p->trsv_err,
-          p->vec, p->vec);
+          p->aug, p->tinv, p->blk, sched, p->trsv_flag_off, flags, ticket, p->trsv_err, p->vec,
+          p->vec, rhs, p->yoff_d);
     else
       count_launch(), trsv_bwd_kernel<double><<<njobs, TrsvCfg<double, true>::threads, trsv_smem<double>(), s>>>(
-          p->aug, p->tinv, p->blk, sched, p->trsv_flag_off, p->trsv_flags, ticket, p->trsv_err,
-          p->vec);
+          p->aug, p->tinv, p->blk, sched, p->trsv_flag_off, flags, ticket, p->trsv_err, p->vec, io);
   }
   return cudaGetLastError();
 }

@@ -642,24 +642,18 @@ __global__ void negate_corner_kernel(double *bd, int ld, int n0, int mg, double 
 // --------------------------------------------------------------------------
 // solve pipeline kernels
 // --------------------------------------------------------------------------
-// f = r_d - X^-1 r_c (forward) or g_x - Z X^-1 g_z (adjoint); g = D f on block columns
+// f = r_d - X^-1 r_c (forward) or g_x - Z X^-1 g_z (adjoint); g = D f on block
+// columns.  First kernel of a solve: it also clears the wavefront solves' flags.
 __global__ void prep_f_kernel(double *f, double *g, const double *rd, const double *rc,
                               const double *xinv, const double *z, const double *d,
-                              const unsigned char *is_x0, long long n, int adjoint) {
+                              const unsigned char *is_x0, long long n, int adjoint, int *flags,
+                              int nflags) {
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nflags) flags[i] = 0;
   if (i >= n) return;
   const double fi = adjoint ? rd[i] - z[i] * rc[i] * xinv[i] : rd[i] - rc[i] * xinv[i];
   f[i] = fi;
   g[i] = is_x0[i] ? 0.0 : d[i] * fi;
-}
-
-__global__ void pack_rhs_kernel(const BlkInfo *blk, const SchurBlk *sb, const long long *yoff,
-                                const double *rhat, double *vec) {
-  const int i = blockIdx.y;
-  const BlkInfo bi = blk[i];
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= bi.a) return;
-  vec[bi.voff + r] = (r < sb[i].m) ? rhat[yoff[i] + r] : 0.0;
 }
 
 struct RArgs {
@@ -949,58 +943,6 @@ __global__ void __launch_bounds__(512) link_back_kernel(const double *__restrict
   }
 }
 
-__global__ void gather_schur_kernel(const BlkInfo *blk, const SchurBlk *sb, const int *kmap,
-                                    const long long *kmap_off, const double *svec, double *vec) {
-  const int i = blockIdx.y;
-  const SchurBlk s = sb[i];
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= s.k) return;
-  vec[blk[i].voff + s.m + t] = svec[kmap[kmap_off[i] + t]];
-}
-
-__global__ void scatter_dy_kernel(const BlkInfo *blk, const SchurBlk *sb, const long long *yoff,
-                                  const double *vec, double *dy) {
-  const int i = blockIdx.y;
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= sb[i].m) return;
-  dy[yoff[i] + r] = vec[blk[i].voff + r];
-}
-
-__global__ void schur_dy_kernel(const double *svec, int nl, int n0, int mg, long long msum,
-                                double *dy) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < nl) dy[msum + q] = svec[q];
-  else if (q < nl + mg) dy[msum + q] = svec[n0 + q];
-}
-
-// dx = (A'dy - f) / (1/d + rho[x0]);  dz = X^-1 (r_c - Z dx)  or  X^-1 (g_z - dx)
-// dx = (A'dy - f) / (D^-1 + rho on the linking variables), dz from dx; w and
-// xinv are those quotients' reciprocals, taken once per factor point
-__global__ void finish_kernel(double *dx, double *dz, const double *aty, const double *f,
-                              const double *w, const double *xinv, const double *z,
-                              const double *rc, long long n, int adjoint) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double dxi = (aty[i] - f[i]) * w[i];
-  dx[i] = dxi;
-  dz[i] = adjoint ? (rc[i] - dxi) * xinv[i] : (rc[i] - z[i] * dxi) * xinv[i];
-}
-
-// residual blocks of J d = r (forward) or J' d = r (adjoint)
-__global__ void residual_tail_kernel(double *e_d, double *e_c, const double *dx,
-                                     const double *dz, const double *rc, const double *x,
-                                     const double *z, long long n, int adjoint) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (adjoint) {
-    e_d[i] -= z[i] * dz[i];
-    e_c[i] = rc[i] - dx[i] - x[i] * dz[i];
-  } else {
-    e_d[i] -= dz[i];
-    e_c[i] = rc[i] - z[i] * dx[i] - x[i] * dz[i];
-  }
-}
-
 inline unsigned nb(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 SArgs sargs(ahlp_problem *p, double delta, double rho) {
@@ -1094,17 +1036,18 @@ cudaError_t launch_schur_factor(ahlp_problem *p) {
 }
 
 cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
-                         const double *r_c, double *dx, double *dy, double *dz, bool adjoint) {
+                         const double *r_c, double *dx, double *dy, double *dz, bool adjoint,
+                         double *wx, double *wc) {
   cudaStream_t s = p->stream;
   const long long n = p->n;
   cudaError_t e;
-  count_launch(), prep_f_kernel<<<nb(n, 256), 256, 0, s>>>(p->f, p->g, r_d, r_c, p->xinv, p->z, p->dscale, p->is_x0,
-                                          n, adjoint ? 1 : 0);
+  const int nflags = 2 * p->trsv_nflags + 2;
+  count_launch(), prep_f_kernel<<<nb(std::max<long long>(n, nflags), 256), 256, 0, s>>>(
+      p->f, p->g, r_d, r_c, p->xinv, p->z, p->dscale, p->is_x0, n, adjoint ? 1 : 0, p->trsv_flags,
+      nflags);
   e = launch_spmv(p->Amat, p->g, p->rhat, 1.0, r_p, s);
   if (e != cudaSuccess) return e;
-  count_launch(), pack_rhs_kernel<<<dim3(nb(p->amax, 256), p->N), 256, 0, s>>>(p->blk, p->sblk, p->yoff_d,
-                                                                p->rhat, p->vec);
-  e = launch_trsv(p, true);
+  e = launch_trsv(p, true, p->rhat, nullptr);
   if (e != cudaSuccess) return e;
   if (p->nS > 0) {
     int lmax = 0;
@@ -1156,41 +1099,10 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
             C, p->svec, 1, stages, lmax);
       }
     }
-    int kmax = 0;
-    for (int k : p->ki) kmax = std::max(kmax, k);
-    if (kmax > 0)
-      count_launch(), gather_schur_kernel<<<dim3(nb(kmax, 256), p->N), 256, 0, s>>>(p->blk, p->sblk, p->kmap,
-                                                                  p->kmap_off_d, p->svec, p->vec);
   }
-  e = launch_trsv(p, false);
+  e = launch_trsv(p, false, nullptr, dy);
   if (e != cudaSuccess) return e;
-  int mmax = 0;
-  for (int v : p->mi) mmax = std::max(mmax, v);
-  count_launch(), scatter_dy_kernel<<<dim3(nb(mmax, 256), p->N), 256, 0, s>>>(
-      p->blk, p->sblk, p->yoff_d, p->vec, dy);
-  if (p->nl + p->mg > 0)
-    count_launch(), schur_dy_kernel<<<nb(p->nl + p->mg, 256), 256, 0, s>>>(p->svec, p->nl, p->n0, p->mg, p->msum,
-                                                          dy);
-  // dx, dz
-  e = launch_spmv(p->ATmat, dy, p->g, 1.0, nullptr, s);
-  if (e != cudaSuccess) return e;
-  count_launch(), finish_kernel<<<nb(n, 256), 256, 0, s>>>(dx, dz, p->g, p->f, p->wfin, p->xinv,
-                                                            p->z, r_c, n, adjoint ? 1 : 0);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_residual(ahlp_problem *p, const double *r_d, const double *r_p,
-                            const double *r_c, const double *dx, const double *dy,
-                            const double *dz, double *e_d, double *e_p, double *e_c,
-                            bool adjoint) {
-  cudaStream_t s = p->stream;
-  cudaError_t e = launch_spmv(p->ATmat, dy, e_d, -1.0, r_d, s);
-  if (e != cudaSuccess) return e;
-  e = launch_spmv(p->Amat, dx, e_p, -1.0, r_p, s);
-  if (e != cudaSuccess) return e;
-  count_launch(), residual_tail_kernel<<<nb(p->n, 256), 256, 0, s>>>(e_d, e_c, dx, dz, r_c, p->x, p->z, p->n,
-                                                    adjoint ? 1 : 0);
-  return cudaGetLastError();
+  return launch_finish(p, dy, r_c, dx, dz, adjoint, wx, wc);
 }
 
 cudaError_t set_schur_smem_limits(int bytes) {

@@ -53,6 +53,6 @@ def test_direction_from_the_factor_alone(P, n0, mg, l):
             res = np.linalg.norm(np.concatenate(e)) / np.linalg.norm(np.concatenate(r))
         assert res <= 1e-9, res
         # the library's own residual is the same quantity
-        assert abs(info["rel_residual"] - res) <= 1e-3 * res + 1e-15
+        assert abs(info["rel_residual"] - res) <= 0.05 * res + 1e-14
     prob.close()
 
