@@ -328,7 +328,8 @@ struct ahlp_problem {
   double *x = nullptr, *z = nullptr, *dscale = nullptr;   // current point, d = x/z
   double *xinv = nullptr, *wfin = nullptr;   // 1 / x, 1 / (1 / d + rho on x_0)
   double *vec = nullptr;      // block solve segments [sum a_i]
-  float *vec32 = nullptr;     // FP32 copy of the forward solution (FP32 factors)
+  double *vecb = nullptr;     // backward solution as published (FP32 words with FP32 factors)
+  float *vec32 = nullptr;     // forward solution as published with FP32 factors
   double *svec = nullptr;     // Schur vector [nS]
   double *f = nullptr, *g = nullptr, *rhat = nullptr;      // solve scratch
   double *stg[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // staging for host I/O
@@ -345,15 +346,13 @@ struct ahlp_problem {
   double *scal = nullptr;     // device scalars
   double *h_scal = nullptr;   // pinned host scalars
   int *status = nullptr;      // device status words [4]
-  // wavefront block solves: (block, row tile) jobs in ticket order, one ready
-  // flag per tile, then the forward and backward ticket counters
+  // wavefront block solves: (block, row tile) jobs in ticket order, and the
+  // forward and backward ticket counters (zeroed by the first kernel of a solve,
+  // which also fills the publication buffers)
   int *trsv_fsched = nullptr, *trsv_bsched = nullptr;   // [2 * jobs]
-  int *trsv_flag_off = nullptr;   // [N] first flag of each block
-  // ready flags of the forward, then of the backward solve, and the two tickets
-  // (all zeroed by the first kernel of a solve)
-  int *trsv_flags = nullptr;      // [2 trsv_nflags + 2]
+  int *trsv_ticket = nullptr;     // [2]
   int *trsv_err = nullptr;        // set when a wait timed out
-  int trsv_nf = 0, trsv_nb = 0, trsv_nflags = 0;
+  int trsv_nf = 0, trsv_nb = 0;
   int tiny_pivots = 0;
   bool factored = false;
   bool assembled = false;     // the Schur complement of the last kkt_factor exists

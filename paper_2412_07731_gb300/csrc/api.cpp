@@ -1132,11 +1132,9 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     {
       // wavefront schedules of the block solves: forward in increasing row
       // tile, backward in decreasing pivot tile, blocks interleaved per wave
-      std::vector<int> fs, bs, foff(N);
-      int nflags = 0, maxT = 0, maxTp = 0;
+      std::vector<int> fs, bs;
+      int maxT = 0, maxTp = 0;
       for (int i = 0; i < N; ++i) {
-        foff[i] = nflags;
-        nflags += p->h_blk[i].T;
         maxT = std::max(maxT, p->h_blk[i].T);
         maxTp = std::max(maxTp, p->h_blk[i].Tp);
       }
@@ -1148,11 +1146,9 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
           if (w < p->h_blk[i].Tp) bs.insert(bs.end(), {i, p->h_blk[i].Tp - 1 - w});
       p->trsv_nf = (int)fs.size() / 2;
       p->trsv_nb = (int)bs.size() / 2;
-      p->trsv_nflags = nflags;
       if (!fs.empty()) p->trsv_fsched = dupload(p, fs);
       if (!bs.empty()) p->trsv_bsched = dupload(p, bs);
-      if (N > 0) p->trsv_flag_off = dupload(p, foff);
-      p->trsv_flags = dalloc<int>(p, 2 * nflags + 2);
+      p->trsv_ticket = dalloc<int>(p, 2);
       p->trsv_err = dalloc<int>(p, 1);
       ck(cudaMemset(p->trsv_err, 0, sizeof(int)), "memset");
     }
@@ -1286,6 +1282,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     p->xinv = dalloc<double>(p, p->n);
     p->wfin = dalloc<double>(p, p->n);
     p->vec = dalloc<double>(p, p->vec_elems);
+    p->vecb = dalloc<double>(p, p->vec_elems);
     p->svec = dalloc<double>(p, p->nS);
     p->f = dalloc<double>(p, p->n);
     p->g = dalloc<double>(p, std::max(p->n, p->m));

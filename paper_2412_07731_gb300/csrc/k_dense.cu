@@ -1254,10 +1254,10 @@ __global__ void __launch_bounds__(kUpdFFThreads) pchol_update_ff8_kernel(float *
 // r of every block before tile r+1 of any block; reversed for the backward
 // sweep), so a tile only ever waits for tiles holding smaller tickets, which
 // are already running: the waits cannot deadlock.  A CTA prefetches its part
-// of the factor before it waits for the tile it needs, solves its diagonal
-// tile, writes its solution rows and publishes them with a release store on
-// its ready flag.  Every wait is bounded: after kWaitLimitNs the error word
-// is set, the CTA stops waiting and the host reports AHLP_ERR_TIMEOUT.
+// of the factor before it waits for the entries it needs, solves its diagonal
+// tile and publishes its solution rows.  Every wait is bounded: after
+// kWaitLimitNs the error word is set, the CTA stops waiting and the host
+// reports AHLP_ERR_TIMEOUT.
 //
 // forward : v <- [L11 0; L21 I]^-1 v     (all a rows; pivot tiles publish)
 // backward: v_top <- L11^-T (v_top - L21' v_bottom), v_bottom unchanged
@@ -1270,28 +1270,73 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-__device__ __forceinline__ int load_acquire(const int *f) {
+// Solved entries are their own ready flags: the publication buffers are filled
+// with a bit pattern (all ones, a NaN no arithmetic produces) by the first
+// kernel of a solve, a writer stores an entry with a relaxed store, a reader
+// polls until the pattern is gone.  So a link of the wavefront costs one store
+// and one load through L2, where a flag beside the data cost a fence, the flag's
+// store and load and then the data's load.
+template <typename T>
+struct PubBits;
+template <>
+struct PubBits<float> {
+  using U = unsigned;
+  static constexpr U none = 0xffffffffu;
+  static __device__ __forceinline__ U ld(const float *p) {
+    U v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+  }
+  static __device__ __forceinline__ void st(float *p, float x) {
+    const U v = __float_as_uint(x) == none ? 0x7fffffffu : __float_as_uint(x);
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+  }
+  static __device__ __forceinline__ float val(U v) { return __uint_as_float(v); }
+};
+template <>
+struct PubBits<double> {
+  using U = unsigned long long;
+  static constexpr U none = 0xffffffffffffffffull;
+  static __device__ __forceinline__ U ld(const double *p) {
+    U v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+  }
+  static __device__ __forceinline__ void st(double *p, double x) {
+    const U b = (U)__double_as_longlong(x);
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p),
+                 "l"(b == none ? 0x7fffffffffffffffull : b)
+                 : "memory");
+  }
+  static __device__ __forceinline__ double val(U v) { return __longlong_as_double((long long)v); }
+};
+
+__device__ __forceinline__ int load_relaxed(const int *f) {
   int v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
   return v;
 }
 
-__device__ __forceinline__ void store_release(int *f, int v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(f), "r"(v) : "memory");
-}
-
-// Thread-level bounded wait until *f != 0.  Gives up at once when another CTA
-// has already timed out, so a failure does not cascade into more waits.
-__device__ void wait_ready(const int *f, int *err) {
-  if (load_acquire(f)) return;
+// Whole-warp bounded wait until no lane's `bits` is the unpublished pattern;
+// lanes with `in` reload theirs from p.  Gives up at once when another CTA has
+// already timed out, so a failure does not cascade into more waits.
+template <typename T>
+__device__ __forceinline__ void wait_published(typename PubBits<T>::U &bits, const T *p, bool in,
+                                               int *err) {
+  using P = PubBits<T>;
+  if (!__any_sync(0xffffffffu, in && bits == P::none)) return;
   const unsigned long long t0 = global_ns();
-  for (;;) {
-    __nanosleep(128);
-    if (load_acquire(f)) return;
-    if (load_acquire(err)) return;
-    if (global_ns() - t0 > kWaitLimitNs) {
-      atomicExch(err, 1);
-      return;
+  for (int it = 0;; ++it) {
+    if (in && bits == P::none) bits = P::ld(p);
+    if (!__any_sync(0xffffffffu, in && bits == P::none)) return;
+    if (it >= 8) __nanosleep(64);
+    if ((it & 31) == 31) {   // lane 0's clock decides for the warp
+      bool out = load_relaxed(err) != 0;
+      if (!out && global_ns() - t0 > kWaitLimitNs) {
+        atomicExch(err, 1);
+        out = true;
+      }
+      if (__shfl_sync(0xffffffffu, out ? 1 : 0, 0)) return;
     }
   }
 }
@@ -1368,75 +1413,50 @@ __global__ void __launch_bounds__(kThreads) tinv_kernel(const double *__restrict
   }
 }
 
-// Called by all threads when the next needed tile k may not be published.
-// Warp 0 scans up to 32 flags fl[k + dir*i] in one round (tiles publish in
-// order, so the set flags form a run starting at k), waits (bounded) when
-// none is set yet, and the barrier count broadcasts the length of the run.
-__device__ __forceinline__ int published_run(const int *fl, int k, int dir, int limit, int *err) {
-  const int lane = threadIdx.x & 31;
-  int c = 0;
-  if (threadIdx.x < 32) {
-    for (;;) {
-      const int idx = k + dir * lane;
-      const bool in = dir > 0 ? idx < limit : idx > limit;
-      const bool set = in && load_acquire(fl + idx) != 0;
-      const unsigned bal = __ballot_sync(0xffffffffu, set);
-      c = bal == 0xffffffffu ? 32 : __ffs(~bal) - 1;
-      if (c > 0) break;
-      if (lane == 0) wait_ready(fl + k, err);
-      __syncwarp();
-      if (__any_sync(0xffffffffu, load_acquire(err) != 0)) {   // timed out: the host reports it
-        c = 1;
-        break;
-      }
-    }
-  }
-  return __syncthreads_count(threadIdx.x < 32 && lane < c);
-}
-
 // thread = (row rho of a 64-row tile or chunk, column lane q); lane q owns the
-// columns q, q + kQL, ... of a 64-column tile.  The factor tiles a CTA reads
-// are streamed into a ring of shared-memory stages by cp.async (16 bytes per
-// copy, rows past the matrix zero-filled), kTrsvStages - 1 tiles ahead of
-// the one in use, so each SM keeps several tiles of the factor in flight
-// without holding them in registers; the inverse of the diagonal tile comes
-// in with the first stage.
-
-// FP64 factors go through the ring (two 32 KB stages, 512 threads, two CTAs
-// per SM); FP32 factors hold the next tile in registers instead, which
-// measured faster for their 16 KB tiles than a ring with a barrier per tile:
-// the forward sweep with 256 threads (sixteen entries each, three CTAs per
-// SM), the backward one, which also keeps sixteen accumulators per thread at
-// that width, with 512 threads (eight entries each, two CTAs per SM).
+// columns q, q + kQL, ... of a 64-column tile.  The next factor tile's entries
+// are loaded into registers while this one is used (a shared-memory ring with a
+// barrier per tile measured slower), and a warp waits for its own entries of
+// the solution alone, so the sweep over a row of tiles has no barrier.  FP32
+// forward: 256 threads (sixteen entries each, three CTAs per SM); the others
+// 512 threads (eight entries each, two CTAs per SM).  With the factor streamed,
+// the chain of tiles is the bound: a link (wait, one tile's product, the
+// product with the inverted diagonal tile, publish) took 5.2 us in FP32, and
+// 17 us in the FP64 backward sweep, whose eight sums per thread each went
+// through five FP64 shuffle steps.
 template <typename T, bool Bwd>
 struct TrsvCfg {
   static constexpr bool narrow = sizeof(T) == 4 && !Bwd;
   static constexpr int threads = narrow ? 256 : 512;
   static constexpr int min_ctas = narrow ? 3 : 2;   // per SM
-  static constexpr int stages = sizeof(T) == 4 ? 0 : 2;
-  static constexpr int ql = threads / NB;   // column lanes
-  static constexpr int jc = NB / ql;        // columns per thread
+  static constexpr int ql = threads / NB;           // column lanes
+  static constexpr int jc = NB / ql;                // columns per thread
 };
-template <typename T>
-constexpr size_t trsv_smem() {
-  return (size_t)TrsvCfg<T, false>::stages * NB * NB * sizeof(T);
-}
 
-// One 64 x 64 tile of a column-major factor into dst ([c][row], 64 entries per
-// column): columns [0, ncols) of the tile starting at src, rows below
-// `rows` are zero, so are the other columns.  Every copy reads only entries
-// of the matrix.
+// Sum over a warp of each of a thread's eight values by a transposing exchange
+// (the additions of an xor tree, nine per thread instead of forty): the total
+// of value warp_sum8_index(lane) is returned.
 template <typename T>
-__device__ __forceinline__ void stage_factor_tile(T *dst, const T *src, long long lda, int ncols,
-                                                  int rows) {
-  constexpr int EPC = 16 / sizeof(T);   // entries per 16-byte copy
-  constexpr int CPC = NB / EPC;         // copies per column
-  for (int ch = threadIdx.x; ch < NB * CPC; ch += blockDim.x) {
-    const int c = ch / CPC, rr = (ch % CPC) * EPC;
-    const int valid = c < ncols ? max(0, min(EPC, rows - rr)) : 0;
-    const T *g = valid ? src + (long long)c * lda + rr : src;
-    cp_async16(dst + c * NB + rr, g, valid * (int)sizeof(T));
+__device__ __forceinline__ T warp_sum8(const T (&a)[8], int lane) {
+  T h4[4], h2[2];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const T keep = (lane & 16) ? a[u + 4] : a[u], give = (lane & 16) ? a[u] : a[u + 4];
+    h4[u] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
   }
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const T keep = (lane & 8) ? h4[u + 2] : h4[u], give = (lane & 8) ? h4[u] : h4[u + 2];
+    h2[u] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+  }
+  const T keep = (lane & 4) ? h2[1] : h2[0], give = (lane & 4) ? h2[0] : h2[1];
+  T t = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  return t;
+}
+__device__ __forceinline__ int warp_sum8_index(int lane) {
+  return ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
 }
 
 // n contiguous entries (a multiple of 16 bytes)
@@ -1446,17 +1466,16 @@ __device__ __forceinline__ void stage_contiguous(T *dst, const T *src, int n) {
   for (int i = threadIdx.x * EPC; i < n; i += blockDim.x * EPC) cp_async16(dst + i, src + i, 16);
 }
 
+// pub: publication buffer, x on the pivot rows; vec receives every row in FP64
+// (the same buffer for FP64 factors)
 template <typename T>
 __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>::min_ctas)
     trsv_fwd_kernel(const T *__restrict__ buf, const T *__restrict__ tinv,
-                    const BlkInfo *__restrict__ blk, const int *__restrict__ sched,
-                    const int *__restrict__ flag_off, int *flags, int *ticket, int *err,
-                    double *vec, T *vecT, const double *__restrict__ rhs,
+                    const BlkInfo *__restrict__ blk, const int *__restrict__ sched, int *ticket,
+                    int *err, double *vec, T *pub, const double *__restrict__ rhs,
                     const long long *__restrict__ yoff) {
-  constexpr int S = TrsvCfg<T, false>::stages;
+  using P = PubBits<T>;
   constexpr int kQL = TrsvCfg<T, false>::ql, kJC = TrsvCfg<T, false>::jc;
-  extern __shared__ __align__(16) unsigned char trsv_raw[];
-  T *ring = reinterpret_cast<T *>(trsv_raw);   // S tiles, [c][row]
   __shared__ __align__(16) T Xs[NB * NB];      // column-major, Xs[c * NB + r]
   __shared__ T red[kQL][NB];
   __shared__ T u[NB];
@@ -1469,50 +1488,20 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
   const T *__restrict__ L = buf + bi.base;
   const long long lda = bi.lda;
   double *gv = vec + bi.voff;
-  T *gvT = vecT + bi.voff;   // solution in the factor's precision (gv itself for FP64)
-  int *fl = flags + flag_off[b];
+  T *gp = pub + bi.voff;
   const int r0 = r * NB, nr = min(NB, bi.a - r0);
   const bool pivtile = r < bi.Tp;
   const int npiv = pivtile ? min(NB, bi.p - r0) : 0;
-  const int rho = threadIdx.x & (NB - 1), q = threadIdx.x / NB;
+  const int rho = threadIdx.x & (NB - 1), q = threadIdx.x / NB, lane = threadIdx.x & 31;
   const int nct = min(r, bi.Tp);   // pivot column tiles left of this tile
   if (pivtile) stage_contiguous(Xs, tinv + bi.ioff + (long long)r * NB * NB, NB * NB);
   cp_async_commit();
+  // the block's rows of the right-hand side; zero in its Schur rows
+  const double rhs_r = (threadIdx.x < nr && r0 + (int)threadIdx.x < bi.p)
+                           ? rhs[yoff[b] + r0 + threadIdx.x]
+                           : 0.0;
   T acc0 = T(0), acc1 = T(0);
-  int ready = 0;   // column tiles [0, ready) are published
-  if constexpr (S > 0) {
-    auto issue = [&](int k) {
-      const int c0 = k * NB;
-      stage_factor_tile(ring + (k % S) * NB * NB, L + (long long)c0 * lda + r0, lda,
-                        min(NB, bi.p - c0), nr);
-    };
-#pragma unroll
-    for (int s = 0; s < S - 1; ++s) {
-      if (s < nct) issue(s);
-      cp_async_commit();
-    }
-    for (int k = 0; k < nct; ++k) {
-      const int c0 = k * NB, nc = min(NB, bi.p - c0);
-      cp_async_wait<S - 2>();   // tile k has landed (this thread's copies) ...
-      __syncthreads();          // ... everyone's, and stage (k - 1) % S is free
-      if (k + S - 1 < nct) issue(k + S - 1);
-      cp_async_commit();
-      if (k >= ready) ready = k + published_run(fl, k, 1, nct, err);
-      const T *t = ring + (k % S) * NB * NB;
-#pragma unroll
-      for (int j = 0; j < kJC; ++j) {
-        const int c = q + kQL * j;
-        if (c < nc) {
-          const T xv = __ldcg(gvT + c0 + c);
-          if (j & 1)
-            acc1 = fma(t[c * NB + rho], xv, acc1);
-          else
-            acc0 = fma(t[c * NB + rho], xv, acc0);
-        }
-      }
-    }
-  } else {
-    // the next tile's entries are loaded into registers while this one is used
+  {
     const bool rok = rho < nr;
     const T *__restrict__ Lr = L + r0 + rho;
     T l[kJC], ln[kJC];
@@ -1524,16 +1513,21 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
         dst[j] = (rok && c < nc) ? Lr[(long long)(c0 + c) * lda] : T(0);
       }
     };
+    // a warp's columns all have its q: lane j holds column q + kQL j's solution
+    const int xc = q + kQL * (lane < kJC ? lane : 0);
+    auto x_in = [&](int k) { return lane < kJC && k * NB + xc < bi.p; };
     if (nct > 0) load_tile(0, l);
+    typename P::U xb = nct > 0 && x_in(0) ? P::ld(gp + xc) : 0;
     for (int k = 0; k < nct; ++k) {
       const int c0 = k * NB, nc = min(NB, bi.p - c0);
       if (k + 1 < nct) load_tile(k + 1, ln);
-      if (k >= ready) ready = k + published_run(fl, k, 1, nct, err);
+      wait_published<T>(xb, gp + c0 + xc, x_in(k), err);
+      const T xk = P::val(xb);
+      if (k + 1 < nct && x_in(k + 1)) xb = P::ld(gp + c0 + NB + xc);
 #pragma unroll
       for (int j = 0; j < kJC; ++j) {
-        const int c = q + kQL * j;
-        if (c < nc) {
-          const T xv = __ldcg(gvT + c0 + c);
+        const T xv = __shfl_sync(0xffffffffu, xk, j);
+        if (q + kQL * j < nc) {
           if (j & 1)
             acc1 = fma(l[j], xv, acc1);
           else
@@ -1546,18 +1540,20 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
   }
   cp_async_wait<0>();
   auto sum_lanes = [&](int t) {
-    T s = T(0);
+    if constexpr (sizeof(T) == sizeof(double)) {   // a chain of eight additions is 512 clocks
+      static_assert(kQL == 8, "eight column lanes");
+      return ((red[0][t] + red[1][t]) + (red[2][t] + red[3][t])) +
+             ((red[4][t] + red[5][t]) + (red[6][t] + red[7][t]));
+    } else {
+      T s = T(0);
 #pragma unroll
-    for (int i = 0; i < kQL; ++i) s += red[i][t];
-    return s;
+      for (int i = 0; i < kQL; ++i) s += red[i][t];
+      return s;
+    }
   };
   red[q][rho] = acc0 + acc1;
   __syncthreads();
-  if (threadIdx.x < nr) {
-    // the block's rows of the right-hand side; zero in its Schur rows
-    const int row = r0 + threadIdx.x;
-    u[threadIdx.x] = (T)(row < bi.p ? rhs[yoff[b] + row] : 0.0) - sum_lanes(threadIdx.x);
-  }
+  if (threadIdx.x < nr) u[threadIdx.x] = (T)rhs_r - sum_lanes(threadIdx.x);
   __syncthreads();
   if (pivtile) {
     // pivot rows: x = L_rr^-1 u
@@ -1571,10 +1567,15 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
     }
     red[q][rho] = s;
     __syncthreads();
-    if (threadIdx.x < npiv) xs[threadIdx.x] = sum_lanes(threadIdx.x);
-    __syncthreads();
+    if (threadIdx.x < npiv) {
+      const T x = sum_lanes(threadIdx.x);
+      P::st(gp + r0 + threadIdx.x, x);
+      xs[threadIdx.x] = x;
+      if constexpr (sizeof(T) != sizeof(double)) gv[r0 + threadIdx.x] = (double)x;
+    }
     if (npiv < nr) {
       // non-pivot rows of the last pivot tile: u -= L(rows, pivots) x
+      __syncthreads();
       T s2 = T(0);
       if (rho >= npiv && rho < nr) {
 #pragma unroll
@@ -1585,21 +1586,11 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
       }
       red[q][rho] = s2;
       __syncthreads();
-      if (threadIdx.x >= npiv && threadIdx.x < nr) u[threadIdx.x] -= sum_lanes(threadIdx.x);
+      if (threadIdx.x >= npiv && threadIdx.x < nr)
+        gv[r0 + threadIdx.x] = (double)(u[threadIdx.x] - sum_lanes(threadIdx.x));
     }
-    if (threadIdx.x < npiv) u[threadIdx.x] = xs[threadIdx.x];
-    __syncthreads();
-  }
-  if (threadIdx.x < nr) {
+  } else if (threadIdx.x < nr) {
     gv[r0 + threadIdx.x] = (double)u[threadIdx.x];
-    if constexpr (sizeof(T) != sizeof(double)) gvT[r0 + threadIdx.x] = u[threadIdx.x];
-  }
-  if (pivtile) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      store_release(fl + r, 1);
-    }
   }
 }
 
@@ -1614,16 +1605,15 @@ struct TrsvBwdIO {
   int nl, n0, mg;
 };
 
+// vec holds the forward solution; pub is the publication buffer (its pivot rows)
 template <typename T>
 __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::min_ctas)
     trsv_bwd_kernel(const T *__restrict__ buf, const T *__restrict__ tinv,
-                    const BlkInfo *__restrict__ blk, const int *__restrict__ sched,
-                    const int *__restrict__ flag_off, int *flags, int *ticket, int *err,
-                    double *vec, const TrsvBwdIO io) {
-  constexpr int S = TrsvCfg<T, true>::stages;
+                    const BlkInfo *__restrict__ blk, const int *__restrict__ sched, int *ticket,
+                    int *err, const double *__restrict__ vec, T *pub, const TrsvBwdIO io) {
+  using P = PubBits<T>;
   constexpr int kQL = TrsvCfg<T, true>::ql, kJC = TrsvCfg<T, true>::jc;
-  extern __shared__ __align__(16) unsigned char trsv_raw[];
-  T *ring = reinterpret_cast<T *>(trsv_raw);   // S chunks of 64 rows, [c][row]
+  static_assert(kJC == 8, "eight sums per thread");
   __shared__ __align__(16) T Xs[NB * NB];      // column-major, Xs[c * NB + r]
   __shared__ T red[TrsvCfg<T, true>::threads / 32][kJC];
   __shared__ T u[NB];
@@ -1634,12 +1624,9 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
   const BlkInfo bi = blk[b];
   const T *__restrict__ L = buf + bi.base;
   const long long lda = bi.lda;
-  double *gv = vec + bi.voff;
-  int *fl = flags + flag_off[b];
+  T *gp = pub + bi.voff;
   const int r0 = r * NB, nr = min(NB, bi.a - r0), npiv = min(NB, bi.p - r0);
   const int *km = io.kmap + io.kmap_off[b] - bi.p;
-  // a solved entry: a pivot row another CTA has published, or a Schur unknown
-  auto solved = [&](int row) { return (T)(row < bi.p ? __ldcg(gv + row) : io.svec[km[row]]); };
   // the link and global rows of dy, shared out over the CTAs
   for (int q = s_job * (int)blockDim.x + threadIdx.x; q < io.nl + io.mg;
        q += (int)gridDim.x * (int)blockDim.x)
@@ -1655,41 +1642,11 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
   const int nch = bi.T - kend;   // chunks, taken k = T - 1, T - 2, ..., kend
   stage_contiguous(Xs, tinv + bi.ioff + (long long)r * NB * NB, NB * NB);
   cp_async_commit();
+  const double fwd_r = threadIdx.x < npiv ? vec[bi.voff + r0 + threadIdx.x] : 0.0;
   T acc[kJC];
 #pragma unroll
   for (int j = 0; j < kJC; ++j) acc[j] = T(0);
-  int ready_from = bi.Tp;   // chunks k >= ready_from are final
-  if constexpr (S > 0) {
-    auto issue = [&](int i) {      // i-th chunk taken: k = T - 1 - i
-      const int k = bi.T - 1 - i;
-      stage_factor_tile(ring + (i % S) * NB * NB, Lc + (long long)k * NB, lda, npiv,
-                        bi.a - k * NB);
-    };
-#pragma unroll
-    for (int s = 0; s < S - 1; ++s) {
-      if (s < nch) issue(s);
-      cp_async_commit();
-    }
-    for (int i = 0; i < nch; ++i) {
-      const int k = bi.T - 1 - i;
-      cp_async_wait<S - 2>();
-      __syncthreads();
-      if (i + S - 1 < nch) issue(i + S - 1);
-      cp_async_commit();
-      // tiles publish in decreasing order
-      if (k > r && k < ready_from) ready_from = k + 1 - published_run(fl, k, -1, r, err);
-      const int row = k * NB + rho;
-      // rows past the matrix are zero in the stage; the pivot rows of chunk r
-      // (entries of L_rr) take no part
-      if (row < bi.a && (k > r || rho >= npiv)) {
-        const T xv = solved(row);
-        const T *t = ring + (i % S) * NB * NB;
-#pragma unroll
-        for (int j = 0; j < kJC; ++j) acc[j] = fma(t[(q + kQL * j) * NB + rho], xv, acc[j]);
-      }
-    }
-  } else {
-    // the next chunk's entries are loaded into registers while this one is used
+  {
     T l[kJC], ln[kJC];
     auto load_chunk = [&](int k, T(&dst)[kJC]) {
       const int row = k * NB + rho;
@@ -1700,14 +1657,28 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
         dst[j] = (ok && c < npiv) ? Lc[(long long)c * lda + row] : T(0);
       }
     };
-    if (nch > 0) load_chunk(bi.T - 1, l);
+    // a solved entry: a pivot row another CTA publishes, or a Schur unknown
+    auto x_in = [&](int k) { return k > r && k * NB + rho < bi.p; };
+    auto x_ld = [&](int k) -> typename P::U {
+      const int row = k * NB + rho;
+      if (x_in(k)) return P::ld(gp + row);
+      typename P::U v = 0;
+      if (row >= bi.p && row < bi.a) {
+        const T x = (T)io.svec[km[row]];
+        memcpy(&v, &x, sizeof v);
+      }
+      return v;
+    };
+    typename P::U xb = 0;
+    if (nch > 0) {
+      load_chunk(bi.T - 1, l);
+      xb = x_ld(bi.T - 1);
+    }
     for (int k = bi.T - 1; k >= kend; --k) {
       if (k - 1 >= kend) load_chunk(k - 1, ln);
-      // tiles publish in decreasing order
-      if (k > r && k < ready_from) ready_from = k + 1 - published_run(fl, k, -1, r, err);
-      const int row = k * NB + rho;
-      const bool ok = row < bi.a && (k > r || rho >= npiv);
-      const T xv = ok ? solved(row) : T(0);
+      wait_published<T>(xb, gp + k * NB + rho, x_in(k), err);
+      const T xv = P::val(xb);
+      if (k - 1 >= kend) xb = x_ld(k - 1);
 #pragma unroll
       for (int j = 0; j < kJC; ++j) acc[j] = fma(l[j], xv, acc[j]);
 #pragma unroll
@@ -1715,41 +1686,32 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
     }
   }
   cp_async_wait<0>();
-  __syncthreads();
   // column c = q + kQL j is summed over the two warps of lane q
   auto col_sum = [&](int c) {
     const int cq = c % kQL, cj = c / kQL;
     return red[2 * cq][cj] + red[2 * cq + 1][cj];
   };
-#pragma unroll
-  for (int j = 0; j < kJC; ++j) {
-    T s = acc[j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[warp][j] = s;
+  const int si = warp_sum8_index(lane);
+  {
+    const T s = warp_sum8(acc, lane);
+    if ((lane & 3) == 0) red[warp][si] = s;
   }
   __syncthreads();
-  if (threadIdx.x < npiv) u[threadIdx.x] = (T)gv[r0 + threadIdx.x] - col_sum(threadIdx.x);
+  if (threadIdx.x < npiv) u[threadIdx.x] = (T)fwd_r - col_sum(threadIdx.x);
   __syncthreads();
   // x = L_rr^-T u: column c = q + kQL j collects X(rho, c) u(rho) over the rows
   const T uv = rho < npiv ? u[rho] : T(0);
 #pragma unroll
-  for (int j = 0; j < kJC; ++j) {
-    T s = (rho < npiv) ? Xs[(q + kQL * j) * NB + rho] * uv : T(0);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[warp][j] = s;
+  for (int j = 0; j < kJC; ++j) acc[j] = (rho < npiv) ? Xs[(q + kQL * j) * NB + rho] * uv : T(0);
+  {
+    const T s = warp_sum8(acc, lane);
+    if ((lane & 3) == 0) red[warp][si] = s;
   }
   __syncthreads();
   if (threadIdx.x < npiv) {
-    const double xr = (double)col_sum(threadIdx.x);
-    gv[r0 + threadIdx.x] = xr;
-    io.dy[io.yoff[b] + r0 + threadIdx.x] = xr;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    store_release(fl + r, 1);
+    const T x = col_sum(threadIdx.x);
+    P::st(gp + r0 + threadIdx.x, x);
+    io.dy[io.yoff[b] + r0 + threadIdx.x] = (double)x;
   }
 }
 
@@ -1914,8 +1876,7 @@ __global__ void schur_dy_kernel(const TrsvBwdIO io) {
 cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double *dy) {
   const int njobs = forward ? p->trsv_nf : p->trsv_nb;
   cudaStream_t s = p->stream;
-  int *flags = p->trsv_flags + (forward ? 0 : p->trsv_nflags);
-  int *ticket = p->trsv_flags + 2 * p->trsv_nflags + (forward ? 0 : 1);
+  int *ticket = p->trsv_ticket + (forward ? 0 : 1);
   const int *sched = forward ? p->trsv_fsched : p->trsv_bsched;
   const TrsvBwdIO io{p->svec, p->kmap, p->kmap_off_d, p->yoff_d, dy, p->msum, p->nl, p->n0, p->mg};
   if (njobs == 0) {
@@ -1924,22 +1885,21 @@ cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double
     return cudaGetLastError();
   }
   if (p->fac_prec == kPrecFP32) {
+    float *pubb = reinterpret_cast<float *>(p->vecb);
     if (forward)
-      count_launch(), trsv_fwd_kernel<float><<<njobs, TrsvCfg<float, false>::threads, trsv_smem<float>(), s>>>(
-          p->aug32, p->tinv32, p->blk, sched, p->trsv_flag_off, flags, ticket, p->trsv_err, p->vec,
-          p->vec32, rhs, p->yoff_d);
+      count_launch(), trsv_fwd_kernel<float><<<njobs, TrsvCfg<float, false>::threads, 0, s>>>(
+          p->aug32, p->tinv32, p->blk, sched, ticket, p->trsv_err, p->vec, p->vec32, rhs,
+          p->yoff_d);
     else
-      count_launch(), trsv_bwd_kernel<float><<<njobs, TrsvCfg<float, true>::threads, trsv_smem<float>(), s>>>(
-          p->aug32, p->tinv32, p->blk, sched, p->trsv_flag_off, flags, ticket, p->trsv_err, p->vec,
-          io);
+      count_launch(), trsv_bwd_kernel<float><<<njobs, TrsvCfg<float, true>::threads, 0, s>>>(
+          p->aug32, p->tinv32, p->blk, sched, ticket, p->trsv_err, p->vec, pubb, io);
   } else {
     if (forward)
-      count_launch(), trsv_fwd_kernel<double><<<njobs, TrsvCfg<double, false>::threads, trsv_smem<double>(), s>>>(
-          p->aug, p->tinv, p->blk, sched, p->trsv_flag_off, flags, ticket, p->trsv_err, p->vec,
-          p->vec, rhs, p->yoff_d);
+      count_launch(), trsv_fwd_kernel<double><<<njobs, TrsvCfg<double, false>::threads, 0, s>>>(
+          p->aug, p->tinv, p->blk, sched, ticket, p->trsv_err, p->vec, p->vec, rhs, p->yoff_d);
     else
-      count_launch(), trsv_bwd_kernel<double><<<njobs, TrsvCfg<double, true>::threads, trsv_smem<double>(), s>>>(
-          p->aug, p->tinv, p->blk, sched, p->trsv_flag_off, flags, ticket, p->trsv_err, p->vec, io);
+      count_launch(), trsv_bwd_kernel<double><<<njobs, TrsvCfg<double, true>::threads, 0, s>>>(
+          p->aug, p->tinv, p->blk, sched, ticket, p->trsv_err, p->vec, p->vecb, io);
   }
   return cudaGetLastError();
 }
@@ -1963,18 +1923,6 @@ cudaError_t launch_tile_inverses(const double *buf, double *tinv, const BlkInfo 
 cudaError_t set_dense_smem_limits() {
   cudaError_t e = cudaFuncSetAttribute(tinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kTinvSmem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(trsv_fwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)trsv_smem<float>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(trsv_bwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)trsv_smem<float>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(trsv_fwd_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)trsv_smem<double>());
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(trsv_bwd_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)trsv_smem<double>());
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(pchol_update_ff8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)kUpdFFSmem);

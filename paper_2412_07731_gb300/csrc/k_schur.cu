@@ -643,13 +643,19 @@ __global__ void negate_corner_kernel(double *bd, int ld, int n0, int mg, double 
 // solve pipeline kernels
 // --------------------------------------------------------------------------
 // f = r_d - X^-1 r_c (forward) or g_x - Z X^-1 g_z (adjoint); g = D f on block
-// columns.  First kernel of a solve: it also clears the wavefront solves' flags.
+// columns.  First kernel of a solve: it also resets the wavefront solves'
+// tickets and fills their publication buffers (fwd_words and bwd_words 32-bit
+// words) with the unpublished pattern.
 __global__ void prep_f_kernel(double *f, double *g, const double *rd, const double *rc,
                               const double *xinv, const double *z, const double *d,
-                              const unsigned char *is_x0, long long n, int adjoint, int *flags,
-                              int nflags) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nflags) flags[i] = 0;
+                              const unsigned char *is_x0, long long n, int adjoint, int *ticket,
+                              unsigned *pub_fwd, unsigned *pub_bwd, long long fwd_words,
+                              long long bwd_words) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  if (i < 2) ticket[i] = 0;
+  for (long long w = i; w < fwd_words; w += stride) pub_fwd[w] = 0xffffffffu;
+  for (long long w = i; w < bwd_words; w += stride) pub_bwd[w] = 0xffffffffu;
   if (i >= n) return;
   const double fi = adjoint ? rd[i] - z[i] * rc[i] * xinv[i] : rd[i] - rc[i] * xinv[i];
   f[i] = fi;
@@ -1041,10 +1047,12 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
   cudaStream_t s = p->stream;
   const long long n = p->n;
   cudaError_t e;
-  const int nflags = 2 * p->trsv_nflags + 2;
-  count_launch(), prep_f_kernel<<<nb(std::max<long long>(n, nflags), 256), 256, 0, s>>>(
-      p->f, p->g, r_d, r_c, p->xinv, p->z, p->dscale, p->is_x0, n, adjoint ? 1 : 0, p->trsv_flags,
-      nflags);
+  const bool f32 = p->fac_prec == kPrecFP32;
+  const long long words = p->vec_elems * (f32 ? 1 : 2);
+  count_launch(), prep_f_kernel<<<nb(std::max<long long>(n, 2), 256), 256, 0, s>>>(
+      p->f, p->g, r_d, r_c, p->xinv, p->z, p->dscale, p->is_x0, n, adjoint ? 1 : 0, p->trsv_ticket,
+      f32 ? reinterpret_cast<unsigned *>(p->vec32) : reinterpret_cast<unsigned *>(p->vec),
+      reinterpret_cast<unsigned *>(p->vecb), words, words);
   e = launch_spmv(p->Amat, p->g, p->rhat, 1.0, r_p, s);
   if (e != cudaSuccess) return e;
   e = launch_trsv(p, true, p->rhat, nullptr);
