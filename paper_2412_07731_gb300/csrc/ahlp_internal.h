@@ -66,6 +66,42 @@ constexpr int kTagBorderX = 1 << 20;   // pivot reports of the border x_0 factor
 constexpr int kTagBorderG = 2 << 20;   // pivot reports of the border y_g factor
 
 #ifdef __CUDACC__
+// First statement of every kernel that launch_pdl starts: returns when the
+// kernels before this one are complete and their writes are visible; from then
+// on the next kernel of the stream may be scheduled (it waits in turn).
+// pdl_wait leaves that to the kernel's end: for kernels that fill the GPU, whose
+// successors would only hold shared memory and registers.  Pointers to data that
+// other kernels write are not marked __restrict__ here: such loads count as
+// invariant and could be moved above the wait.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_begin() {
+  pdl_wait();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch with programmatic stream serialisation: the kernel's launch and the
+// scheduling of its CTAs overlap the tail of the kernel before it.  Dependent
+// kernels of a few CTAs follow each other in 1.5 us instead of 4.1 us, and most
+// of a solve's kernels are that small.  Only for kernels that begin with
+// pdl_begin().
+template <typename... P, typename... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                       A &&...args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 // Pivot safeguard shared by every Cholesky in the library.  A pivot that is
 // not above tol * (the diagonal entry it started from) has lost all its
 // significant digits to cancellation.  It is clamped to that threshold, which
@@ -375,7 +411,7 @@ struct ahlp_problem {
 
 namespace ahlp {
 
-// Every kernel launch of the library is written `count_launch(), k<<<...>>>(...)`
+// Every kernel launch of the library is written `count_launch(), launch_pdl(k, ...)`
 // so the number of launches can be reported (arrowhead_lp_launch_count).
 void count_launch();
 long long launch_count();

@@ -76,6 +76,7 @@ __device__ void sub_gtg(double *dst, int rows, int cols, const double *G, const 
 // Factor of the pairs of one level: earlier-level updates of T_j, its
 // Cholesky and inverse, and GL_j, GR_j.  One CTA per pair.
 __global__ void __launch_bounds__(kBcrThreads) bcr_factor_kernel(BArgs A) {
+  pdl_begin();
   extern __shared__ double sm[];
   const int lm = A.lmax;
   double *T = sm, *Li = sm + lm * lm, *C = sm + 2 * lm * lm;
@@ -217,6 +218,7 @@ __global__ void __launch_bounds__(kBcrThreads) bcr_factor_kernel(BArgs A) {
 // Z_j = Linv_j (E_j' - earlier-level terms), thread (row, column) over 32 x 4,
 // blockIdx.y over groups of four border columns
 __global__ void __launch_bounds__(kBcrThreads) bcr_z_kernel(BArgs A) {
+  pdl_begin();
   const int j = A.order[blockIdx.x];
   int lv, jb, je;
   pair_info(A, j, lv, jb, je);
@@ -276,7 +278,7 @@ __device__ __forceinline__ double bcr_lanes_sum(double v) {
 }
 
 // s += sum_q G[q] z[q], q = lane, lane + 8, ... < k
-__device__ __forceinline__ void bcr_dot(const double *__restrict__ G, const double *z, int k,
+__device__ __forceinline__ void bcr_dot(const double *G, const double *z, int k,
                                         int stride, int q0, double &s) {
 #pragma unroll 4
   for (int q = q0; q < k; q += kBcrLanes) s = fma(G[(long long)q * stride], z[q], s);
@@ -285,6 +287,7 @@ __device__ __forceinline__ void bcr_dot(const double *__restrict__ G, const doub
 // forward solve of one level, in place on the link part of u, one CTA per
 // pair: u_j = Linv_j (r_j - earlier-level terms)
 __global__ void __launch_bounds__(kBcrSolveThreads) bcr_fwd_kernel(BArgs A, double *u) {
+  pdl_begin();
   const int j = A.order[blockIdx.x];
   int lv, jb, je;
   pair_info(A, j, lv, jb, je);
@@ -334,6 +337,7 @@ __global__ void __launch_bounds__(kBcrSolveThreads) bcr_fwd_kernel(BArgs A, doub
 
 // backward solve of one level: x_j = Linv_j' (u_j - GL_j x_a - GR_j x_b)
 __global__ void __launch_bounds__(kBcrSolveThreads) bcr_bwd_kernel(BArgs A, double *u) {
+  pdl_begin();
   const int j = A.order[blockIdx.x];
   int lv, jb, je;
   pair_info(A, j, lv, jb, je);
@@ -405,9 +409,9 @@ cudaError_t launch_bcr_factor(ahlp_problem *p) {
     if (n == 0) continue;
     BArgs A = bargs(p);
     A.order = p->bcr_order + p->bcr_loff[v];
-    count_launch(), bcr_factor_kernel<<<n, kBcrThreads, smem, s>>>(A);
+    count_launch(), launch_pdl(bcr_factor_kernel, n, kBcrThreads, smem, s, A);
     if (p->B > 0)
-      count_launch(), bcr_z_kernel<<<dim3(n, (p->B + 3) / 4), kBcrThreads, 0, s>>>(A);
+      count_launch(), launch_pdl(bcr_z_kernel, dim3(n, (p->B + 3) / 4), kBcrThreads, 0, s, A);
   }
   return cudaGetLastError();
 }
@@ -422,9 +426,9 @@ cudaError_t launch_bcr_solve(ahlp_problem *p, double *u, bool forward) {
     BArgs A = bargs(p);
     A.order = p->bcr_order + p->bcr_loff[v];
     if (forward)
-      count_launch(), bcr_fwd_kernel<<<n, kBcrSolveThreads, 0, s>>>(A, u);
+      count_launch(), launch_pdl(bcr_fwd_kernel, n, kBcrSolveThreads, 0, s, A, u);
     else
-      count_launch(), bcr_bwd_kernel<<<n, kBcrSolveThreads, 0, s>>>(A, u);
+      count_launch(), launch_pdl(bcr_bwd_kernel, n, kBcrSolveThreads, 0, s, A, u);
   }
   return cudaGetLastError();
 }

@@ -45,6 +45,7 @@ struct FormArgs {
 
 template <typename T, bool kLo>
 __global__ void __launch_bounds__(kThreads) form_aug_kernel(FormArgs<T> A) {
+  pdl_begin();
   __shared__ T t[NB * NB];   // column-major tile
   __shared__ float tl[kLo ? NB * NB : 1];
   const FormTile ft = A.tiles[blockIdx.x];
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(kThreads) form_aug_kernel(FormArgs<T> A) {
 __global__ void dscale_kernel(const double *x, const double *z, double *d, double *xinv,
                               double *w, long long n, double rho_x, double rho,
                               const unsigned char *is_x0) {
+  pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double di = (rho_x > 0.0 && !is_x0[i]) ? x[i] / (z[i] + rho_x * x[i]) : x[i] / z[i];
@@ -142,6 +144,7 @@ __global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(double *buf, cons
                                                                int k, const double *diag0,
                                                                double tol, int *status,
                                                                double drop) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.x];
   if (k >= bi.Tp) return;
   __shared__ double t[NB][NB + 1];
@@ -312,6 +315,7 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkInfo *blk, int k,
                                                               __half *stage, int *dexp,
                                                               long long slots) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const int I = k + 1 + blockIdx.x;
@@ -382,6 +386,7 @@ constexpr int kPotrf32Threads = 256;
 __global__ void __launch_bounds__(kPotrf32Threads) pchol_potrf_f32_kernel(
     float *buf, float *tinv, const BlkInfo *blk, int k, const double *diag0, float tol,
     int *status, float drop) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.x];
   if (k >= bi.Tp) return;
   __shared__ float t[NB][NB + 1];
@@ -558,6 +563,7 @@ template <typename T>
 __global__ void __launch_bounds__(kThreads) pchol_trsm_inv_kernel(T *buf, const T *tinv,
                                                                   const BlkInfo *blk, int k,
                                                                   float *pstage) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const int I = k + 1 + blockIdx.x;
@@ -674,8 +680,9 @@ __device__ __forceinline__ void ff_renorm(float &sh, float &sl) {
 // hi + lo -> FP64 copy of the float-float factor, used by the solves; four
 // entries per thread and step (16-byte loads of each word, two 16-byte
 // stores; the buffers are cudaMalloc-aligned), the last n % 4 one by one
-__global__ void ff_expand_kernel(const float *__restrict__ hi, const float *__restrict__ lo,
-                                 double *__restrict__ out, long long n) {
+__global__ void ff_expand_kernel(const float *hi, const float *lo,
+                                 double *out, long long n) {
+  pdl_begin();
   const long long n4 = n / 4;
   const float4 *h4 = reinterpret_cast<const float4 *>(hi);
   const float4 *l4 = reinterpret_cast<const float4 *>(lo);
@@ -695,6 +702,7 @@ __global__ void __launch_bounds__(kThreads) pchol_potrf_ff_kernel(float *hi, flo
                                                                   const BlkInfo *blk, int k,
                                                                   const double *diag0, double tol,
                                                                   int *status, double drop) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.x];
   if (k >= bi.Tp) return;
   __shared__ double t[NB][NB + 1];
@@ -813,6 +821,7 @@ constexpr size_t kTrsmFFSmem =
 __global__ void __launch_bounds__(kFFRowThreads) pchol_trsm_ff_kernel(float *hi, float *lo,
                                                                      const BlkInfo *blk, int k,
                                                                      __half *dstage, int *dexp) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const int I0 = k + 1 + kFFRowTiles * blockIdx.x;
@@ -943,6 +952,7 @@ __global__ void __launch_bounds__(kFFRowThreads) pchol_trsm_ff_kernel(float *hi,
 constexpr int KC = 16;
 template <typename T>
 __global__ void __launch_bounds__(kThreads) pchol_update_kernel(T *buf, const BlkInfo *blk, int k) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const long long t = bi.T - k - 1;
@@ -1030,6 +1040,7 @@ __device__ __forceinline__ void cp_async_wait() {
 __global__ void __launch_bounds__(kUpdF32Threads) pchol_update_f32_kernel(float *buf,
                                                                          const BlkInfo *blk,
                                                                          int k) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const long long t = bi.T - k - 1;
@@ -1144,6 +1155,7 @@ constexpr size_t kUpdFFSmem = 4 * NB * NB * sizeof(float);
 __global__ void __launch_bounds__(kUpdFFThreads) pchol_update_ff8_kernel(float *hi, float *lo,
                                                                         const BlkInfo *blk,
                                                                         int k) {
+  pdl_begin();
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const long long t = bi.T - k - 1;
@@ -1350,10 +1362,11 @@ __device__ __forceinline__ void wait_published(typename PubBits<T>::U &bits, con
 // tiles of 32 blocks (1130 tiles): 326 -> 150 us against one thread per column.
 constexpr size_t kTinvSmem = (2 * NB * (NB + 1) + 16 * NB + NB) * sizeof(double);
 
-__global__ void __launch_bounds__(kThreads) tinv_kernel(const double *__restrict__ buf,
-                                                        double *__restrict__ tinv,
+__global__ void __launch_bounds__(kThreads) tinv_kernel(const double *buf,
+                                                        double *tinv,
                                                         const BlkInfo *__restrict__ blk,
                                                         const int *__restrict__ sched) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char tinv_raw[];   // kTinvSmem bytes
   double(*Ls)[NB + 1] = reinterpret_cast<double(*)[NB + 1]>(tinv_raw);
   double(*Xs)[NB + 1] = Ls + NB;
@@ -1361,7 +1374,7 @@ __global__ void __launch_bounds__(kThreads) tinv_kernel(const double *__restrict
   double *rinv = Tm + 16 * NB;
   const int b = sched[2 * blockIdx.x], k = sched[2 * blockIdx.x + 1];
   const BlkInfo bi = blk[b];
-  const double *__restrict__ L = buf + bi.base;
+  const double *L = buf + bi.base;
   const int r0 = k * NB, nr = min(NB, bi.a - r0), npiv = min(NB, bi.p - r0);
   for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
     const int r = i % NB, c = i / NB;
@@ -1406,7 +1419,7 @@ __global__ void __launch_bounds__(kThreads) tinv_kernel(const double *__restrict
     }
     __syncthreads();
   }
-  double *__restrict__ out = tinv + bi.ioff + (long long)k * NB * NB;
+  double *out = tinv + bi.ioff + (long long)k * NB * NB;
   for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
     const int r = i % NB, c = i / NB;
     out[i] = r < npiv ? Xs[r][c] : Ls[r][c];
@@ -1470,10 +1483,11 @@ __device__ __forceinline__ void stage_contiguous(T *dst, const T *src, int n) {
 // (the same buffer for FP64 factors)
 template <typename T>
 __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>::min_ctas)
-    trsv_fwd_kernel(const T *__restrict__ buf, const T *__restrict__ tinv,
+    trsv_fwd_kernel(const T *buf, const T *tinv,
                     const BlkInfo *__restrict__ blk, const int *__restrict__ sched, int *ticket,
-                    int *err, double *vec, T *pub, const double *__restrict__ rhs,
+                    int *err, double *vec, T *pub, const double *rhs,
                     const long long *__restrict__ yoff) {
+  pdl_begin();
   using P = PubBits<T>;
   constexpr int kQL = TrsvCfg<T, false>::ql, kJC = TrsvCfg<T, false>::jc;
   __shared__ __align__(16) T Xs[NB * NB];      // column-major, Xs[c * NB + r]
@@ -1485,7 +1499,7 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
   __syncthreads();
   const int b = sched[2 * s_job], r = sched[2 * s_job + 1];
   const BlkInfo bi = blk[b];
-  const T *__restrict__ L = buf + bi.base;
+  const T *L = buf + bi.base;
   const long long lda = bi.lda;
   double *gv = vec + bi.voff;
   T *gp = pub + bi.voff;
@@ -1503,7 +1517,7 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
   T acc0 = T(0), acc1 = T(0);
   {
     const bool rok = rho < nr;
-    const T *__restrict__ Lr = L + r0 + rho;
+    const T *Lr = L + r0 + rho;
     T l[kJC], ln[kJC];
     auto load_tile = [&](int k, T(&dst)[kJC]) {
       const int c0 = k * NB, nc = min(NB, bi.p - c0);
@@ -1608,9 +1622,10 @@ struct TrsvBwdIO {
 // vec holds the forward solution; pub is the publication buffer (its pivot rows)
 template <typename T>
 __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::min_ctas)
-    trsv_bwd_kernel(const T *__restrict__ buf, const T *__restrict__ tinv,
+    trsv_bwd_kernel(const T *buf, const T *tinv,
                     const BlkInfo *__restrict__ blk, const int *__restrict__ sched, int *ticket,
-                    int *err, const double *__restrict__ vec, T *pub, const TrsvBwdIO io) {
+                    int *err, const double *vec, T *pub, const TrsvBwdIO io) {
+  pdl_begin();
   using P = PubBits<T>;
   constexpr int kQL = TrsvCfg<T, true>::ql, kJC = TrsvCfg<T, true>::jc;
   static_assert(kJC == 8, "eight sums per thread");
@@ -1622,7 +1637,7 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
   __syncthreads();
   const int b = sched[2 * s_job], r = sched[2 * s_job + 1];   // r < Tp
   const BlkInfo bi = blk[b];
-  const T *__restrict__ L = buf + bi.base;
+  const T *L = buf + bi.base;
   const long long lda = bi.lda;
   T *gp = pub + bi.voff;
   const int r0 = r * NB, nr = min(NB, bi.a - r0), npiv = min(NB, bi.p - r0);
@@ -1634,7 +1649,7 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
   // lane q dots the tile's columns q, q + kQL, ... with the rows of each chunk
   const int rho = threadIdx.x & (NB - 1), q = threadIdx.x / NB;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const T *__restrict__ Lc = L + (long long)r0 * lda;
+  const T *Lc = L + (long long)r0 * lda;
   // chunks of rows below the pivots, bottom first: non-pivot rows are inputs,
   // pivot tiles publish upwards.  Chunk r itself holds the non-pivot rows of
   // the last pivot tile (if any).
@@ -1739,22 +1754,22 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
     }
     if constexpr (sizeof(T) == sizeof(float)) {
       if (prof) kt_mark(prof, 0, s);
-      count_launch(), pchol_potrf_f32_kernel<<<nblk, kPotrf32Threads, 0, s>>>(
-                          buf, tinv, info, k, diag0, (float)tol, status, (float)drop);
+      count_launch(), launch_pdl(pchol_potrf_f32_kernel, nblk, kPotrf32Threads, 0, s, buf, tinv,
+                                 info, k, diag0, (float)tol, status, (float)drop);
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
-        count_launch(), pchol_trsm_inv_kernel<T><<<dim3((unsigned)maxPanel, nblk), kThreads,
-                                                   trsm_smem<T>(), s>>>(
-                            buf, tinv, info, k, tc ? tc->pstage : nullptr);
+        count_launch(), launch_pdl(pchol_trsm_inv_kernel<T>, dim3((unsigned)maxPanel, nblk),
+                                   kThreads, trsm_smem<T>(), s, buf, tinv, info, k,
+                                   tc ? tc->pstage : nullptr);
     } else {
       if (prof) kt_mark(prof, 0, s);
-      count_launch(), pchol_potrf_kernel<<<nblk, kThreads, 0, s>>>(buf, info, k, diag0, tol,
+      count_launch(), launch_pdl(pchol_potrf_kernel, nblk, kThreads, 0, s, buf, info, k, diag0,
+                                 tol,
                                                                    status, drop);
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
-        count_launch(), pchol_trsm_kernel<T><<<dim3((unsigned)maxPanel, nblk), kThreads,
-                                               trsm_smem<T>(), s>>>(
-                            buf, info, k, dz ? dz->dz_stage : nullptr,
+        count_launch(), launch_pdl(pchol_trsm_kernel<T>, dim3((unsigned)maxPanel, nblk), kThreads,
+                                   trsm_smem<T>(), s, buf, info, k, dz ? dz->dz_stage : nullptr,
                             dz ? dz->dz_exp : nullptr, dz ? dz->stage_slots : 0);
     }
     if (prof) kt_mark(prof, 2, s);
@@ -1764,15 +1779,15 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
           cudaError_t e = launch_update_tc(tc, k, s);
           if (e != cudaSuccess) return e;
         } else {
-          count_launch(), pchol_update_f32_kernel<<<dim3((unsigned)maxTrail, nblk),
-                                                    kUpdF32Threads, 0, s>>>(buf, info, k);
+          count_launch(), launch_pdl(pchol_update_f32_kernel, dim3((unsigned)maxTrail, nblk),
+                                     kUpdF32Threads, 0, s, buf, info, k);
         }
       } else if (dz) {
         cudaError_t e = launch_update_dz(dz, k, s);
         if (e != cudaSuccess) return e;
       } else {
-        count_launch(), pchol_update_kernel<T><<<dim3((unsigned)maxTrail, nblk), kThreads, 0, s>>>(
-                            buf, info, k);
+        count_launch(), launch_pdl(pchol_update_kernel<T>, dim3((unsigned)maxTrail, nblk),
+                                   kThreads, 0, s, buf, info, k);
       }
     }
     if (prof) kt_mark(prof, 3, s);
@@ -1787,8 +1802,9 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
 // ---------------------------------------------------------------------------
 cudaError_t launch_dscale(ahlp_problem *p) {
   if (p->n <= 0) return cudaSuccess;
-  count_launch(), dscale_kernel<<<(unsigned)((p->n + 255) / 256), 256, 0, p->stream>>>(
-      p->x, p->z, p->dscale, p->xinv, p->wfin, p->n, p->fac_rho_x, p->fac_rho, p->is_x0);
+  count_launch(), launch_pdl(dscale_kernel, (unsigned)((p->n + 255) / 256), 256, 0, p->stream,
+                             p->x, p->z, p->dscale, p->xinv, p->wfin, p->n, p->fac_rho_x,
+                             p->fac_rho, p->is_x0);
   return cudaGetLastError();
 }
 
@@ -1797,15 +1813,18 @@ cudaError_t launch_form(ahlp_problem *p, double delta) {
   if (p->fac_prec == kPrecFP32) {
     FormArgs<float> A{nullptr, p->ftiles, p->tile_ent, p->ent_pos, p->ent_cb, p->con_idx,
                       p->con_coef, p->dscale, p->blk, p->aug32, p->diag0, p->cdiag0, delta};
-    count_launch(), form_aug_kernel<float, false><<<(unsigned)p->ntiles, kThreads, 0, p->stream>>>(A);
+    count_launch(), launch_pdl(form_aug_kernel<float, false>, (unsigned)p->ntiles, kThreads, 0,
+                               p->stream, A);
   } else if (p->fac_prec == kPrecFF) {
     FormArgs<float> A{p->aug_lo, p->ftiles, p->tile_ent, p->ent_pos, p->ent_cb, p->con_idx,
                       p->con_coef, p->dscale, p->blk, p->aug32, p->diag0, p->cdiag0, delta};
-    count_launch(), form_aug_kernel<float, true><<<(unsigned)p->ntiles, kThreads, 0, p->stream>>>(A);
+    count_launch(), launch_pdl(form_aug_kernel<float, true>, (unsigned)p->ntiles, kThreads, 0,
+                               p->stream, A);
   } else {
     FormArgs<double> A{nullptr, p->ftiles, p->tile_ent, p->ent_pos, p->ent_cb, p->con_idx,
                        p->con_coef, p->dscale, p->blk, p->aug, p->diag0, p->cdiag0, delta};
-    count_launch(), form_aug_kernel<double, false><<<(unsigned)p->ntiles, kThreads, 0, p->stream>>>(A);
+    count_launch(), launch_pdl(form_aug_kernel<double, false>, (unsigned)p->ntiles, kThreads, 0,
+                               p->stream, A);
   }
   return cudaGetLastError();
 }
@@ -1827,23 +1846,23 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
       if (t * (t + 1) / 2 > maxTrail) maxTrail = t * (t + 1) / 2;
     }
     if (prof) kt_mark(prof, 0, s);
-    count_launch(), pchol_potrf_ff_kernel<<<nblk, kThreads, 0, s>>>(hi, lo, info, k, diag0, tol,
+    count_launch(), launch_pdl(pchol_potrf_ff_kernel, nblk, kThreads, 0, s, hi, lo, info, k, diag0,
+                               tol,
                                                                     status, drop);
     if (prof) kt_mark(prof, 1, s);
     if (maxPanel > 0)
-      count_launch(), pchol_trsm_ff_kernel<<<dim3((unsigned)((maxPanel + kFFRowTiles - 1) /
+      count_launch(), launch_pdl(pchol_trsm_ff_kernel,
+                                 dim3((unsigned)((maxPanel + kFFRowTiles - 1) /
                                                              kFFRowTiles),
-                                                  nblk),
-                                             kFFRowThreads, kTrsmFFSmem, s>>>(
-                          hi, lo, info, k, oz ? oz->dstage : nullptr, oz ? oz->dexp : nullptr);
+                                                  nblk), kFFRowThreads, kTrsmFFSmem, s, hi, lo, info, k, oz ? oz->dstage : nullptr, oz ? oz->dexp : nullptr);
     if (prof) kt_mark(prof, 2, s);
     if (maxTrail > 0) {
       if (oz) {
         cudaError_t e = launch_update_oz(oz, k, s);
         if (e != cudaSuccess) return e;
       } else {
-        count_launch(), pchol_update_ff8_kernel<<<dim3((unsigned)maxTrail, nblk), kUpdFFThreads,
-                                                  kUpdFFSmem, s>>>(hi, lo, info, k);
+        count_launch(), launch_pdl(pchol_update_ff8_kernel, dim3((unsigned)maxTrail, nblk),
+                                   kUpdFFThreads, kUpdFFSmem, s, hi, lo, info, k);
       }
     }
     if (prof) kt_mark(prof, 3, s);
@@ -1851,7 +1870,7 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
     if (e != cudaSuccess) return e;
   }
   if (elems > 0)
-    count_launch(), ff_expand_kernel<<<152 * 8, 256, 0, s>>>(hi, lo, out, elems);
+    count_launch(), launch_pdl(ff_expand_kernel, 152 * 8, 256, 0, s, hi, lo, out, elems);
   return cudaGetLastError();
 }
 
@@ -1869,6 +1888,7 @@ cudaError_t launch_pchol_f32(float *buf, float *tinv, const BlkInfo *info,
 }
 
 __global__ void schur_dy_kernel(const TrsvBwdIO io) {
+  pdl_begin();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < io.nl + io.mg) io.dy[io.msum + q] = io.svec[q < io.nl ? q : q + io.n0];
 }
@@ -1881,25 +1901,29 @@ cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double
   const TrsvBwdIO io{p->svec, p->kmap, p->kmap_off_d, p->yoff_d, dy, p->msum, p->nl, p->n0, p->mg};
   if (njobs == 0) {
     if (!forward && p->nl + p->mg > 0)
-      count_launch(), schur_dy_kernel<<<(p->nl + p->mg + 255) / 256, 256, 0, s>>>(io);
+      count_launch(), launch_pdl(schur_dy_kernel, (p->nl + p->mg + 255) / 256, 256, 0, s, io);
     return cudaGetLastError();
   }
   if (p->fac_prec == kPrecFP32) {
     float *pubb = reinterpret_cast<float *>(p->vecb);
     if (forward)
-      count_launch(), trsv_fwd_kernel<float><<<njobs, TrsvCfg<float, false>::threads, 0, s>>>(
-          p->aug32, p->tinv32, p->blk, sched, ticket, p->trsv_err, p->vec, p->vec32, rhs,
+      count_launch(), launch_pdl(trsv_fwd_kernel<float>, njobs, TrsvCfg<float, false>::threads, 0,
+                                 s, p->aug32, p->tinv32, p->blk, sched, ticket, p->trsv_err,
+                                 p->vec, p->vec32, rhs,
           p->yoff_d);
     else
-      count_launch(), trsv_bwd_kernel<float><<<njobs, TrsvCfg<float, true>::threads, 0, s>>>(
-          p->aug32, p->tinv32, p->blk, sched, ticket, p->trsv_err, p->vec, pubb, io);
+      count_launch(), launch_pdl(trsv_bwd_kernel<float>, njobs, TrsvCfg<float, true>::threads, 0,
+                                 s, p->aug32, p->tinv32, p->blk, sched, ticket, p->trsv_err,
+                                 p->vec, pubb, io);
   } else {
     if (forward)
-      count_launch(), trsv_fwd_kernel<double><<<njobs, TrsvCfg<double, false>::threads, 0, s>>>(
-          p->aug, p->tinv, p->blk, sched, ticket, p->trsv_err, p->vec, p->vec, rhs, p->yoff_d);
+      count_launch(), launch_pdl(trsv_fwd_kernel<double>, njobs, TrsvCfg<double, false>::threads,
+                                 0, s, p->aug, p->tinv, p->blk, sched, ticket, p->trsv_err, p->vec,
+                                 p->vec, rhs, p->yoff_d);
     else
-      count_launch(), trsv_bwd_kernel<double><<<njobs, TrsvCfg<double, true>::threads, 0, s>>>(
-          p->aug, p->tinv, p->blk, sched, ticket, p->trsv_err, p->vec, p->vecb, io);
+      count_launch(), launch_pdl(trsv_bwd_kernel<double>, njobs, TrsvCfg<double, true>::threads, 0,
+                                 s, p->aug, p->tinv, p->blk, sched, ticket, p->trsv_err, p->vec,
+                                 p->vecb, io);
   }
   return cudaGetLastError();
 }
@@ -1908,15 +1932,15 @@ cudaError_t launch_tinv(ahlp_problem *p) {
   // FP32 factors write their inverse tiles in pchol_potrf_f32_kernel; FP64 and
   // float-float factors (through their FP64 copy) get them here
   if (p->trsv_nb == 0 || p->fac_prec == kPrecFP32) return cudaSuccess;
-  count_launch(), tinv_kernel<<<p->trsv_nb, kThreads, kTinvSmem, p->stream>>>(
-      p->aug, p->tinv, p->blk, p->trsv_bsched);
+  count_launch(), launch_pdl(tinv_kernel, p->trsv_nb, kThreads, kTinvSmem, p->stream, p->aug,
+                             p->tinv, p->blk, p->trsv_bsched);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tile_inverses(const double *buf, double *tinv, const BlkInfo *info,
                                  const int *sched, int njobs, cudaStream_t s) {
   if (njobs > 0)
-    count_launch(), tinv_kernel<<<njobs, kThreads, kTinvSmem, s>>>(buf, tinv, info, sched);
+    count_launch(), launch_pdl(tinv_kernel, njobs, kThreads, kTinvSmem, s, buf, tinv, info, sched);
   return cudaGetLastError();
 }
 

@@ -139,6 +139,7 @@ struct DzArgs {
 __global__ void __launch_bounds__(kDzThreads, 1)
     pchol_update_dz_kernel(const DzArgs args, const __grid_constant__ CUtensorMap mapA,
                            const __grid_constant__ CUtensorMap mapB, int njobs) {
+  pdl_wait();
   extern __shared__ __align__(1024) unsigned char dz_raw[];
   __shared__ __align__(8) uint64_t full[kDzStages], empty[kDzStages], tfull, tempty;
   __shared__ uint32_t tmem_slot;
@@ -357,7 +358,8 @@ cudaError_t launch_update_dz(ahlp_problem *p, int k, cudaStream_t s) {
   memcpy(&mA, p->dz_map[0], sizeof mA);
   memcpy(&mB, p->dz_map[1], sizeof mB);
   const int grid = (int)std::min<long long>(jobs, p->num_sms);
-  count_launch(), pchol_update_dz_kernel<<<grid, kDzThreads, kDzSmem, s>>>(a, mA, mB, (int)jobs);
+  count_launch(), launch_pdl(pchol_update_dz_kernel, grid, kDzThreads, kDzSmem, s, a, mA, mB,
+                             (int)jobs);
   return cudaGetLastError();
 }
 

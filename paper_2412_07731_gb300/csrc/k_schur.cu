@@ -54,6 +54,7 @@ __device__ __forceinline__ int border_local(const SchurBlk &s, int n0, int rb) {
 }
 
 __global__ void assemble_T_kernel(SArgs A) {
+  pdl_begin();
   const int j = blockIdx.y;
   const int lj = A.l[j];
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -75,6 +76,7 @@ __global__ void assemble_T_kernel(SArgs A) {
 }
 
 __global__ void assemble_H_kernel(SArgs A) {
+  pdl_begin();
   const int j = blockIdx.y;   // H_j couples pair j+1 (rows) and pair j (cols) through block j+1
   const int lr = A.l[j + 1], lc = A.l[j];
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -87,6 +89,7 @@ __global__ void assemble_H_kernel(SArgs A) {
 }
 
 __global__ void assemble_E_kernel(SArgs A) {
+  pdl_begin();
   const int j = blockIdx.y;
   const int lj = A.l[j];
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -101,6 +104,7 @@ __global__ void assemble_E_kernel(SArgs A) {
 }
 
 __global__ void assemble_SB_kernel(SArgs A) {
+  pdl_begin();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= A.B * A.B) return;
   const int rb = idx % A.B, sb = idx / A.B;
@@ -125,6 +129,7 @@ __global__ void assemble_SB_kernel(SArgs A) {
 
 __global__ void scatter_add_kernel(double *dst, const long long *idx, const double *val,
                                    long long n) {
+  pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[idx[i]] += val[i];
 }
@@ -176,6 +181,7 @@ __device__ __forceinline__ void fwd_subst_regs(double (&z)[kChainRegL], int lj, 
 }
 
 __global__ void __launch_bounds__(512) chain_factor_kernel(CArgs A) {
+  pdl_begin();
   extern __shared__ double T[];   // lmax * lmax
   __shared__ double s_inv;
   __shared__ double Tinv[128];
@@ -393,6 +399,7 @@ __global__ void __launch_bounds__(512) chain_factor_kernel(CArgs A) {
 // only, the operators take one CTA per pair, and Z one warp per border column.
 // --------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) chain_critical_kernel(CArgs A) {
+  pdl_begin();
   extern __shared__ double T[];   // lmax * lmax
   __shared__ double Tinv[kChainRegL], Dg[kChainRegL];
   const int tid = threadIdx.x, bd = blockDim.x;
@@ -481,6 +488,7 @@ __global__ void __launch_bounds__(256) chain_critical_kernel(CArgs A) {
 
 // Linv_j = L_j^-1, Yf_j = Linv_j X_{j-1}, Yb_j = Linv_j' X_j': one CTA per pair
 __global__ void __launch_bounds__(128) chain_ops_kernel(CArgs A) {
+  pdl_begin();
   extern __shared__ double Ls[];   // L_j then Linv_j, lmax * lmax each
   __shared__ double Tinv[kChainRegL];
   const int j = blockIdx.x, tid = threadIdx.x, bd = blockDim.x;
@@ -550,6 +558,7 @@ __global__ void __launch_bounds__(128) chain_ops_kernel(CArgs A) {
 // row r of the current link block): Z_j = Linv_j (E_j' - X_{j-1} Z_{j-1}).
 // Segments outside the column's link rows [zlo, zhi) hold zeros and are skipped.
 __global__ void __launch_bounds__(256) chain_z_kernel(CArgs A, const int *zlo, const int *zhi) {
+  pdl_begin();
   const int rb = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (rb >= A.B) return;   // whole warps leave together
@@ -604,6 +613,7 @@ __global__ void __launch_bounds__(256) chain_z_kernel(CArgs A, const int *zlo, c
 // independent partial sums.
 __global__ void border_prep_kernel(const double *SB, const double *Z, int B, int nl, double *bd,
                                    int ld, double *bdiag0, const int *zlo, const int *zhi) {
+  pdl_begin();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= B * B) return;
   const int rb = idx % B, sb = idx / B;
@@ -627,6 +637,7 @@ __global__ void border_prep_kernel(const double *SB, const double *Z, int B, int
 // after eliminating the x_0 pivots the y_g corner holds -P; flip its sign
 __global__ void negate_corner_kernel(double *bd, int ld, int n0, int mg, double *bdiag0,
                                      const double *sb_ref) {
+  pdl_begin();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= mg * mg) return;
   const int r = idx % mg, s = idx / mg;
@@ -651,6 +662,7 @@ __global__ void prep_f_kernel(double *f, double *g, const double *rd, const doub
                               const unsigned char *is_x0, long long n, int adjoint, int *ticket,
                               unsigned *pub_fwd, unsigned *pub_bwd, long long fwd_words,
                               long long bwd_words) {
+  pdl_begin();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
   if (i < 2) ticket[i] = 0;
@@ -678,6 +690,7 @@ struct RArgs {
 // a fixed shuffle tree adds the lanes.  Launch: link_ctas CTAs of 256 threads
 // for the link rows, then ceil(B / 8) CTAs for the border rows.
 __global__ void schur_rhs_kernel(RArgs A, int link_ctas) {
+  pdl_begin();
   if ((int)blockIdx.x < link_ctas) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= A.nl) return;
@@ -722,6 +735,7 @@ constexpr int kChainSolveThreads = 1024;
 __global__ void __launch_bounds__(kChainSolveThreads) chain_solve_kernel(CArgs A, double *u,
                                                                          int dir, int stages,
                                                                          int lmax) {
+  pdl_begin();
   extern __shared__ double opbuf[];               // operators of one batch, then its tmp rows
   double *tbuf = opbuf + (size_t)stages * lmax * lmax;
   __shared__ double ubuf[2][kChainMaxL];          // solution of the previous pair
@@ -828,10 +842,11 @@ __global__ void __launch_bounds__(kChainSolveThreads) chain_solve_kernel(CArgs A
 // two rows, so the columns of L it streams serve both.
 constexpr int kBinvThreads = 256;
 
-__global__ void __launch_bounds__(kBinvThreads) border_inv_kernel(const double *__restrict__ L,
-                                                                  const double *__restrict__ X,
+__global__ void __launch_bounds__(kBinvThreads) border_inv_kernel(const double *L,
+                                                                  const double *X,
                                                                   int B, int ld, double *Wr,
                                                                   double *Wc) {
+  pdl_begin();
   __shared__ double xs[NB][NB + 1];   // xs[c][q] = X_jj(q, c)
   __shared__ double v[2][NB];
   const int r0 = 2 * blockIdx.x, r1 = min(r0 + 1, B - 1);
@@ -877,9 +892,10 @@ __global__ void __launch_bounds__(kBinvThreads) border_inv_kernel(const double *
 }
 
 // border rhs: sB -= Z' uT, one CTA per border row over its column's link rows
-__global__ void __launch_bounds__(128) border_rhs_kernel(const double *__restrict__ Z, int nl,
+__global__ void __launch_bounds__(128) border_rhs_kernel(const double *Z, int nl,
                                                          const int *zlo, const int *zhi,
                                                          double *svec) {
+  pdl_begin();
   __shared__ double part[4];
   const int rb = blockIdx.x;
   const double *zc = Z + (long long)rb * nl;
@@ -901,9 +917,10 @@ __global__ void __launch_bounds__(128) border_rhs_kernel(const double *__restric
 }
 
 // t = J W b (fwd, W's rows) or x = W' t (columns), one warp per entry
-__global__ void __launch_bounds__(256) border_w_kernel(const double *__restrict__ W, int B, int ld,
-                                                       int n0, const double *__restrict__ in,
+__global__ void __launch_bounds__(256) border_w_kernel(const double *W, int B, int ld,
+                                                       int n0, const double *in,
                                                        double *out, int fwd) {
+  pdl_begin();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= B) return;
   const double *w = W + (long long)i * ld;
@@ -924,8 +941,9 @@ __global__ void __launch_bounds__(256) border_w_kernel(const double *__restrict_
 
 // uT -= Z sB: a CTA takes 32 link rows, 16 threads per row share the border
 // columns (one thread per row walked all of them: 28 us at 100, 156 us at 601)
-__global__ void __launch_bounds__(512) link_back_kernel(const double *__restrict__ Z, int B,
+__global__ void __launch_bounds__(512) link_back_kernel(const double *Z, int B,
                                                         int nl, double *svec) {
+  pdl_begin();
   __shared__ double part[16][32];
   const int rr = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int q = blockIdx.x * 32 + rr;
@@ -972,16 +990,22 @@ cudaError_t launch_schur_assemble(ahlp_problem *p, double delta, double rho) {
   int lmax = 0;
   for (int j = 0; j + 1 < p->N; ++j) lmax = std::max(lmax, (int)(p->link_off[j + 1] - p->link_off[j]));
   if (p->N > 1 && lmax > 0) {
-    count_launch(), assemble_T_kernel<<<dim3(nb((long long)lmax * lmax, 256), p->N - 1), 256, 0, s>>>(A);
+    count_launch(), launch_pdl(assemble_T_kernel, dim3(nb((long long)lmax * lmax, 256), p->N - 1),
+                               256, 0, s, A);
     if (p->N > 2)
-      count_launch(), assemble_H_kernel<<<dim3(nb((long long)lmax * lmax, 256), p->N - 2), 256, 0, s>>>(A);
+      count_launch(), launch_pdl(assemble_H_kernel, dim3(nb((long long)lmax * lmax, 256),
+                                 p->N - 2), 256, 0, s, A);
     if (p->B > 0)
-      count_launch(), assemble_E_kernel<<<dim3(nb((long long)lmax * p->B, 256), p->N - 1), 256, 0, s>>>(A);
+      count_launch(), launch_pdl(assemble_E_kernel, dim3(nb((long long)lmax * p->B, 256),
+                                 p->N - 1), 256, 0, s, A);
   }
-  if (p->B > 0) count_launch(), assemble_SB_kernel<<<nb((long long)p->B * p->B, 256), 256, 0, s>>>(A);
-  if (p->nf0 > 0) count_launch(), scatter_add_kernel<<<nb(p->nf0, 256), 256, 0, s>>>(p->Et, p->f0_idx, p->f0_val, p->nf0);
+  if (p->B > 0) count_launch(), launch_pdl(assemble_SB_kernel, nb((long long)p->B * p->B, 256),
+                                        256, 0, s, A);
+  if (p->nf0 > 0) count_launch(), launch_pdl(scatter_add_kernel, nb(p->nf0, 256), 256, 0, s, p->Et,
+                                        p->f0_idx, p->f0_val, p->nf0);
   if (p->nfg0 > 0)
-    count_launch(), scatter_add_kernel<<<nb(p->nfg0, 256), 256, 0, s>>>(p->SB, p->fg0_idx, p->fg0_val, p->nfg0);
+    count_launch(), launch_pdl(scatter_add_kernel, nb(p->nfg0, 256), 256, 0, s, p->SB, p->fg0_idx,
+                               p->fg0_val, p->nfg0);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // keep the assembled matrix for diagnostics
@@ -1005,19 +1029,23 @@ cudaError_t launch_schur_factor(ahlp_problem *p) {
       if (e != cudaSuccess) return e;
     } else if (p->nchain_seg > 0 && lmax <= kChainRegL) {
       const CArgs A = cargs(p);
-      count_launch(), chain_critical_kernel<<<p->nchain_seg, 256, (size_t)lmax * lmax * 8, s>>>(A);
-      count_launch(), chain_ops_kernel<<<p->N - 1, 128, (size_t)2 * lmax * lmax * 8, s>>>(A);
+      count_launch(), launch_pdl(chain_critical_kernel, p->nchain_seg, 256,
+                                 (size_t)lmax * lmax * 8, s, A);
+      count_launch(), launch_pdl(chain_ops_kernel, p->N - 1, 128, (size_t)2 * lmax * lmax * 8, s,
+                                 A);
       if (p->B > 0)
-        count_launch(), chain_z_kernel<<<(unsigned)((p->B + 7) / 8), 256, 0, s>>>(A, p->zlo,
+        count_launch(), launch_pdl(chain_z_kernel, (unsigned)((p->B + 7) / 8), 256, 0, s, A,
+                                   p->zlo,
                                                                                    p->zhi);
     } else if (p->nchain_seg > 0) {
-      count_launch(), chain_factor_kernel<<<p->nchain_seg, 512, (size_t)lmax * lmax * 8, s>>>(
-          cargs(p));
+      count_launch(), launch_pdl(chain_factor_kernel, p->nchain_seg, 512, (size_t)lmax * lmax * 8,
+                                 s, cargs(p));
     }
   }
   if (p->B > 0) {
-    count_launch(), border_prep_kernel<<<nb((long long)p->B * p->B, 256), 256, 0, s>>>(
-        p->SB, p->Et, p->B, p->nl, p->border, p->Bld, p->border_diag0, p->zlo, p->zhi);
+    count_launch(), launch_pdl(border_prep_kernel, nb((long long)p->B * p->B, 256), 256, 0, s,
+                               p->SB, p->Et, p->B, p->nl, p->border, p->Bld, p->border_diag0,
+                               p->zlo, p->zhi);
     std::vector<BlkInfo> hx(1, p->h_bx);
     if (p->n0 > 0) {
       cudaError_t e = launch_pchol(p->border, p->bx_info, hx, p->border_diag0, p->fac_pivot_tol,
@@ -1025,8 +1053,8 @@ cudaError_t launch_schur_factor(ahlp_problem *p) {
       if (e != cudaSuccess) return e;
     }
     if (p->mg > 0) {
-      count_launch(), negate_corner_kernel<<<nb((long long)p->mg * p->mg, 256), 256, 0, s>>>(
-          p->border, p->Bld, p->n0, p->mg, p->border_diag0, p->sb_ref);
+      count_launch(), launch_pdl(negate_corner_kernel, nb((long long)p->mg * p->mg, 256), 256, 0,
+                                 s, p->border, p->Bld, p->n0, p->mg, p->border_diag0, p->sb_ref);
       std::vector<BlkInfo> hp(1, p->h_bp);
       cudaError_t e = launch_pchol(p->border, p->bp_info, hp, p->border_diag0, p->fac_pivot_tol,
                                    p->status, s);
@@ -1035,8 +1063,8 @@ cudaError_t launch_schur_factor(ahlp_problem *p) {
     const int T = (p->B + NB - 1) / NB;
     cudaError_t e = launch_tile_inverses(p->border, p->border_tinv, p->bw_info, p->bw_sched, T, s);
     if (e != cudaSuccess) return e;
-    count_launch(), border_inv_kernel<<<(p->B + 1) / 2, kBinvThreads, 0, s>>>(
-        p->border, p->border_tinv, p->B, p->Bld, p->border_wr, p->border_wc);
+    count_launch(), launch_pdl(border_inv_kernel, (p->B + 1) / 2, kBinvThreads, 0, s, p->border,
+                               p->border_tinv, p->B, p->Bld, p->border_wr, p->border_wc);
   }
   return cudaGetLastError();
 }
@@ -1049,8 +1077,9 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
   cudaError_t e;
   const bool f32 = p->fac_prec == kPrecFP32;
   const long long words = p->vec_elems * (f32 ? 1 : 2);
-  count_launch(), prep_f_kernel<<<nb(std::max<long long>(n, 2), 256), 256, 0, s>>>(
-      p->f, p->g, r_d, r_c, p->xinv, p->z, p->dscale, p->is_x0, n, adjoint ? 1 : 0, p->trsv_ticket,
+  count_launch(), launch_pdl(prep_f_kernel, nb(std::max<long long>(n, 2), 256), 256, 0, s, p->f,
+                             p->g, r_d, r_c, p->xinv, p->z, p->dscale, p->is_x0, n,
+                             adjoint ? 1 : 0, p->trsv_ticket,
       f32 ? reinterpret_cast<unsigned *>(p->vec32) : reinterpret_cast<unsigned *>(p->vec),
       reinterpret_cast<unsigned *>(p->vecb), words, words);
   e = launch_spmv(p->Amat, p->g, p->rhat, 1.0, r_p, s);
@@ -1066,7 +1095,8 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
             p->xoff[p->N], p->svec};
     {
       const int link_ctas = (int)nb(p->nl, 256);
-      count_launch(), schur_rhs_kernel<<<link_ctas + (int)nb(p->B, 8), 256, 0, s>>>(R, link_ctas);
+      count_launch(), launch_pdl(schur_rhs_kernel, link_ctas + (int)nb(p->B, 8), 256, 0, s, R,
+                                 link_ctas);
     }
     CArgs C = cargs(p);
     // one stage = one operator (<= lmax^2) plus one pair's rows (<= lmax); the
@@ -1081,21 +1111,24 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
         e = launch_bcr_solve(p, p->svec, true);
         if (e != cudaSuccess) return e;
       } else {
-        count_launch(), chain_solve_kernel<<<p->nchain_seg, kChainSolveThreads, csm, s>>>(
-            C, p->svec, 0, stages, lmax);
+        count_launch(), launch_pdl(chain_solve_kernel, p->nchain_seg, kChainSolveThreads, csm, s,
+                                   C, p->svec, 0, stages, lmax);
       }
     }
     if (p->B > 0) {
       if (p->nl > 0)
-        count_launch(), border_rhs_kernel<<<p->B, 128, 0, s>>>(p->Et, p->nl, p->zlo, p->zhi,
+        count_launch(), launch_pdl(border_rhs_kernel, p->B, 128, 0, s, p->Et, p->nl, p->zlo,
+                                   p->zhi,
                                                                p->svec);
       double *sb = p->svec + p->nl;
-      count_launch(), border_w_kernel<<<nb(p->B, 8), 256, 0, s>>>(p->border_wr, p->B, p->Bld,
+      count_launch(), launch_pdl(border_w_kernel, nb(p->B, 8), 256, 0, s, p->border_wr, p->B,
+                                 p->Bld,
                                                                   p->n0, sb, p->border_t, 1);
-      count_launch(), border_w_kernel<<<nb(p->B, 8), 256, 0, s>>>(p->border_wc, p->B, p->Bld,
+      count_launch(), launch_pdl(border_w_kernel, nb(p->B, 8), 256, 0, s, p->border_wc, p->B,
+                                 p->Bld,
                                                                   p->n0, p->border_t, sb, 0);
       if (p->nl > 0)
-        count_launch(), link_back_kernel<<<nb(p->nl, 32), 512, 0, s>>>(p->Et, p->B, p->nl,
+        count_launch(), launch_pdl(link_back_kernel, nb(p->nl, 32), 512, 0, s, p->Et, p->B, p->nl,
                                                                        p->svec);
     }
     if (p->nl > 0 && lmax > 0 && p->nchain_seg > 0) {
@@ -1103,8 +1136,8 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
         e = launch_bcr_solve(p, p->svec, false);
         if (e != cudaSuccess) return e;
       } else {
-        count_launch(), chain_solve_kernel<<<p->nchain_seg, kChainSolveThreads, csm, s>>>(
-            C, p->svec, 1, stages, lmax);
+        count_launch(), launch_pdl(chain_solve_kernel, p->nchain_seg, kChainSolveThreads, csm, s,
+                                   C, p->svec, 1, stages, lmax);
       }
     }
   }

@@ -96,6 +96,7 @@ struct TcArgs {
 };
 
 __global__ void __launch_bounds__(kTcThreads) pchol_update_tc_kernel(const TcArgs args) {
+  pdl_wait();
   extern __shared__ __align__(1024) unsigned char tc_raw[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t tmem_slot;
@@ -247,6 +248,7 @@ constexpr uint32_t kTc2Smem = 2 * kTc2Stage + kTcM * kTcN * 4 + 1024;  // 2 stag
 
 __global__ void __launch_bounds__(kTc2Threads, 1) pchol_update_tc2_kernel(const TcArgs args,
                                                                          int njobs) {
+  pdl_wait();
   extern __shared__ __align__(1024) unsigned char tc2_raw[];
   __shared__ __align__(8) uint64_t full[2], empty[2], tfull[2], tempty[2];
   __shared__ uint32_t tmem_slot;
@@ -513,6 +515,7 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *tm, int x, int y
 }
 
 __global__ void __launch_bounds__(kTcThreads) pchol_update_oz_kernel(const OzArgs args) {
+  pdl_wait();
   extern __shared__ __align__(1024) unsigned char oz_raw[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t tmem_slot;
@@ -722,6 +725,7 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *tm, int x, in
 
 __global__ void __launch_bounds__(kOz2Threads, 1) pchol_update_oz2_kernel(const OzArgs args,
                                                                          int njobs) {
+  pdl_wait();
   extern __shared__ __align__(1024) unsigned char oz2_raw[];
   __shared__ __align__(8) uint64_t full[kOz2Stages], empty[kOz2Stages], tfull, tempty;
   __shared__ uint32_t tmem_slot;
@@ -1102,9 +1106,11 @@ cudaError_t launch_update_tc(ahlp_problem *p, int k, cudaStream_t s) {
            p->status, p->tc_jtab ? p->tc_jtab + p->tc_jtab_off[k] : nullptr};
   if (p->fp32_update == 3) {   // persistent pipeline: one CTA per SM
     const int grid = (int)std::min<long long>(jobs, p->num_sms);
-    count_launch(), pchol_update_tc2_kernel<<<grid, kTc2Threads, kTc2Smem, s>>>(a, (int)jobs);
+    count_launch(), launch_pdl(pchol_update_tc2_kernel, grid, kTc2Threads, kTc2Smem, s, a,
+                               (int)jobs);
   } else {
-    count_launch(), pchol_update_tc_kernel<<<(unsigned)jobs, kTcThreads, kSmemBytes, s>>>(a);
+    count_launch(), launch_pdl(pchol_update_tc_kernel, (unsigned)jobs, kTcThreads, kSmemBytes, s,
+                               a);
   }
   return cudaGetLastError();
 }
@@ -1154,9 +1160,10 @@ cudaError_t launch_update_oz(ahlp_problem *p, int k, cudaStream_t s) {
            p->tc_jtab ? p->tc_jtab + p->tc_jtab_off[k] : nullptr};
   if (p->ff_update == 3) {   // persistent pipeline: one CTA per SM
     const int grid = (int)std::min<long long>(jobs, p->num_sms);
-    count_launch(), pchol_update_oz2_kernel<<<grid, kOz2Threads, kOz2Smem, s>>>(a, (int)jobs);
+    count_launch(), launch_pdl(pchol_update_oz2_kernel, grid, kOz2Threads, kOz2Smem, s, a,
+                               (int)jobs);
   } else {
-    count_launch(), pchol_update_oz_kernel<<<(unsigned)jobs, kTcThreads, kOzSmem, s>>>(a);
+    count_launch(), launch_pdl(pchol_update_oz_kernel, (unsigned)jobs, kTcThreads, kOzSmem, s, a);
   }
   return cudaGetLastError();
 }

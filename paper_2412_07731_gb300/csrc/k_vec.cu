@@ -106,6 +106,7 @@ struct RedSet {
 
 __global__ void __launch_bounds__(kRedThreads) reduce_set_kernel(const RedSet S, double *part,
                                                                  int *cnt) {
+  pdl_begin();
   __shared__ double sh[kRedThreads / 32];
   const RedArgs &r = S.r[blockIdx.y];
   const int nb = S.nb[blockIdx.y];
@@ -284,6 +285,7 @@ __device__ __forceinline__ void sp_short(const SpSeg &S, const SpTailArgs &T, lo
 template <int TAIL>
 __global__ void __launch_bounds__(kSpThreads) spmv_kernel(const SpSeg a, const SpSeg b,
                                                           const SpTailArgs T) {
+  pdl_begin();
   __shared__ double part[8];
   long long c = blockIdx.x;
   const long long na = (a.rows + kSpThreads - 1) / kSpThreads;
@@ -296,16 +298,19 @@ __global__ void __launch_bounds__(kSpThreads) spmv_kernel(const SpSeg a, const S
 }
 
 __global__ void axpby_k(double *y, const double *x, double a, double b, long long n) {
+  pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = a * x[i] + b * y[i];
 }
 
 __global__ void fill_k(double *y, double v, long long n) {
+  pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = v;
 }
 
 __global__ void mul_k(double *y, const double *a, const double *b, double sc, long long n) {
+  pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = sc * a[i] * b[i];
 }
@@ -313,6 +318,7 @@ __global__ void mul_k(double *y, const double *a, const double *b, double sc, lo
 // r_c = sigma_mu - x z - dxa dza
 __global__ void ipm_rc_k(double *rc, const double *x, const double *z, const double *dxa,
                          const double *dza, double smu, long long n) {
+  pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) rc[i] = smu - x[i] * z[i] - (dxa ? dxa[i] * dza[i] : 0.0);
 }
@@ -320,6 +326,7 @@ __global__ void ipm_rc_k(double *rc, const double *x, const double *z, const dou
 __global__ void centrality_rc_k(double *rc2, const double *rc, const double *x, const double *dx,
                                 double ap, const double *z, const double *dz, double ad,
                                 double lo, double hi, long long n) {
+  pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double v = (x[i] + ap * dx[i]) * (z[i] + ad * dz[i]);
@@ -329,6 +336,7 @@ __global__ void centrality_rc_k(double *rc2, const double *rc, const double *x, 
 }
 
 __global__ void add_scalar_k(double *y, const double *x, double s, long long n) {
+  pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = x[i] + s;
 }
@@ -337,11 +345,12 @@ __global__ void add_scalar_k(double *y, const double *x, double s, long long n) 
 // at a time: w is read once per eight, and the eight per-thread sums are added
 // across a warp by a transposing exchange (9 FP64 additions instead of 40).
 // The last CTA adds the partial sums in a fixed order.
-__global__ void __launch_bounds__(kRedThreads) mdot_kernel(const double *__restrict__ V,
+__global__ void __launch_bounds__(kRedThreads) mdot_kernel(const double *V,
                                                            long long ld, int k,
-                                                           const double *__restrict__ w,
+                                                           const double *w,
                                                            long long len, double *part,
                                                            double *out, int *cnt) {
+  pdl_begin();
   __shared__ double sh[8][kRedThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -395,13 +404,14 @@ __global__ void __launch_bounds__(kRedThreads) mdot_kernel(const double *__restr
 // pieces (w0, w1, w2 of lengths n0, n1 and the rest; V_i contiguous).  With
 // nrm2 the last CTA also leaves nrm2[0] = <w, w> and nrm2[1] = 1 / |w| (1 when
 // <w, w> is not positive).
-__global__ void __launch_bounds__(kRedThreads) maxpy_kernel(const double *__restrict__ V,
+__global__ void __launch_bounds__(kRedThreads) maxpy_kernel(const double *V,
                                                             long long ld, int k,
-                                                            const double *__restrict__ coef,
+                                                            const double *coef,
                                                             double sc, double *w0, long long n0,
                                                             double *w1, long long n1, double *w2,
                                                             long long len, double *part,
                                                             double *nrm2, int *cnt) {
+  pdl_begin();
   __shared__ double cs[kMaxKrylov + 1];
   __shared__ double sh[kRedThreads / 32];
   for (int i = threadIdx.x; i < k; i += blockDim.x) cs[i] = sc * coef[i];
@@ -431,6 +441,7 @@ __global__ void __launch_bounds__(kRedThreads) maxpy_kernel(const double *__rest
 
 // y = a x, a on the device (da) or not
 __global__ void scale_k(double *y, const double *x, const double *da, double a, long long n) {
+  pdl_begin();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = (da ? *da : a) * x[i];
 }
@@ -442,8 +453,8 @@ inline unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) /
 cudaError_t launch_mdot(ahlp_problem *p, const double *V, long long ld, int k, const double *w,
                         long long len, double *out) {
   if (k <= 0) return cudaSuccess;
-  count_launch(), mdot_kernel<<<red_blocks(len, kMdotBlocks), kRedThreads, 0, p->stream>>>(
-      V, ld, k, w, len, p->mdot_part, out, p->red_cnt + kRedSetMax);
+  count_launch(), launch_pdl(mdot_kernel, red_blocks(len, kMdotBlocks), kRedThreads, 0, p->stream,
+                             V, ld, k, w, len, p->mdot_part, out, p->red_cnt + kRedSetMax);
   return cudaGetLastError();
 }
 
@@ -456,8 +467,9 @@ cudaError_t launch_maxpy3(ahlp_problem *p, const double *V, long long ld, int k,
                           const double *coef, double *w0, long long n0, double *w1, long long n1,
                           double *w2, long long len, double sign, double *nrm2) {
   if (k <= 0 || len <= 0) return cudaSuccess;
-  count_launch(), maxpy_kernel<<<red_blocks(len, kMaxpyBlocks), kRedThreads, 0, p->stream>>>(
-      V, ld, k, coef, sign, w0, n0, w1, n1, w2, len, p->red_part, nrm2,
+  count_launch(), launch_pdl(maxpy_kernel, red_blocks(len, kMaxpyBlocks), kRedThreads, 0,
+                             p->stream, V, ld, k, coef, sign, w0, n0, w1, n1, w2, len, p->red_part,
+                             nrm2,
       p->red_cnt + kRedSetMax + 1);
   return cudaGetLastError();
 }
@@ -465,13 +477,13 @@ cudaError_t launch_maxpy3(ahlp_problem *p, const double *V, long long ld, int k,
 cudaError_t launch_scale(double *y, const double *x, const double *da, double a, long long len,
                          cudaStream_t s) {
   if (len <= 0) return cudaSuccess;
-  count_launch(), scale_k<<<blocks_for(len, 256), 256, 0, s>>>(y, x, da, a, len);
+  count_launch(), launch_pdl(scale_k, blocks_for(len, 256), 256, 0, s, y, x, da, a, len);
   return cudaGetLastError();
 }
 
 cudaError_t launch_add_scalar(double *y, const double *x, double s, long long n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  count_launch(), add_scalar_k<<<blocks_for(n, 256), 256, 0, st>>>(y, x, s, n);
+  count_launch(), launch_pdl(add_scalar_k, blocks_for(n, 256), 256, 0, st, y, x, s, n);
   return cudaGetLastError();
 }
 
@@ -487,7 +499,8 @@ cudaError_t launch_reduce_set(ahlp_problem *p, const RedOne *ops, int n) {
       S.nb[i] = red_blocks(o.len, kRedBlocks);
       nb = std::max(nb, S.nb[i]);
     }
-    count_launch(), reduce_set_kernel<<<dim3(nb, c), kRedThreads, 0, p->stream>>>(S, p->red_part,
+    count_launch(), launch_pdl(reduce_set_kernel, dim3(nb, c), kRedThreads, 0, p->stream, S,
+                               p->red_part,
                                                                                 p->red_cnt);
   }
   return cudaGetLastError();
@@ -518,7 +531,8 @@ cudaError_t launch_spmv(const SpMat &A, const double *x, double *y, double alpha
                         const double *yadd, cudaStream_t s) {
   if (A.rows <= 0) return cudaSuccess;
   const SpSeg a = sp_seg(A, x, y, alpha, yadd);
-  count_launch(), spmv_kernel<SP_STORE><<<sp_ctas(a), kSpThreads, 0, s>>>(a, SpSeg{}, SpTailArgs{});
+  count_launch(), launch_pdl(spmv_kernel<SP_STORE>, sp_ctas(a), kSpThreads, 0, s, a, SpSeg{},
+                             SpTailArgs{});
   return cudaGetLastError();
 }
 
@@ -538,7 +552,8 @@ cudaError_t launch_finish(ahlp_problem *p, const double *dy, const double *rc, d
   T.wx = wx;
   T.wc = wc;
   T.adjoint = adjoint ? 1 : 0;
-  count_launch(), spmv_kernel<SP_FINISH><<<sp_ctas(a), kSpThreads, 0, p->stream>>>(a, SpSeg{}, T);
+  count_launch(), launch_pdl(spmv_kernel<SP_FINISH>, sp_ctas(a), kSpThreads, 0, p->stream, a,
+                             SpSeg{}, T);
   return cudaGetLastError();
 }
 
@@ -556,7 +571,8 @@ cudaError_t launch_residual(ahlp_problem *p, const double *r_d, const double *r_
   T.rc = r_c;
   T.e_c = e_c;
   T.adjoint = adjoint ? 1 : 0;
-  count_launch(), spmv_kernel<SP_RESID><<<sp_ctas(a) + sp_ctas(b), kSpThreads, 0, p->stream>>>(a, b,
+  count_launch(), launch_pdl(spmv_kernel<SP_RESID>, sp_ctas(a) + sp_ctas(b), kSpThreads, 0,
+                             p->stream, a, b,
                                                                                               T);
   return cudaGetLastError();
 }
@@ -564,27 +580,28 @@ cudaError_t launch_residual(ahlp_problem *p, const double *r_d, const double *r_
 cudaError_t launch_axpby(double *y, const double *x, double a, double b, long long n,
                          cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  count_launch(), axpby_k<<<blocks_for(n, 256), 256, 0, s>>>(y, x, a, b, n);
+  count_launch(), launch_pdl(axpby_k, blocks_for(n, 256), 256, 0, s, y, x, a, b, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fill(double *y, double v, long long n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  count_launch(), fill_k<<<blocks_for(n, 256), 256, 0, s>>>(y, v, n);
+  count_launch(), launch_pdl(fill_k, blocks_for(n, 256), 256, 0, s, y, v, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_mul(double *y, const double *a, const double *b, double scale, long long n,
                        cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  count_launch(), mul_k<<<blocks_for(n, 256), 256, 0, s>>>(y, a, b, scale, n);
+  count_launch(), launch_pdl(mul_k, blocks_for(n, 256), 256, 0, s, y, a, b, scale, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ipm_rc(double *rc, const double *x, const double *z, const double *dxa,
                           const double *dza, double sigma_mu, long long n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  count_launch(), ipm_rc_k<<<blocks_for(n, 256), 256, 0, s>>>(rc, x, z, dxa, dza, sigma_mu, n);
+  count_launch(), launch_pdl(ipm_rc_k, blocks_for(n, 256), 256, 0, s, rc, x, z, dxa, dza, sigma_mu,
+                             n);
   return cudaGetLastError();
 }
 
@@ -592,7 +609,8 @@ cudaError_t launch_centrality_rc(double *rc2, const double *rc, const double *x,
                                  const double *dx, double ap, const double *z, const double *dz,
                                  double ad, double lo, double hi, long long n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  count_launch(), centrality_rc_k<<<blocks_for(n, 256), 256, 0, s>>>(rc2, rc, x, dx, ap, z, dz, ad,
+  count_launch(), launch_pdl(centrality_rc_k, blocks_for(n, 256), 256, 0, s, rc2, rc, x, dx, ap, z,
+                             dz, ad,
                                                                      lo, hi, n);
   return cudaGetLastError();
 }
