@@ -186,20 +186,21 @@ typedef struct {
                            timings; 0: up to max_correctors regardless (1)     */
   int32_t fp32_update;  /* trailing updates of FP32 block factors: 0 = tensor
                            cores when available (tcgen05, TF32 hi/lo split
-                           operands, FP32 accumulation), 1 = FP32 pipe,
+                           operands, FP32 accumulation; 2 or 3 by the number
+                           of tiles of a step, the same factor), 1 = FP32 pipe,
                            2 = tensor cores, one CTA per 128 x 64 output tile,
                            3 = tensor cores, one persistent CTA per SM that
                            overlaps the copies, products and reduce of
                            consecutive tiles (2 and 3: AHLP_ERR_UNSUPPORTED
                            when the driver cannot encode tensor maps) (0)      */
-  int32_t ff_update;    /* trailing updates of float-float block factors: 0 or 2 =
+  int32_t ff_update;    /* trailing updates of float-float block factors: 2 =
                            tensor cores (each panel entry as six FP16 integer
                            digits under a per-row exponent, the digit products
                            accumulated exactly in FP32, 49 bits in all), one
                            CTA per 128 x 64 output tile; 3 = the same products
                            in one persistent CTA per SM that overlaps the
                            copies, products and C-tile update of consecutive
-                           tiles (bitwise the same factor); 1 = double-float
+                           tiles (bitwise the same factor); 0 = 3; 1 = double-float
                            arithmetic on the FP32 pipe.  0, 2 and 3 fall back
                            to 1 when the driver cannot encode tensor maps (0) */
   int32_t schur_chain;  /* factor and solves of the block-tridiagonal link chain

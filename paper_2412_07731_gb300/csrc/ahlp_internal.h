@@ -294,7 +294,8 @@ struct ahlp_problem {
   int *dexp = nullptr;
   bool oz_ready = false;
   void *oz_tmap = nullptr;           // [2N] CUtensorMap: each block's hi, then lo matrix
-  int ff_update = 0;                 // trailing update of float-float factors: 1 FP32 pipe, 2 tensor cores
+  int ff_update = 0;                 // trailing update of float-float factors: 1 FP32 pipe, 2 tensor
+                                     // cores (one CTA per job), 3 tensor cores (persistent)
   // per block, T x T: lower tile (I, J) of the formed augmented matrix has entries
   std::vector<std::vector<unsigned char>> tile_nz;
   // tile-sparse update jobs (option tile_sparse): per step, the kept jobs of the
@@ -304,7 +305,7 @@ struct ahlp_problem {
   long long tc_jobs_dense = 0, tc_jobs_kept = 0;
   int fp32_update = 0;               // trailing update of FP32 factors: 1 SIMT, 2 tensor
                                      // cores (one CTA per job), 3 tensor cores (persistent
-                                     // warp-specialised pipeline)
+                                     // warp-specialised pipeline), 0 either, by the jobs of a step
   int num_sms = 1;
   double fac_flops = 0;   // algorithmic flops of one batched partial Cholesky
   double tri_elems = 0;   // lower-triangle entries of all augmented matrices
@@ -342,6 +343,7 @@ struct ahlp_problem {
   std::vector<int> bcr_loff;
   int bcr_lmax = 0;
   double *bcr_GL = nullptr, *bcr_GR = nullptr;
+  double *bcr_pub = nullptr;   // [2 nl] published forward, then backward chain solution
   bool fac_bcr = false;   // the current Schur factor's chain is the cyclic-reduction one
   long long *yoff_d = nullptr;       // [N] start of y_i
   long long *kmap_off_d = nullptr;   // [N]
@@ -383,10 +385,10 @@ struct ahlp_problem {
   double *h_scal = nullptr;   // pinned host scalars
   int *status = nullptr;      // device status words [4]
   // wavefront block solves: (block, row tile) jobs in ticket order, and the
-  // forward and backward ticket counters (zeroed by the first kernel of a solve,
-  // which also fills the publication buffers)
+  // ticket counters of the forward and backward block and chain solves (zeroed by
+  // the first kernel of a solve, which also fills the publication buffers)
   int *trsv_fsched = nullptr, *trsv_bsched = nullptr;   // [2 * jobs]
-  int *trsv_ticket = nullptr;     // [2]
+  int *trsv_ticket = nullptr;     // [4]
   int *trsv_err = nullptr;        // set when a wait timed out
   int trsv_nf = 0, trsv_nb = 0;
   int tiny_pivots = 0;
@@ -457,9 +459,10 @@ cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double
 cudaError_t launch_schur_assemble(ahlp_problem *p, double delta, double rho);
 cudaError_t launch_schur_factor(ahlp_problem *p);
 // cyclic reduction of the link chain: factor (T_j, Linv_j, GL_j, GR_j, and Z
-// into Et) and the forward / backward solves in place on the link part of u
+// into Et); forward solve of svec's link part into bcr_pub, backward solve in
+// place on svec's link part
 cudaError_t launch_bcr_factor(ahlp_problem *p);
-cudaError_t launch_bcr_solve(ahlp_problem *p, double *u, bool forward);
+cudaError_t launch_bcr_solve(ahlp_problem *p, bool forward);
 cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
                          const double *r_c, double *dx, double *dy, double *dz, bool adjoint,
                          double *wx = nullptr, double *wc = nullptr);

@@ -1148,7 +1148,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
       p->trsv_nb = (int)bs.size() / 2;
       if (!fs.empty()) p->trsv_fsched = dupload(p, fs);
       if (!bs.empty()) p->trsv_bsched = dupload(p, bs);
-      p->trsv_ticket = dalloc<int>(p, 2);
+      p->trsv_ticket = dalloc<int>(p, 4);
       p->trsv_err = dalloc<int>(p, 1);
       ck(cudaMemset(p->trsv_err, 0, sizeof(int)), "memset");
     }
@@ -1227,6 +1227,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
           p->bcr_info = dupload(p, info);
           p->bcr_GL = dalloc<double>(p, (long long)(N - 1) * lm * lm);
           p->bcr_GR = dalloc<double>(p, (long long)(N - 1) * lm * lm);
+          p->bcr_pub = dalloc<double>(p, 2LL * p->nl);
           ck(set_bcr_smem_limits(lm), "smem limit");
         }
       }
@@ -1482,14 +1483,14 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
                        "kkt_factor: tensor-core update requested, but the driver cannot "
                        "encode tensor maps");
     }
-    p->fp32_update = tc ? (p->opt.fp32_update == 3 ? 3 : 2) : 1;
+    p->fp32_update = tc ? p->opt.fp32_update : 1;
     ck(launch_pchol_f32(p->aug32, p->tinv32, p->blk, p->h_blk, p->diag0, p->fac_pivot_tol,
                         p->status, s, tc, prof, drop ? kDropFP32 : 0.0),
        "pchol");
   }
   else if (p->fac_prec == kPrecFF) {
     ahlp_problem *oz = (p->opt.ff_update != 1 && oz_setup(p)) ? p : nullptr;
-    p->ff_update = oz ? (p->opt.ff_update == 3 ? 3 : 2) : 1;
+    p->ff_update = oz ? (p->opt.ff_update == 2 ? 2 : 3) : 1;
     ck(launch_pchol_ff(p->aug32, p->aug_lo, p->aug, p->aug_elems, p->blk, p->h_blk, p->diag0,
                        p->fac_pivot_tol, p->status, s, oz, prof, drop ? kDropFF : 0.0),
        "pchol");

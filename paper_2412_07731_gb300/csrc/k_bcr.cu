@@ -26,6 +26,7 @@
 #include <algorithm>
 
 #include "ahlp_internal.h"
+#include "publish.h"
 
 namespace ahlp {
 
@@ -262,14 +263,19 @@ __global__ void __launch_bounds__(kBcrThreads) bcr_z_kernel(BArgs A) {
   }
 }
 
-// The two solve kernels work on a few thousand multiply-adds per pair, so they
-// are bound by latency: a thread that walks a dot product alone pays the load
-// and the FP64 latency of every term in turn (13.5 us per level with a thread
-// per row).  Eight lanes share a row instead, each taking every eighth entry of
-// every term; the terms' loads are independent of each other and run ahead of
-// the multiply-adds, and a row ends in three shuffles.
+// The solves.  A pair needs a few thousand multiply-adds and then the solutions
+// of its neighbours, so they are bound by latency.  One launch per sweep, a CTA
+// per pair: CTAs take the pairs in elimination order by ticket (the backward
+// sweep in reverse), so a pair only waits for pairs whose CTAs already run, and
+// a pair's solution is published entry by entry (publish.h).  While it waits, a
+// CTA reads its coupling blocks once, which brings them into its L1.  Eight
+// lanes share a row; left and right terms go to the two halves of the CTA.  A
+// launch per level took 8.4 us (forward) and 6.8 us (backward) at 64 pairs of 20
+// rows, 91 us for both sweeps' six levels; a thread per row had taken 18.6 and
+// 15.1 us per level.
 constexpr int kBcrLanes = 8;
 constexpr int kBcrSolveThreads = 512;   // 32 rows at a time, left and right terms apart
+constexpr int kBcrMaxTerms = 64;        // earlier-level terms of a pair, both sides
 
 __device__ __forceinline__ double bcr_lanes_sum(double v) {
 #pragma unroll
@@ -277,101 +283,163 @@ __device__ __forceinline__ double bcr_lanes_sum(double v) {
   return v;
 }
 
-// s += sum_q G[q] z[q], q = lane, lane + 8, ... < k
-__device__ __forceinline__ void bcr_dot(const double *G, const double *z, int k,
-                                        int stride, int q0, double &s) {
+// s += sum_q G[q] z[q], q = q0, q0 + 8, ... < k
+__device__ __forceinline__ void bcr_dot(const double *G, const double *z, int k, int stride,
+                                        int q0, double &s) {
 #pragma unroll 4
   for (int q = q0; q < k; q += kBcrLanes) s = fma(G[(long long)q * stride], z[q], s);
 }
 
-// forward solve of one level, in place on the link part of u, one CTA per
-// pair: u_j = Linv_j (r_j - earlier-level terms)
-__global__ void __launch_bounds__(kBcrSolveThreads) bcr_fwd_kernel(BArgs A, double *u) {
+// the same entries of G read and dropped
+__device__ __forceinline__ void bcr_touch(const double *G, int k, int stride, int q0) {
+#pragma unroll 4
+  for (int q = q0; q < k; q += kBcrLanes) {
+    const double v = G[(long long)q * stride];
+    asm volatile("" ::"d"(v));
+  }
+}
+
+// zs[i] = the published entry pub[at[i / lm] + i % lm], i % lm < cnt[i / lm]
+__device__ __forceinline__ void bcr_collect(double *zs, const double *pub, const int *cnt,
+                                            const long long *at, int nterm, int lm, int *err) {
+  const int total = nterm * lm;
+  for (int i0 = threadIdx.x & ~31; i0 < total; i0 += blockDim.x) {   // whole warps
+    const int i = i0 + (threadIdx.x & 31);
+    const int t = i < total ? i / lm : 0, q = i - t * lm;
+    const bool in = i < total && q < cnt[t];
+    const double *p = pub + (in ? at[t] + q : 0);
+    PubBits<double>::U bits = in ? PubBits<double>::ld(p) : 0;
+    wait_published<double>(bits, p, in, err);
+    if (in) zs[i] = PubBits<double>::val(bits);
+  }
+}
+
+// forward: u_j = Linv_j (r_j - earlier-level terms); r in svec's link part, u
+// published in pub
+__global__ void __launch_bounds__(kBcrSolveThreads) bcr_fwd_kernel(BArgs A, const double *svec,
+                                                                   double *pub, int *ticket,
+                                                                   int *err) {
   pdl_begin();
-  const int j = A.order[blockIdx.x];
+  extern __shared__ double zs[];   // [terms][lmax]
+  __shared__ double r[96], part[2][96];
+  __shared__ int cnt[kBcrMaxTerms];         // term 2w + side: rows, 0: none
+  __shared__ long long at[kBcrMaxTerms];    // and where its solution starts
+  __shared__ int s_job;
+  if (threadIdx.x == 0) s_job = atomicAdd(ticket, 1);
+  __syncthreads();
+  const int j = A.order[s_job];
   int lv, jb, je;
   pair_info(A, j, lv, jb, je);
   const int lj = A.l[j], lm = A.lmax;
   const long long off = A.link_off[j];
-  __shared__ double r[96], part[2][96];
-  __shared__ int tk[2][32];           // rows of each earlier-level term, 0: none
-  __shared__ long long tu[2][32];     // and where its solution starts
   const int side = threadIdx.x / (kBcrSolveThreads / 2);
   const int lane = threadIdx.x & (kBcrLanes - 1);
   const int row0 = (threadIdx.x % (kBcrSolveThreads / 2)) / kBcrLanes;
   constexpr int rows = kBcrSolveThreads / 2 / kBcrLanes;
-  if (threadIdx.x < 64 && (threadIdx.x & 31) < lv) {
-    const int sd = threadIdx.x >> 5, w = threadIdx.x & 31;
-    const int m = sd ? j + (1 << w) : j - (1 << w);
-    const bool in = sd ? m < je : m >= jb;
-    tk[sd][w] = in ? A.l[m] : 0;
-    tu[sd][w] = in ? A.link_off[m] : 0;
+  if (threadIdx.x < 2 * lv) {
+    const int w = threadIdx.x >> 1, m = (threadIdx.x & 1) ? j + (1 << w) : j - (1 << w);
+    const bool in = (threadIdx.x & 1) ? m < je : m >= jb;
+    cnt[threadIdx.x] = in ? A.l[m] : 0;
+    at[threadIdx.x] = in ? A.link_off[m] : 0;
   }
+  __syncthreads();
+  const double *Gs = side ? A.GL : A.GR;
+  const double *Li = A.Linv + A.td_off[j];
+  for (int i = row0; i < lj; i += rows) {
+    for (int w = 0; w < lv; ++w) {
+      const int k = cnt[2 * w + side];
+      const long long m = side ? j + (1 << w) : j - (1 << w);
+      bcr_touch(Gs + m * lm * lm + (long long)i * k, k, 1, lane);
+    }
+    if (side == 0) bcr_touch(Li + i, i + 1, lj, lane);
+  }
+  bcr_collect(zs, pub, cnt, at, 2 * lv, lm, err);
   __syncthreads();
   for (int i0 = 0; i0 < lj; i0 += rows) {
     const int i = i0 + row0;
     double s = 0.0;
     if (i < lj)
       for (int w = 0; w < lv; ++w) {
-        const int k = tk[side][w];
+        const int k = cnt[2 * w + side];
         const long long m = side ? j + (1 << w) : j - (1 << w);
-        bcr_dot((side ? A.GL : A.GR) + m * lm * lm + (long long)i * k, u + tu[side][w], k, 1,
-                lane, s);
+        bcr_dot(Gs + m * lm * lm + (long long)i * k, zs + (2 * w + side) * lm, k, 1, lane, s);
       }
     s = bcr_lanes_sum(s);
     if (lane == 0 && i < lj) part[side][i] = s;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < lj; i += kBcrSolveThreads)
-    r[i] = u[off + i] - (part[0][i] + part[1][i]);
+    r[i] = svec[off + i] - (part[0][i] + part[1][i]);
   __syncthreads();
-  const double *Li = A.Linv + A.td_off[j];
   for (int i0 = 0; i0 < lj; i0 += 2 * rows) {
     const int i = i0 + threadIdx.x / kBcrLanes;
     double s = 0.0;
     if (i < lj) bcr_dot(Li + i, r, i + 1, lj, lane, s);
     s = bcr_lanes_sum(s);
-    if (lane == 0 && i < lj) u[off + i] = s;
+    if (lane == 0 && i < lj) PubBits<double>::st(pub + off + i, s);
   }
 }
 
-// backward solve of one level: x_j = Linv_j' (u_j - GL_j x_a - GR_j x_b)
-__global__ void __launch_bounds__(kBcrSolveThreads) bcr_bwd_kernel(BArgs A, double *u) {
+// backward: x_j = Linv_j' (v_j - GL_j x_a - GR_j x_b); x goes to svec's link part
+// (which may be v) and is published in pub
+__global__ void __launch_bounds__(kBcrSolveThreads) bcr_bwd_kernel(BArgs A, int npairs,
+                                                                   const double *v, double *svec,
+                                                                   double *pub,
+                                                                   int *ticket, int *err) {
   pdl_begin();
-  const int j = A.order[blockIdx.x];
+  extern __shared__ double zs[];   // [2][lmax]
+  __shared__ double r[96], part[2][96];
+  __shared__ int cnt[2];
+  __shared__ long long at[2];
+  __shared__ int s_job;
+  if (threadIdx.x == 0) s_job = atomicAdd(ticket, 1);
+  __syncthreads();
+  const int j = A.order[npairs - 1 - s_job];
   int lv, jb, je;
   pair_info(A, j, lv, jb, je);
   const int lj = A.l[j], lm = A.lmax;
   const long long off = A.link_off[j];
-  __shared__ double r[96], part[2][96];
   const int side = threadIdx.x / (kBcrSolveThreads / 2);
   const int lane = threadIdx.x & (kBcrLanes - 1);
   const int row0 = (threadIdx.x % (kBcrSolveThreads / 2)) / kBcrLanes;
   constexpr int rows = kBcrSolveThreads / 2 / kBcrLanes;
-  const int a = side ? j + (1 << lv) : j - (1 << lv);   // this side's neighbour
-  const bool in = side ? a < je : a >= jb;
-  const int ka = in ? A.l[a] : 0;
-  const long long oa = in ? A.link_off[a] : 0;
+  if (threadIdx.x < 2) {
+    const int m = threadIdx.x ? j + (1 << lv) : j - (1 << lv);
+    const bool in = threadIdx.x ? m < je : m >= jb;
+    cnt[threadIdx.x] = in ? A.l[m] : 0;
+    at[threadIdx.x] = in ? A.link_off[m] : 0;
+  }
+  __syncthreads();
+  const double *G = (side ? A.GR : A.GL) + (long long)j * lm * lm;   // l_j x l_neighbour
+  const double *Li = A.Linv + A.td_off[j];
+  const int k = cnt[side];
+  for (int i = row0; i < lj; i += rows) {
+    bcr_touch(G + i, k, lj, lane);
+    if (side == 0) bcr_touch(Li + (long long)i * lj + i, lj - i, 1, lane);
+  }
+  bcr_collect(zs, pub, cnt, at, 2, lm, err);
+  __syncthreads();
   for (int i0 = 0; i0 < lj; i0 += rows) {
     const int i = i0 + row0;
     double s = 0.0;
-    if (i < lj)   // l_j x l_a
-      bcr_dot((side ? A.GR : A.GL) + (long long)j * lm * lm + i, u + oa, ka, lj, lane, s);
+    if (i < lj) bcr_dot(G + i, zs + side * lm, k, lj, lane, s);
     s = bcr_lanes_sum(s);
     if (lane == 0 && i < lj) part[side][i] = s;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < lj; i += kBcrSolveThreads)
-    r[i] = u[off + i] - (part[0][i] + part[1][i]);
+    r[i] = v[off + i] - (part[0][i] + part[1][i]);
   __syncthreads();
-  const double *Li = A.Linv + A.td_off[j];
   for (int i0 = 0; i0 < lj; i0 += 2 * rows) {
     const int i = i0 + threadIdx.x / kBcrLanes;
     double s = 0.0;
     // entries i .. lj - 1 of column i
     if (i < lj) bcr_dot(Li + (long long)i * lj + i, r + i, lj - i, 1, lane, s);
     s = bcr_lanes_sum(s);
-    if (lane == 0 && i < lj) u[off + i] = s;
+    if (lane == 0 && i < lj) {
+      PubBits<double>::st(pub + off + i, s);
+      svec[off + i] = s;
+    }
   }
 }
 
@@ -416,24 +484,26 @@ cudaError_t launch_bcr_factor(ahlp_problem *p) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_bcr_solve(ahlp_problem *p, double *u, bool forward) {
-  cudaStream_t s = p->stream;
-  const int nlev = (int)p->bcr_loff.size() - 1;
-  for (int w = 0; w < nlev; ++w) {
-    const int v = forward ? w : nlev - 1 - w;
-    const int n = p->bcr_loff[v + 1] - p->bcr_loff[v];
-    if (n == 0) continue;
-    BArgs A = bargs(p);
-    A.order = p->bcr_order + p->bcr_loff[v];
-    if (forward)
-      count_launch(), launch_pdl(bcr_fwd_kernel, n, kBcrSolveThreads, 0, s, A, u);
-    else
-      count_launch(), launch_pdl(bcr_bwd_kernel, n, kBcrSolveThreads, 0, s, A, u);
-  }
+cudaError_t launch_bcr_solve(ahlp_problem *p, bool forward) {
+  const int n = p->bcr_loff.back(), nlev = (int)p->bcr_loff.size() - 1;
+  if (n == 0) return cudaSuccess;
+  const BArgs A = bargs(p);
+  const size_t row = (size_t)p->bcr_lmax * sizeof(double);
+  if (forward)
+    count_launch(), launch_pdl(bcr_fwd_kernel, n, kBcrSolveThreads, 2 * (nlev - 1) * row,
+                               p->stream, A, p->svec, p->bcr_pub, p->trsv_ticket + 2, p->trsv_err);
+  else
+    count_launch(), launch_pdl(bcr_bwd_kernel, n, kBcrSolveThreads, 2 * row, p->stream, A, n,
+                               p->B > 0 ? p->svec : p->bcr_pub, p->svec, p->bcr_pub + p->nl,
+                               p->trsv_ticket + 3, p->trsv_err);
   return cudaGetLastError();
 }
 
 cudaError_t set_bcr_smem_limits(int lmax) {
+  const int full = kBcrMaxTerms * lmax * (int)sizeof(double);
+  cudaError_t e = cudaFuncSetAttribute(bcr_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       full);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(bcr_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               3 * lmax * lmax * (int)sizeof(double));
 }

@@ -654,20 +654,26 @@ __global__ void negate_corner_kernel(double *bd, int ld, int n0, int mg, double 
 // solve pipeline kernels
 // --------------------------------------------------------------------------
 // f = r_d - X^-1 r_c (forward) or g_x - Z X^-1 g_z (adjoint); g = D f on block
-// columns.  First kernel of a solve: it also resets the wavefront solves'
-// tickets and fills their publication buffers (fwd_words and bwd_words 32-bit
-// words) with the unpublished pattern.
+// columns.  First kernel of a solve: it also resets the ticket counters of the
+// wavefront and chain solves and fills their publication buffers (nw 32-bit words
+// each) with the unpublished pattern.
+struct PubFill {
+  int *ticket;
+  unsigned *buf[3];
+  long long nw[3];
+};
+
 __global__ void prep_f_kernel(double *f, double *g, const double *rd, const double *rc,
                               const double *xinv, const double *z, const double *d,
-                              const unsigned char *is_x0, long long n, int adjoint, int *ticket,
-                              unsigned *pub_fwd, unsigned *pub_bwd, long long fwd_words,
-                              long long bwd_words) {
+                              const unsigned char *is_x0, long long n, int adjoint,
+                              const PubFill P) {
   pdl_begin();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  if (i < 2) ticket[i] = 0;
-  for (long long w = i; w < fwd_words; w += stride) pub_fwd[w] = 0xffffffffu;
-  for (long long w = i; w < bwd_words; w += stride) pub_bwd[w] = 0xffffffffu;
+  if (i < 4) P.ticket[i] = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    for (long long w = i; w < P.nw[k]; w += stride) P.buf[k][w] = 0xffffffffu;
   if (i >= n) return;
   const double fi = adjoint ? rd[i] - z[i] * rc[i] * xinv[i] : rd[i] - rc[i] * xinv[i];
   f[i] = fi;
@@ -891,10 +897,11 @@ __global__ void __launch_bounds__(kBinvThreads) border_inv_kernel(const double *
   }
 }
 
-// border rhs: sB -= Z' uT, one CTA per border row over its column's link rows
+// border rhs: sB -= Z' uT, one CTA per border row over its column's link rows;
+// uT is the chain's forward solution, sB svec's border part
 __global__ void __launch_bounds__(128) border_rhs_kernel(const double *Z, int nl,
                                                          const int *zlo, const int *zhi,
-                                                         double *svec) {
+                                                         const double *uT, double *svec) {
   pdl_begin();
   __shared__ double part[4];
   const int rb = blockIdx.x;
@@ -904,10 +911,10 @@ __global__ void __launch_bounds__(128) border_rhs_kernel(const double *Z, int nl
   int q = zlo[rb] + threadIdx.x;
 #pragma unroll 4
   for (; q + 128 < q1; q += 256) {
-    s0 = fma(zc[q], svec[q], s0);
-    s1 = fma(zc[q + 128], svec[q + 128], s1);
+    s0 = fma(zc[q], uT[q], s0);
+    s1 = fma(zc[q + 128], uT[q + 128], s1);
   }
-  if (q < q1) s0 = fma(zc[q], svec[q], s0);
+  if (q < q1) s0 = fma(zc[q], uT[q], s0);
   double acc = s0 + s1;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -939,10 +946,11 @@ __global__ void __launch_bounds__(256) border_w_kernel(const double *W, int B, i
   if (lane == 0) out[i] = fwd && i < n0 ? -s : s;
 }
 
-// uT -= Z sB: a CTA takes 32 link rows, 16 threads per row share the border
+// svec's link part = uT - Z sB: a CTA takes 32 link rows, 16 threads per row share the border
 // columns (one thread per row walked all of them: 28 us at 100, 156 us at 601)
 __global__ void __launch_bounds__(512) link_back_kernel(const double *Z, int B,
-                                                        int nl, double *svec) {
+                                                        int nl, const double *uT,
+                                                        double *svec) {
   pdl_begin();
   __shared__ double part[16][32];
   const int rr = threadIdx.x & 31, g = threadIdx.x >> 5;
@@ -963,7 +971,7 @@ __global__ void __launch_bounds__(512) link_back_kernel(const double *Z, int B,
     double s = 0.0;
 #pragma unroll
     for (int i = 0; i < 16; ++i) s += part[i][rr];
-    svec[q] -= s;
+    svec[q] = uT[q] - s;
   }
 }
 
@@ -1077,11 +1085,15 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
   cudaError_t e;
   const bool f32 = p->fac_prec == kPrecFP32;
   const long long words = p->vec_elems * (f32 ? 1 : 2);
-  count_launch(), launch_pdl(prep_f_kernel, nb(std::max<long long>(n, 2), 256), 256, 0, s, p->f,
+  const PubFill fill{p->trsv_ticket,
+                     {f32 ? reinterpret_cast<unsigned *>(p->vec32)
+                          : reinterpret_cast<unsigned *>(p->vec),
+                      reinterpret_cast<unsigned *>(p->vecb),
+                      reinterpret_cast<unsigned *>(p->bcr_pub)},
+                     {words, words, p->fac_bcr && p->bcr_pub ? 4LL * p->nl : 0}};
+  count_launch(), launch_pdl(prep_f_kernel, nb(std::max<long long>(n, 4), 256), 256, 0, s, p->f,
                              p->g, r_d, r_c, p->xinv, p->z, p->dscale, p->is_x0, n,
-                             adjoint ? 1 : 0, p->trsv_ticket,
-      f32 ? reinterpret_cast<unsigned *>(p->vec32) : reinterpret_cast<unsigned *>(p->vec),
-      reinterpret_cast<unsigned *>(p->vecb), words, words);
+                             adjoint ? 1 : 0, fill);
   e = launch_spmv(p->Amat, p->g, p->rhat, 1.0, r_p, s);
   if (e != cudaSuccess) return e;
   e = launch_trsv(p, true, p->rhat, nullptr);
@@ -1108,7 +1120,7 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
     const size_t csm = (size_t)stages * ((size_t)lmax * lmax + lmax) * sizeof(double);
     if (p->nl > 0 && lmax > 0 && p->nchain_seg > 0) {
       if (p->fac_bcr) {
-        e = launch_bcr_solve(p, p->svec, true);
+        e = launch_bcr_solve(p, true);
         if (e != cudaSuccess) return e;
       } else {
         count_launch(), launch_pdl(chain_solve_kernel, p->nchain_seg, kChainSolveThreads, csm, s,
@@ -1116,24 +1128,24 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
       }
     }
     if (p->B > 0) {
+      // the chain's forward solution: published by the cyclic reduction, in place
+      // in svec otherwise
+      const double *uT = p->nl > 0 && p->fac_bcr ? p->bcr_pub : p->svec;
+      double *sb = p->svec + p->nl;
       if (p->nl > 0)
         count_launch(), launch_pdl(border_rhs_kernel, p->B, 128, 0, s, p->Et, p->nl, p->zlo,
-                                   p->zhi,
-                                                               p->svec);
-      double *sb = p->svec + p->nl;
+                                   p->zhi, uT, p->svec);
       count_launch(), launch_pdl(border_w_kernel, nb(p->B, 8), 256, 0, s, p->border_wr, p->B,
-                                 p->Bld,
-                                                                  p->n0, sb, p->border_t, 1);
+                                 p->Bld, p->n0, sb, p->border_t, 1);
       count_launch(), launch_pdl(border_w_kernel, nb(p->B, 8), 256, 0, s, p->border_wc, p->B,
-                                 p->Bld,
-                                                                  p->n0, p->border_t, sb, 0);
+                                 p->Bld, p->n0, p->border_t, sb, 0);
       if (p->nl > 0)
         count_launch(), launch_pdl(link_back_kernel, nb(p->nl, 32), 512, 0, s, p->Et, p->B, p->nl,
-                                                                       p->svec);
+                                   uT, p->svec);
     }
     if (p->nl > 0 && lmax > 0 && p->nchain_seg > 0) {
       if (p->fac_bcr) {
-        e = launch_bcr_solve(p, p->svec, false);
+        e = launch_bcr_solve(p, false);
         if (e != cudaSuccess) return e;
       } else {
         count_launch(), launch_pdl(chain_solve_kernel, p->nchain_seg, kChainSolveThreads, csm, s,

@@ -1104,7 +1104,12 @@ cudaError_t launch_update_tc(ahlp_problem *p, int k, cudaStream_t s) {
   TcArgs a{p->pstage, p->tc_joff + (size_t)k * (p->h_blk.size() + 1), p->blk,
            reinterpret_cast<const CUtensorMap *>(p->tc_tmap), (int)p->h_blk.size(), k,
            p->status, p->tc_jtab ? p->tc_jtab + p->tc_jtab_off[k] : nullptr};
-  if (p->fp32_update == 3) {   // persistent pipeline: one CTA per SM
+  // Both kernels give the same factor.  The persistent pipeline (one CTA per SM)
+  // wins once its CTAs have several jobs to overlap: 96 uneven blocks, thousands
+  // of jobs per step, 15.4 -> 12.4 ms per factor; with about one job per SM its
+  // longer start costs more than it hides (8 blocks of 1000 rows 0.81 against
+  // 0.80 ms, 16 of 300..700 rows 0.555 against 0.543).
+  if (p->fp32_update == 3 || (p->fp32_update == 0 && jobs >= 2LL * p->num_sms)) {
     const int grid = (int)std::min<long long>(jobs, p->num_sms);
     count_launch(), launch_pdl(pchol_update_tc2_kernel, grid, kTc2Threads, kTc2Smem, s, a,
                                (int)jobs);
