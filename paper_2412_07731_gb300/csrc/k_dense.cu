@@ -110,17 +110,19 @@ __global__ void dscale_kernel(const double *x, const double *z, double *d, doubl
 // --------------------------------------------------------------------------
 // partial Cholesky, step k: diagonal tile
 // --------------------------------------------------------------------------
-// The FP64 pipe issues one warp instruction per 64 clocks and partition, so the
-// tile is bound by its chain of dependent FP64 operations (64 pivots) and by
-// the number of FP64 warp instructions, not by bandwidth.  Four 16-column
-// panels; a panel is factored in registers by four warps, one per partition:
-// every warp holds its own copy of the 16 x 16 diagonal block and 16 rows
-// below it (lane = row and column parity, eight entries each), so no column
-// waits for another warp, and a pivot costs one reciprocal square root (a
-// single third-order step from the FP32 one), a scaling and an update.  Then
-// all eight warps apply the panel to the lower triangle right of it, lanes
-// packed over the triangle.  28 us per 64 x 64 tile on one CTA (124 us with a
-// barrier, a square root and a division per column).
+// FP64 and float-float diagonal tiles.  The FP64 pipe takes one warp instruction
+// per 64 clocks and partition (76 with all four busy), comparisons and
+// conversions included, so the tile is bound by the FP64 instructions on its
+// chain of 64 pivots, not by bandwidth.  Four 16-column panels; a panel is
+// factored in registers by four warps, one per partition: every warp holds its
+// own copy of the 16 x 16 diagonal block and 16 rows below it (lane = row and
+// column parity, eight entries each), so no column waits for another warp.  A
+// pivot costs its test in integers, one reciprocal square root (five FP64
+// instructions), two scalings and the updates; the diagonal entries themselves
+// follow at the end, all at once.  Then all eight warps apply the panel to the
+// lower triangle right of it, lanes packed over the triangle.  51 us per tile on
+// one CTA (76 us with FP64 pivot tests and the diagonal on the chain, 124 us with
+// a barrier, a square root and a division per column).
 // 1 / sqrt(p) of a positive finite p: y0 = rsqrtf of the mantissa (p scaled
 // by an even power of two into [1, 4)), then Householder's third-order
 // iteration y = y0 + y0 e (1/2 + 3/8 e), e = 1 - m y0^2, whose error is ~e^3.
@@ -129,35 +131,49 @@ __device__ __forceinline__ double rsqrt_f64(double p) {
   const int ex = hi >> 20;
   if (ex == 0 || ex >= 0x7ff) return rsqrt(p);   // subnormal or infinite
   const int k = (ex - 1023) >> 1;
-  const double m = __hiloint2double(hi - (k << 21), __double2loint(p));   // [1, 4)
-  // FP32 value of m from its bits (truncated)
-  const int mh = __double2hiint(m);
-  const float f = __int_as_float(((mh - 0x38000000) << 3) | (int)((unsigned)__double2loint(m) >> 29));
-  const double y0 = (double)rsqrtf(f);
+  const int mh = hi - (k << 21), ml = __double2loint(p);
+  const double m = __hiloint2double(mh, ml);   // [1, 4)
+  // FP32 value of m from its bits (truncated), and y0's bits as FP64 (y0 in (1/2, 1])
+  const float y = rsqrtf(__int_as_float(((mh - 0x38000000) << 3) | (int)((unsigned)ml >> 29)));
+  const int yb = __float_as_int(y);
+  const double y0 = __hiloint2double((yb >> 3) + 0x38000000, yb << 29);
   const double e = fma(-m * y0, y0, 1.0);
-  const double y = fma(y0 * e, fma(0.375, e, 0.5), y0);
-  return __hiloint2double(__double2hiint(y) - (k << 20), __double2loint(y));
+  const double r = fma(y0 * e, fma(0.375, e, 0.5), y0);
+  return __hiloint2double(__double2hiint(r) - (k << 20), __double2loint(r));
 }
 
 constexpr int kPW = 16;   // panel width
 
-__global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(double *buf, const BlkInfo *blk,
-                                                               int k, const double *diag0,
-                                                               double tol, int *status,
-                                                               double drop) {
+// kFF: the matrix is hi + lo (lo null otherwise)
+template <bool kFF, typename T>
+__global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(T *buf, float *lo,
+                                                               const BlkInfo *blk, int k,
+                                                               const double *diag0, double tol,
+                                                               int *status, double drop) {
   pdl_begin();
   const BlkInfo bi = blk[blockIdx.x];
   if (k >= bi.Tp) return;
   __shared__ double t[NB][NB + 1];
+  __shared__ double s_piv[NB], s_inv[NB];
   const int r0 = k * NB;
   const int nr = min(NB, bi.a - r0);
   const int npiv = min(NB, bi.p - r0);
-  double *g = buf + bi.base + (long long)r0 * bi.lda + r0;
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
-    const int r = i % NB, c = i / NB;
-    t[r][c] = (r < nr && c < nr && r >= c) ? g[(long long)c * bi.lda + r] : 0.0;
+  const long long g0 = bi.base + (long long)r0 * bi.lda + r0;
+  {
+    const int r = threadIdx.x & (NB - 1), cs = threadIdx.x / NB;
+#pragma unroll 8
+    for (int c = cs; c < NB; c += kThreads / NB) {
+      double v = 0.0;
+      if (r < nr && c < nr && r >= c) {
+        const long long el = g0 + (long long)c * bi.lda + r;
+        if constexpr (kFF) v = (double)buf[el] + (double)lo[el];
+        else v = buf[el];
+      }
+      t[r][c] = v;
+    }
   }
   __syncthreads();
+  const double cap = kFF ? kDropCapFF : 1e300;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rr = lane & 15, hc = lane >> 4;   // row of 16, column parity
   for (int c0 = 0; c0 < npiv; c0 += kPW) {
@@ -171,36 +187,45 @@ __global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(double *buf, cons
         o[j] = own ? t[row][c0 + 2 * j + hc] : 0.0;
       }
       const double dref = c0 + rr < npiv ? diag0[bi.d0off + r0 + c0 + rr] : 0.0;
+      // the pivot must exceed lim: positive doubles compare as their bits
+      const double lim = tol * dref;
+      const long long limb = max(__double_as_longlong(lim), 0ll);
 #pragma unroll
       for (int u = 0; u < kPW; ++u) {
         if (c0 + u < npiv) {   // uniform over the CTA
           const int src = (u & 1) * 16;
           double piv = __shfl_sync(0xffffffffu, d[u >> 1], src + u);
-          const double orig = __shfl_sync(0xffffffffu, dref, u);
+          const long long lb = __shfl_sync(0xffffffffu, limb, u);
           const double v = __shfl_sync(0xffffffffu, d[u >> 1], src + rr);
           const double vo = __shfl_sync(0xffffffffu, o[u >> 1], src + rr);
-          // the safeguard of pivot_fix, reported by one lane
-          const double lim = tol * orig;
-          if (!(piv == piv) || !(piv > lim) || !(piv > 0.0)) {
-            if (threadIdx.x == 0)
-              pivot_fix(piv, orig, tol, status, bi.tag + (int)blockIdx.x, r0 + c0 + u, drop);
-            piv = drop > 0.0 ? fmin(drop * fmax(orig, 1.0), 1e300) : lim > 0.0 ? lim : 1.0;
+          const long long pb = __double_as_longlong(piv);
+          if (pb <= lb || pb > 0x7ff0000000000000ll) {   // too small, negative or NaN
+            const double orig = __shfl_sync(0xffffffffu, dref, u);
+            if (threadIdx.x == 0) {
+              double q = piv;
+              pivot_fix(q, orig, tol, status, bi.tag + (int)blockIdx.x, r0 + c0 + u, drop, cap);
+            }
+            const double lm = tol * orig;
+            piv = drop > 0.0 ? fmin(drop * fmax(orig, 1.0), cap) : lm > 0.0 ? lm : 1.0;
           }
           const double inv = rsqrt_f64(piv);
-          double lcc = piv * inv;
-          lcc = fma(fma(-lcc, lcc, piv), 0.5 * inv, lcc);
-          const double ld = rr == u ? lcc : v * inv;
-          const double lo = vo * inv;
-          if (hc == (u & 1)) {
-            d[u >> 1] = ld;
-            o[u >> 1] = lo;
+          if (threadIdx.x == 0) {
+            s_piv[c0 + u] = piv;
+            s_inv[c0 + u] = inv;
+          }
+          const double ld = v * inv;   // rows u + 1 .. (the diagonal entry comes later)
+          if (hc == (u & 1)) d[u >> 1] = ld;
+          double lor = 0.0;
+          if (own) {   // uniform over the warp
+            lor = vo * inv;
+            if (hc == (u & 1)) o[u >> 1] = lor;
           }
 #pragma unroll
           for (int j = u >> 1; j < 8; ++j) {   // columns q = 2j + hc > u
             const double lq = __shfl_sync(0xffffffffu, ld, 2 * j + hc);
             if (2 * j + hc > u) {
               d[j] = fma(-ld, lq, d[j]);
-              o[j] = fma(-lo, lq, o[j]);
+              if (own) o[j] = fma(-lor, lq, o[j]);
             }
           }
         }
@@ -234,9 +259,24 @@ __global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(double *buf, cons
     }
     __syncthreads();
   }
+  if (threadIdx.x < npiv) {   // sqrt(piv) = piv inv, one correction
+    const double piv = s_piv[threadIdx.x], inv = s_inv[threadIdx.x];
+    const double l = piv * inv;
+    t[threadIdx.x][threadIdx.x] = fma(fma(-l, l, piv), 0.5 * inv, l);
+  }
+  __syncthreads();
   for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
     const int r = i % NB, c = i / NB;
-    if (r < nr && c < nr && r >= c) g[(long long)c * bi.lda + r] = t[r][c];
+    if (r < nr && c < nr && r >= c) {
+      const long long el = g0 + (long long)c * bi.lda + r;
+      if constexpr (kFF) {
+        const float h = (float)t[r][c];
+        buf[el] = h;
+        lo[el] = (float)(t[r][c] - (double)h);
+      } else {
+        buf[el] = t[r][c];
+      }
+    }
   }
 }
 
@@ -380,8 +420,12 @@ __global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkI
 // it (a rank-16 update).  The code of a panel step is small and runs four
 // times; a fully unrolled 64-column version was bound by instruction fetch.
 // The inverse goes by 16x16 blocks: the diagonal blocks by substitution in
-// parallel, then each block row below as two small products with the rows
-// above it, so its sequential depth is 16 rows rather than 64.
+// parallel, each lane's column in registers, then each block row below as two
+// small products with the rows above it, so its sequential depth is 16 rows
+// rather than 64.  Everything outside the panels' chain of pivots is bound by
+// the latency of shared-memory reads, so loops are unrolled and every thread
+// works on several entries at once (71.5 k -> 46 k clocks per tile, the same
+// roundings).
 // --------------------------------------------------------------------------
 constexpr int kPotrf32Threads = 256;
 __global__ void __launch_bounds__(kPotrf32Threads) pchol_potrf_f32_kernel(
@@ -397,10 +441,14 @@ __global__ void __launch_bounds__(kPotrf32Threads) pchol_potrf_f32_kernel(
   const int nr = min(NB, bi.a - r0);
   const int npiv = min(NB, bi.p - r0);
   float *g = buf + bi.base + (long long)r0 * bi.lda + r0;
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
-    const int r = i % NB, c = i / NB;
-    t[r][c] = (r < nr && c < nr && r >= c) ? g[(long long)c * bi.lda + r] : 0.0f;
-    X[r][c] = 0.0f;
+  {
+    const int r = threadIdx.x & (NB - 1), cs = threadIdx.x / NB;
+#pragma unroll
+    for (int u = 0; u < NB / (kPotrf32Threads / NB); ++u) {
+      const int c = cs + u * (kPotrf32Threads / NB);
+      t[r][c] = (r < nr && c < nr && r >= c) ? g[(long long)c * bi.lda + r] : 0.0f;
+      X[r][c] = 0.0f;
+    }
   }
   __syncthreads();
   const double *d0 = diag0 + bi.d0off + r0;
@@ -465,23 +513,62 @@ __global__ void __launch_bounds__(kPotrf32Threads) pchol_potrf_f32_kernel(
     __syncthreads();
     // rank-16 update of the lower triangle right of the panel:
     // t[r][q] -= sum_c t[r][c] t[q][c], c0 + 16 <= q <= r < nr, c < npiv
+    // thread (tx, ty) takes the entries (tx, ty) of the 16x16 blocks (a, b), b <= a,
+    // each sum in two chains (even and odd columns of the panel)
     const int q0 = c0 + kPW;
     const int cend = min(c0 + kPW, npiv);
     if (q0 < nr) {
-      const int w = nr - q0;
-      for (int idx = threadIdx.x; idx < w * w; idx += blockDim.x) {
-        const int rr = idx % w, qq = idx / w;
-        if (rr < qq) continue;
-        const int r = q0 + rr, q = q0 + qq;
-        float s0 = 0.0f, s1 = 0.0f;
-        int c = c0;
-        for (; c + 1 < cend; c += 2) {
-          s0 = fmaf(t[r][c], t[q][c], s0);
-          s1 = fmaf(t[r][c + 1], t[q][c + 1], s1);
+      const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+      const int nbl = (nr - q0 + kPW - 1) / kPW;   // 1..3
+      float s0[3][3], s1[3][3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) s0[a][b] = s1[a][b] = 0.0f;
+      if (cend == c0 + kPW) {
+#pragma unroll 4
+        for (int c = c0; c < c0 + kPW; c += 2) {
+          float ra[3], rb[3], qa[3], qb[3];
+#pragma unroll
+          for (int a = 0; a < 3; ++a)
+            if (a < nbl) {
+              ra[a] = t[q0 + 16 * a + tx][c];
+              rb[a] = t[q0 + 16 * a + tx][c + 1];
+              qa[a] = t[q0 + 16 * a + ty][c];
+              qb[a] = t[q0 + 16 * a + ty][c + 1];
+            }
+#pragma unroll
+          for (int a = 0; a < 3; ++a)
+            if (a < nbl) {
+#pragma unroll
+              for (int b = 0; b <= a; ++b) {
+                s0[a][b] = fmaf(ra[a], qa[b], s0[a][b]);
+                s1[a][b] = fmaf(rb[a], qb[b], s1[a][b]);
+              }
+            }
         }
-        if (c < cend) s0 = fmaf(t[r][c], t[q][c], s0);
-        t[r][q] -= s0 + s1;
+      } else {
+        for (int c = c0; c < cend; ++c)
+#pragma unroll
+          for (int a = 0; a < 3; ++a)
+            if (a < nbl) {
+#pragma unroll
+              for (int b = 0; b <= a; ++b) {
+                const float x = t[q0 + 16 * a + tx][c], y = t[q0 + 16 * b + ty][c];
+                if ((c - c0) & 1) s1[a][b] = fmaf(x, y, s1[a][b]);
+                else s0[a][b] = fmaf(x, y, s0[a][b]);
+              }
+            }
       }
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        if (a < nbl) {
+#pragma unroll
+          for (int b = 0; b <= a; ++b) {
+            const int r = q0 + 16 * a + tx, q = q0 + 16 * b + ty;
+            if (r < nr && q <= r) t[r][q] -= s0[a][b] + s1[a][b];
+          }
+        }
     }
     __syncthreads();
   }
@@ -492,45 +579,60 @@ __global__ void __launch_bounds__(kPotrf32Threads) pchol_potrf_f32_kernel(
   const int nbk = (npiv + kPW - 1) / kPW;
   {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w < 4 && lane < kPW) {
-      const int b0 = w * kPW, j = b0 + lane;
-      for (int i = b0; i < b0 + kPW; ++i) {
-        float v = 0.0f;
-        if (i < npiv && i >= j) {
-          float s0 = i == j ? 1.0f : 0.0f, s1 = 0.0f;
-          int q = j;
-          for (; q + 1 < i; q += 2) {
-            s0 = fmaf(-t[i][q], X[q][j], s0);
-            s1 = fmaf(-t[i][q + 1], X[q + 1][j], s1);
-          }
-          if (q < i) s0 = fmaf(-t[i][q], X[q][j], s0);
-          v = (s0 + s1) / t[i][i];
+    if (w < 4 && lane < kPW && w * kPW < npiv) {
+      // x[i]: rows b0 + i of column b0 + lane; the terms of rows above the
+      // column's diagonal are zero, so every lane runs all of them
+      const int b0 = w * kPW;
+      float x[kPW];
+#pragma unroll
+      for (int i = 0; i < kPW; ++i) {
+        float se = i == lane ? 1.0f : 0.0f, so = 0.0f;   // even and odd rows q
+#pragma unroll
+        for (int q = 0; q < i; ++q) {
+          if (q & 1) so = fmaf(-t[b0 + i][b0 + q], x[q], so);
+          else se = fmaf(-t[b0 + i][b0 + q], x[q], se);
         }
-        X[i][j] = v;
+        x[i] = (b0 + i < npiv && i >= lane) ? (se + so) / t[b0 + i][b0 + i] : 0.0f;
       }
+#pragma unroll
+      for (int i = 0; i < kPW; ++i) X[b0 + i][b0 + lane] = x[i];
     }
   }
   __syncthreads();
   for (int bi2 = 1; bi2 < nbk; ++bi2) {
-    const int i0 = bi2 * kPW, wc = i0;   // columns 0 .. i0-1 of block row bi2
-    for (int e = threadIdx.x; e < kPW * wc; e += blockDim.x) {
-      const int r = e % kPW, c = e / kPW;
-      float s0 = 0.0f, s1 = 0.0f;
-      int q = (c / kPW) * kPW;
-      for (; q + 1 < i0; q += 2) {
-        s0 = fmaf(t[i0 + r][q], X[q][c], s0);
-        s1 = fmaf(t[i0 + r][q + 1], X[q + 1][c], s1);
-      }
-      if (q < i0) s0 = fmaf(t[i0 + r][q], X[q][c], s0);
-      Tm[r][c] = s0 + s1;
+    // block row bi2, columns 0 .. i0-1: thread (row r, column c) of each block
+    const int i0 = bi2 * kPW;
+    const int r = threadIdx.x % kPW, c = threadIdx.x / kPW;
+    float s0[3], s1[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) s0[b] = s1[b] = 0.0f;
+#pragma unroll 4
+    for (int q = 0; q < i0; q += 2) {   // block b starts at its own row 16 b
+      const float ta = t[i0 + r][q], tb = t[i0 + r][q + 1];
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+        if (b < bi2 && q >= b * kPW) {
+          s0[b] = fmaf(ta, X[q][b * kPW + c], s0[b]);
+          s1[b] = fmaf(tb, X[q + 1][b * kPW + c], s1[b]);
+        }
     }
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+      if (b < bi2) Tm[r][b * kPW + c] = s0[b] + s1[b];
     __syncthreads();
-    for (int e = threadIdx.x; e < kPW * wc; e += blockDim.x) {
-      const int r = e % kPW, c = e / kPW;
-      float s = 0.0f;
-      for (int q = 0; q <= r; ++q) s = fmaf(X[i0 + r][i0 + q], Tm[q][c], s);
-      X[i0 + r][c] = i0 + r < npiv ? -s : 0.0f;
+    float s[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int q = 0; q < kPW; ++q) {
+      const float xv = X[i0 + r][i0 + q];
+      if (q <= r) {
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+          if (b < bi2) s[b] = fmaf(xv, Tm[q][b * kPW + c], s[b]);
+      }
     }
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+      if (b < bi2) X[i0 + r][b * kPW + c] = i0 + r < npiv ? -s[b] : 0.0f;
     __syncthreads();
   }
   float *out = tinv + bi.ioff + (long long)k * NB * NB;
@@ -648,16 +750,6 @@ __global__ void __launch_bounds__(kThreads) pchol_trsm_inv_kernel(T *buf, const 
 // The __f*_rn intrinsics keep the compiler from contracting the error-free
 // transformations into FMAs.
 // --------------------------------------------------------------------------
-__device__ __forceinline__ double ff_get(const float *hi, const float *lo, long long i) {
-  return (double)hi[i] + (double)lo[i];
-}
-
-__device__ __forceinline__ void ff_put(float *hi, float *lo, long long i, double v) {
-  const float h = (float)v;
-  hi[i] = h;
-  lo[i] = (float)(v - (double)h);
-}
-
 // (sh, sl) += (ah + al)(bh + bl), al*bl dropped
 __device__ __forceinline__ void ff_mac(float &sh, float &sl, float ah, float al, float bh,
                                        float bl) {
@@ -697,50 +789,6 @@ __global__ void ff_expand_kernel(const float *hi, const float *lo,
   for (long long i = 4 * n4 + (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += stride)
     out[i] = (double)hi[i] + (double)lo[i];
-}
-
-__global__ void __launch_bounds__(kThreads) pchol_potrf_ff_kernel(float *hi, float *lo,
-                                                                  const BlkInfo *blk, int k,
-                                                                  const double *diag0, double tol,
-                                                                  int *status, double drop) {
-  pdl_begin();
-  const BlkInfo bi = blk[blockIdx.x];
-  if (k >= bi.Tp) return;
-  __shared__ double t[NB][NB + 1];
-  __shared__ double s_inv;
-  const int r0 = k * NB;
-  const int nr = min(NB, bi.a - r0);
-  const int npiv = min(NB, bi.p - r0);
-  const long long g0 = bi.base + (long long)r0 * bi.lda + r0;
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
-    const int r = i % NB, c = i / NB;
-    t[r][c] = (r < nr && c < nr && r >= c) ? ff_get(hi, lo, g0 + (long long)c * bi.lda + r) : 0.0;
-  }
-  __syncthreads();
-  for (int c = 0; c < npiv; ++c) {
-    if (threadIdx.x == 0) {
-      double piv = t[c][c];
-      pivot_fix(piv, diag0[bi.d0off + r0 + c], tol, status, bi.tag + (int)blockIdx.x, r0 + c,
-                drop, kDropCapFF);
-      const double l = sqrt(piv);
-      t[c][c] = l;
-      s_inv = 1.0 / l;
-    }
-    __syncthreads();
-    const double inv = s_inv;
-    for (int r = c + 1 + threadIdx.x; r < nr; r += blockDim.x) t[r][c] *= inv;
-    __syncthreads();
-    const int m = nr - c - 1;
-    for (int idx = threadIdx.x; idx < m * m; idx += blockDim.x) {
-      const int rr = idx % m, ss = idx / m;
-      if (rr >= ss) t[c + 1 + rr][c + 1 + ss] -= t[c + 1 + rr][c] * t[c + 1 + ss][c];
-    }
-    __syncthreads();
-  }
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
-    const int r = i % NB, c = i / NB;
-    if (r < nr && c < nr && r >= c) ff_put(hi, lo, g0 + (long long)c * bi.lda + r, t[r][c]);
-  }
 }
 
 // With dstage (the tensor-core float-float update, k_tc.cu) the finished
@@ -1685,9 +1733,8 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
                                    tc ? tc->pstage : nullptr);
     } else {
       if (prof) kt_mark(prof, 0, s);
-      count_launch(), launch_pdl(pchol_potrf_kernel, nblk, kThreads, 0, s, buf, info, k, diag0,
-                                 tol,
-                                                                   status, drop);
+      count_launch(), launch_pdl(pchol_potrf_kernel<false, double>, nblk, kThreads, 0, s, buf,
+                                 nullptr, info, k, diag0, tol, status, drop);
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
         count_launch(), launch_pdl(pchol_trsm_kernel<T>, dim3((unsigned)maxPanel, nblk), kThreads,
@@ -1768,9 +1815,8 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
       if (t * (t + 1) / 2 > maxTrail) maxTrail = t * (t + 1) / 2;
     }
     if (prof) kt_mark(prof, 0, s);
-    count_launch(), launch_pdl(pchol_potrf_ff_kernel, nblk, kThreads, 0, s, hi, lo, info, k, diag0,
-                               tol,
-                                                                    status, drop);
+    count_launch(), launch_pdl(pchol_potrf_kernel<true, float>, nblk, kThreads, 0, s, hi, lo, info,
+                               k, diag0, tol, status, drop);
     if (prof) kt_mark(prof, 1, s);
     if (maxPanel > 0)
       count_launch(), launch_pdl(pchol_trsm_ff_kernel,
