@@ -295,15 +295,17 @@ __device__ __forceinline__ void dz_stage_tile(F x, int nri, int npiv, __half *st
                                               long long slots, long long slot) {
   const int r = threadIdx.x >> 2, sl = threadIdx.x & 3, c0 = sl * 16;
   const bool row = r < nri;
-  int mx = 0;   // largest biased exponent
+  int mx = 0;   // largest high word (exponent and leading bits); 1 for a tiny nonzero
 #pragma unroll
   for (int j = 0; j < 16; ++j)
-    if (row && c0 + j < npiv)
-      mx = max(mx, (__double2hiint(x(r, c0 + j)) >> 20) & 0x7ff);
+    if (row && c0 + j < npiv) {
+      const double xv = x(r, c0 + j);
+      mx = max(mx, max(__double2hiint(xv) & 0x7fffffff, __double2loint(xv) ? 1 : 0));
+    }
   mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
   mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-  const bool fin = mx < 0x7ff;
-  const int E = mx - 1021;   // |x| < 2^(E - 1)
+  const bool fin = mx < 0x7ff00000;
+  const int E = mx ? (mx >> 20) - 1021 : 0;   // |x| < 2^(E - 1); a zero row takes 0
   if (sl == 0) dexp[slot * NB + r] = fin ? E : kDzNotFinite;
   __half *st = stage + ((long long)(sl * kDzQ) * slots + slot) * 1024 + (r >> 3) * 128 + (r & 7) * 8;
 #pragma unroll

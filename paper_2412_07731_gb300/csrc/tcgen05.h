@@ -44,8 +44,13 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// bounded wait for phase `parity` of the barrier; false when it ran out
+// bounded wait for phase `parity` of the barrier; false when it ran out.  The
+// timer is read only after some failed tries: most waits end at once, and one
+// timer read per wait would sit between consecutive MMAs.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+#pragma unroll 1
+  for (int i = 0; i < 16; ++i)
+    if (mbar_try(bar, parity)) return true;
   const unsigned long long t0 = globaltimer();
   while (!mbar_try(bar, parity))
     if (globaltimer() - t0 > kWaitNs) return false;

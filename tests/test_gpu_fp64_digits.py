@@ -78,6 +78,17 @@ def test_backward_error_with_several_jobs_per_cta(P):
     _check(P, lp, 5, 6.0, blocks=(0, 17, 31, 46, 58, 59))
 
 
+def test_backward_error_with_mixed_last_tiles(P):
+    """500 small blocks: a CTA's jobs of one step mix blocks whose pivot tile is full with
+    blocks whose last one has one, two or three slices of 16 columns, so the operand
+    buffers are reused with different numbers of slices."""
+    rng = np.random.default_rng(6)
+    m = [int(v) for v in rng.integers(66, 200, 500)]
+    lp = random_block_lp(24, N=500, m_sizes=m, n_sizes=[3 * v // 2 for v in m], nnz_per_col=6,
+                         n0=70, w_density=0.1, l=1)
+    _check(P, lp, 7, 4.0, blocks=[int(b) for b in rng.integers(0, 500, 40)])
+
+
 def test_nan_pivot_is_reported(P):
     """A block whose diagonal overflows to infinity: rows with a NaN or an infinity pass
     through the digit staging, and the factor is refused as before."""
