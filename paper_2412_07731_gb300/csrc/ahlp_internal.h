@@ -378,11 +378,11 @@ struct ahlp_problem {
   int *red_cnt = nullptr;     // arrivals at the reductions' last CTAs (0 between launches)
   double *mdot_part = nullptr;  // multi-dot partials [kMaxKrylov+1][304]
   double *gm_V = nullptr, *gm_Z = nullptr;   // Krylov bases, allocated on first use
-  double *gm_coef = nullptr;    // device coefficients for multi-axpy
   double *gm_h = nullptr;       // Arnoldi column on the device: both Gram-Schmidt passes and |w|^2
   int gm_cap = 0;               // vectors allocated in gm_Z (gm_V has one more)
   double *scal = nullptr;     // device scalars
-  double *h_scal = nullptr;   // pinned host scalars
+  double *h_scal = nullptr;   // pinned host scalars; [511] holds the sequence word below
+  unsigned read_seq = 0;      // value the device writes there when a read-back has arrived
   int *status = nullptr;      // device status words [4]
   // wavefront block solves: (block, row tile) jobs in ticket order, and the
   // ticket counters of the forward and backward block and chain solves (zeroed by
@@ -507,10 +507,11 @@ cudaError_t launch_mdot(ahlp_problem *p, const double *V, long long ld, int k, c
 // nrm2 also nrm2[0] = <w, w> and nrm2[1] = 1 / |w| (1 when <w, w> is not positive)
 cudaError_t launch_maxpy(ahlp_problem *p, const double *V, long long ld, int k, const double *coef,
                          double *w, long long len, double sign = 1.0, double *nrm2 = nullptr);
-// the same for w in three pieces of lengths n0, n1 and len - n0 - n1
+// w += sum_i coef[i] V_i, coefficients from the host, for w in three pieces of
+// lengths n0, n1 and len - n0 - n1
 cudaError_t launch_maxpy3(ahlp_problem *p, const double *V, long long ld, int k,
                           const double *coef, double *w0, long long n0, double *w1, long long n1,
-                          double *w2, long long len, double sign = 1.0, double *nrm2 = nullptr);
+                          double *w2, long long len);
 // y = a x, the factor on the device when da is not null
 cudaError_t launch_scale(double *y, const double *x, const double *da, double a, long long len,
                          cudaStream_t s);
@@ -518,6 +519,16 @@ cudaError_t launch_scale(double *y, const double *x, const double *da, double a,
 // also the first and third parts of J (dx, dy, dz) (adjoint: J')
 cudaError_t launch_finish(ahlp_problem *p, const double *dy, const double *rc, double *dx,
                           double *dz, bool adjoint, double *wx, double *wc);
+// dst <- src over n 32-bit words, two pieces, then *seq = val, all in host memory
+cudaError_t launch_publish(const unsigned *src, unsigned *dst, int n, const unsigned *src2,
+                           unsigned *dst2, int n2, unsigned *seq, unsigned val, cudaStream_t s);
+// up to four copies of doubles in one launch
+struct CopySet {
+  const double *src[4];
+  double *dst[4];
+  long long n[4];
+};
+cudaError_t launch_copies(const CopySet &c, cudaStream_t s);
 cudaError_t launch_mul(double *y, const double *a, const double *b, double scale, long long n,
                        cudaStream_t s);   // y = scale * a .* b
 // centrality corrector right-hand side: rc2 = rc + t, where v = (x + ap dx) .* (z + ad dz)
@@ -560,6 +571,13 @@ bool is_device_ptr(const void *ptr);
 const double *stage_in(ahlp_problem *p, const double *v, long long n, double *staging);
 int set_err(ahlp_problem *p, int code, const std::string &msg);
 void read_scalars(ahlp_problem *p, int k);
+// Read up to two pieces of device memory (32-bit words) back into pinned host
+// memory: a kernel writes them there, then a sequence word the host polls.
+// Everything launched on the stream before it is complete on return.  A memcpy
+// and a stream synchronisation cost about 9 us more, and a solve reads back once
+// per Krylov step and twice besides.
+void read_back(ahlp_problem *p, const void *src, void *dst, int words, const void *src2 = nullptr,
+               void *dst2 = nullptr, int words2 = 0);
 // ff_nan_up: a NaN pivot of a float-float factor refactors in FP64 (else the
 // call returns AHLP_ERR_NOT_SPD and the caller picks the next safeguard)
 int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol,

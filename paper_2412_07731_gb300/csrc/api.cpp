@@ -1299,11 +1299,11 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     p->red_cnt = dalloc<int>(p, kRedSetMax + 2);
     ck(cudaMemset(p->red_cnt, 0, (kRedSetMax + 2) * sizeof(int)), "memset");
     p->mdot_part = dalloc<double>(p, (long long)(kMaxKrylov + 1) * kMdotParts);
-    p->gm_coef = dalloc<double>(p, kMaxKrylov + 1);
     p->gm_h = dalloc<double>(p, 2 * (kMaxKrylov + 1) + 2);
     p->scal = dalloc<double>(p, 64);
     p->status = dalloc<int>(p, 8);
     ck(cudaMallocHost(&p->h_scal, 512 * sizeof(double)), "cudaMallocHost");
+    memset(p->h_scal, 0, 512 * sizeof(double));   // the sequence word starts at read_seq
     for (auto &e : p->ev) ck(cudaEventCreate(&e), "cudaEventCreate");
     ck(set_dense_smem_limits(), "smem limit");
     ck(set_schur_smem_limits(128 * 128 * 8), "smem limit");
@@ -1381,13 +1381,44 @@ int set_err(ahlp_problem *p, int code, const std::string &msg) {
   return code;
 }
 
-// read k device scalars into p->h_scal (synchronises the stream)
-void read_scalars(ahlp_problem *p, int k) {
-  p->bytes_d2h += k * (long long)sizeof(double);
-  ck(cudaMemcpyAsync(p->h_scal, p->scal, k * sizeof(double), cudaMemcpyDeviceToHost, p->stream),
-     "D2H scalars");
-  ck(cudaStreamSynchronize(p->stream), "stream sync");
+void read_back(ahlp_problem *p, const void *src, void *dst, int words, const void *src2,
+               void *dst2, int words2) {
+  p->bytes_d2h += 4LL * (words + words2);
+  unsigned *seq = reinterpret_cast<unsigned *>(p->h_scal + 511);
+  const unsigned val = ++p->read_seq;
+  ck(launch_publish(static_cast<const unsigned *>(src), static_cast<unsigned *>(dst), words,
+                    static_cast<const unsigned *>(src2), static_cast<unsigned *>(dst2), words2,
+                    seq, val, p->stream),
+     "read-back");
+  for (;;) {
+    for (int i = 0; i < 4096; ++i)
+      if (__atomic_load_n(seq, __ATOMIC_ACQUIRE) == val) return;
+    // a failed launch never writes the word: the stream then reports it
+    const cudaError_t e = cudaStreamQuery(p->stream);
+    if (e == cudaErrorNotReady) {
+      cudaGetLastError();
+      continue;
+    }
+    ck(e, "read-back");
+    if (__atomic_load_n(seq, __ATOMIC_ACQUIRE) != val)
+      throw Fail{AHLP_ERR_CUDA, "read-back did not arrive"};
+    return;
+  }
 }
+
+// milliseconds between two recorded events, waiting for the later one if need be
+static float event_ms(cudaEvent_t a, cudaEvent_t b) {
+  float ms = 0.0f;
+  if (cudaEventElapsedTime(&ms, a, b) == cudaErrorNotReady) {
+    cudaGetLastError();
+    ck(cudaEventSynchronize(b), "event");
+    cudaEventElapsedTime(&ms, a, b);
+  }
+  return ms;
+}
+
+// read k device scalars into p->h_scal (waits for the stream)
+void read_scalars(ahlp_problem *p, int k) { read_back(p, p->scal, p->h_scal, 2 * k); }
 
 void kt_mark(ahlp_problem *p, int cls, cudaStream_t s) {
   const size_t i = p->kt_cls.size();
@@ -1408,11 +1439,9 @@ void kt_collect(ahlp_problem *p) {
   for (size_t i = 0; i + 1 < p->kt_cls.size(); ++i) {
     const int c = p->kt_cls[i];
     if (c < 0 || c > 2) continue;
-    float ms = 0.0f;
-    if (cudaEventElapsedTime(&ms, p->kt_pool[i], p->kt_pool[i + 1]) == cudaSuccess) {
-      p->kt_ms[c] += ms;
-      ++p->kt_n[c];
-    }
+    const float ms = event_ms(p->kt_pool[i], p->kt_pool[i + 1]);
+    p->kt_ms[c] += ms;
+    ++p->kt_n[c];
   }
   p->kt_cls.clear();
 }
@@ -1444,9 +1473,7 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
   p->factored = false;
   p->fac_delta = delta;
   p->fac_rho = rho;
-  ck(cudaMemsetAsync(p->status, 0, 8 * sizeof(int), s), "memset");
   ck(cudaEventRecord(p->ev[0], s), "event");
-  ck(cudaMemsetAsync(p->cdiag0, 0, std::max(p->cdiag_elems, 1LL) * sizeof(double), s), "memset");
   ck(launch_dscale(p), "dscale");
   if (p->fac_prec == kPrecFP32 && p->n > 0) {
     // adaptive precision: once D = X Z^-1 spans more than fp32_cond_max the
@@ -1455,10 +1482,7 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
     const RedOne span[2] = {{RED_MAXABS, p->dscale, nullptr, p->n, p->scal + 2},
                             {RED_MIN, p->dscale, nullptr, p->n, p->scal + 3}};
     ck(launch_reduce_set(p, span, 2), "reduce");
-    p->bytes_d2h += 2 * sizeof(double);
-    ck(cudaMemcpyAsync(p->h_scal + 2, p->scal + 2, 2 * sizeof(double), cudaMemcpyDeviceToHost, s),
-       "D2H");
-    ck(cudaStreamSynchronize(s), "sync");
+    read_back(p, p->scal + 2, p->h_scal + 2, 4);
     if (!(p->h_scal[2] <= p->opt.fp32_cond_max * p->h_scal[3])) {
       if (p->opt.verbose)
         printf("D spans %.2e > fp32_cond_max: block factors move to float-float\n",
@@ -1505,13 +1529,11 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
   p->assembled = true;
   ck(launch_schur_factor(p), "schur factor");
   ck(cudaEventRecord(p->ev[3], s), "event");
-  int st[8];
-  p->bytes_d2h += sizeof(st);
-  ck(cudaMemcpyAsync(st, p->status, sizeof(st), cudaMemcpyDeviceToHost, s), "D2H status");
-  ck(cudaStreamSynchronize(s), "factor sync");
-  cudaEventElapsedTime(&p->stage_ms[0], p->ev[0], p->ev[1]);
-  cudaEventElapsedTime(&p->stage_ms[1], p->ev[1], p->ev[2]);
-  cudaEventElapsedTime(&p->stage_ms[2], p->ev[2], p->ev[3]);
+  const int *st = reinterpret_cast<const int *>(p->h_scal + 480);
+  read_back(p, p->status, p->h_scal + 480, 8);
+  p->stage_ms[0] = event_ms(p->ev[0], p->ev[1]);
+  p->stage_ms[1] = event_ms(p->ev[1], p->ev[2]);
+  p->stage_ms[2] = event_ms(p->ev[2], p->ev[3]);
   if (prof) kt_collect(p);
   p->tiny_pivots = st[1];
   if (st[4] != 0)
@@ -1548,7 +1570,6 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
                double *dy, double *dz, bool adjoint, ahlp_solve_info *info, double tol_override) {
   cudaStream_t s = p->stream;
   ck(cudaEventRecord(p->ev[4], s), "event");
-  ck(cudaMemsetAsync(p->trsv_err, 0, sizeof(int), s), "memset");
   ck(launch_solve(p, rd, rp, rc, dx, dy, dz, adjoint), "solve");
   const long long n = p->n, m = p->m, L = 2 * n + m;
   bool have_rhs = false;   // the right-hand side's norm is on the device
@@ -1562,10 +1583,8 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
                              {RED_DOT, rc, rc, n, p->scal + 12}};
     ck(launch_reduce_set(p, norms, have_rhs ? 1 : 4), "reduce");
     have_rhs = true;
-    p->bytes_d2h += 4 * sizeof(double);
-    ck(cudaMemcpyAsync(p->h_scal + 10, p->scal + 10, 4 * sizeof(double), cudaMemcpyDeviceToHost, s),
-       "D2H");
-    ck(cudaStreamSynchronize(s), "sync");
+    ck(cudaEventRecord(p->ev[5], s), "event");
+    read_back(p, p->scal + 10, p->h_scal + 10, 8, p->trsv_err, p->h_scal + 490, 1);
     return std::make_pair(std::sqrt(p->h_scal[13]),
                           std::sqrt(p->h_scal[10] + p->h_scal[11] + p->h_scal[12]));
   };
@@ -1594,7 +1613,7 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
       p->gm_cap = kmax;
     }
     double *V = p->gm_V, *Z = p->gm_Z;
-    double *cbuf = p->h_scal + 64, *hcol = p->h_scal + 256;
+    double *hcol = p->h_scal + 256;
     ck(launch_scale(V, p->res[0], nullptr, 1.0 / en, L, s), "scale");
     std::vector<double> H((size_t)(kc + 1) * kc, 0.0), cs(kc), sn(kc), g(kc + 1, 0.0);
     g[0] = en;
@@ -1617,9 +1636,7 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
       ck(launch_mdot(p, V, L, nh, W, L, gh + nh), "mdot");
       ck(launch_maxpy(p, V, L, nh, gh + nh, W, L, -1.0, gh + 2 * nh), "maxpy");
       ck(launch_scale(W, W, gh + 2 * nh + 1, 0.0, L, s), "scale");
-      p->bytes_d2h += (2 * nh + 1) * 8;
-      ck(cudaMemcpyAsync(hcol, gh, (2 * nh + 1) * 8, cudaMemcpyDeviceToHost, s), "D2H");
-      ck(cudaStreamSynchronize(s), "sync");
+      read_back(p, gh, hcol, 2 * (2 * nh + 1));
       for (int i = 0; i <= j; ++i) h[i] = (h[i] + hcol[i]) + hcol[nh + i];
       const double hn = std::sqrt(hcol[2 * nh]);
       h[j + 1] = hn;
@@ -1649,23 +1666,17 @@ int solve_impl(ahlp_problem *p, const double *rd, const double *rp, const double
       const double d = H[(size_t)i * (kc + 1) + i];
       y[i] = d != 0.0 ? t / d : 0.0;
     }
-    for (int i = 0; i < j; ++i) cbuf[i] = y[i];
-    p->bytes_h2d += j * 8;
-    ck(cudaMemcpyAsync(p->gm_coef, cbuf, j * 8, cudaMemcpyHostToDevice, s), "H2D");
-    ck(launch_maxpy3(p, Z, L, j, p->gm_coef, dx, n, dy, m, dz, L), "maxpy");
+    ck(launch_maxpy3(p, Z, L, j, y.data(), dx, n, dy, m, dz, L), "maxpy");
     steps += j;
     std::tie(en, rn) = residual_norms();
     rel = rn > 0 ? en / rn : en;
     if (!(rel <= 0.5 * prev)) break;
     prev = rel;
   }
-  ck(cudaEventRecord(p->ev[5], s), "event");
-  int timed_out = 0;
-  p->bytes_d2h += sizeof(int);
-  ck(cudaMemcpyAsync(&timed_out, p->trsv_err, sizeof(int), cudaMemcpyDeviceToHost, s), "D2H");
-  ck(cudaEventSynchronize(p->ev[5]), "sync");
-  ck(cudaStreamSynchronize(s), "sync");
-  cudaEventElapsedTime(&p->stage_ms[3], p->ev[4], p->ev[5]);
+  // the last residual's read-back saw everything above complete
+  p->stage_ms[3] = event_ms(p->ev[4], p->ev[5]);
+  const int timed_out = *reinterpret_cast<const int *>(p->h_scal + 490);
+  if (timed_out) ck(cudaMemsetAsync(p->trsv_err, 0, sizeof(int), s), "memset");
   if (timed_out)
     return set_err(p, AHLP_ERR_TIMEOUT, "kkt_solve: a block-solve wait exceeded its time limit");
   if (info) {
@@ -1691,6 +1702,7 @@ int kkt_factor(ahlp_problem *p, const double *x, const double *z, double delta, 
     const double r = rho < 0 ? p->opt.rho : rho;
     p->fac_rho_x = r > 0 ? r : 0.0;
     if (p->n > 0) {
+      // the caller's vectors: a copy takes any device's memory at any alignment
       ck(cudaMemcpyAsync(p->x, dx, p->n * 8, cudaMemcpyDeviceToDevice, p->stream), "copy x");
       ck(cudaMemcpyAsync(p->z, dz, p->n * 8, cudaMemcpyDeviceToDevice, p->stream), "copy z");
     }

@@ -121,8 +121,7 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
       }
     };
     auto factor_at = [&](const double *xx, const double *zz) {
-      ck(cudaMemcpyAsync(p->x, xx, n * 8, cudaMemcpyDeviceToDevice, s), "copy");
-      ck(cudaMemcpyAsync(p->z, zz, n * 8, cudaMemcpyDeviceToDevice, s), "copy");
+      ck(launch_copies(CopySet{{xx, zz}, {p->x, p->z}, {n, n}}, s), "copy");
       // a frozen LP of a batch sits at its converged, extremely ill-conditioned
       // point; its direction is zero (its right-hand sides are zeroed), so its
       // blocks are factored at x = z = 1 instead -- the LPs share no rows or
@@ -163,29 +162,27 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
       std::vector<double> nd(nlp);   // squared norm of each LP's slice
       for (int c0 = 0; c0 < nlp; c0 += 6) {
         const int cn = std::min(6, nlp - c0);
+        RedOne ops[42];
         for (int k = 0; k < cn; ++k) {
           const auto &r = p->lp_rng[c0 + k];
-          double *sc = p->scal + 20 + 5 * k;
-          ck(launch_reduce(p, RED_DOT, rd + r.xb0, rd + r.xb0, r.xb1 - r.xb0, sc + 0), "reduce");
-          ck(launch_reduce(p, RED_DOT, rd + r.x00, rd + r.x00, r.x01 - r.x00, sc + 1), "reduce");
-          ck(launch_reduce(p, RED_DOT, rc + r.xb0, rc + r.xb0, r.xb1 - r.xb0, sc + 2), "reduce");
-          ck(launch_reduce(p, RED_DOT, rc + r.x00, rc + r.x00, r.x01 - r.x00, sc + 3), "reduce");
-          ck(launch_reduce(p, RED_DOT, rp + r.yb0, rp + r.yb0, r.yb1 - r.yb0, sc + 4), "reduce");
+          double *sc = p->scal + 20 + 7 * k;
+          RedOne *o = ops + 7 * k;
+          o[0] = {RED_DOT, rd + r.xb0, rd + r.xb0, r.xb1 - r.xb0, sc + 0};
+          o[1] = {RED_DOT, rd + r.x00, rd + r.x00, r.x01 - r.x00, sc + 1};
+          o[2] = {RED_DOT, rc + r.xb0, rc + r.xb0, r.xb1 - r.xb0, sc + 2};
+          o[3] = {RED_DOT, rc + r.x00, rc + r.x00, r.x01 - r.x00, sc + 3};
+          o[4] = {RED_DOT, rp + r.yb0, rp + r.yb0, r.yb1 - r.yb0, sc + 4};
+          // the link and global rows of the LP
+          o[5] = {RED_DOT, rp + r.yl0, rp + r.yl0, r.yl1 - r.yl0, sc + 5};
+          o[6] = {RED_DOT, rp + r.yg0, rp + r.yg0, r.yg1 - r.yg0, sc + 6};
         }
-        read_scalars(p, 20 + 5 * cn);
+        ck(launch_reduce_set(p, ops, 7 * cn), "reduce");
+        read_scalars(p, 20 + 7 * cn);
         for (int k = 0; k < cn; ++k) {
-          const double *h = p->h_scal + 20 + 5 * k;
+          const double *h = p->h_scal + 20 + 7 * k;
           nd[c0 + k] = h[0] + h[1] + h[2] + h[3] + h[4];
+          nd[c0 + k] += h[5] + h[6];
         }
-        // the link and global rows of each LP
-        for (int k = 0; k < cn; ++k) {
-          const auto &r = p->lp_rng[c0 + k];
-          double *sc = p->scal + 20 + 2 * k;
-          ck(launch_reduce(p, RED_DOT, rp + r.yl0, rp + r.yl0, r.yl1 - r.yl0, sc + 0), "reduce");
-          ck(launch_reduce(p, RED_DOT, rp + r.yg0, rp + r.yg0, r.yg1 - r.yg0, sc + 1), "reduce");
-        }
-        read_scalars(p, 20 + 2 * cn);
-        for (int k = 0; k < cn; ++k) nd[c0 + k] += p->h_scal[20 + 2 * k] + p->h_scal[21 + 2 * k];
       }
       const long long n = p->n, m = p->m;
       ck(cudaMemcpyAsync(v[V_SD], rd, n * 8, cudaMemcpyDeviceToDevice, s), "copy");
@@ -303,15 +300,15 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
     auto lp_xreduce = [&](int op, const double *a, const double *bv, std::vector<double> &out) {
       for (int c0 = 0; c0 < nlp; c0 += 16) {
         const int cn = std::min(16, nlp - c0);
+        RedOne ops[32];
         for (int k = 0; k < cn; ++k) {
           const auto &r = p->lp_rng[c0 + k];
-          ck(launch_reduce(p, op, a + r.xb0, bv ? bv + r.xb0 : nullptr, r.xb1 - r.xb0,
-                           p->scal + 20 + 2 * k),
-             "reduce");
-          ck(launch_reduce(p, op, a + r.x00, bv ? bv + r.x00 : nullptr, r.x01 - r.x00,
-                           p->scal + 21 + 2 * k),
-             "reduce");
+          ops[2 * k] = {op, a + r.xb0, bv ? bv + r.xb0 : nullptr, r.xb1 - r.xb0,
+                        p->scal + 20 + 2 * k};
+          ops[2 * k + 1] = {op, a + r.x00, bv ? bv + r.x00 : nullptr, r.x01 - r.x00,
+                            p->scal + 21 + 2 * k};
         }
+        ck(launch_reduce_set(p, ops, 2 * cn), "reduce");
         read_scalars(p, 20 + 2 * cn);
         for (int k = 0; k < cn; ++k) {
           const double u = p->h_scal[20 + 2 * k], w = p->h_scal[21 + 2 * k];
@@ -325,18 +322,21 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
       for (int b = 0; b < nlp; ++b) {
         const auto &r = p->lp_rng[b];
         double *sc = p->scal + 20;
-        ck(launch_reduce(p, RED_MAXABS, v[V_RP] + r.yb0, nullptr, r.yb1 - r.yb0, sc + 0), "reduce");
-        ck(launch_reduce(p, RED_MAXABS, v[V_RP] + r.yl0, nullptr, r.yl1 - r.yl0, sc + 1), "reduce");
-        ck(launch_reduce(p, RED_MAXABS, v[V_RP] + r.yg0, nullptr, r.yg1 - r.yg0, sc + 2), "reduce");
-        ck(launch_reduce(p, RED_MAXABS, v[V_RD] + r.xb0, nullptr, r.xb1 - r.xb0, sc + 3), "reduce");
-        ck(launch_reduce(p, RED_MAXABS, v[V_RD] + r.x00, nullptr, r.x01 - r.x00, sc + 4), "reduce");
-        ck(launch_reduce(p, RED_DOT, p->c + r.xb0, X + r.xb0, r.xb1 - r.xb0, sc + 5), "reduce");
-        ck(launch_reduce(p, RED_DOT, p->c + r.x00, X + r.x00, r.x01 - r.x00, sc + 6), "reduce");
-        ck(launch_reduce(p, RED_DOT, p->b + r.yb0, Y + r.yb0, r.yb1 - r.yb0, sc + 7), "reduce");
-        ck(launch_reduce(p, RED_DOT, p->b + r.yl0, Y + r.yl0, r.yl1 - r.yl0, sc + 8), "reduce");
-        ck(launch_reduce(p, RED_DOT, p->b + r.yg0, Y + r.yg0, r.yg1 - r.yg0, sc + 9), "reduce");
-        ck(launch_reduce(p, RED_DOT, X + r.xb0, Z + r.xb0, r.xb1 - r.xb0, sc + 10), "reduce");
-        ck(launch_reduce(p, RED_DOT, X + r.x00, Z + r.x00, r.x01 - r.x00, sc + 11), "reduce");
+        const RedOne meas[12] = {
+            {RED_MAXABS, v[V_RP] + r.yb0, nullptr, r.yb1 - r.yb0, sc + 0},
+            {RED_MAXABS, v[V_RP] + r.yl0, nullptr, r.yl1 - r.yl0, sc + 1},
+            {RED_MAXABS, v[V_RP] + r.yg0, nullptr, r.yg1 - r.yg0, sc + 2},
+            {RED_MAXABS, v[V_RD] + r.xb0, nullptr, r.xb1 - r.xb0, sc + 3},
+            {RED_MAXABS, v[V_RD] + r.x00, nullptr, r.x01 - r.x00, sc + 4},
+            {RED_DOT, p->c + r.xb0, X + r.xb0, r.xb1 - r.xb0, sc + 5},
+            {RED_DOT, p->c + r.x00, X + r.x00, r.x01 - r.x00, sc + 6},
+            {RED_DOT, p->b + r.yb0, Y + r.yb0, r.yb1 - r.yb0, sc + 7},
+            {RED_DOT, p->b + r.yl0, Y + r.yl0, r.yl1 - r.yl0, sc + 8},
+            {RED_DOT, p->b + r.yg0, Y + r.yg0, r.yg1 - r.yg0, sc + 9},
+            {RED_DOT, X + r.xb0, Z + r.xb0, r.xb1 - r.xb0, sc + 10},
+            {RED_DOT, X + r.x00, Z + r.x00, r.x01 - r.x00, sc + 11},
+        };
+        ck(launch_reduce_set(p, meas, 12), "reduce");
         read_scalars(p, 32);
         const double *h = p->h_scal + 20;
         const double pinf = std::max({h[0], h[1], h[2]}) / (1.0 + r.bnorm);
@@ -395,14 +395,16 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
       st = solve(p->c, zero_m, ones, v[V_DXA], Y, Z);
       if (st != AHLP_OK) throw Fail{st, p->err};
       ck(cudaMemcpyAsync(X, v[V_DX], n * 8, cudaMemcpyDeviceToDevice, s), "copy");
-      ck(launch_reduce(p, RED_MIN, X, nullptr, n, p->scal + 0), "reduce");
-      ck(launch_reduce(p, RED_MIN, Z, nullptr, n, p->scal + 1), "reduce");
+      const RedOne mins[2] = {{RED_MIN, X, nullptr, n, p->scal + 0},
+                              {RED_MIN, Z, nullptr, n, p->scal + 1}};
+      ck(launch_reduce_set(p, mins, 2), "reduce");
       read_scalars(p, 2);
       ck(launch_add_scalar(X, X, std::max(-1.5 * p->h_scal[0], 0.0), n, s), "shift");
       ck(launch_add_scalar(Z, Z, std::max(-1.5 * p->h_scal[1], 0.0), n, s), "shift");
-      ck(launch_reduce(p, RED_DOT, X, Z, n, p->scal + 0), "reduce");
-      ck(launch_reduce(p, RED_SUM, X, nullptr, n, p->scal + 1), "reduce");
-      ck(launch_reduce(p, RED_SUM, Z, nullptr, n, p->scal + 2), "reduce");
+      const RedOne sums[3] = {{RED_DOT, X, Z, n, p->scal + 0},
+                              {RED_SUM, X, nullptr, n, p->scal + 1},
+                              {RED_SUM, Z, nullptr, n, p->scal + 2}};
+      ck(launch_reduce_set(p, sums, 3), "reduce");
       read_scalars(p, 3);
       const double xz = p->h_scal[0], sx = p->h_scal[1], sz = p->h_scal[2];
       const double ax = sz > 0 ? 0.5 * xz / sz : 1.0, az = sx > 0 ? 0.5 * xz / sx : 1.0;
@@ -418,13 +420,14 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
       ck(launch_spmv(p->Amat, X, v[V_RP], -1.0, p->b, s), "spmv");
       ck(launch_spmv(p->ATmat, Y, v[V_RD], -1.0, p->c, s), "spmv");
       ck(launch_axpby(v[V_RD], Z, -1.0, 1.0, n, s), "axpby");
-      ck(launch_reduce(p, RED_MAXABS, v[V_RP], nullptr, m, p->scal + 0), "reduce");
-      ck(launch_reduce(p, RED_MAXABS, v[V_RD], nullptr, n, p->scal + 1), "reduce");
-      ck(launch_reduce(p, RED_DOT, p->c, X, n, p->scal + 2), "reduce");
-      ck(launch_reduce(p, RED_DOT, p->b, Y, m, p->scal + 3), "reduce");
-      ck(launch_reduce(p, RED_DOT, X, Z, n, p->scal + 4), "reduce");
-      ck(launch_reduce(p, RED_MAXABS, X, nullptr, n, p->scal + 5), "reduce");
-      ck(launch_reduce(p, RED_MAXABS, Y, nullptr, m, p->scal + 6), "reduce");
+      const RedOne meas[7] = {{RED_MAXABS, v[V_RP], nullptr, m, p->scal + 0},
+                              {RED_MAXABS, v[V_RD], nullptr, n, p->scal + 1},
+                              {RED_DOT, p->c, X, n, p->scal + 2},
+                              {RED_DOT, p->b, Y, m, p->scal + 3},
+                              {RED_DOT, X, Z, n, p->scal + 4},
+                              {RED_MAXABS, X, nullptr, n, p->scal + 5},
+                              {RED_MAXABS, Y, nullptr, m, p->scal + 6}};
+      ck(launch_reduce_set(p, meas, 7), "reduce");
       read_scalars(p, 7);
       const double *hs = p->h_scal;
       R.pinf = hs[0] / (1.0 + p->bnorm_inf);
@@ -534,8 +537,9 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
             }
           }
         } else {
-          ck(launch_reduce(p, RED_MINSTEP, X, v[V_DXA], n, p->scal + 0), "reduce");
-          ck(launch_reduce(p, RED_MINSTEP, Z, v[V_DZA], n, p->scal + 1), "reduce");
+          const RedOne rat[2] = {{RED_MINSTEP, X, v[V_DXA], n, p->scal + 0},
+                                 {RED_MINSTEP, Z, v[V_DZA], n, p->scal + 1}};
+          ck(launch_reduce_set(p, rat, 2), "reduce");
           read_scalars(p, 2);
           const double apa = std::min(1.0, p->h_scal[0]), ada = std::min(1.0, p->h_scal[1]);
           ck(launch_step_dot(p, X, v[V_DXA], apa, Z, v[V_DZA], ada, n, p->scal + 0),
@@ -571,8 +575,9 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
                            : p->opt.max_correctors;
       if (kmax > 0 && nlp == 0) {
         auto steps = [&](const double *dxv, const double *dzv, double &a_p, double &a_d) {
-          ck(launch_reduce(p, RED_MINSTEP, X, dxv, n, p->scal + 0), "reduce");
-          ck(launch_reduce(p, RED_MINSTEP, Z, dzv, n, p->scal + 1), "reduce");
+          const RedOne rat[2] = {{RED_MINSTEP, X, dxv, n, p->scal + 0},
+                                 {RED_MINSTEP, Z, dzv, n, p->scal + 1}};
+          ck(launch_reduce_set(p, rat, 2), "reduce");
           read_scalars(p, 2);
           a_p = std::min(1.0, p->h_scal[0]);
           a_d = std::min(1.0, p->h_scal[1]);
@@ -673,8 +678,9 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
         lp_axpy(Z, v[V_DZ], lp_ad, false);
         continue;
       }
-      ck(launch_reduce(p, RED_MINSTEP, X, v[V_DX], n, p->scal + 0), "reduce");
-      ck(launch_reduce(p, RED_MINSTEP, Z, v[V_DZ], n, p->scal + 1), "reduce");
+      const RedOne rat[2] = {{RED_MINSTEP, X, v[V_DX], n, p->scal + 0},
+                             {RED_MINSTEP, Z, v[V_DZ], n, p->scal + 1}};
+      ck(launch_reduce_set(p, rat, 2), "reduce");
       read_scalars(p, 2);
       const double ap = std::min(1.0, eta * p->h_scal[0]), ad = std::min(1.0, eta * p->h_scal[1]);
       ck(launch_axpby(X, v[V_DX], ap, 1.0, n, s), "update");

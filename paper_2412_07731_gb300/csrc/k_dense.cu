@@ -17,6 +17,8 @@
 #include <cuda_fp16.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "ahlp_internal.h"
 #include "publish.h"
 
@@ -95,11 +97,15 @@ __global__ void __launch_bounds__(kThreads) form_aug_kernel(FormArgs<T> A) {
 // two per-variable quotients every solve at this point needs (FP64 division
 // is a long instruction sequence on this part): xinv = 1 / x and
 // w = 1 / (1 / d + rho on the linking variables).
+// It also clears the factor's status words and the corner diagonals.
 __global__ void dscale_kernel(const double *x, const double *z, double *d, double *xinv,
                               double *w, long long n, double rho_x, double rho,
-                              const unsigned char *is_x0) {
+                              const unsigned char *is_x0, int *status, double *cdiag0,
+                              long long ncd) {
   pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < 8) status[i] = 0;
+  for (long long q = i; q < ncd; q += (long long)gridDim.x * blockDim.x) cdiag0[q] = 0.0;
   if (i >= n) return;
   const double di = (rho_x > 0.0 && !is_x0[i]) ? x[i] / (z[i] + rho_x * x[i]) : x[i] / z[i];
   d[i] = di;
@@ -1772,10 +1778,10 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
 
 // ---------------------------------------------------------------------------
 cudaError_t launch_dscale(ahlp_problem *p) {
-  if (p->n <= 0) return cudaSuccess;
-  count_launch(), launch_pdl(dscale_kernel, (unsigned)((p->n + 255) / 256), 256, 0, p->stream,
-                             p->x, p->z, p->dscale, p->xinv, p->wfin, p->n, p->fac_rho_x,
-                             p->fac_rho, p->is_x0);
+  count_launch(), launch_pdl(dscale_kernel, (unsigned)((std::max(p->n, 8LL) + 255) / 256), 256, 0,
+                             p->stream, p->x, p->z, p->dscale, p->xinv, p->wfin, p->n,
+                             p->fac_rho_x, p->fac_rho, p->is_x0, p->status, p->cdiag0,
+                             p->cdiag_elems);
   return cudaGetLastError();
 }
 

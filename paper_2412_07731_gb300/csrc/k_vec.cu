@@ -401,20 +401,25 @@ __global__ void __launch_bounds__(kRedThreads) mdot_kernel(const double *V,
 }
 
 // w[e] += sum_i coef[i] V_i[e], fixed order over i, for vectors in up to three
-// pieces (w0, w1, w2 of lengths n0, n1 and the rest; V_i contiguous).  With
+// pieces (w0, w1, w2 of lengths n0, n1 and the rest; V_i contiguous); the
+// coefficients come from the device (coef, times sc) or by value.  With
 // nrm2 the last CTA also leaves nrm2[0] = <w, w> and nrm2[1] = 1 / |w| (1 when
 // <w, w> is not positive).
-__global__ void __launch_bounds__(kRedThreads) maxpy_kernel(const double *V,
-                                                            long long ld, int k,
-                                                            const double *coef,
-                                                            double sc, double *w0, long long n0,
-                                                            double *w1, long long n1, double *w2,
+struct HostCoefs {
+  double c[kMaxKrylov];
+};
+
+__global__ void __launch_bounds__(kRedThreads) maxpy_kernel(const double *V, long long ld, int k,
+                                                            const double *coef, double sc,
+                                                            const HostCoefs hc, double *w0,
+                                                            long long n0, double *w1,
+                                                            long long n1, double *w2,
                                                             long long len, double *part,
                                                             double *nrm2, int *cnt) {
   pdl_begin();
   __shared__ double cs[kMaxKrylov + 1];
   __shared__ double sh[kRedThreads / 32];
-  for (int i = threadIdx.x; i < k; i += blockDim.x) cs[i] = sc * coef[i];
+  for (int i = threadIdx.x; i < k; i += blockDim.x) cs[i] = coef ? sc * coef[i] : hc.c[i];
   __syncthreads();
   const long long stride = (long long)gridDim.x * blockDim.x;
   double q = 0.0;
@@ -439,6 +444,28 @@ __global__ void __launch_bounds__(kRedThreads) maxpy_kernel(const double *V,
   }
 }
 
+__global__ void publish_k(const unsigned *src, unsigned *dst, int n, const unsigned *src2,
+                          unsigned *dst2, int n2, unsigned *seq, unsigned val) {
+  pdl_begin();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
+  for (int i = threadIdx.x; i < n2; i += blockDim.x) dst2[i] = src2[i];
+  __threadfence_system();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence_system();
+    *reinterpret_cast<volatile unsigned *>(seq) = val;
+  }
+}
+
+__global__ void copies_k(const CopySet c) {
+  pdl_begin();
+  const double *src = c.src[blockIdx.y];
+  double *dst = c.dst[blockIdx.y];
+  const long long n = c.n[blockIdx.y], stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
+    dst[i] = src[i];
+}
+
 // y = a x, a on the device (da) or not
 __global__ void scale_k(double *y, const double *x, const double *da, double a, long long n) {
   pdl_begin();
@@ -460,17 +487,36 @@ cudaError_t launch_mdot(ahlp_problem *p, const double *V, long long ld, int k, c
 
 cudaError_t launch_maxpy(ahlp_problem *p, const double *V, long long ld, int k, const double *coef,
                          double *w, long long len, double sign, double *nrm2) {
-  return launch_maxpy3(p, V, ld, k, coef, w, len, w, 0, w, len, sign, nrm2);
+  if (k <= 0 || len <= 0) return cudaSuccess;
+  count_launch(), launch_pdl(maxpy_kernel, red_blocks(len, kMaxpyBlocks), kRedThreads, 0,
+                             p->stream, V, ld, k, coef, sign, HostCoefs{}, w, len, w, 0, w, len,
+                             p->red_part, nrm2, p->red_cnt + kRedSetMax + 1);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_maxpy3(ahlp_problem *p, const double *V, long long ld, int k,
                           const double *coef, double *w0, long long n0, double *w1, long long n1,
-                          double *w2, long long len, double sign, double *nrm2) {
+                          double *w2, long long len) {
   if (k <= 0 || len <= 0) return cudaSuccess;
+  HostCoefs hc{};
+  for (int i = 0; i < k; ++i) hc.c[i] = coef[i];
   count_launch(), launch_pdl(maxpy_kernel, red_blocks(len, kMaxpyBlocks), kRedThreads, 0,
-                             p->stream, V, ld, k, coef, sign, w0, n0, w1, n1, w2, len, p->red_part,
-                             nrm2,
-      p->red_cnt + kRedSetMax + 1);
+                             p->stream, V, ld, k, nullptr, 1.0, hc, w0, n0, w1, n1, w2, len,
+                             p->red_part, nullptr, p->red_cnt + kRedSetMax + 1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_publish(const unsigned *src, unsigned *dst, int n, const unsigned *src2,
+                           unsigned *dst2, int n2, unsigned *seq, unsigned val, cudaStream_t s) {
+  count_launch(), launch_pdl(publish_k, 1, 64, 0, s, src, dst, n, src2, dst2, n2, seq, val);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_copies(const CopySet &c, cudaStream_t s) {
+  const long long n = std::max(std::max(c.n[0], c.n[1]), std::max(c.n[2], c.n[3]));
+  if (n <= 0) return cudaSuccess;
+  const unsigned g = (unsigned)std::min<long long>((n + 255) / 256, 1216);
+  count_launch(), launch_pdl(copies_k, dim3(g, 4), 256, 0, s, c);
   return cudaGetLastError();
 }
 
