@@ -278,7 +278,13 @@ struct ahlp_problem {
   // block over its FP32 augmented matrix
   float *pstage = nullptr;
   long long stage_slots = 0;
-  int *tc_joff = nullptr;            // [maxTp][N + 1]
+  int *tc_joff = nullptr;            // [maxTp][2 N + 2] (StepJobs::joff)
+  // diagonal tiles of the next step, counted off by an update's CTAs: [maxTp][N],
+  // cleared by launch_dscale; blocks a step's jobs do not touch; blocks per step
+  int *la_ready = nullptr, *la_miss = nullptr;
+  long long la_elems = 0;
+  std::vector<long long> la_miss_off;
+  std::vector<int> la_pot;
   std::vector<long long> tc_jobs;    // [maxTp]
   // FP64 factors on the tensor cores: each panel tile of the current step as
   // eight FP16 digit planes, one exponent per row, and the CUtensorMaps of the
@@ -420,6 +426,12 @@ long long launch_count();
 
 // ---- kernels (launch wrappers) --------------------------------------------
 // All wrappers enqueue on p->stream and return the cudaError_t of the launch.
+// What a diagonal factorisation that runs beside the step before it waits for:
+// ready[b] >= target (ready == nullptr: for that whole kernel, as usual).
+struct LookAhead {
+  int *ready = nullptr;
+  int target = 0;
+};
 cudaError_t launch_dscale(ahlp_problem *p);   // dscale = x / (z + fac_rho_x x)
 cudaError_t launch_form(ahlp_problem *p, double delta);
 // prof (nullable): a handle whose kernel-class timer records the launches
@@ -544,14 +556,14 @@ cudaError_t launch_step_dot(ahlp_problem *p, const double *x, const double *dx, 
 // staging, job offsets and tensor maps for the FP32 factors (needs aug32);
 // false when the driver has no tensor-map encoder
 bool tc_setup(ahlp_problem *p);
-cudaError_t launch_update_tc(ahlp_problem *p, int k, cudaStream_t s);
+cudaError_t launch_update_tc(ahlp_problem *p, int k, cudaStream_t s, LookAhead *la);
 // the same for float-float factors: FP16 digit staging and job offsets
 bool oz_setup(ahlp_problem *p);
-cudaError_t launch_update_oz(ahlp_problem *p, int k, cudaStream_t s);
+cudaError_t launch_update_oz(ahlp_problem *p, int k, cudaStream_t s, LookAhead *la);
 
 // the same for FP64 factors: eight-digit staging, job offsets, tensor maps
 bool dz_setup(ahlp_problem *p);
-cudaError_t launch_update_dz(ahlp_problem *p, int k, cudaStream_t s);
+cudaError_t launch_update_dz(ahlp_problem *p, int k, cudaStream_t s, LookAhead *la);
 // update jobs of every step (called by the three set-ups)
 void jobs_setup(ahlp_problem *p);
 

@@ -97,15 +97,17 @@ __global__ void __launch_bounds__(kThreads) form_aug_kernel(FormArgs<T> A) {
 // two per-variable quotients every solve at this point needs (FP64 division
 // is a long instruction sequence on this part): xinv = 1 / x and
 // w = 1 / (1 / d + rho on the linking variables).
-// It also clears the factor's status words and the corner diagonals.
+// It also clears the factor's status words, the corner diagonals and the counts of
+// updated diagonal tiles.
 __global__ void dscale_kernel(const double *x, const double *z, double *d, double *xinv,
                               double *w, long long n, double rho_x, double rho,
                               const unsigned char *is_x0, int *status, double *cdiag0,
-                              long long ncd) {
+                              long long ncd, int *ready, long long nready) {
   pdl_begin();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < 8) status[i] = 0;
   for (long long q = i; q < ncd; q += (long long)gridDim.x * blockDim.x) cdiag0[q] = 0.0;
+  for (long long q = i; q < nready; q += (long long)gridDim.x * blockDim.x) ready[q] = 0;
   if (i >= n) return;
   const double di = (rho_x > 0.0 && !is_x0[i]) ? x[i] / (z[i] + rho_x * x[i]) : x[i] / z[i];
   d[i] = di;
@@ -150,15 +152,51 @@ __device__ __forceinline__ double rsqrt_f64(double p) {
 
 constexpr int kPW = 16;   // panel width
 
+// Start and end of a diagonal factorisation.  With la.ready the kernel runs beside
+// the update of the step before: it was launched as that update's programmatic
+// dependent, so the update's CTAs have all started (they never wait for this
+// kernel, and everything before them is complete), a block waits for its own tile
+// only, and the whole update is waited for at the end, on behalf of the panel
+// kernel behind.  The wait is bounded (1 s), then status[4] is set.
+__device__ __forceinline__ bool diag_begin(const LookAhead &la, bool active, int *status) {
+  if (!la.ready || !active) {
+    pdl_begin();
+    return active;
+  }
+  if (threadIdx.x == 0) {
+    const int *f = la.ready + blockIdx.x;
+    const unsigned long long t0 = global_ns();
+    for (int it = 0; load_relaxed(f) < la.target; ++it) {
+      __nanosleep(100);
+      if ((it & 31) == 31 && global_ns() - t0 > kWaitLimitNs) {
+        atomicExch(&status[4], 1);
+        break;
+      }
+    }
+    __threadfence();   // the tile's writes, ordered before the count, are visible
+  }
+  __syncthreads();
+  return true;
+}
+
+__device__ __forceinline__ void diag_end(const LookAhead &la) {
+  if (la.ready) pdl_begin();
+}
+
+// Unused shared memory of an FP64 or float-float diagonal tile beside an update:
+// at most two per SM, since they share its FP64 pipe (three: 28.4 against 27.7 ms
+// per FP64 factor and solve of 32 uneven blocks).
+constexpr int kDiagPad = 60000;
+
 // kFF: the matrix is hi + lo (lo null otherwise)
 template <bool kFF, typename T>
 __global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(T *buf, float *lo,
                                                                const BlkInfo *blk, int k,
                                                                const double *diag0, double tol,
-                                                               int *status, double drop) {
-  pdl_begin();
+                                                               int *status, double drop,
+                                                               const LookAhead la) {
   const BlkInfo bi = blk[blockIdx.x];
-  if (k >= bi.Tp) return;
+  if (!diag_begin(la, k < bi.Tp, status)) return;
   __shared__ double t[NB][NB + 1];
   __shared__ double s_piv[NB], s_inv[NB];
   const int r0 = k * NB;
@@ -284,6 +322,7 @@ __global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(T *buf, float *lo
       }
     }
   }
+  diag_end(la);
 }
 
 // One 64 x 64 FP64 panel tile as eight FP16 digit planes for the tensor-core
@@ -438,10 +477,9 @@ __global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkI
 constexpr int kPotrf32Threads = 256;
 __global__ void __launch_bounds__(kPotrf32Threads) pchol_potrf_f32_kernel(
     float *buf, float *tinv, const BlkInfo *blk, int k, const double *diag0, float tol,
-    int *status, float drop) {
-  pdl_begin();
+    int *status, float drop, const LookAhead la) {
   const BlkInfo bi = blk[blockIdx.x];
-  if (k >= bi.Tp) return;
+  if (!diag_begin(la, k < bi.Tp, status)) return;
   __shared__ float t[NB][NB + 1];
   __shared__ float X[NB][NB + 1];
   __shared__ float Tm[kPW][NB];
@@ -649,6 +687,7 @@ __global__ void __launch_bounds__(kPotrf32Threads) pchol_potrf_f32_kernel(
     if (r < nr && c < nr && r >= c) g[(long long)c * bi.lda + r] = t[r][c];
     out[i] = r < npiv ? X[r][c] : (c < npiv ? t[r][c] : 0.0f);
   }
+  diag_end(la);
 }
 
 // Panel tile (I, k) below the diagonal: X = A_Ik L_kk^-T on the pivot columns
@@ -1722,7 +1761,9 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
   if (nblk == 0) return cudaSuccess;
   int maxTp = 0;
   for (auto &b : h) maxTp = b.Tp > maxTp ? b.Tp : maxTp;
+  LookAhead la;   // this step's diagonal tiles, beside the update before
   for (int k = 0; k < maxTp; ++k) {
+    LookAhead next;
     long long maxPanel = 0, maxTrail = 0;
     for (auto &b : h) {
       if (k >= b.Tp) continue;
@@ -1733,7 +1774,7 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
     if constexpr (sizeof(T) == sizeof(float)) {
       if (prof) kt_mark(prof, 0, s);
       count_launch(), launch_pdl(pchol_potrf_f32_kernel, nblk, kPotrf32Threads, 0, s, buf, tinv,
-                                 info, k, diag0, (float)tol, status, (float)drop);
+                                 info, k, diag0, (float)tol, status, (float)drop, la);
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
         count_launch(), launch_pdl(pchol_trsm_inv_kernel<T>, dim3((unsigned)maxPanel, nblk),
@@ -1741,8 +1782,9 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
                                    tc ? tc->pstage : nullptr);
     } else {
       if (prof) kt_mark(prof, 0, s);
-      count_launch(), launch_pdl(pchol_potrf_kernel<false, double>, nblk, kThreads, 0, s, buf,
-                                 nullptr, info, k, diag0, tol, status, drop);
+      count_launch(), launch_pdl(pchol_potrf_kernel<false, double>, nblk, kThreads,
+                                 la.ready ? kDiagPad : 0, s, buf,
+                                 nullptr, info, k, diag0, tol, status, drop, la);
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
         count_launch(), launch_pdl(pchol_trsm_kernel<T>, dim3((unsigned)maxPanel, nblk), kThreads,
@@ -1753,14 +1795,14 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
     if (maxTrail > 0) {
       if constexpr (sizeof(T) == sizeof(float)) {
         if (tc) {
-          cudaError_t e = launch_update_tc(tc, k, s);
+          cudaError_t e = launch_update_tc(tc, k, s, &next);
           if (e != cudaSuccess) return e;
         } else {
           count_launch(), launch_pdl(pchol_update_f32_kernel, dim3((unsigned)maxTrail, nblk),
                                      kUpdF32Threads, 0, s, buf, info, k);
         }
       } else if (dz) {
-        cudaError_t e = launch_update_dz(dz, k, s);
+        cudaError_t e = launch_update_dz(dz, k, s, &next);
         if (e != cudaSuccess) return e;
       } else {
         count_launch(), launch_pdl(pchol_update_kernel<T>, dim3((unsigned)maxTrail, nblk),
@@ -1768,6 +1810,7 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
       }
     }
     if (prof) kt_mark(prof, 3, s);
+    la = next;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -1781,7 +1824,7 @@ cudaError_t launch_dscale(ahlp_problem *p) {
   count_launch(), launch_pdl(dscale_kernel, (unsigned)((std::max(p->n, 8LL) + 255) / 256), 256, 0,
                              p->stream, p->x, p->z, p->dscale, p->xinv, p->wfin, p->n,
                              p->fac_rho_x, p->fac_rho, p->is_x0, p->status, p->cdiag0,
-                             p->cdiag_elems);
+                             p->cdiag_elems, p->la_ready, p->la_elems);
   return cudaGetLastError();
 }
 
@@ -1814,7 +1857,9 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
   if (nblk == 0) return cudaSuccess;
   int maxTp = 0;
   for (auto &b : h) maxTp = b.Tp > maxTp ? b.Tp : maxTp;
+  LookAhead la;   // this step's diagonal tiles, beside the update before
   for (int k = 0; k < maxTp; ++k) {
+    LookAhead next;
     long long maxPanel = 0, maxTrail = 0;
     for (auto &b : h) {
       if (k >= b.Tp) continue;
@@ -1823,8 +1868,9 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
       if (t * (t + 1) / 2 > maxTrail) maxTrail = t * (t + 1) / 2;
     }
     if (prof) kt_mark(prof, 0, s);
-    count_launch(), launch_pdl(pchol_potrf_kernel<true, float>, nblk, kThreads, 0, s, hi, lo, info,
-                               k, diag0, tol, status, drop);
+    count_launch(), launch_pdl(pchol_potrf_kernel<true, float>, nblk, kThreads,
+                               la.ready ? kDiagPad : 0, s, hi, lo, info,
+                               k, diag0, tol, status, drop, la);
     if (prof) kt_mark(prof, 1, s);
     if (maxPanel > 0)
       count_launch(), launch_pdl(pchol_trsm_ff_kernel,
@@ -1834,7 +1880,7 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
     if (prof) kt_mark(prof, 2, s);
     if (maxTrail > 0) {
       if (oz) {
-        cudaError_t e = launch_update_oz(oz, k, s);
+        cudaError_t e = launch_update_oz(oz, k, s, &next);
         if (e != cudaSuccess) return e;
       } else {
         count_launch(), launch_pdl(pchol_update_ff8_kernel, dim3((unsigned)maxTrail, nblk),
@@ -1842,6 +1888,7 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
       }
     }
     if (prof) kt_mark(prof, 3, s);
+    la = next;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -1921,8 +1968,14 @@ cudaError_t launch_tile_inverses(const double *buf, double *tinv, const BlkInfo 
 }
 
 cudaError_t set_dense_smem_limits() {
-  cudaError_t e = cudaFuncSetAttribute(tinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kTinvSmem);
+  cudaError_t e = cudaFuncSetAttribute(pchol_potrf_kernel<false, double>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kDiagPad);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(pchol_potrf_kernel<true, float>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, kDiagPad);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(tinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kTinvSmem);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(pchol_update_ff8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)kUpdFFSmem);

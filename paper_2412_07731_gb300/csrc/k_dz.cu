@@ -128,18 +128,16 @@ __device__ __forceinline__ double dz_scale(long long p, int sc) {
 
 struct DzArgs {
   const int *dexp;         // per slot 64 row exponents
-  const int *joff;
-  const BlkInfo *blk;
   double *buf;             // the augmented matrices
-  int nblk, k;
   int *status;
-  const int4 *jt;          // this step's tile-sparse job table, or nullptr
+  StepJobs S;
 };
 
 __global__ void __launch_bounds__(kDzThreads, 1)
     pchol_update_dz_kernel(const DzArgs args, const __grid_constant__ CUtensorMap mapA,
-                           const __grid_constant__ CUtensorMap mapB, int njobs) {
+                           const __grid_constant__ CUtensorMap mapB) {
   pdl_wait();
+  jobs_begin(args.S, kDzEpiWarps);
   extern __shared__ __align__(1024) unsigned char dz_raw[];
   __shared__ __align__(8) uint64_t full[kDzStages], empty[kDzStages], tfull, tempty;
   __shared__ uint32_t tmem_slot;
@@ -147,8 +145,7 @@ __global__ void __launch_bounds__(kDzThreads, 1)
   unsigned char *base = dz_raw + ((1024 - (smem_u32(dz_raw) & 1023)) & 1023);
   volatile int *vfail = &s_fail;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int myjobs = (int)blockIdx.x < njobs ? (njobs - 1 - (int)blockIdx.x) / (int)gridDim.x + 1
-                                             : 0;
+  const int myjobs = my_jobs(args.S);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_slot)),
@@ -177,10 +174,9 @@ __global__ void __launch_bounds__(kDzThreads, 1)
     if (lane == 0) {
       int u = 0;   // units issued
       for (int j = 0; j < myjobs && !*vfail; ++j) {
-        const Job jb = decode_job(args.joff, args.nblk, args.k, args.blk,
-                                  (int)blockIdx.x + j * (int)gridDim.x, args.jt);
-        const BlkInfo &bi = args.blk[jb.b];
-        const int npiv = min(NB, bi.p - args.k * NB), soff = (int)bi.soff;
+        const Job jb = decode_job(args.S, job_index(args.S, j));
+        const BlkInfo &bi = args.S.blk[jb.b];
+        const int npiv = min(NB, bi.p - args.S.k * NB), soff = (int)bi.soff;
         const int ns = (npiv + kDzSliceK - 1) / kDzSliceK;
         bool ok = true;
         for (int sl = 0; sl < ns; ++sl, ++u) {
@@ -209,9 +205,8 @@ __global__ void __launch_bounds__(kDzThreads, 1)
     if (lane == 0) {
       int u = 0, last = -1;   // last unit whose MMAs were committed
       for (int j = 0; j < myjobs && !*vfail; ++j) {
-        const Job jb = decode_job(args.joff, args.nblk, args.k, args.blk,
-                                  (int)blockIdx.x + j * (int)gridDim.x, args.jt);
-        const int npiv = min(NB, args.blk[jb.b].p - args.k * NB);
+        const Job jb = decode_job(args.S, job_index(args.S, j));
+        const int npiv = min(NB, args.S.blk[jb.b].p - args.S.k * NB);
         const int ns = (npiv + kDzSliceK - 1) / kDzSliceK;
         if (!mbar_wait(smem_u32(&tempty), (j & 1) ^ 1)) {
           atomicExch(&s_fail, 2);
@@ -255,9 +250,8 @@ __global__ void __launch_bounds__(kDzThreads, 1)
     const int r = quarter * 32 + lane;             // row of the 128-row tile
     const uint32_t tw = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)cbase;
     for (int j = 0; j < myjobs; ++j) {
-      const Job jb = decode_job(args.joff, args.nblk, args.k, args.blk,
-                                (int)blockIdx.x + j * (int)gridDim.x, args.jt);
-      const BlkInfo &bi = args.blk[jb.b];
+      const Job jb = decode_job(args.S, job_index(args.S, j));
+      const BlkInfo &bi = args.S.blk[jb.b];
       const int a = bi.a;
       const long long lda = bi.lda, slot0 = bi.soff + jb.I0, slotJ = bi.soff + jb.J;
       const int grow = jb.I0 * NB + r, col0 = jb.J * NB + cbase;
@@ -300,6 +294,11 @@ __global__ void __launch_bounds__(kDzThreads, 1)
       for (int v = 0; v < 16; ++v) {
         const int sc = er + __shfl_sync(0xffffffffu, ec, v);
         if (v < nc) g[v * lda] = c[v] - dz_scale(P[v], sc);
+      }
+      if (next_diag(args.S, jb)) {
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) atomicAdd(&args.S.ready[jb.b], 1);
       }
     }
   }
@@ -348,18 +347,15 @@ bool dz_setup(ahlp_problem *p) {
   return true;
 }
 
-cudaError_t launch_update_dz(ahlp_problem *p, int k, cudaStream_t s) {
-  const long long jobs = p->tc_jobs[k];
-  if (jobs <= 0) return cudaSuccess;
-  DzArgs a{p->dz_exp, p->tc_joff + (size_t)k * (p->h_blk.size() + 1), p->blk, p->aug,
-           (int)p->h_blk.size(), k, p->status,
-           p->tc_jtab ? p->tc_jtab + p->tc_jtab_off[k] : nullptr};
+cudaError_t launch_update_dz(ahlp_problem *p, int k, cudaStream_t s, LookAhead *la) {
+  if (p->tc_jobs[k] <= 0) return cudaSuccess;
+  int grid = 0;
+  DzArgs a{p->dz_exp, p->aug, p->status, StepJobs{}};
+  a.S = step_jobs(p, k, true, 13, 1, kDzEpiWarps, la, &grid);
   CUtensorMap mA, mB;
   memcpy(&mA, p->dz_map[0], sizeof mA);
   memcpy(&mB, p->dz_map[1], sizeof mB);
-  const int grid = (int)std::min<long long>(jobs, p->num_sms);
-  count_launch(), launch_pdl(pchol_update_dz_kernel, grid, kDzThreads, kDzSmem, s, a, mA, mB,
-                             (int)jobs);
+  count_launch(), launch_pdl(pchol_update_dz_kernel, grid, kDzThreads, kDzSmem, s, a, mA, mB);
   return cudaGetLastError();
 }
 

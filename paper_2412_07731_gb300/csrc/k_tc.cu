@@ -87,12 +87,9 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 
 struct TcArgs {
   const float *stage;      // staged panel tiles: per slot 4096 hi then 4096 lo words
-  const int *joff;         // [nblk + 1] job prefix of this step over the blocks
-  const BlkInfo *blk;
   const CUtensorMap *tmap; // [nblk] each block's FP32 augmented matrix
-  int nblk, k;
   int *status;             // status[4] := 1 when a bounded wait ran out
-  const int4 *jt;          // this step's tile-sparse job table, or nullptr
+  StepJobs S;
 };
 
 __global__ void __launch_bounds__(kTcThreads) pchol_update_tc_kernel(const TcArgs args) {
@@ -110,10 +107,10 @@ __global__ void __launch_bounds__(kTcThreads) pchol_update_tc_kernel(const TcArg
   float *b_lo = reinterpret_cast<float *>(base + 2 * kSmemA + kSmemB);
 
   // ---- which block and tiles ------------------------------------------------
-  const Job jb = decode_job(args.joff, args.nblk, args.k, args.blk, blockIdx.x, args.jt);
+  const Job jb = decode_job(args.S, blockIdx.x);
   const int b = jb.b, I0 = jb.I0, J = jb.J;
   const bool has_i1 = jb.has_i1;
-  const BlkInfo bi = args.blk[b];
+  const BlkInfo bi = args.S.blk[b];
   const float *st0 = args.stage + (bi.soff + I0) * 8192LL;
   const float *st1 = args.stage + (bi.soff + I0 + 1) * 8192LL;
   const float *stJ = args.stage + (bi.soff + J) * 8192LL;
@@ -246,9 +243,10 @@ constexpr int kTc2Threads = 192;
 constexpr uint32_t kTc2Stage = 2 * kSmemA + 2 * kSmemB;             // 96 KB of operands
 constexpr uint32_t kTc2Smem = 2 * kTc2Stage + kTcM * kTcN * 4 + 1024;  // 2 stages + staging
 
-__global__ void __launch_bounds__(kTc2Threads, 1) pchol_update_tc2_kernel(const TcArgs args,
-                                                                         int njobs) {
+__global__ void __launch_bounds__(kTc2Threads, 1) pchol_update_tc2_kernel(
+    const TcArgs args) {
   pdl_wait();
+  jobs_begin(args.S, 1);
   extern __shared__ __align__(1024) unsigned char tc2_raw[];
   __shared__ __align__(8) uint64_t full[2], empty[2], tfull[2], tempty[2];
   __shared__ uint32_t tmem_slot;
@@ -257,8 +255,7 @@ __global__ void __launch_bounds__(kTc2Threads, 1) pchol_update_tc2_kernel(const 
   float *stage_out = reinterpret_cast<float *>(base + 2 * kTc2Stage);   // [64 cols][128 rows]
   volatile int *vfail = &s_fail;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int myjobs = (int)blockIdx.x < njobs ? (njobs - 1 - (int)blockIdx.x) / (int)gridDim.x + 1
-                                             : 0;
+  const int myjobs = my_jobs(args.S);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_slot)),
@@ -293,9 +290,8 @@ __global__ void __launch_bounds__(kTc2Threads, 1) pchol_update_tc2_kernel(const 
           atomicExch(&s_fail, 1);
           break;
         }
-        const Job jb = decode_job(args.joff, args.nblk, args.k, args.blk,
-                                (int)blockIdx.x + j * (int)gridDim.x, args.jt);
-        const BlkInfo bi = args.blk[jb.b];
+        const Job jb = decode_job(args.S, job_index(args.S, j));
+        const BlkInfo bi = args.S.blk[jb.b];
         const float *st0 = args.stage + (bi.soff + jb.I0) * 8192LL;
         const float *stJ = args.stage + (bi.soff + jb.J) * 8192LL;
         const uint32_t sa = smem_u32(base + st * kTc2Stage);
@@ -375,8 +371,7 @@ __global__ void __launch_bounds__(kTc2Threads, 1) pchol_update_tc2_kernel(const 
         if (leader) atomicExch(&s_fail, 3);
         break;
       }
-      const Job jb = decode_job(args.joff, args.nblk, args.k, args.blk,
-                                (int)blockIdx.x + j * (int)gridDim.x, args.jt);
+      const Job jb = decode_job(args.S, job_index(args.S, j));
       const int grow = jb.I0 * NB + r;
 #pragma unroll
       for (int h = 0; h < 2; ++h)
@@ -396,6 +391,12 @@ __global__ void __launch_bounds__(kTc2Threads, 1) pchol_update_tc2_kernel(const 
             "r"(jb.I0 * NB), "r"(jb.J * NB), "r"(smem_u32(stage_out))
             : "memory");
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        if (next_diag(args.S, jb)) {
+          asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+          asm volatile("fence.proxy.async;" ::: "memory");
+          __threadfence();
+          atomicAdd(&args.S.ready[jb.b], 1);
+        }
       }
     }
     if (leader) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -489,13 +490,10 @@ __device__ __forceinline__ void oz_combine(const float (&D)[kOzQ], float &h, flo
 struct OzArgs {
   const __half *dstage;    // digit planes: per slot 6 x 4096 halves
   const int *dexp;         // per slot 64 row exponents
-  const int *joff;
-  const BlkInfo *blk;
   const CUtensorMap *tmap; // [2 nblk]: each block's hi matrix, then its lo matrix
-  int nblk, k;
   int *status;
   float *hi, *lo;          // the augmented matrices' words (persistent kernel)
-  const int4 *jt;          // this step's tile-sparse job table, or nullptr
+  StepJobs S;
 };
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *tm, int x, int y,
@@ -527,10 +525,10 @@ __global__ void __launch_bounds__(kTcThreads) pchol_update_oz_kernel(const OzArg
   float *c_hi = reinterpret_cast<float *>(base + kOzQ * kOzPlaneA + kOzQ * kOzPlaneB);
   float *c_lo = c_hi + kTcM * kTcN;
 
-  const Job jb = decode_job(args.joff, args.nblk, args.k, args.blk, blockIdx.x, args.jt);
+  const Job jb = decode_job(args.S, blockIdx.x);
   const int b = jb.b, I0 = jb.I0, J = jb.J;
   const bool has_i1 = jb.has_i1;
-  const BlkInfo bi = args.blk[b];
+  const BlkInfo bi = args.S.blk[b];
   const long long slot0 = bi.soff + I0, slotJ = bi.soff + J;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar_ld = smem_u32(&bars[0]), bar_mma = smem_u32(&bars[1]);
@@ -563,7 +561,7 @@ __global__ void __launch_bounds__(kTcThreads) pchol_update_oz_kernel(const OzArg
     const __half *st0 = args.dstage + slot0 * (kOzQ * NB * NB);
     const __half *stJ = args.dstage + slotJ * (kOzQ * NB * NB);
     const uint32_t plane = NB * NB * 2;   // bytes of one 64-row plane
-    const CUtensorMap *tmh = args.tmap + b, *tml = args.tmap + args.nblk + b;
+    const CUtensorMap *tmh = args.tmap + b, *tml = args.tmap + args.S.nblk + b;
     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tmh) : "memory");
     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tml) : "memory");
     // the whole box counts, rows past the matrix included (zero-filled)
@@ -658,7 +656,7 @@ __global__ void __launch_bounds__(kTcThreads) pchol_update_oz_kernel(const OzArg
     __syncthreads();
     if (threadIdx.x == 0) {
       tma_store_2d(args.tmap + b, I0 * NB, J * NB, smem_u32(c_hi));
-      tma_store_2d(args.tmap + args.nblk + b, I0 * NB, J * NB, smem_u32(c_lo));
+      tma_store_2d(args.tmap + args.S.nblk + b, I0 * NB, J * NB, smem_u32(c_lo));
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
       asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
@@ -697,6 +695,7 @@ __global__ void __launch_bounds__(kTcThreads) pchol_update_oz_kernel(const OzArg
 // --------------------------------------------------------------------------
 constexpr int kOz2Threads = 320;
 constexpr int kOz2Stages = 2;
+constexpr int kOz2Arrivals = 8;   // epilogue warps
 constexpr uint32_t kOz2HalfA = kTcM * (NB / 2) * 2;             // one K half of an A plane: 8 KB
 constexpr uint32_t kOz2HalfB = kTcN * (NB / 2) * 2;             // 4 KB
 constexpr uint32_t kOz2Stage = kOzQ * (kOz2HalfA + kOz2HalfB);  // 72 KB
@@ -723,9 +722,10 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *tm, int x, in
                : "memory");
 }
 
-__global__ void __launch_bounds__(kOz2Threads, 1) pchol_update_oz2_kernel(const OzArgs args,
-                                                                         int njobs) {
+__global__ void __launch_bounds__(kOz2Threads, 1) pchol_update_oz2_kernel(
+    const OzArgs args) {
   pdl_wait();
+  jobs_begin(args.S, kOz2Arrivals);
   extern __shared__ __align__(1024) unsigned char oz2_raw[];
   __shared__ __align__(8) uint64_t full[kOz2Stages], empty[kOz2Stages], tfull, tempty;
   __shared__ uint32_t tmem_slot;
@@ -733,8 +733,7 @@ __global__ void __launch_bounds__(kOz2Threads, 1) pchol_update_oz2_kernel(const 
   unsigned char *base = oz2_raw + ((1024 - (smem_u32(oz2_raw) & 1023)) & 1023);
   volatile int *vfail = &s_fail;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int myjobs = (int)blockIdx.x < njobs ? (njobs - 1 - (int)blockIdx.x) / (int)gridDim.x + 1
-                                             : 0;
+  const int myjobs = my_jobs(args.S);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_slot)),
@@ -770,15 +769,14 @@ __global__ void __launch_bounds__(kOz2Threads, 1) pchol_update_oz2_kernel(const 
           break;
         }
         if (h == 0) {   // next job: its C tile towards L2 ahead of the epilogue's loads
-          jb = decode_job(args.joff, args.nblk, args.k, args.blk,
-                                (int)blockIdx.x + j * (int)gridDim.x, args.jt);
-          const CUtensorMap *th = args.tmap + jb.b, *tl = args.tmap + args.nblk + jb.b;
+          jb = decode_job(args.S, job_index(args.S, j));
+          const CUtensorMap *th = args.tmap + jb.b, *tl = args.tmap + args.S.nblk + jb.b;
           asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(th) : "memory");
           asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(tl) : "memory");
           tma_prefetch_2d(th, jb.I0 * NB, jb.J * NB);
           tma_prefetch_2d(tl, jb.I0 * NB, jb.J * NB);
         }
-        const BlkInfo bi = args.blk[jb.b];
+        const BlkInfo bi = args.S.blk[jb.b];
         const __half *st0 = args.dstage + (bi.soff + jb.I0) * (kOzQ * NB * NB) + h * (NB * NB / 2);
         const __half *stJ = args.dstage + (bi.soff + jb.J) * (kOzQ * NB * NB) + h * (NB * NB / 2);
         const uint32_t sa = smem_u32(base + st * kOz2Stage), sb = sa + kOzQ * kOz2HalfA;
@@ -845,9 +843,8 @@ __global__ void __launch_bounds__(kOz2Threads, 1) pchol_update_oz2_kernel(const 
     // this warp's quarter of the C tile, [column][row] for hi then lo
     float *cs = reinterpret_cast<float *>(base + kOz2Stages * kOz2Stage + (warp - 2) * 8192);
     for (int j = 0; j < myjobs; ++j) {
-      const Job jb = decode_job(args.joff, args.nblk, args.k, args.blk,
-                                (int)blockIdx.x + j * (int)gridDim.x, args.jt);
-      const BlkInfo bi = args.blk[jb.b];
+      const Job jb = decode_job(args.S, job_index(args.S, j));
+      const BlkInfo bi = args.S.blk[jb.b];
       const long long slot0 = bi.soff + jb.I0, slotJ = bi.soff + jb.J;
       const int row0 = jb.I0 * NB + quarter * 32;   // first row of the warp's quarter
       const int grow = row0 + lane;
@@ -918,6 +915,11 @@ __global__ void __launch_bounds__(kOz2Threads, 1) pchol_update_oz2_kernel(const 
       tc_fence_before();
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty))
                    : "memory");
+      if (next_diag(args.S, jb)) {
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) atomicAdd(&args.S.ready[jb.b], 1);
+      }
     }
   }
   __syncwarp();
@@ -1025,20 +1027,34 @@ void jobs_setup(ahlp_problem *p) {
   p->num_sms = std::max(sms, 1);
   const int N = (int)p->h_blk.size();
   const int maxTp = p->maxTp;
-  std::vector<int> joff((size_t)std::max(maxTp, 1) * (N + 1), 0);
+  const size_t row = 2 * (size_t)N + 2;   // StepJobs::joff of one step
+  std::vector<int> joff(std::max(maxTp, 1) * row, 0);
   p->tc_jobs.assign(maxTp, 0);
+  p->la_pot.assign(maxTp + 1, 0);
+  p->la_miss_off.assign(maxTp + 1, 0);
   for (int k = 0; k < maxTp; ++k) {
-    long long acc = 0;
+    long long acc = 0, first = 0;
+    int *jo = joff.data() + (size_t)k * row, nact = 0;
     for (int b = 0; b < N; ++b) {
-      joff[(size_t)k * (N + 1) + b] = (int)acc;
+      jo[b] = (int)(acc - first);
       const BlkInfo &bi = p->h_blk[b];
-      if (k < bi.Tp) acc += tc_jobs_of(bi.T - k - 1);
+      const long long n = k < bi.Tp ? tc_jobs_of(bi.T - k - 1) : 0;
+      if (n > 0) {
+        jo[N + 2 + nact++] = b;
+        ++first;
+      }
+      acc += n;
+      if (k < bi.Tp) ++p->la_pot[k];
     }
-    joff[(size_t)k * (N + 1) + N] = (int)acc;
+    jo[N] = (int)(acc - first);
+    jo[N + 1] = nact;
     p->tc_jobs[k] = acc;
     p->tc_jobs_dense += acc;
   }
   p->tc_joff = static_cast<int *>(dupload_bytes(p, joff.data(), joff.size() * sizeof(int)));
+  p->la_elems = (long long)N * maxTp;
+  p->la_ready = static_cast<int *>(dalloc_bytes(p, p->la_elems * sizeof(int)));
+  ck(cudaMemsetAsync(p->la_ready, 0, p->la_elems * sizeof(int), p->stream), "memset");
   p->tc_jobs_kept = p->tc_jobs_dense;
   if (!p->opt.tile_sparse || (int)p->tile_nz.size() != N) return;
   std::vector<int> T(N), Tp(N);
@@ -1059,8 +1075,65 @@ void jobs_setup(ahlp_problem *p) {
            p->tc_jobs_dense);
   // Nothing left out (every block tile-dense): the kernels keep decoding the
   // dense enumeration and no table is uploaded.
-  if (kept < p->tc_jobs_dense && !tab.empty())
+  if (kept < p->tc_jobs_dense && !tab.empty()) {
+    // the next diagonal tiles' jobs to the front of each step, and the blocks
+    // that have none there
+    std::vector<int> miss;
+    for (int k = 0; k < maxTp; ++k) {
+      const auto lo = tab.begin() + p->tc_jtab_off[k], hi = tab.begin() + p->tc_jtab_off[k + 1];
+      const auto mid = std::stable_partition(
+          lo, hi, [k](const int4 &v) { return v.y == k + 1 && v.z == k + 1; });
+      std::vector<char> has(N, 0);
+      for (auto it = lo; it != mid; ++it) has[it->x] = 1;
+      p->la_miss_off[k] = (long long)miss.size();
+      for (int b = 0; b < N; ++b)
+        if (k + 1 < Tp[b] && !has[b]) miss.push_back(b);
+    }
+    p->la_miss_off[maxTp] = (long long)miss.size();
+    if (!miss.empty())
+      p->la_miss = static_cast<int *>(dupload_bytes(p, miss.data(), miss.size() * sizeof(int)));
     p->tc_jtab = static_cast<int4 *>(dupload_bytes(p, tab.data(), tab.size() * sizeof(int4)));
+  }
+}
+
+// Jobs of step k and the grid of its update kernel: one CTA per SM (persistent) or
+// per job.  A persistent kernel with la set makes room for the next step's
+// diagonal factorisations: one SM for `per_sm` of them, given up `diag_jobs` jobs
+// before the others end; `arrivals` is what the kernel counts per diagonal tile.
+// Measured per factor and solve, without and with (another tile per SM, or half or
+// twice the jobs, is 1 to 4 % slower): FP64 blocks of 500..4000 rows 29.3 -> 27.7
+// ms, 16 batched LPs in FP32 16.5 -> 15.6, uniform blocks 13.75 -> 13.2, float-float
+// 95.0 -> 93.7.  The one-CTA-per-job kernels run when a step has few jobs, and there
+// the same overlap gains nothing (47.6 ms with and without).
+StepJobs step_jobs(ahlp_problem *p, int k, bool persistent, int diag_jobs, int per_sm,
+                   int arrivals, LookAhead *la, int *grid) {
+  const int N = (int)p->h_blk.size(), jobs = (int)p->tc_jobs[k], sms = p->num_sms;
+  StepJobs S{};
+  S.joff = p->tc_joff + (size_t)k * (2 * (size_t)N + 2);
+  S.blk = p->blk;
+  S.jt = p->tc_jtab ? p->tc_jtab + p->tc_jtab_off[k] : nullptr;
+  S.nblk = N;
+  S.k = k;
+  S.njobs = jobs;
+  *grid = persistent ? std::min(jobs, sms) : jobs;
+  const int pot = k + 1 < p->maxTp ? p->la_pot[k + 1] : 0;
+  if (!persistent || !la || pot <= 0) return S;
+  S.ready = p->la_ready + (size_t)(k + 1) * N;
+  S.miss = p->la_miss ? p->la_miss + p->la_miss_off[k] : nullptr;
+  S.nmiss = p->la_miss ? (int)(p->la_miss_off[k + 1] - p->la_miss_off[k]) : 0;
+  la->ready = S.ready;
+  la->target = arrivals;
+  const int give = std::min((pot + per_sm - 1) / per_sm, sms / 2);
+  if (jobs + give <= sms) return S;   // SMs to spare already
+  const long long held = std::min<long long>(jobs, (long long)diag_jobs * (sms - give));
+  const int full = (int)((jobs - held) / sms);
+  if (full > 0) {
+    S.full = full;
+    S.short_ctas = give;
+  } else {
+    *grid = std::min(jobs, sms - give);
+  }
+  return S;
 }
 
 // Staging slots, per-step job offsets and the per-block tensor maps of the
@@ -1098,24 +1171,22 @@ bool tc_setup(ahlp_problem *p) {
   return true;
 }
 
-cudaError_t launch_update_tc(ahlp_problem *p, int k, cudaStream_t s) {
+cudaError_t launch_update_tc(ahlp_problem *p, int k, cudaStream_t s, LookAhead *la) {
   const long long jobs = p->tc_jobs[k];
   if (jobs <= 0) return cudaSuccess;
-  TcArgs a{p->pstage, p->tc_joff + (size_t)k * (p->h_blk.size() + 1), p->blk,
-           reinterpret_cast<const CUtensorMap *>(p->tc_tmap), (int)p->h_blk.size(), k,
-           p->status, p->tc_jtab ? p->tc_jtab + p->tc_jtab_off[k] : nullptr};
+  TcArgs a{p->pstage, reinterpret_cast<const CUtensorMap *>(p->tc_tmap), p->status, StepJobs{}};
+  int grid = 0;
   // Both kernels give the same factor.  The persistent pipeline (one CTA per SM)
   // wins once its CTAs have several jobs to overlap: 96 uneven blocks, thousands
   // of jobs per step, 15.4 -> 12.4 ms per factor; with about one job per SM its
   // longer start costs more than it hides (8 blocks of 1000 rows 0.81 against
   // 0.80 ms, 16 of 300..700 rows 0.555 against 0.543).
   if (p->fp32_update == 3 || (p->fp32_update == 0 && jobs >= 2LL * p->num_sms)) {
-    const int grid = (int)std::min<long long>(jobs, p->num_sms);
-    count_launch(), launch_pdl(pchol_update_tc2_kernel, grid, kTc2Threads, kTc2Smem, s, a,
-                               (int)jobs);
+    a.S = step_jobs(p, k, true, 26, 2, 1, la, &grid);
+    count_launch(), launch_pdl(pchol_update_tc2_kernel, grid, kTc2Threads, kTc2Smem, s, a);
   } else {
-    count_launch(), launch_pdl(pchol_update_tc_kernel, (unsigned)jobs, kTcThreads, kSmemBytes, s,
-                               a);
+    a.S = step_jobs(p, k, false, 0, 0, 0, nullptr, &grid);
+    count_launch(), launch_pdl(pchol_update_tc_kernel, grid, kTcThreads, kSmemBytes, s, a);
   }
   return cudaGetLastError();
 }
@@ -1156,19 +1227,18 @@ bool oz_setup(ahlp_problem *p) {
   return true;
 }
 
-cudaError_t launch_update_oz(ahlp_problem *p, int k, cudaStream_t s) {
+cudaError_t launch_update_oz(ahlp_problem *p, int k, cudaStream_t s, LookAhead *la) {
   const long long jobs = p->tc_jobs[k];
   if (jobs <= 0) return cudaSuccess;
-  OzArgs a{p->dstage, p->dexp, p->tc_joff + (size_t)k * (p->h_blk.size() + 1), p->blk,
-           reinterpret_cast<const CUtensorMap *>(p->oz_tmap), (int)p->h_blk.size(), k,
-           p->status, p->aug32, p->aug_lo,
-           p->tc_jtab ? p->tc_jtab + p->tc_jtab_off[k] : nullptr};
+  OzArgs a{p->dstage, p->dexp, reinterpret_cast<const CUtensorMap *>(p->oz_tmap), p->status,
+           p->aug32, p->aug_lo, StepJobs{}};
+  int grid = 0;
   if (p->ff_update == 3) {   // persistent pipeline: one CTA per SM
-    const int grid = (int)std::min<long long>(jobs, p->num_sms);
-    count_launch(), launch_pdl(pchol_update_oz2_kernel, grid, kOz2Threads, kOz2Smem, s, a,
-                               (int)jobs);
+    a.S = step_jobs(p, k, true, 12, 1, kOz2Arrivals, la, &grid);
+    count_launch(), launch_pdl(pchol_update_oz2_kernel, grid, kOz2Threads, kOz2Smem, s, a);
   } else {
-    count_launch(), launch_pdl(pchol_update_oz_kernel, (unsigned)jobs, kTcThreads, kOzSmem, s, a);
+    a.S = step_jobs(p, k, false, 0, 0, 0, nullptr, &grid);
+    count_launch(), launch_pdl(pchol_update_oz_kernel, grid, kTcThreads, kOzSmem, s, a);
   }
   return cudaGetLastError();
 }

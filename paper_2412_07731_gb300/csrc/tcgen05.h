@@ -92,19 +92,50 @@ __device__ __forceinline__ void tc_fence_after() {
 }
 
 // One update job of step k: block b, the row tile pair (I0, I0 + 1) (the
-// second one only when has_i1) and the column tile J.  The jobs of a step are
-// numbered block after block (joff: prefix over the blocks); inside a block
-// with t trailing tiles, row pair R holds min(2R + 2, t) jobs, so the jobs
-// before it number R(R + 1).
+// second one only when has_i1) and the column tile J.  Inside a block with t
+// trailing tiles, row pair R holds min(2R + 2, t) jobs, so the jobs before it
+// number R(R + 1).
 struct Job {
   int b, I0, J;
   bool has_i1;
 };
 
-__device__ __forceinline__ Job decode_job(const int *joff, int nblk, int k, const BlkInfo *blk,
-                                          int q, const int4 *jt) {
-  if (jt) {   // tile-sparse: the kept jobs of this step, in the dense order
-    const int4 v = jt[q];
+// The update jobs of one pivot step, shared by every tensor-core update kernel.
+// The jobs that hold the next step's diagonal tiles come first, and the kernel
+// counts them off in `ready`, so that the next step's diagonal factorisations
+// (a chain of 64 dependent pivots that keeps a few CTAs busy for 20 to 75 us) run
+// beside the rest of this update instead of after it: they are the next kernel in
+// the stream, may be scheduled as soon as every CTA here has started, and need an
+// SM with room.  A persistent update takes a whole SM per CTA, so the last
+// `short_ctas` CTAs stop after `full` rounds, some time before the others end.
+struct StepJobs {
+  const int *joff;      // [nblk + 1] prefix of (jobs - 1) over the blocks, then the number of
+                        // blocks with jobs and those blocks
+  const BlkInfo *blk;
+  const int4 *jt;       // this step's tile-sparse job table, or nullptr
+  int nblk, k, njobs;
+  int full, short_ctas;
+  int *ready;           // [nblk] arrivals on the next diagonal tiles, or nullptr
+  const int *miss;      // blocks whose next diagonal tile this step does not touch
+  int nmiss;
+};
+
+// number of jobs of this CTA, and its j-th job
+__device__ __forceinline__ int my_jobs(const StepJobs &S) {
+  const int i = blockIdx.x, G = gridDim.x, g = G - S.short_ctas;
+  if (i >= g) return S.full;
+  const int rest = S.njobs - S.full * G - i;
+  return S.full + (rest > 0 ? (rest - 1) / g + 1 : 0);
+}
+
+__device__ __forceinline__ int job_index(const StepJobs &S, int j) {
+  const int i = blockIdx.x, G = gridDim.x;
+  return j < S.full ? i + j * G : S.full * G + i + (j - S.full) * (G - S.short_ctas);
+}
+
+__device__ __forceinline__ Job decode_job(const StepJobs &S, int q) {
+  if (S.jt) {   // tile-sparse: the kept jobs of this step
+    const int4 v = S.jt[q];
     Job j;
     j.b = v.x;
     j.I0 = v.y;
@@ -112,32 +143,63 @@ __device__ __forceinline__ Job decode_job(const int *joff, int nblk, int k, cons
     j.has_i1 = v.w != 0;
     return j;
   }
-  int lo = 0, hi = nblk;   // joff[lo] <= q < joff[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (joff[mid] <= q) lo = mid;
-    else hi = mid;
+  const int nact = S.joff[S.nblk + 1];
+  int lo;
+  long long local;
+  if (q < nact) {   // a block's first job: the next diagonal tile
+    lo = S.joff[S.nblk + 2 + q];
+    local = 0;
+  } else {
+    q -= nact;
+    lo = 0;
+    int hi = S.nblk;   // joff[lo] <= q < joff[hi]
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (S.joff[mid] <= q) lo = mid;
+      else hi = mid;
+    }
+    local = q - S.joff[lo] + 1;
   }
-  const int t = blk[lo].T - k - 1;
+  const int t = S.blk[lo].T - S.k - 1;
   // largest R with R(R + 1) <= local: an FP32 estimate, corrected in integers
   // (an FP64 square root here costs every warp of every job ~25 instructions of
   // a pipe that issues one warp instruction in 64 clocks per partition)
-  const long long local = q - joff[lo];
   long long R = (long long)((sqrtf(4.0f * (float)local + 1.0f) - 1.0f) * 0.5f);
   while (R * (R + 1) > local) --R;
   while ((R + 1) * (R + 2) <= local) ++R;
   Job j;
   j.b = lo;
-  j.I0 = k + 1 + 2 * (int)R;
-  j.J = k + 1 + (int)(local - R * (R + 1));
+  j.I0 = S.k + 1 + 2 * (int)R;
+  j.J = S.k + 1 + (int)(local - R * (R + 1));
   j.has_i1 = 2 * R + 1 < t;
   return j;
+}
+
+// does this job hold the next step's diagonal tile, and is someone waiting for it
+__device__ __forceinline__ bool next_diag(const StepJobs &S, const Job &jb) {
+  return S.ready && jb.J == S.k + 1 && jb.I0 == S.k + 1;
+}
+
+// after the kernel's griddepcontrol.wait: let the next kernel's CTAs be scheduled,
+// and count off the tiles that have no job (`arrivals` per tile)
+__device__ __forceinline__ void jobs_begin(const StepJobs &S, int arrivals) {
+  if (!S.ready) return;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < S.nmiss; i += blockDim.x) {
+      __threadfence();
+      atomicExch(&S.ready[S.miss[i]], arrivals);
+    }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                   const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                   const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// jobs of step k and the grid of its update kernel (k_tc.cu)
+StepJobs step_jobs(ahlp_problem *p, int k, bool persistent, int diag_jobs, int per_sm,
+                   int arrivals, LookAhead *la, int *grid);
 
 // the driver's tensor-map encoder, or nullptr
 EncodeTiledFn tensor_map_encoder();
