@@ -332,14 +332,16 @@ __global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(T *buf, float *lo
 // Plane p of the K slice of columns 16 sl .. 16 sl + 15 is a 64 x 16 K-major
 // operand of 8-row x 16-byte core matrices, 2 KB at ((8 sl + p) * slots +
 // slot): entry (r, c) at (r/8)*128 + ((c%16)/8)*64 + (r%8)*8 + c%8.  Rows past
-// the matrix and columns past the pivots are zero.  Thread (row r = tid / 4,
-// slice tid % 4); x(r, c) returns the entry.  A row holding a NaN or an
-// infinity gets the exponent kDzNotFinite and no digits.
+// the matrix and columns past the pivots are zero.  Rows row0 .. row0 + nrow - 1,
+// thread (row row0 + tid / 4, slice tid % 4); x(r, c) returns the entry.  A row
+// holding a NaN or an infinity gets the exponent kDzNotFinite and no digits.
 template <typename F>
-__device__ __forceinline__ void dz_stage_tile(F x, int nri, int npiv, __half *stage, int *dexp,
-                                              long long slots, long long slot) {
-  const int r = threadIdx.x >> 2, sl = threadIdx.x & 3, c0 = sl * 16;
-  const bool row = r < nri;
+__device__ __forceinline__ void dz_stage_rows(F x, int row0, int nrow, int nri, int npiv,
+                                              __half *stage, int *dexp, long long slots,
+                                              long long slot) {
+  const int r = row0 + (threadIdx.x >> 2), sl = threadIdx.x & 3, c0 = sl * 16;
+  const bool mine = r < row0 + nrow;
+  const bool row = mine && r < nri;
   int mx = 0;   // largest high word (exponent and leading bits); 1 for a tiny nonzero
 #pragma unroll
   for (int j = 0; j < 16; ++j)
@@ -351,7 +353,7 @@ __device__ __forceinline__ void dz_stage_tile(F x, int nri, int npiv, __half *st
   mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
   const bool fin = mx < 0x7ff00000;
   const int E = mx ? (mx >> 20) - 1021 : 0;   // |x| < 2^(E - 1); a zero row takes 0
-  if (sl == 0) dexp[slot * NB + r] = fin ? E : kDzNotFinite;
+  if (mine && sl == 0) dexp[slot * NB + r] = fin ? E : kDzNotFinite;
   __half *st = stage + ((long long)(sl * kDzQ) * slots + slot) * 1024 + (r >> 3) * 128 + (r & 7) * 8;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {   // 8 columns: one 16-byte run per plane
@@ -390,8 +392,9 @@ __device__ __forceinline__ void dz_stage_tile(F x, int nri, int npiv, __half *st
                                   __floats2half2_rn(1152.0f, 1152.0f));
         w[q] = *reinterpret_cast<const uint32_t *>(&f);
       }
-      *reinterpret_cast<uint4 *>(st + (long long)p * slots * 1024 + h * 64) =
-          make_uint4(w[0], w[1], w[2], w[3]);
+      if (mine)
+        *reinterpret_cast<uint4 *>(st + (long long)p * slots * 1024 + h * 64) =
+            make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
 }
@@ -399,57 +402,95 @@ __device__ __forceinline__ void dz_stage_tile(F x, int nri, int npiv, __half *st
 // panel tiles below the diagonal tile: X = A_Ik L_kk^-T on the pivot columns,
 // and the non-pivot (Schur) columns of the tile updated with the new X.  With
 // stage (FP64 factors, tensor-core update) the tile's digits are written too.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) pchol_trsm_kernel(T *buf, const BlkInfo *blk, int k,
-                                                              __half *stage, int *dexp,
-                                                              long long slots) {
+//
+// Bound by the FP64 pipe: 64^3 / 2 multiply-adds per tile, 34 us of one SM.  So the
+// inner loop is nothing but those: a row lives in the registers of G lanes (column
+// 4j + g in register j of lane group g, for G = 4), the owner of column c scales
+// it, a shuffle hands it to the row's other lanes, and each lane subtracts it from
+// its columns right of c, with L_sc broadcast from shared memory; no barrier and no
+// shared-memory store.  Every entry's operations and their order are those of
+// the plain right-looking loop.  Lanes idle at the diagonal cost 8 % (G = 2), 17 %
+// (4) and 35 % (8) more instructions, but a warp's 32 / G rows finish in 37, 20 and
+// 12 us, so G grows as the tiles get fewer than the SMs' partitions (trsm_lanes).
+constexpr int kTrsmThreads = 128;
+constexpr size_t kTrsmSmem = NB * (NB + 1) * sizeof(double);
+template <int G>
+__global__ void __launch_bounds__(kTrsmThreads, G == 2 ? 3 : 4) pchol_trsm_kernel(double *buf, const BlkInfo *blk,
+                                                                  int k, __half *stage, int *dexp,
+                                                                  long long slots) {
   pdl_begin();
+  constexpr int R = 32 / G, kRows = kTrsmThreads / G, kC = NB / G;
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
-  const int I = k + 1 + blockIdx.x;
+  const int I = k + 1 + blockIdx.x / (NB / kRows), row0 = (blockIdx.x % (NB / kRows)) * kRows;
   if (I >= bi.T) return;
-  extern __shared__ __align__(16) unsigned char trsm_raw[];   // two (NB x NB+1) tiles
-  T(*L)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(trsm_raw);
-  T(*X)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(trsm_raw + sizeof(T) * NB * (NB + 1));
-  __shared__ T rinv[NB];
+  extern __shared__ __align__(16) unsigned char trsm_raw[];
+  double *L = reinterpret_cast<double *>(trsm_raw);   // column c at c * NB
+  __shared__ double rinv[NB];
   const int r0 = k * NB;
   const int nr = min(NB, bi.a - r0);
   const int npiv = min(NB, bi.p - r0);
   const int ri = I * NB;
   const int nri = min(NB, bi.a - ri);
-  const T *gl = buf + bi.base + (long long)r0 * bi.lda + r0;
-  T *gx = buf + bi.base + (long long)r0 * bi.lda + ri;
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
+  const double *gl = buf + bi.base + (long long)r0 * bi.lda + r0;
+  double *gx = buf + bi.base + (long long)r0 * bi.lda + ri;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rl = lane % R, g = lane / R, row = row0 + warp * R + rl;
+  double x[kC];   // columns G j + g of the row
+#pragma unroll
+  for (int j = 0; j < kC; ++j) {
+    const int s = G * j + g;
+    x[j] = (row < nri && s < nr) ? gx[(long long)s * bi.lda + row] : 0.0;
+  }
+#pragma unroll 8
+  for (int i = threadIdx.x; i < NB * NB; i += kTrsmThreads) {
     const int r = i % NB, c = i / NB;
-    L[r][c] = (r < nr && c < nr && r >= c) ? gl[(long long)c * bi.lda + r] : T(0);
-    X[r][c] = (r < nri && c < nr) ? gx[(long long)c * bi.lda + r] : T(0);
+    L[i] = (r < nr && c < nr && r >= c) ? gl[(long long)c * bi.lda + r] : 0.0;
   }
   __syncthreads();
-  // one reciprocal per column (a division by every thread at every column took
-  // two thirds of this kernel: FP64 divisions are ~20 instructions of a pipe
-  // with two lanes per clock)
-  if (threadIdx.x < npiv) rinv[threadIdx.x] = T(1) / L[threadIdx.x][threadIdx.x];
+  // one reciprocal per column
+  if (threadIdx.x < npiv) rinv[threadIdx.x] = 1.0 / L[threadIdx.x * (NB + 1)];
   __syncthreads();
-  for (int c = 0; c < npiv; ++c) {
-    const T inv = rinv[c];
-    for (int r = threadIdx.x; r < nri; r += blockDim.x) X[r][c] *= inv;
-    __syncthreads();
-    const int ns = nr - c - 1;
-    for (int idx = threadIdx.x; idx < nri * ns; idx += blockDim.x) {
-      const int r = idx % nri, s = c + 1 + idx / nri;
-      X[r][s] -= X[r][c] * L[s][c];
+#pragma unroll
+  for (int c = 0; c < NB; ++c) {
+    if (c < npiv) {   // uniform
+      const int jc = c / G, gc = c % G;
+      const double v = x[jc] * rinv[c];
+      const double xc = __shfl_sync(0xffffffffu, v, gc * R + rl);
+      const double *Lc = L + c * NB + g;
+      if (gc < G - 1) {
+        const double u = fma(-xc, Lc[G * jc], x[jc]);
+        x[jc] = g > gc ? u : g == gc ? v : x[jc];
+      } else if (g == gc) {
+        x[jc] = v;
+      }
+#pragma unroll
+      for (int j = jc + 1; j < kC; ++j) x[j] = fma(-xc, Lc[G * j], x[j]);
     }
+  }
+#pragma unroll
+  for (int j = 0; j < kC; ++j) {
+    const int s = G * j + g;
+    if (row < nri && s < nr) gx[(long long)s * bi.lda + row] = x[j];
+  }
+  if (stage) {   // through shared memory, over L
     __syncthreads();
+    double(*X)[NB + 1] = reinterpret_cast<double(*)[NB + 1]>(trsm_raw);
+#pragma unroll
+    for (int j = 0; j < kC; ++j) X[warp * R + rl][G * j + g] = x[j];
+    __syncthreads();
+    for (int h = 0; h < kRows; h += 32)
+      dz_stage_rows([&](int r, int c) { return X[r - row0][c]; }, row0 + h, min(32, kRows), nri,
+                    npiv, stage, dexp, slots, bi.soff + I);
   }
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
-    const int r = i % NB, c = i / NB;
-    if (r < nri && c < nr) gx[(long long)c * bi.lda + r] = X[r][c];
-  }
-  if constexpr (sizeof(T) == sizeof(double)) {
-    if (stage)
-      dz_stage_tile([&](int r, int c) { return X[r][c]; }, nri, npiv, stage, dexp, slots,
-                    bi.soff + I);
-  }
+}
+
+// lane groups per row: as many as keep every warp of the step's tiles (2 G per
+// tile) on a partition of its own.  One tile: 70 us with a column's updates spread
+// over a CTA between two barriers.
+constexpr int kSMs = 152;
+inline int trsm_lanes(long long tiles) {
+  return tiles * 16 <= 4 * kSMs ? 8 : tiles * 8 <= 4 * kSMs ? 4 : 2;
 }
 
 // --------------------------------------------------------------------------
@@ -1046,13 +1087,17 @@ __global__ void __launch_bounds__(kFFRowThreads) pchol_trsm_ff_kernel(float *hi,
 // trailing update: C_IJ -= L_Ik L_Jk' over the pivot columns of step k (the
 // FP64 factor; FP32 and float-float have their own kernels below).
 constexpr int KC = 16;
-template <typename T>
+// S x S CTAs per tile: a tile keeps one SM's FP64 pipe busy for 69 us, so a step
+// with fewer tiles than SMs spreads them (79 us at S = 1)
+template <typename T, int S>
 __global__ void __launch_bounds__(kThreads) pchol_update_kernel(T *buf, const BlkInfo *blk, int k) {
+  constexpr int M = NB / S, A = M / 16;
   pdl_begin();
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const long long t = bi.T - k - 1;
-  const long long q = blockIdx.x;
+  const long long q = blockIdx.x / (S * S);
+  const int sub = blockIdx.x % (S * S), sI = sub / S, sJ = sub % S;
   if (q >= t * (t + 1) / 2) return;
   long long ii = (long long)((sqrt(8.0 * (double)q + 1.0) - 1.0) * 0.5);
   while (ii * (ii + 1) / 2 > q) --ii;
@@ -1060,20 +1105,21 @@ __global__ void __launch_bounds__(kThreads) pchol_update_kernel(T *buf, const Bl
   const long long jj = q - ii * (ii + 1) / 2;
   const int I = k + 1 + (int)ii, J = k + 1 + (int)jj;
   const int npiv = min(NB, bi.p - k * NB);
-  const int rI = I * NB, rJ = J * NB;
-  const int nrI = min(NB, bi.a - rI), nrJ = min(NB, bi.a - rJ);
-  __shared__ T As[KC][NB];
-  __shared__ T Bs[KC][NB];
+  if (I == J && sI < sJ) return;
+  const int rI = I * NB + sI * M, rJ = J * NB + sJ * M;
+  const int nrI = min(M, bi.a - rI), nrJ = min(M, bi.a - rJ);   // may be negative
+  __shared__ T As[KC][M];
+  __shared__ T Bs[KC][M];
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  T acc[4][4];
+  T acc[A][A];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < A; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
+    for (int j = 0; j < A; ++j) acc[i][j] = T(0);
   const T *colk = buf + bi.base + (long long)(k * NB) * bi.lda;
   for (int kc = 0; kc < npiv; kc += KC) {
-    for (int idx = threadIdx.x; idx < KC * NB; idx += blockDim.x) {
-      const int r = idx % NB, kk = idx / NB;
+    for (int idx = threadIdx.x; idx < KC * M; idx += blockDim.x) {
+      const int r = idx % M, kk = idx / M;
       const bool kin = (kc + kk) < npiv;
       const T *col = colk + (long long)(kc + kk) * bi.lda;
       As[kk][r] = (kin && r < nrI) ? col[rI + r] : T(0);
@@ -1082,26 +1128,26 @@ __global__ void __launch_bounds__(kThreads) pchol_update_kernel(T *buf, const Bl
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < KC; ++kk) {
-      T av[4], bv[4];
+      T av[A], bv[A];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[kk][tx + 16 * i];
+      for (int i = 0; i < A; ++i) av[i] = As[kk][tx + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][ty + 16 * j];
+      for (int j = 0; j < A; ++j) bv[j] = Bs[kk][ty + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < A; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+        for (int j = 0; j < A; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
     }
     __syncthreads();
   }
   T *gc = buf + bi.base + (long long)rJ * bi.lda + rI;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < A; ++j) {
     const int c = ty + 16 * j;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < A; ++i) {
       const int r = tx + 16 * i;
-      if (r < nrI && c < nrJ && (I != J || r >= c)) gc[(long long)c * bi.lda + r] -= acc[i][j];
+      if (r < nrI && c < nrJ && (I != J || sI != sJ || r >= c)) gc[(long long)c * bi.lda + r] -= acc[i][j];
     }
   }
 }
@@ -1752,6 +1798,17 @@ constexpr size_t trsm_smem() {
   return 2 * NB * (NB + 1) * sizeof(T);
 }
 
+void launch_trsm64(int lanes, double *buf, const BlkInfo *info, unsigned panels, int nblk, int k,
+                   ahlp_problem *dz, cudaStream_t s) {
+  auto *const kern = lanes == 8   ? pchol_trsm_kernel<8>
+                     : lanes == 4 ? pchol_trsm_kernel<4>
+                                  : pchol_trsm_kernel<2>;
+  const unsigned ctas = panels * (NB / (kTrsmThreads / lanes));
+  count_launch(), launch_pdl(kern, dim3(ctas, nblk), kTrsmThreads, kTrsmSmem, s, buf, info, k,
+                             dz ? dz->dz_stage : nullptr, dz ? dz->dz_exp : nullptr,
+                             dz ? dz->stage_slots : 0);
+}
+
 template <typename T>
 cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkInfo> &h,
                     const double *diag0, double tol, int *status, cudaStream_t s,
@@ -1764,10 +1821,12 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
   LookAhead la;   // this step's diagonal tiles, beside the update before
   for (int k = 0; k < maxTp; ++k) {
     LookAhead next;
-    long long maxPanel = 0, maxTrail = 0;
+    long long maxPanel = 0, maxTrail = 0, panels = 0, trails = 0;
     for (auto &b : h) {
       if (k >= b.Tp) continue;
       long long t = b.T - k - 1;
+      panels += t;
+      trails += t * (t + 1) / 2;
       if (t > maxPanel) maxPanel = t;
       if (t * (t + 1) / 2 > maxTrail) maxTrail = t * (t + 1) / 2;
     }
@@ -1787,9 +1846,7 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
                                  nullptr, info, k, diag0, tol, status, drop, la);
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
-        count_launch(), launch_pdl(pchol_trsm_kernel<T>, dim3((unsigned)maxPanel, nblk), kThreads,
-                                   trsm_smem<T>(), s, buf, info, k, dz ? dz->dz_stage : nullptr,
-                            dz ? dz->dz_exp : nullptr, dz ? dz->stage_slots : 0);
+        launch_trsm64(trsm_lanes(panels), buf, info, (unsigned)maxPanel, nblk, k, dz, s);
     }
     if (prof) kt_mark(prof, 2, s);
     if (maxTrail > 0) {
@@ -1805,8 +1862,12 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
         cudaError_t e = launch_update_dz(dz, k, s, &next);
         if (e != cudaSuccess) return e;
       } else {
-        count_launch(), launch_pdl(pchol_update_kernel<T>, dim3((unsigned)maxTrail, nblk),
-                                   kThreads, 0, s, buf, info, k);
+        auto *const kern = trails <= kSMs / 8 ? pchol_update_kernel<T, 4>
+                           : trails <= kSMs   ? pchol_update_kernel<T, 2>
+                                              : pchol_update_kernel<T, 1>;
+        const unsigned sub = trails <= kSMs / 8 ? 16 : trails <= kSMs ? 4 : 1;
+        count_launch(), launch_pdl(kern, dim3((unsigned)maxTrail * sub, nblk), kThreads, 0, s, buf,
+                                   info, k);
       }
     }
     if (prof) kt_mark(prof, 3, s);
@@ -1982,10 +2043,6 @@ cudaError_t set_dense_smem_limits() {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(pchol_trsm_ff_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)kTrsmFFSmem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(pchol_trsm_kernel<double>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)trsm_smem<double>());
   if (e != cudaSuccess) return e;
   return e;
 }
