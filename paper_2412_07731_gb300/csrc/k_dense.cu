@@ -750,81 +750,114 @@ __device__ __forceinline__ float tf32_round(float x) {
 // (entry (r, c) at (r/8)*512 + (c/4)*32 + (r%8)*4 + c%4; hi in words
 // 0..4095, lo in 4096..8191).  Rows past the matrix and columns past the
 // pivots are zero.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) pchol_trsm_inv_kernel(T *buf, const T *tinv,
-                                                                  const BlkInfo *blk, int k,
-                                                                  float *pstage) {
+//
+// Bound by its traffic (a tile read, written and staged twice: 64 KB) once the
+// product does not wait for shared memory: both operands are copied as they
+// lie in memory, 16 bytes at a time and all requested before the first is used, and
+// a thread's 4 x 4 entries of the product take one 16-byte read of each per pivot
+// column (eight 4-byte reads each way when a thread's rows lay 16 apart).
+__global__ void __launch_bounds__(kThreads, 4)
+    pchol_trsm_inv_kernel(float *buf, const float *tinv, const BlkInfo *blk, int k,
+                          float *pstage) {
   pdl_begin();
   const BlkInfo bi = blk[blockIdx.y];
   if (k >= bi.Tp) return;
   const int I = k + 1 + blockIdx.x;
   if (I >= bi.T) return;
-  extern __shared__ __align__(16) unsigned char trsm_raw[];   // two (NB x NB+1) tiles
-  T(*A)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(trsm_raw);
-  T(*V)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(trsm_raw + sizeof(T) * NB * (NB + 1));
+  __shared__ __align__(16) float A[NB][NB];   // A[c][r]: the tile, column c
+  __shared__ __align__(16) float V[NB][NB];   // V[q][c]: inverse (c < npiv) or factor entry (c, q)
   const int r0 = k * NB;
   const int nr = min(NB, bi.a - r0);
   const int npiv = min(NB, bi.p - r0);
   const int ri = I * NB;
   const int nri = min(NB, bi.a - ri);
-  T *gx = buf + bi.base + (long long)r0 * bi.lda + ri;
-  const T *ti = tinv + bi.ioff + (long long)k * NB * NB;
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
-    const int r = i % NB, c = i / NB;
-    A[r][c] = (r < nri && c < nr) ? gx[(long long)c * bi.lda + r] : T(0);
-    V[r][c] = ti[i];   // V[r][c]: inverse (r < npiv) or factor (r >= npiv) entry (r, c)
+  float *gx = buf + bi.base + (long long)r0 * bi.lda + ri;   // base, lda: multiples of 8
+  const float *ti = tinv + bi.ioff + (long long)k * NB * NB;
+  {
+    constexpr int kU = NB * NB / 4 / kThreads;
+    float4 a[kU], v[kU];
+    const int r = (threadIdx.x & 15) * 4;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int c = (threadIdx.x >> 4) + u * (kThreads / 16);
+      a[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      // a tile's last rows read into the column's padding (lda >= a, rounded up)
+      if (c < nr && r < nri)
+        a[u] = *reinterpret_cast<const float4 *>(gx + (long long)c * bi.lda + r);
+      v[u] = *reinterpret_cast<const float4 *>(ti + c * NB + r);
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int c = (threadIdx.x >> 4) + u * (kThreads / 16);
+      if (r + 1 >= nri) a[u].y = 0.0f;
+      if (r + 2 >= nri) a[u].z = 0.0f;
+      if (r + 3 >= nri) a[u].w = 0.0f;
+      *reinterpret_cast<float4 *>(&A[c][r]) = a[u];
+      *reinterpret_cast<float4 *>(&V[c][r]) = v[u];
+    }
   }
   __syncthreads();
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  T acc[4][4];
+  const int tr = (threadIdx.x & 15) * 4, tc = (threadIdx.x >> 4) * 4;   // 4 x 4 entries
+  float acc[4][4];   // [column][row]
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int b = 0; b < 4; ++b)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+    for (int a = 0; a < 4; ++a) acc[b][a] = 0.0f;
+#pragma unroll 8
   for (int q = 0; q < npiv; ++q) {
-    T av[4], bv[4];
+    const float4 av = *reinterpret_cast<const float4 *>(&A[q][tr]);
+    const float4 bv = *reinterpret_cast<const float4 *>(&V[q][tc]);   // zero for q > column
+    const float x[4] = {av.x, av.y, av.z, av.w}, y[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
-    for (int a = 0; a < 4; ++a) av[a] = A[tx + 16 * a][q];
+    for (int b = 0; b < 4; ++b)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) bv[b] = V[ty + 16 * b][q];   // (L^-1)(c, q), zero for q > c
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+      for (int a = 0; a < 4; ++a) acc[b][a] = fmaf(x[a], y[b], acc[b][a]);
   }
-  __syncthreads();
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = ty + 16 * b;
-      if (c < npiv) A[tx + 16 * a][c] = acc[a][b];
-    }
-  __syncthreads();
-  if (npiv < nr) {
-    const int ns = nr - npiv;
-    for (int idx = threadIdx.x; idx < nri * ns; idx += blockDim.x) {
-      const int r = idx % nri, sc = npiv + idx / nri;
-      T u = A[r][sc];
-      for (int c = 0; c < npiv; ++c) u = fma(-A[r][c], V[sc][c], u);
-      A[r][sc] = u;
-    }
+  if (npiv < nr) {   // the last pivot tile's other columns
     __syncthreads();
-  }
-  for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
-    const int r = i % NB, c = i / NB;
-    if (r < nri && c < nr) gx[(long long)c * bi.lda + r] = A[r][c];
-  }
-  if constexpr (sizeof(T) == sizeof(float)) {
-    if (pstage) {
-      float *st = pstage + (bi.soff + I) * 8192LL;
-      for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        const int r = (e >> 9) * 8 + ((e >> 2) & 7), c = ((e >> 5) & 15) * 4 + (e & 3);
-        const float v = (r < nri && c < npiv) ? (float)A[r][c] : 0.0f;
-        const float h = tf32_round(v);
-        st[e] = h;
-        st[NB * NB + e] = tf32_round(v - h);
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      if (tc + b < npiv) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) A[tc + b][tr + a] = acc[b][a];
       }
+    __syncthreads();
+    const int ns = nr - npiv;
+    for (int idx = threadIdx.x; idx < NB * ns; idx += kThreads) {
+      const int r = idx % NB, sc = npiv + idx / NB;
+      if (r >= nri) continue;
+      float u = A[sc][r];
+      for (int c = 0; c < npiv; ++c) u = fmaf(-A[c][r], V[c][sc], u);
+      gx[(long long)sc * bi.lda + r] = u;
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    if (tc + b >= npiv) continue;
+    float *g = gx + (long long)(tc + b) * bi.lda + tr;
+    if (tr + 3 < nri) {
+      *reinterpret_cast<float4 *>(g) = make_float4(acc[b][0], acc[b][1], acc[b][2], acc[b][3]);
+    } else {
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+        if (tr + a < nri) g[a] = acc[b][a];
+    }
+  }
+  if (pstage) {
+    float *st = pstage + (bi.soff + I) * 8192LL + tc * 8;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const int r = tr + a;
+      float h[4], l[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const float v = (r < nri && tc + b < npiv) ? acc[b][a] : 0.0f;
+        h[b] = tf32_round(v);
+        l[b] = tf32_round(v - h[b]);
+      }
+      float *o = st + (r >> 3) * 512 + (r & 7) * 4;
+      *reinterpret_cast<float4 *>(o) = make_float4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<float4 *>(o + NB * NB) = make_float4(l[0], l[1], l[2], l[3]);
     }
   }
 }
@@ -1793,11 +1826,6 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
   }
 }
 
-template <typename T>
-constexpr size_t trsm_smem() {
-  return 2 * NB * (NB + 1) * sizeof(T);
-}
-
 void launch_trsm64(int lanes, double *buf, const BlkInfo *info, unsigned panels, int nblk, int k,
                    ahlp_problem *dz, cudaStream_t s) {
   auto *const kern = lanes == 8   ? pchol_trsm_kernel<8>
@@ -1836,8 +1864,8 @@ cudaError_t pchol_t(T *buf, T *tinv, const BlkInfo *info, const std::vector<BlkI
                                  info, k, diag0, (float)tol, status, (float)drop, la);
       if (prof) kt_mark(prof, 1, s);
       if (maxPanel > 0)
-        count_launch(), launch_pdl(pchol_trsm_inv_kernel<T>, dim3((unsigned)maxPanel, nblk),
-                                   kThreads, trsm_smem<T>(), s, buf, tinv, info, k,
+        count_launch(), launch_pdl(pchol_trsm_inv_kernel, dim3((unsigned)maxPanel, nblk),
+                                   kThreads, 0, s, buf, tinv, info, k,
                                    tc ? tc->pstage : nullptr);
     } else {
       if (prof) kt_mark(prof, 0, s);
