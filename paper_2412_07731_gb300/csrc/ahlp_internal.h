@@ -292,6 +292,10 @@ struct ahlp_problem {
   __half *dz_stage = nullptr;
   int *dz_exp = nullptr;
   unsigned char dz_map[2][128] = {};
+  bool fac_dz = false;      // the last FP64 factor's updates ran on the tensor cores
+  // FP64 factors keep to the FP64 pipe: set when a digit factor broke down (a NaN
+  // pivot or a stalled direction), for the rest of a solve
+  bool fp64_pipe = false;
   void *tc_tmap = nullptr;           // [N] CUtensorMap
   bool tc_ready = false;
   // float-float factors on the tensor cores: each panel tile as six FP16

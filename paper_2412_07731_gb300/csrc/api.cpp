@@ -1519,10 +1519,12 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
                        p->fac_pivot_tol, p->status, s, oz, prof, drop ? kDropFF : 0.0),
        "pchol");
   }
-  else
+  else {
+    p->fac_dz = p->maxT > 1 && !p->fp64_pipe && dz_setup(p);
     ck(launch_pchol(p->aug, p->blk, p->h_blk, p->diag0, p->fac_pivot_tol, p->status, s, prof,
-                    drop ? kDropFP64 : 0.0, p->maxT > 1 && dz_setup(p) ? p : nullptr),
+                    drop ? kDropFP64 : 0.0, p->fac_dz ? p : nullptr),
        "pchol");
+  }
   ck(launch_tinv(p), "diagonal tile inverses");
   ck(cudaEventRecord(p->ev[2], s), "event");
   ck(launch_schur_assemble(p, delta, rho), "schur assemble");
@@ -1557,6 +1559,12 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
         printf("%s with %s block factors; refactoring in %s\n", buf,
                p->fac_prec == kPrecFP32 ? "FP32" : "float-float", up == kPrecFF ? "float-float" : "FP64");
       p->fac_prec = up;
+      return factor_impl(p, delta, rho, pivot_tol, ff_nan_up);
+    }
+    if (p->fac_prec == kPrecFP64 && p->fac_dz && ff_nan_up) {
+      // the digits keep an entry to 2^-63 of its row's largest; FP64 arithmetic may
+      // still do where a row's entries differ by more
+      p->fp64_pipe = true;
       return factor_impl(p, delta, rho, pivot_tol, ff_nan_up);
     }
     return set_err(p, AHLP_ERR_NOT_SPD, buf);
@@ -1707,6 +1715,7 @@ int kkt_factor(ahlp_problem *p, const double *x, const double *z, double delta, 
       ck(cudaMemcpyAsync(p->z, dz, p->n * 8, cudaMemcpyDeviceToDevice, p->stream), "copy z");
     }
     p->fac_prec = p->opt.precision == AHLP_PREC_MIXED ? kPrecFP32 : kPrecFP64;
+    p->fp64_pipe = false;
     return factor_impl(p, delta < 0 ? p->opt.delta : delta, rho < 0 ? p->opt.rho : rho,
                        p->opt.pivot_tol);
   } catch (const Fail &f) {
