@@ -636,16 +636,18 @@ UPDATE_KERNEL = {("FP32", 1): "pchol_update_f32_kernel (FP32 pipe)",
                  ("FP32", 3): "pchol_update_tc2_kernel (tcgen05, persistent)",
                  ("float-float", 1): "pchol_update_ff8_kernel (double-float, FP32 pipe)",
                  ("float-float", 2): "pchol_update_oz_kernel (tcgen05 digits, one CTA per tile)",
-                 ("float-float", 3): "pchol_update_oz2_kernel (tcgen05 digits, persistent)"}
+                 ("float-float", 3): "pchol_update_oz2_kernel (tcgen05 digits, persistent)",
+                 ("FP64", 2): "pchol_update_dz_kernel (tcgen05 digits, persistent)"}
 
 
 def kernel_roofline(P, prob, lp, x, z, prec_name, peaks):
     """The trailing-update kernel of the block factor in precision prec_name at
     the iterate (x, z) where the timed window ended: CUDA events around its
-    launches (option profile_kernels), median of three factors after one
+    launches (option profile_kernels; the events keep the next step's diagonal
+    tiles from running beside an update), median of three factors after one
     warm-up.  Its algorithmic bytes are the lower-triangle entries it reads
     and writes (4 bytes each way for FP32, 8 for float-float's two words,
-    8 for FP64); for FP64 the bound is the FP64 pipe instead."""
+    8 for FP64)."""
     from paper_2412_07731_gb300 import _lib as L
     saved = L.Options.from_buffer_copy(prob.options)
     o = L.Options.from_buffer_copy(saved)
@@ -668,20 +670,15 @@ def kernel_roofline(P, prob, lp, x, z, prec_name, peaks):
     med = lambda key: statistics.median([t[key] for t in times[1:]])  # noqa: E731
     upd_ms, launches = med("update_ms"), med("update_launches")
     jobs = P.kkt_update_jobs(prob)
-    variant = (saved.fp32_update if prec_name == "FP32" else saved.ff_update) or 2
-    tensor_upd = prec_name != "FP64" and variant in (2, 3)
+    # option 0 picks the persistent kernels on a workload of this size
+    variant = 2 if prec_name == "FP64" else (
+        saved.fp32_update if prec_name == "FP32" else saved.ff_update) or 3
+    tensor_upd = variant in (2, 3)
     elems, flops = update_geometry(lp, jobs=jobs if tensor_upd else None)
     out = {"kernel": f"trailing update of the {prec_name} block factor: "
-                     f"{UPDATE_KERNEL.get((prec_name, variant), 'FP64 pipe')}",
+                     f"{UPDATE_KERNEL[(prec_name, variant)]}",
            "launches": launches,
            "ms_per_factor": upd_ms, "diag_ms": med("diag_ms"), "panel_ms": med("panel_ms")}
-    if prec_name == "FP64":
-        ach = flops / (upd_ms / 1e3) / 1e12
-        out.update({"bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS,
-                    "unit": "TFLOP/s", "frac": ach / FP64_PEAK_TFLOPS, "traffic": None,
-                    "flop_per_launch": flops / launches,
-                    "peak_source": "nominal GB300 FP64 rate"})
-        return out
     word = 4 if prec_name == "FP32" else 8
     bytes_ = 2.0 * word * elems
     gbs = bytes_ / (upd_ms / 1e3) / 1e9
@@ -703,7 +700,7 @@ def kernel_roofline(P, prob, lp, x, z, prec_name, peaks):
                 "tensor": {"flop_per_factor": flops,
                            "achieved_tflops": flops / (upd_ms / 1e3) / 1e12,
                            "note": "FP32: 3 TF32 MMAs per product (hi*hi, hi*lo, lo*hi); "
-                                   "float-float: 21 FP16 digit MMAs per product"}})
+                                   "float-float: 21 and FP64: 36 FP16 digit MMAs per product"}})
     return out
 
 
@@ -719,9 +716,9 @@ def roofline(lp, win, peaks, opts=None, jobs=None):
     the most time in the timed window; achieved = its algorithmic flops per
     factor / its mean CUDA-event time per factor.  When its trailing updates
     run on the tensor cores (TF32 hi/lo splits: 3 MMAs per product; FP16
-    digits: 21), the factor is reported against the tensor peak of that
-    operand type, counting the updates' tensor flops (sustained BF16 peak,
-    the factor being timed inside long steps)."""
+    digits: 21 for float-float, 36 for FP64), the factor is reported against
+    the tensor peak of that operand type, counting the updates' tensor flops
+    (sustained BF16 peak, the factor being timed inside long steps)."""
     a = win.acc
     flops = block_factor_flops(lp)
     kinds = [
@@ -741,11 +738,11 @@ def roofline(lp, win, peaks, opts=None, jobs=None):
     variant = None
     if opts is not None:
         variant = (opts.fp32_update if name == "FP32" else
-                   opts.ff_update if name == "float-float" else None)
+                   opts.ff_update if name == "float-float" else 2)
     if variant in (0, 2, 3):   # tensor-core trailing updates
         _, upd_flops = update_geometry(lp, jobs=jobs)
         per, ratio, op = ((3, TF32_PER_BF16, "TF32") if name == "FP32" else
-                          (21, FP16_PER_BF16, "FP16"))
+                          (21 if name == "float-float" else 36, FP16_PER_BF16, "FP16"))
         tpeak = peaks["bf16_tflops_sustained"] * ratio
         achieved = per * upd_flops / (ms / 1e3) / 1e12
         out = {"bound": "tensor", "achieved": achieved, "peak": tpeak, "unit": "TFLOP/s",
