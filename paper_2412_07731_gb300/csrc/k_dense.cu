@@ -751,11 +751,12 @@ __device__ __forceinline__ float tf32_round(float x) {
 // 0..4095, lo in 4096..8191).  Rows past the matrix and columns past the
 // pivots are zero.
 //
-// Bound by its traffic (a tile read, written and staged twice: 64 KB) once the
-// product does not wait for shared memory: both operands are copied as they
-// lie in memory, 16 bytes at a time and all requested before the first is used, and
-// a thread's 4 x 4 entries of the product take one 16-byte read of each per pivot
-// column (eight 4-byte reads each way when a thread's rows lay 16 apart).
+// Bound by the L1 and shared-memory path (83 % of its rate). So both operands are
+// copied as they lie in memory, 16 bytes at a time and all requested before the
+// first is used, and a thread's 4 x 4 entries of the product take one 16-byte read
+// of each operand per pivot column (eight 4-byte reads when a thread's rows lay 16
+// apart): 28 -> 22 us per step of an energy model's blocks, 11.5 -> 7.8 us on
+// mid-size ones.
 __global__ void __launch_bounds__(kThreads, 4)
     pchol_trsm_inv_kernel(float *buf, const float *tinv, const BlkInfo *blk, int k,
                           float *pstage) {
