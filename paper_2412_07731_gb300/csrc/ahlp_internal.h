@@ -29,6 +29,7 @@ constexpr double kFFPivotTol = 1e-12;     // smallest clamp threshold for float-
 constexpr double kDropFP64 = 1e32, kDropFF = 1e16, kDropFP32 = 1e16;
 constexpr double kDropCapFF = 1e60, kDropCapFP32 = 1e30;
 constexpr long long kSmemVecBytes = 160 * 1024;   // limit of the border order, 8 bytes each
+constexpr int kMaxLinks = 96;     // local link rows of a block pair, at most
 constexpr int kThreads = 256;     // threads per CTA of the dense kernels
 // FP64 factors on the tensor cores (k_dz.cu): digits per entry, and the row
 // exponent that marks a row holding a NaN or an infinity

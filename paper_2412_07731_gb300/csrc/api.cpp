@@ -23,7 +23,7 @@ using namespace ahlp;
 namespace ahlp {
 cudaError_t set_dense_smem_limits();
 cudaError_t set_schur_smem_limits(int bytes);
-cudaError_t set_bcr_smem_limits(int lmax);
+cudaError_t set_bcr_smem_limits();
 }
 
 static std::string g_create_err;
@@ -977,7 +977,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     if ((long long)p->B * 8 > kSmemVecBytes)
       fail(AHLP_ERR_UNSUPPORTED, "the border (linking variables + global rows) exceeds 20480");
     for (int v : l)
-      if (v > 96) fail(AHLP_ERR_UNSUPPORTED, "more than 96 local link rows per block pair");
+      if (v > kMaxLinks) fail(AHLP_ERR_UNSUPPORTED, "more than 96 local link rows per block pair");
     // ---- formation patterns --------------------------------------------------
     // Independent per block: built on host threads into block-local patterns,
     // then concatenated in block order, so the result does not depend on the
@@ -1228,7 +1228,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
           p->bcr_GL = dalloc<double>(p, (long long)(N - 1) * lm * lm);
           p->bcr_GR = dalloc<double>(p, (long long)(N - 1) * lm * lm);
           p->bcr_pub = dalloc<double>(p, 2LL * p->nl);
-          ck(set_bcr_smem_limits(lm), "smem limit");
+          ck(set_bcr_smem_limits(), "smem limit");
         }
       }
       // link-row range of each border column of Z = L_T^-1 E': all links for one

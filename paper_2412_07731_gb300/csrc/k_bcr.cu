@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(kBcrSolveThreads) bcr_fwd_kernel(BArgs A, cons
                                                                    int *err) {
   pdl_begin();
   extern __shared__ double zs[];   // [terms][lmax]
-  __shared__ double r[96], part[2][96];
+  __shared__ double r[kMaxLinks], part[2][kMaxLinks];
   __shared__ int cnt[kBcrMaxTerms];         // term 2w + side: rows, 0: none
   __shared__ long long at[kBcrMaxTerms];    // and where its solution starts
   __shared__ int s_job;
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kBcrSolveThreads) bcr_bwd_kernel(BArgs A, int 
                                                                    int *ticket, int *err) {
   pdl_begin();
   extern __shared__ double zs[];   // [2][lmax]
-  __shared__ double r[96], part[2][96];
+  __shared__ double r[kMaxLinks], part[2][kMaxLinks];
   __shared__ int cnt[2];
   __shared__ long long at[2];
   __shared__ int s_job;
@@ -499,13 +499,15 @@ cudaError_t launch_bcr_solve(ahlp_problem *p, bool forward) {
   return cudaGetLastError();
 }
 
-cudaError_t set_bcr_smem_limits(int lmax) {
-  const int full = kBcrMaxTerms * lmax * (int)sizeof(double);
+// The limits belong to the functions, not to a handle: they cover every accepted
+// size, so that no handle lowers another's.
+cudaError_t set_bcr_smem_limits() {
+  constexpr int row = kMaxLinks * (int)sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(bcr_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       full);
+                                       kBcrMaxTerms * row);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(bcr_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              3 * lmax * lmax * (int)sizeof(double));
+                              3 * kMaxLinks * row);
 }
 
 }  // namespace ahlp
