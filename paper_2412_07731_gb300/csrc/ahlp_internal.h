@@ -610,4 +610,15 @@ struct Fail {
   std::string msg;
 };
 
+// Device memory that a handle takes while a scope is open is given back at its
+// end unless the scope is kept: a set-up whose later allocation fails leaves
+// nothing behind.  Pointers go to the handle once everything has succeeded.
+struct AllocScope {
+  explicit AllocScope(ahlp_problem *q) : p(q), mark(q->allocs.size()) {}
+  ~AllocScope();
+  ahlp_problem *p;
+  size_t mark;
+  bool keep = false;
+};
+
 }  // namespace ahlp

@@ -1332,6 +1332,12 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
 // ===========================================================================
 namespace ahlp {
 
+AllocScope::~AllocScope() {
+  if (keep) return;
+  for (size_t i = mark; i < p->allocs.size(); ++i) cudaFree(p->allocs[i].ptr);
+  p->allocs.resize(mark);
+}
+
 void *dalloc_bytes(ahlp_problem *p, size_t bytes) {
   return dalloc<unsigned char>(p, (long long)std::max<size_t>(bytes, 1));
 }
@@ -1453,14 +1459,21 @@ int factor_impl(ahlp_problem *p, double delta, double rho, double pivot_tol, boo
                      : p->fac_prec == kPrecFF ? std::max(pivot_tol, kFFPivotTol)
                                               : pivot_tol;
   if (p->fac_prec != kPrecFP64 && !p->aug32) {
-    p->aug32 = dalloc<float>(p, p->aug_elems);
-    p->tinv32 = dalloc<float>(p, std::max(p->tinv_elems, 1LL));
+    AllocScope mem(p);
+    float *aug = dalloc<float>(p, p->aug_elems);
+    float *tinv = dalloc<float>(p, std::max(p->tinv_elems, 1LL));
     p->vec32 = dalloc<float>(p, std::max(p->vec_elems, 1LL));
+    p->aug32 = aug;
+    p->tinv32 = tinv;
+    mem.keep = true;
   }
   if (p->fac_prec == kPrecFF && !p->aug_lo) p->aug_lo = dalloc<float>(p, p->aug_elems);
   if (p->fac_prec != kPrecFP32 && !p->aug) {
-    p->aug = dalloc<double>(p, p->aug_elems);
+    AllocScope mem(p);
+    double *aug = dalloc<double>(p, p->aug_elems);
     p->tinv = dalloc<double>(p, std::max(p->tinv_elems, 1LL));
+    p->aug = aug;
+    mem.keep = true;
   }
   cudaStream_t s = p->stream;
   // strictly positive point required (Sec. 2.3: x, z > 0)

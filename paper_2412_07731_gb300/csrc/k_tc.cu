@@ -1028,10 +1028,10 @@ void jobs_setup(ahlp_problem *p) {
   const int N = (int)p->h_blk.size();
   const int maxTp = p->maxTp;
   const size_t row = 2 * (size_t)N + 2;   // StepJobs::joff of one step
-  std::vector<int> joff(std::max(maxTp, 1) * row, 0);
-  p->tc_jobs.assign(maxTp, 0);
-  p->la_pot.assign(maxTp + 1, 0);
-  p->la_miss_off.assign(maxTp + 1, 0);
+  std::vector<int> joff(std::max(maxTp, 1) * row, 0), pot(maxTp + 1, 0), miss;
+  std::vector<long long> jobs(maxTp, 0), jtab_off, miss_off(maxTp + 1, 0);
+  std::vector<int4> tab;
+  long long dense = 0;
   for (int k = 0; k < maxTp; ++k) {
     long long acc = 0, first = 0;
     int *jo = joff.data() + (size_t)k * row, nact = 0;
@@ -1044,56 +1044,68 @@ void jobs_setup(ahlp_problem *p) {
         ++first;
       }
       acc += n;
-      if (k < bi.Tp) ++p->la_pot[k];
+      if (k < bi.Tp) ++pot[k];
     }
     jo[N] = (int)(acc - first);
     jo[N + 1] = nact;
-    p->tc_jobs[k] = acc;
-    p->tc_jobs_dense += acc;
+    jobs[k] = acc;
+    dense += acc;
   }
-  p->tc_joff = static_cast<int *>(dupload_bytes(p, joff.data(), joff.size() * sizeof(int)));
-  p->la_elems = (long long)N * maxTp;
-  p->la_ready = static_cast<int *>(dalloc_bytes(p, p->la_elems * sizeof(int)));
-  ck(cudaMemsetAsync(p->la_ready, 0, p->la_elems * sizeof(int), p->stream), "memset");
-  p->tc_jobs_kept = p->tc_jobs_dense;
-  if (!p->opt.tile_sparse || (int)p->tile_nz.size() != N) return;
-  std::vector<int> T(N), Tp(N);
-  std::vector<const unsigned char *> nz(N);
-  for (int b = 0; b < N; ++b) {
-    T[b] = p->h_blk[b].T;
-    Tp[b] = p->h_blk[b].Tp;
-    // no pattern: every tile counts as nonzero
-    nz[b] = p->tile_nz[b].size() == (size_t)T[b] * T[b] ? p->tile_nz[b].data() : nullptr;
-  }
-  std::vector<int4> tab;
-  const long long kept =
-      tile_sparse_jobs(N, T.data(), Tp.data(), nz.data(), maxTp, tab, p->tc_jtab_off);
-  for (int k = 0; k < maxTp; ++k) p->tc_jobs[k] = p->tc_jtab_off[k + 1] - p->tc_jtab_off[k];
-  p->tc_jobs_kept = kept;
-  if (p->opt.verbose)
-    printf("       tile-sparse trailing updates: %lld of %lld tile jobs kept\n", kept,
-           p->tc_jobs_dense);
-  // Nothing left out (every block tile-dense): the kernels keep decoding the
-  // dense enumeration and no table is uploaded.
-  if (kept < p->tc_jobs_dense && !tab.empty()) {
+  long long kept = dense;
+  if (p->opt.tile_sparse && (int)p->tile_nz.size() == N) {
+    std::vector<int> T(N), Tp(N);
+    std::vector<const unsigned char *> nz(N);
+    for (int b = 0; b < N; ++b) {
+      T[b] = p->h_blk[b].T;
+      Tp[b] = p->h_blk[b].Tp;
+      // no pattern: every tile counts as nonzero
+      nz[b] = p->tile_nz[b].size() == (size_t)T[b] * T[b] ? p->tile_nz[b].data() : nullptr;
+    }
+    kept = tile_sparse_jobs(N, T.data(), Tp.data(), nz.data(), maxTp, tab, jtab_off);
+    for (int k = 0; k < maxTp; ++k) jobs[k] = jtab_off[k + 1] - jtab_off[k];
+    if (p->opt.verbose)
+      printf("       tile-sparse trailing updates: %lld of %lld tile jobs kept\n", kept, dense);
+    // Nothing left out (every block tile-dense): the kernels keep decoding the
+    // dense enumeration and no table is uploaded.
+    if (kept == dense) tab.clear();
     // the next diagonal tiles' jobs to the front of each step, and the blocks
     // that have none there
-    std::vector<int> miss;
-    for (int k = 0; k < maxTp; ++k) {
-      const auto lo = tab.begin() + p->tc_jtab_off[k], hi = tab.begin() + p->tc_jtab_off[k + 1];
+    for (int k = 0; k < maxTp && !tab.empty(); ++k) {
+      const auto lo = tab.begin() + jtab_off[k], hi = tab.begin() + jtab_off[k + 1];
       const auto mid = std::stable_partition(
           lo, hi, [k](const int4 &v) { return v.y == k + 1 && v.z == k + 1; });
       std::vector<char> has(N, 0);
       for (auto it = lo; it != mid; ++it) has[it->x] = 1;
-      p->la_miss_off[k] = (long long)miss.size();
+      miss_off[k] = (long long)miss.size();
       for (int b = 0; b < N; ++b)
         if (k + 1 < Tp[b] && !has[b]) miss.push_back(b);
     }
-    p->la_miss_off[maxTp] = (long long)miss.size();
-    if (!miss.empty())
-      p->la_miss = static_cast<int *>(dupload_bytes(p, miss.data(), miss.size() * sizeof(int)));
-    p->tc_jtab = static_cast<int4 *>(dupload_bytes(p, tab.data(), tab.size() * sizeof(int4)));
+    miss_off[maxTp] = (long long)miss.size();
   }
+  // the device's copies; the handle takes the tables when all of them exist
+  AllocScope mem(p);
+  const long long nready = (long long)N * maxTp;
+  int *d_joff = static_cast<int *>(dupload_bytes(p, joff.data(), joff.size() * sizeof(int)));
+  int *d_ready = static_cast<int *>(dalloc_bytes(p, nready * sizeof(int)));
+  ck(cudaMemsetAsync(d_ready, 0, nready * sizeof(int), p->stream), "memset");
+  int *d_miss = nullptr;
+  int4 *d_jtab = nullptr;
+  if (!miss.empty())
+    d_miss = static_cast<int *>(dupload_bytes(p, miss.data(), miss.size() * sizeof(int)));
+  if (!tab.empty())
+    d_jtab = static_cast<int4 *>(dupload_bytes(p, tab.data(), tab.size() * sizeof(int4)));
+  mem.keep = true;
+  p->tc_jobs.swap(jobs);
+  p->tc_jobs_dense = dense;
+  p->tc_jobs_kept = kept;
+  p->tc_jtab_off.swap(jtab_off);
+  p->la_pot.swap(pot);
+  p->la_miss_off.swap(miss_off);
+  p->la_miss = d_miss;
+  p->la_ready = d_ready;
+  p->la_elems = nready;
+  p->tc_jtab = d_jtab;
+  p->tc_joff = d_joff;
 }
 
 // Jobs of step k and the grid of its update kernel: one CTA per SM (persistent) or
@@ -1158,6 +1170,7 @@ bool tc_setup(ahlp_problem *p) {
     if (r != CUDA_SUCCESS) return false;
   }
   jobs_setup(p);
+  AllocScope mem(p);
   p->tc_tmap = dupload_bytes(p, maps.data(), sizeof(CUtensorMap) * maps.size());
   p->pstage = static_cast<float *>(
       dalloc_bytes(p, (size_t)std::max(p->stage_slots, 1LL) * 8192 * sizeof(float)));
@@ -1167,7 +1180,7 @@ bool tc_setup(ahlp_problem *p) {
   ck(cudaFuncSetAttribute(pchol_update_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)kTc2Smem),
      "tensor-core update shared memory");
-  p->tc_ready = true;
+  mem.keep = p->tc_ready = true;
   return true;
 }
 
@@ -1212,6 +1225,7 @@ bool oz_setup(ahlp_problem *p) {
       if (r != CUDA_SUCCESS) return false;
     }
   jobs_setup(p);
+  AllocScope mem(p);
   p->oz_tmap = dupload_bytes(p, maps.data(), sizeof(CUtensorMap) * maps.size());
   p->dstage = static_cast<__half *>(
       dalloc_bytes(p, (size_t)std::max(p->stage_slots, 1LL) * kOzQ * NB * NB * sizeof(__half)));
@@ -1223,7 +1237,7 @@ bool oz_setup(ahlp_problem *p) {
   ck(cudaFuncSetAttribute(pchol_update_oz2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                           (int)kOz2Smem),
      "float-float tensor-core update shared memory");
-  p->oz_ready = true;
+  mem.keep = p->oz_ready = true;
   return true;
 }
 
