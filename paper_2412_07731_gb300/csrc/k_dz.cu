@@ -321,35 +321,45 @@ __global__ void __launch_bounds__(kDzThreads, 1)
 
 // Digit staging (plane p of K slice sl of every slot: 2 KB at
 // ((sl * kDzQ + p) * slots + slot)), job offsets and the two tensor maps over
-// the staging.  False when the driver has no tensor-map encoder.
+// the staging.  False when the driver has no tensor-map encoder, or when the
+// device has no room for the staging (64 KB per 64 rows): the FP64 pipe's
+// updates need none.  Nothing is kept then, and the next factor tries again.
 bool dz_setup(ahlp_problem *p) {
   if (p->dz_stage) return true;
   const EncodeTiledFn encode = tensor_map_encoder();
   if (!encode) return false;
-  jobs_setup(p);
-  const long long slots = std::max(p->stage_slots, 1LL);
-  constexpr int planes = kDzQ * NB / kDzSliceK;
-  __half *stage = static_cast<__half *>(dalloc_bytes(p, (size_t)slots * planes * kDzPlane));
-  static_assert(sizeof(p->dz_map) == 2 * sizeof(CUtensorMap), "tensor map size");
-  for (int w = 0; w < 2; ++w) {
-    const cuuint64_t dims[3] = {kDzPlane / 8, (cuuint64_t)slots, (cuuint64_t)planes};
-    const cuuint64_t strides[2] = {kDzPlane, (cuuint64_t)slots * kDzPlane};
-    const cuuint32_t box[3] = {kDzPlane / 8, w == 0 ? 2u : 1u, (cuuint32_t)kDzQ};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    CUtensorMap m;
-    if (encode(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, stage, dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return false;
-    memcpy(p->dz_map[w], &m, sizeof m);
+  try {
+    jobs_setup(p);
+    AllocScope mem(p);
+    const long long slots = std::max(p->stage_slots, 1LL);
+    constexpr int planes = kDzQ * NB / kDzSliceK;
+    __half *stage = static_cast<__half *>(dalloc_bytes(p, (size_t)slots * planes * kDzPlane));
+    int *exps = static_cast<int *>(dalloc_bytes(p, (size_t)slots * NB * sizeof(int)));
+    static_assert(sizeof(p->dz_map) == 2 * sizeof(CUtensorMap), "tensor map size");
+    for (int w = 0; w < 2; ++w) {
+      const cuuint64_t dims[3] = {kDzPlane / 8, (cuuint64_t)slots, (cuuint64_t)planes};
+      const cuuint64_t strides[2] = {kDzPlane, (cuuint64_t)slots * kDzPlane};
+      const cuuint32_t box[3] = {kDzPlane / 8, w == 0 ? 2u : 1u, (cuuint32_t)kDzQ};
+      const cuuint32_t estr[3] = {1, 1, 1};
+      CUtensorMap m;
+      if (encode(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, stage, dims, strides, box, estr,
+                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+      memcpy(p->dz_map[w], &m, sizeof m);
+    }
+    ck(cudaFuncSetAttribute(pchol_update_dz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)kDzSmem),
+       "FP64 tensor-core update shared memory");
+    p->dz_exp = exps;
+    p->dz_stage = stage;
+    mem.keep = true;
+    return true;
+  } catch (const Fail &f) {
+    if (f.code != AHLP_ERR_OOM) throw;
+    return false;
   }
-  p->dz_exp = static_cast<int *>(dalloc_bytes(p, (size_t)slots * NB * sizeof(int)));
-  ck(cudaFuncSetAttribute(pchol_update_dz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                          (int)kDzSmem),
-     "FP64 tensor-core update shared memory");
-  p->dz_stage = stage;
-  return true;
 }
 
 cudaError_t launch_update_dz(ahlp_problem *p, int k, cudaStream_t s, LookAhead *la) {
