@@ -303,10 +303,10 @@ __global__ void __launch_bounds__(kThreads) pchol_potrf_kernel(T *buf, float *lo
     }
     __syncthreads();
   }
-  if (threadIdx.x < npiv) {   // sqrt(piv) = piv inv, one correction
+  if (threadIdx.x < npiv) {   // sqrt(piv) = piv inv, one correction; an infinite pivot stays
     const double piv = s_piv[threadIdx.x], inv = s_inv[threadIdx.x];
     const double l = piv * inv;
-    t[threadIdx.x][threadIdx.x] = fma(fma(-l, l, piv), 0.5 * inv, l);
+    t[threadIdx.x][threadIdx.x] = isinf(piv) ? piv : fma(fma(-l, l, piv), 0.5 * inv, l);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < NB * NB; i += blockDim.x) {
