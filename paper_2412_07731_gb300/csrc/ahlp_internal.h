@@ -28,7 +28,8 @@ constexpr double kFFPivotTol = 1e-12;     // smallest clamp threshold for float-
 // storage words
 constexpr double kDropFP64 = 1e32, kDropFF = 1e16, kDropFP32 = 1e16;
 constexpr double kDropCapFF = 1e60, kDropCapFP32 = 1e30;
-constexpr long long kSmemVecBytes = 160 * 1024;   // limit of the border order, 8 bytes each
+constexpr int kMaxBorder = 20480;   // linking variables and global rows, at most
+constexpr int kTickets = 6;         // ticket counters of a solve
 constexpr int kMaxLinks = 96;     // local link rows of a block pair, at most
 constexpr int kThreads = 256;     // threads per CTA of the dense kernels
 // FP64 factors on the tensor cores (k_dz.cu): digits per entry, and the row
@@ -366,12 +367,14 @@ struct ahlp_problem {
   ahlp::BlkInfo *bx_info = nullptr, *bp_info = nullptr;
   ahlp::BlkInfo h_bx{}, h_bp{};
   double *border_diag0 = nullptr;
-  // the border solves: W = L^-1 of the whole border factor (x_0 and y_g parts),
-  // row-major and column-major (ld Bld), from its inverted diagonal tiles
+  // the border solves: the whole border factor (x_0 and y_g parts) as one more block of
+  // the wavefront sweeps, its inverted diagonal tiles, the jobs of the forward and then
+  // the backward sweep, and the two sweeps' published solutions
   ahlp::BlkInfo *bw_info = nullptr;
   int *bw_sched = nullptr;
-  double *border_tinv = nullptr, *border_wr = nullptr, *border_wc = nullptr;
-  double *border_t = nullptr;        // [B] J W b
+  long long *bw_zero = nullptr;      // [1] the block's offset: 0
+  double *border_tinv = nullptr;
+  double *border_pub = nullptr;      // [2 B]
 
   // ---- vectors ------------------------------------------------------------
   double *x = nullptr, *z = nullptr, *dscale = nullptr;   // current point, d = x/z
@@ -396,10 +399,10 @@ struct ahlp_problem {
   unsigned read_seq = 0;      // value the device writes there when a read-back has arrived
   int *status = nullptr;      // device status words [4]
   // wavefront block solves: (block, row tile) jobs in ticket order, and the
-  // ticket counters of the forward and backward block and chain solves (zeroed by
+  // ticket counters of the forward and backward block, chain and border solves (zeroed by
   // the first kernel of a solve, which also fills the publication buffers)
   int *trsv_fsched = nullptr, *trsv_bsched = nullptr;   // [2 * jobs]
-  int *trsv_ticket = nullptr;     // [4]
+  int *trsv_ticket = nullptr;     // [kTickets]
   int *trsv_err = nullptr;        // set when a wait timed out
   int trsv_nf = 0, trsv_nb = 0;
   int tiny_pivots = 0;
@@ -473,6 +476,8 @@ cudaError_t launch_tinv(ahlp_problem *p);
 // p->vec, or the backward one from p->vec and the Schur solution p->svec, which
 // also writes dy; wait timeouts set p->trsv_err
 cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double *dy);
+// the border system on p->svec's border part, in place
+cudaError_t launch_border_solve(ahlp_problem *p);
 cudaError_t launch_schur_assemble(ahlp_problem *p, double delta, double rho);
 cudaError_t launch_schur_factor(ahlp_problem *p);
 // cyclic reduction of the link chain: factor (T_j, Linv_j, GL_j, GR_j, and Z

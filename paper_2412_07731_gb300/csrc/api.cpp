@@ -972,9 +972,9 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     p->aug_elems = base;
     p->tinv_elems = ioff;
     p->vec_elems = voff;
-    // the border solves keep the border vector in shared memory next to a
-    // staged 64x64 tile; the link-chain kernels keep one l x l block there
-    if ((long long)p->B * 8 > kSmemVecBytes)
+    // the border is one dense FP64 matrix: 10 GB with its copy and its factor at the
+    // limit; the link-chain kernels keep three l x l blocks in shared memory
+    if (p->B > kMaxBorder)
       fail(AHLP_ERR_UNSUPPORTED, "the border (linking variables + global rows) exceeds 20480");
     for (int v : l)
       if (v > kMaxLinks) fail(AHLP_ERR_UNSUPPORTED, "more than 96 local link rows per block pair");
@@ -1148,7 +1148,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
       p->trsv_nb = (int)bs.size() / 2;
       if (!fs.empty()) p->trsv_fsched = dupload(p, fs);
       if (!bs.empty()) p->trsv_bsched = dupload(p, bs);
-      p->trsv_ticket = dalloc<int>(p, 4);
+      p->trsv_ticket = dalloc<int>(p, kTickets);
       p->trsv_err = dalloc<int>(p, 1);
       ck(cudaMemset(p->trsv_err, 0, sizeof(int)), "memset");
     }
@@ -1271,11 +1271,11 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
                                   1, BlkInfo{0, 0, 0, p->Bld, p->B, p->B, T, T, 0, 0, 0, 0}));
       std::vector<int> sched;
       for (int k = 0; k < T; ++k) sched.insert(sched.end(), {0, k});
+      for (int k = T - 1; k >= 0; --k) sched.insert(sched.end(), {0, k});
       p->bw_sched = dupload(p, sched);
+      p->bw_zero = dupload(p, std::vector<long long>(1, 0));
       p->border_tinv = dalloc<double>(p, (long long)T * NB * NB);
-      p->border_wr = dalloc<double>(p, (long long)p->Bld * p->B);
-      p->border_wc = dalloc<double>(p, (long long)p->Bld * p->B);
-      p->border_t = dalloc<double>(p, p->B);
+      p->border_pub = dalloc<double>(p, 2LL * p->B);
     }
     p->x = dalloc<double>(p, p->n);
     p->z = dalloc<double>(p, p->n);

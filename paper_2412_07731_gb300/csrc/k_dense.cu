@@ -1706,14 +1706,16 @@ __global__ void __launch_bounds__(TrsvCfg<T, false>::threads, TrsvCfg<T, false>:
 }
 
 // the backward solve's ends: the Schur solution it reads (its non-pivot rows
-// through the block's index map) and dy = [block rows, link rows, global rows]
+// through the block's index map) and dy = [block rows, link rows, global rows];
+// the forward solution of the first `neg` rows counts with its sign changed (the
+// border, whose x_0 part is negative definite)
 struct TrsvBwdIO {
   const double *svec;
   const int *kmap;
   const long long *kmap_off, *yoff;
   double *dy;
   long long msum;
-  int nl, n0, mg;
+  int nl, n0, mg, neg;
 };
 
 // vec holds the forward solution; pub is the publication buffer (its pivot rows)
@@ -1754,7 +1756,8 @@ __global__ void __launch_bounds__(TrsvCfg<T, true>::threads, TrsvCfg<T, true>::m
   const int nch = bi.T - kend;   // chunks, taken k = T - 1, T - 2, ..., kend
   stage_contiguous(Xs, tinv + bi.ioff + (long long)r * NB * NB, NB * NB);
   cp_async_commit();
-  const double fwd_r = threadIdx.x < npiv ? vec[bi.voff + r0 + threadIdx.x] : 0.0;
+  double fwd_r = threadIdx.x < npiv ? vec[bi.voff + r0 + threadIdx.x] : 0.0;
+  if (r0 + (int)threadIdx.x < io.neg) fwd_r = -fwd_r;
   T acc[kJC];
 #pragma unroll
   for (int j = 0; j < kJC; ++j) acc[j] = T(0);
@@ -2011,7 +2014,8 @@ cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double
   cudaStream_t s = p->stream;
   int *ticket = p->trsv_ticket + (forward ? 0 : 1);
   const int *sched = forward ? p->trsv_fsched : p->trsv_bsched;
-  const TrsvBwdIO io{p->svec, p->kmap, p->kmap_off_d, p->yoff_d, dy, p->msum, p->nl, p->n0, p->mg};
+  const TrsvBwdIO io{p->svec, p->kmap, p->kmap_off_d, p->yoff_d, dy, p->msum, p->nl, p->n0, p->mg,
+                     0};
   if (njobs == 0) {
     if (!forward && p->nl + p->mg > 0)
       count_launch(), launch_pdl(schur_dy_kernel, (p->nl + p->mg + 255) / 256, 256, 0, s, io);
@@ -2038,6 +2042,55 @@ cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double
                                  s, p->aug, p->tinv, p->blk, sched, ticket, p->trsv_err, p->vec,
                                  p->vecb, io);
   }
+  return cudaGetLastError();
+}
+
+// The border solve, in place on svec's border part.  With L the factor of the border
+// (x_0 pivots first, then y_g) and J = diag(-I, I), the solution is L^-T J L^-1 b:
+// the wavefront sweeps of the blocks on one more factor, a chain of B / 64 tiles on as
+// many SMs, 8 us at order 100 and 100 us at 601 for both sweeps (substitution over all
+// of L on one SM: 106 and 349 us).  An explicit inverse of L (two matrix-vector products
+// over many SMs, 16 us at 601) is not used: its residual was ten times substitution's
+// and grew with the order, which cost Krylov steps at ill-conditioned borders (order
+// 420, D over 20 decades: 19 steps against 14), and its B^3 / 3 multiply-adds made the
+// factor slower than the sweeps' gain from about order 700 on (4096: 54 against 29 ms).
+//
+// One tile: two products with its inverse X (column-major), t = J X b and x = X' t, one
+// warp per entry over several CTAs: 5 us, where the sweeps' kernels take 8.
+__global__ void __launch_bounds__(256) border_tile_kernel(const double *X, int B, int n0,
+                                                          const double *in, double *out, int fwd) {
+  pdl_begin();
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= B) return;
+  const int q0 = (fwd ? 0 : i) + lane, q1 = fwd ? i + 1 : B;
+  auto x = [&](int q) { return fwd ? X[q * NB + i] : X[i * NB + q]; };
+  const double s0 = q0 < q1 ? x(q0) * in[q0] : 0.0;
+  const double s1 = q0 + 32 < q1 ? x(q0 + 32) * in[q0 + 32] : 0.0;
+  double s = s0 + s1;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[i] = fwd && i < n0 ? -s : s;
+}
+
+cudaError_t launch_border_solve(ahlp_problem *p) {
+  const int T = (p->B + NB - 1) / NB;
+  double *sb = p->svec + p->nl, *y = p->border_pub, *u = y + p->B;
+  if (T == 1) {
+    const unsigned ctas = (unsigned)(p->B + 7) / 8;
+    count_launch(), launch_pdl(border_tile_kernel, ctas, 256, 0, p->stream, p->border_tinv, p->B,
+                               p->n0, sb, y, 1);
+    count_launch(), launch_pdl(border_tile_kernel, ctas, 256, 0, p->stream, p->border_tinv, p->B,
+                               p->n0, y, sb, 0);
+    return cudaGetLastError();
+  }
+  int *ticket = p->trsv_ticket + 4;
+  const TrsvBwdIO io{nullptr, p->kmap, p->bw_zero, p->bw_zero, sb, 0, 0, 0, 0, p->n0};
+  count_launch(), launch_pdl(trsv_fwd_kernel<double>, T, TrsvCfg<double, false>::threads, 0,
+                             p->stream, p->border, p->border_tinv, p->bw_info, p->bw_sched, ticket,
+                             p->trsv_err, y, y, sb, p->bw_zero);
+  count_launch(), launch_pdl(trsv_bwd_kernel<double>, T, TrsvCfg<double, true>::threads, 0,
+                             p->stream, p->border, p->border_tinv, p->bw_info,
+                             p->bw_sched + 2 * T, ticket + 1, p->trsv_err, y, u, io);
   return cudaGetLastError();
 }
 

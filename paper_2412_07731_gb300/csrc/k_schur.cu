@@ -655,12 +655,12 @@ __global__ void negate_corner_kernel(double *bd, int ld, int n0, int mg, double 
 // --------------------------------------------------------------------------
 // f = r_d - X^-1 r_c (forward) or g_x - Z X^-1 g_z (adjoint); g = D f on block
 // columns.  First kernel of a solve: it also resets the ticket counters of the
-// wavefront and chain solves and fills their publication buffers (nw 32-bit words
+// wavefront, chain and border solves and fills their publication buffers (nw 32-bit words
 // each) with the unpublished pattern.
 struct PubFill {
   int *ticket;
-  unsigned *buf[3];
-  long long nw[3];
+  unsigned *buf[4];
+  long long nw[4];
 };
 
 __global__ void prep_f_kernel(double *f, double *g, const double *rd, const double *rc,
@@ -670,9 +670,9 @@ __global__ void prep_f_kernel(double *f, double *g, const double *rd, const doub
   pdl_begin();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  if (i < 4) P.ticket[i] = 0;
+  if (i < kTickets) P.ticket[i] = 0;
 #pragma unroll
-  for (int k = 0; k < 3; ++k)
+  for (int k = 0; k < 4; ++k)
     for (long long w = i; w < P.nw[k]; w += stride) P.buf[k][w] = 0xffffffffu;
   if (i >= n) return;
   const double fi = adjoint ? rd[i] - z[i] * rc[i] * xinv[i] : rd[i] - rc[i] * xinv[i];
@@ -837,66 +837,6 @@ __global__ void __launch_bounds__(kChainSolveThreads) chain_solve_kernel(CArgs A
   }
 }
 
-// The border solves.  With L the factor of the border (x_0 pivots first, then
-// y_g) and J = diag(-I, I), the border system's solution is L^-T J L^-1 b.
-// Substitution is a chain of 64-column steps on one SM (35 + 71 us per solve
-// of order 100, 126 + 223 us of order 601); the explicit W = L^-1, formed once
-// per factor, makes a solve two matrix-vector products over many SMs.  W's
-// rows are independent of each other: row r solves w L = e_r' from its own
-// 64-column tile leftwards, tile j as v = e_r' - (w L)_j over the columns
-// already done, w_j = v X_jj with the inverted diagonal tile X_jj.  A CTA takes
-// two rows, so the columns of L it streams serve both.
-constexpr int kBinvThreads = 256;
-
-__global__ void __launch_bounds__(kBinvThreads) border_inv_kernel(const double *L,
-                                                                  const double *X,
-                                                                  int B, int ld, double *Wr,
-                                                                  double *Wc) {
-  pdl_begin();
-  __shared__ double xs[NB][NB + 1];   // xs[c][q] = X_jj(q, c)
-  __shared__ double v[2][NB];
-  const int r0 = 2 * blockIdx.x, r1 = min(r0 + 1, B - 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double *w0 = Wr + (long long)r0 * ld, *w1 = Wr + (long long)r1 * ld;
-  const int ti = r0 / NB;
-  for (int j = ti; j >= 0; --j) {
-    const int c0 = j * NB;
-    for (int i = threadIdx.x; i < NB * NB; i += kBinvThreads)
-      xs[i / NB][i % NB] = X[(long long)j * NB * NB + i];
-    for (int c = warp; c < NB; c += kBinvThreads / 32) {
-      double s0 = 0.0, s1 = 0.0;
-      if (c0 + c < B && j < ti) {
-        const double *col = L + (long long)(c0 + c) * ld;
-        for (int q = c0 + NB + lane; q <= r1; q += 32) {   // row r0 is zero at q = r1
-          const double l = col[q];
-          s0 = fma(w0[q], l, s0);
-          s1 = fma(w1[q], l, s1);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        }
-      }
-      if (lane == 0) {
-        v[0][c] = (c0 + c == r0 ? 1.0 : 0.0) - s0;
-        v[1][c] = (c0 + c == r1 ? 1.0 : 0.0) - s1;
-      }
-    }
-    __syncthreads();
-    // thread (row a, column c, half h of the sum over q >= c)
-    const int a = threadIdx.x >> 7, c = (threadIdx.x >> 1) & (NB - 1), h = threadIdx.x & 1;
-    double s = 0.0;
-    for (int q = c + h; q < NB; q += 2) s = fma(v[a][q], xs[c][q], s);
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    if (h == 0 && c0 + c < B) {
-      (a ? w1 : w0)[c0 + c] = s;
-      Wc[(long long)(c0 + c) * ld + (a ? r1 : r0)] = s;
-    }
-    __syncthreads();
-  }
-}
-
 // border rhs: sB -= Z' uT, one CTA per border row over its column's link rows;
 // uT is the chain's forward solution, sB svec's border part
 __global__ void __launch_bounds__(128) border_rhs_kernel(const double *Z, int nl,
@@ -921,29 +861,6 @@ __global__ void __launch_bounds__(128) border_rhs_kernel(const double *Z, int nl
   if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) svec[nl + rb] -= (part[0] + part[1]) + (part[2] + part[3]);
-}
-
-// t = J W b (fwd, W's rows) or x = W' t (columns), one warp per entry
-__global__ void __launch_bounds__(256) border_w_kernel(const double *W, int B, int ld,
-                                                       int n0, const double *in,
-                                                       double *out, int fwd) {
-  pdl_begin();
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (i >= B) return;
-  const double *w = W + (long long)i * ld;
-  const int q1 = fwd ? i + 1 : B;
-  double s0 = 0.0, s1 = 0.0;
-  int q = (fwd ? 0 : i) + lane;
-#pragma unroll 4
-  for (; q + 32 < q1; q += 64) {
-    s0 = fma(w[q], in[q], s0);
-    s1 = fma(w[q + 32], in[q + 32], s1);
-  }
-  if (q < q1) s0 = fma(w[q], in[q], s0);
-  double s = s0 + s1;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[i] = fwd && i < n0 ? -s : s;
 }
 
 // svec's link part = uT - Z sB: a CTA takes 32 link rows, 16 threads per row share the border
@@ -1070,8 +987,6 @@ cudaError_t launch_schur_factor(ahlp_problem *p) {
     const int T = (p->B + NB - 1) / NB;
     cudaError_t e = launch_tile_inverses(p->border, p->border_tinv, p->bw_info, p->bw_sched, T, s);
     if (e != cudaSuccess) return e;
-    count_launch(), launch_pdl(border_inv_kernel, (p->B + 1) / 2, kBinvThreads, 0, s, p->border,
-                               p->border_tinv, p->B, p->Bld, p->border_wr, p->border_wc);
   }
   return cudaGetLastError();
 }
@@ -1088,9 +1003,10 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
                      {f32 ? reinterpret_cast<unsigned *>(p->vec32)
                           : reinterpret_cast<unsigned *>(p->vec),
                       reinterpret_cast<unsigned *>(p->vecb),
-                      reinterpret_cast<unsigned *>(p->bcr_pub)},
-                     {words, words, p->fac_bcr && p->bcr_pub ? 4LL * p->nl : 0}};
-  count_launch(), launch_pdl(prep_f_kernel, nb(std::max<long long>(n, 4), 256), 256, 0, s, p->f,
+                      reinterpret_cast<unsigned *>(p->bcr_pub),
+                      reinterpret_cast<unsigned *>(p->border_pub)},
+                     {words, words, p->fac_bcr && p->bcr_pub ? 4LL * p->nl : 0, 4LL * p->B}};
+  count_launch(), launch_pdl(prep_f_kernel, nb(std::max<long long>(n, kTickets), 256), 256, 0, s, p->f,
                              p->g, r_d, r_c, p->xinv, p->z, p->dscale, p->is_x0, n,
                              adjoint ? 1 : 0, fill);
   e = launch_spmv(p->Amat, p->g, p->rhat, 1.0, r_p, s);
@@ -1130,14 +1046,11 @@ cudaError_t launch_solve(ahlp_problem *p, const double *r_d, const double *r_p,
       // the chain's forward solution: published by the cyclic reduction, in place
       // in svec otherwise
       const double *uT = p->nl > 0 && p->fac_bcr ? p->bcr_pub : p->svec;
-      double *sb = p->svec + p->nl;
       if (p->nl > 0)
         count_launch(), launch_pdl(border_rhs_kernel, p->B, 128, 0, s, p->Et, p->nl, p->zlo,
                                    p->zhi, uT, p->svec);
-      count_launch(), launch_pdl(border_w_kernel, nb(p->B, 8), 256, 0, s, p->border_wr, p->B,
-                                 p->Bld, p->n0, sb, p->border_t, 1);
-      count_launch(), launch_pdl(border_w_kernel, nb(p->B, 8), 256, 0, s, p->border_wc, p->B,
-                                 p->Bld, p->n0, p->border_t, sb, 0);
+      e = launch_border_solve(p);
+      if (e != cudaSuccess) return e;
       if (p->nl > 0)
         count_launch(), launch_pdl(link_back_kernel, nb(p->nl, 32), 512, 0, s, p->Et, p->B, p->nl,
                                    uT, p->svec);
