@@ -386,7 +386,7 @@ struct ahlp_problem {
   double *f = nullptr, *g = nullptr, *rhat = nullptr;      // solve scratch
   double *stg[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // staging for host I/O
   double *res[3] = {nullptr, nullptr, nullptr};            // refinement residual
-  double *cor[3] = {nullptr, nullptr, nullptr};            // refinement correction
+  double *best[3] = {nullptr, nullptr, nullptr};           // a direction while its factor is redone
   double *ipmv[19] = {};      // IPM work vectors (the last three: a batch's balanced rhs)
   double *red_part = nullptr; // reduction partials
   int *red_cnt = nullptr;     // arrivals at the reductions' last CTAs (0 between launches)

@@ -1293,7 +1293,7 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
     p->res[0] = dalloc<double>(p, 2 * p->n + p->m);   // one vector [n | m | n]
     p->res[1] = p->res[0] + p->n;
     p->res[2] = p->res[1] + p->m;
-    for (auto &s : p->cor) s = dalloc<double>(p, mx);
+    for (auto &s : p->best) s = dalloc<double>(p, mx);
     for (auto &s : p->ipmv) s = dalloc<double>(p, mx);
     p->red_part = dalloc<double>(p, kRedSetMax * 304);
     p->red_cnt = dalloc<int>(p, kRedSetMax + 2);
@@ -1736,6 +1736,54 @@ int kkt_factor(ahlp_problem *p, const double *x, const double *z, double delta, 
   }
 }
 
+// Whether the Krylov refinement failed on a direction: a NaN that the right-hand side
+// does not explain, or steps taken that leave the residual far above the target
+// (1e-6 is where ipm_solve and the gradients stop trusting one).  No steps allowed
+// is not a failure: the residual is then that of the regularised system.
+static bool refinement_failed(const ahlp_problem *p, int status, const ahlp_solve_info &i) {
+  if (status == AHLP_ERR_NOT_SPD)
+    return std::isfinite(p->h_scal[10] + p->h_scal[11] + p->h_scal[12]);
+  if (status != AHLP_OK || i.refine_steps == 0) return false;
+  const double above = 10.0 * p->opt.refine_tol;
+  return !(i.rel_residual <= std::max(1e-6, above)) ||
+         (i.refine_steps >= std::min(p->opt.refine_max, kMaxKrylov) && i.rel_residual > above);
+}
+
+// A solve that failed on an FP64 factor with tensor-core updates: factor again on the
+// FP64 pipe at the same point and solve again.  The digits keep an entry relative to
+// its row's largest, and behind clamped pivots, whose rows grow by orders of magnitude,
+// that is a worse preconditioner (nearly degenerate LPs: residuals of 13 after 40 steps
+// where FP64 arithmetic leaves 0.03); without clamped pivots both take the same steps,
+// to 16 decades of D.  The better direction is returned; the factor stays the FP64
+// pipe's until the next kkt_factor, or the digits' where FP64 arithmetic breaks down.
+static int solve_on_pipe(ahlp_problem *p, const double *a, const double *b, const double *c,
+                         double *const *out, bool adjoint, int status, ahlp_solve_info *info) {
+  const long long len[3] = {p->n, p->m, p->n};
+  auto copy = [&](double *const *dst, double *const *src) {
+    for (int i = 0; i < 3; ++i)
+      ck(cudaMemcpyAsync(dst[i], src[i], len[i] * 8, cudaMemcpyDeviceToDevice, p->stream), "copy");
+  };
+  if (p->opt.verbose)
+    printf("kkt_solve: residual %.2e; refactoring on the FP64 pipe\n", info->rel_residual);
+  copy(p->best, out);
+  const ahlp_solve_info first = *info;
+  p->fp64_pipe = true;
+  int st = factor_impl(p, p->fac_delta, p->fac_rho, p->fac_pivot_tol, true);
+  if (st == AHLP_OK) {
+    st = solve_impl(p, a, b, c, out[0], out[1], out[2], adjoint, info);
+    if (status != AHLP_OK || (st == AHLP_OK && info->rel_residual <= first.rel_residual)) return st;
+    if (st != AHLP_OK && st != AHLP_ERR_NOT_SPD) return st;
+  } else {
+    if (st != AHLP_ERR_NOT_SPD) return st;
+    p->fp64_pipe = false;
+    st = factor_impl(p, p->fac_delta, p->fac_rho, p->fac_pivot_tol, true);
+    if (st != AHLP_OK) return st;
+  }
+  copy(out, p->best);
+  *info = first;
+  return status;
+}
+
 static int solve_entry(ahlp_problem *p, const double *a, const double *b, const double *c,
                        double *o1, double *o2, double *o3, ahlp_solve_info *info, bool adjoint) {
   if (!p) return AHLP_ERR_INVALID_ARG;
@@ -1748,7 +1796,13 @@ static int solve_entry(ahlp_problem *p, const double *a, const double *b, const 
     const double *dc = stage_in(p, c, p->n, p->stg[2]);
     const bool d1 = is_device_ptr(o1), d2 = is_device_ptr(o2), d3 = is_device_ptr(o3);
     double *w1 = d1 ? o1 : p->stg[3], *w2 = d2 ? o2 : p->stg[4], *w3 = d3 ? o3 : p->stg[5];
-    int st = solve_impl(p, da, db, dc, w1, w2, w3, adjoint, info);
+    ahlp_solve_info si{};
+    int st = solve_impl(p, da, db, dc, w1, w2, w3, adjoint, &si);
+    if (p->fac_prec == kPrecFP64 && p->fac_dz && refinement_failed(p, st, si)) {
+      double *const out[3] = {w1, w2, w3};
+      st = solve_on_pipe(p, da, db, dc, out, adjoint, st, &si);
+    }
+    if (info && (st == AHLP_OK || st == AHLP_ERR_NOT_SPD)) *info = si;
     if (!d1) ck(cudaMemcpyAsync(o1, w1, p->n * 8, cudaMemcpyDeviceToHost, p->stream), "D2H");
     if (!d2) ck(cudaMemcpyAsync(o2, w2, p->m * 8, cudaMemcpyDeviceToHost, p->stream), "D2H");
     if (!d3) ck(cudaMemcpyAsync(o3, w3, p->n * 8, cudaMemcpyDeviceToHost, p->stream), "D2H");
