@@ -259,7 +259,9 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
       // is tested.
       const double per_lp =
           nlp > 0 ? last_rel * std::sqrt((double)std::max(n_active, 1)) : last_rel;
-      if (!allow_delta && per_lp <= kStallAccept &&
+      // FP64 arithmetic has not been tried while the updates run on the tensor cores
+      const bool digits = p->fac_prec == kPrecFP64 && p->fac_dz && !p->fp64_pipe;
+      if (!allow_delta && per_lp <= kStallAccept && !digits &&
           (p->fac_prec == kPrecFF || p->fac_prec == kPrecFP64)) {
         if (p->opt.verbose)
           printf("       %s accepted (%s factor, residual %.2e)\n", why,
@@ -275,7 +277,7 @@ extern "C" int ipm_solve(ahlp_problem *p, const double *x0, const double *y0, co
       } else if (p->fac_prec != kPrecFP64) {   // FP32 -> float-float -> FP64
         if (p->fac_prec == kPrecFP32 && R.fp64_switch_iter < 0) R.fp64_switch_iter = cur_iter;
         p->fac_prec = p->fac_prec == kPrecFP32 ? kPrecFF : kPrecFP64;
-      } else if (p->fac_dz && !p->fp64_pipe) {
+      } else if (digits) {
         // the tensor-core updates keep an entry to 2^-63 of its row's largest entry,
         // FP64 arithmetic to 2^-53 of itself: once pivots are clamped, the second
         // is the better preconditioner (512 uneven blocks, last iteration: 40 Krylov
