@@ -27,31 +27,64 @@ from . import _lib as L
 
 _ADJOINT_TOL = 1e-6   # relative residual above which the transposed solve has stalled
 
+# the options' own regularisation of the factor, then more (dual delta, primal rho)
+_REGULARISATION = ((-1.0, -1.0), (1e-6, 1e-8), (1e-4, 1e-6))
+_NOT_SPD = -4         # AHLP_ERR_NOT_SPD
+
 
 def _factor_chain(prob, x, z):
-    """kkt_factor at (x, z), answering a NaN pivot with more regularisation
-    (dual delta, primal rho); True on success."""
-    for delta, rho in ((-1.0, -1.0), (1e-6, 1e-8), (1e-4, 1e-6)):
+    """kkt_factor at (x, z), answering a NaN pivot with more regularisation;
+    True on success."""
+    for delta, rho in _REGULARISATION:
         try:
             L.kkt_factor(prob, x, z, delta, rho)
             return True
         except L.AHLPError as e:
-            if e.status != -4:   # AHLP_ERR_NOT_SPD
+            if e.status != _NOT_SPD:
                 raise
     return False
 
 
+class _fp64_options:
+    """The handle's options with FP64 block factors, its own ones restored at the end."""
+
+    def __init__(self, prob):
+        self.prob = prob
+
+    def __enter__(self):
+        self.saved = L.Options.from_buffer_copy(self.prob.options)
+        fp64 = L.Options.from_buffer_copy(self.saved)
+        fp64.precision = L.PREC_FP64
+        L.set_options(self.prob, fp64)
+
+    def __exit__(self, *exc):
+        L.set_options(self.prob, self.saved)
+
+
 def _factor_fp64(prob, x, z):
-    """The same chain with FP64 block factors, the handle's options restored."""
-    opts = L.Options.from_buffer_copy(prob.options)
-    fp64 = L.Options.from_buffer_copy(opts)
-    fp64.precision = L.PREC_FP64
-    L.set_options(prob, fp64)
-    try:
+    """The same chain with FP64 block factors."""
+    with _fp64_options(prob):
         if not _factor_chain(prob, x, z):
             raise RuntimeError("no usable factor at the returned point")
-    finally:
-        L.set_options(prob, opts)
+
+
+def _adjoint_fp64(prob, x, z, g):
+    """The transposed solve with FP64 block factors, answering a stall like a NaN
+    pivot: a factor may be accepted and still precondition too badly, and more
+    regularisation can mend that."""
+    info = None
+    with _fp64_options(prob):
+        for delta, rho in _REGULARISATION:
+            try:
+                L.kkt_factor(prob, x, z, delta, rho)
+                lam, info = L.kkt_adjoint_solve(prob, *g)
+            except L.AHLPError as e:
+                if e.status != _NOT_SPD:
+                    raise
+                continue
+            if info["rel_residual"] <= _ADJOINT_TOL:
+                return lam
+    raise RuntimeError(f"adjoint KKT solve did not converge: {info}")
 
 
 def _factor_at_optimum(prob, x, z):
@@ -99,11 +132,9 @@ class LPSolve(torch.autograd.Function):
         (lx, ly, _), info = L.kkt_adjoint_solve(prob, gx, gy, gz)
         if not info["rel_residual"] <= _ADJOINT_TOL:
             # the factor of the final iterate is not a good enough
-            # preconditioner (mixed precision at an extreme D): refactor in FP64
-            _factor_fp64(prob, x, z)
-            (lx, ly, _), info = L.kkt_adjoint_solve(prob, gx, gy, gz)
-            if not info["rel_residual"] <= _ADJOINT_TOL:
-                raise RuntimeError(f"adjoint KKT solve did not converge: {info}")
+            # preconditioner (mixed precision at an extreme D, or rows that
+            # depend on each other up to rounding)
+            lx, ly, _ = _adjoint_fp64(prob, x, z, (gx, gy, gz))
         return lx, ly, None
 
 
