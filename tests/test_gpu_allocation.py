@@ -46,7 +46,10 @@ from paper_2412_07731_gb300._lib import kkt_block_factor_dense
 shim = ctypes.CDLL(sys.argv[1])
 shim.shim_failed.restype = ctypes.c_long
 prec, shape = sys.argv[2], sys.argv[3]
-if shape == "banded":       # a tile-sparse job table, blocks without a job at the next diagonal tile
+if shape == "large":        # more than 152 trailing tiles: the FP64 pipe's undivided updates
+    lp = random_block_lp(6, N=2, m_sizes=[1300, 500], n_sizes=[1950, 750], nnz_per_col=4, n0=5,
+                         w_density=0.3, l=2)
+elif shape == "banded":     # a tile-sparse job table, blocks without a job at the next diagonal tile
     lp = config3(days=2)
 else:
     lp = random_block_lp(5, N=3, m_sizes=[200, 150, 90], n_sizes=[300, 230, 140], nnz_per_col=4,
@@ -117,6 +120,7 @@ def shim(tmp_path_factory):
 # at least: offsets and counters; digit planes and exponents | tensor maps and staging;
 # on banded blocks also the job table and the blocks without a diagonal job
 @pytest.mark.parametrize("prec,shape,least", [("fp64", "random", 4), ("fp64", "banded", 5),
+                                              ("fp64", "large", 4),
                                               ("fp32", "random", 4), ("ff", "random", 5)])
 def test_every_failed_allocation_leaves_the_handle_usable(shim, prec, shape, least):
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
