@@ -68,7 +68,17 @@ constexpr int kTagBorderX = 1 << 20;   // pivot reports of the border x_0 factor
 constexpr int kTagBorderG = 2 << 20;   // pivot reports of the border y_g factor
 
 #ifdef __CUDACC__
-// First statement of every kernel that launch_pdl starts: returns when the
+// Every device wait of the library gives up after this long; the host then reports
+// AHLP_ERR_TIMEOUT.
+constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // 1 s
+
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// First statement of nearly every kernel that launch_pdl starts: returns when the
 // kernels before this one are complete and their writes are visible; from then
 // on the next kernel of the stream may be scheduled (it waits in turn).
 // pdl_wait leaves that to the kernel's end: for kernels that fill the GPU, whose
@@ -86,8 +96,10 @@ __device__ __forceinline__ void pdl_begin() {
 // Launch with programmatic stream serialisation: the kernel's launch and the
 // scheduling of its CTAs overlap the tail of the kernel before it.  Dependent
 // kernels of a few CTAs follow each other in 1.5 us instead of 4.1 us, and most
-// of a solve's kernels are that small.  Only for kernels that begin with
-// pdl_begin().
+// of a solve's kernels are that small.  Only for kernels in which every thread passes
+// griddepcontrol.wait before it touches what earlier kernels wrote: with pdl_begin or
+// pdl_wait first, or, in diagonal factorisations beside an update, after the wait for
+// that update's counts (diag_begin), with griddepcontrol.wait at the end (diag_end).
 template <typename... P, typename... A>
 inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                        A &&...args) {
@@ -235,7 +247,6 @@ struct ahlp_problem {
   long long n = 0, m = 0, msum = 0;   // n_total, m_total, sum of m_i
   std::vector<int> mi, ni, ki, lprev, lnext;
   std::vector<long long> xoff, yoff, link_off;   // link_off has N entries (pairs + 1)
-  int amax = 0;          // largest augmented order
   ahlp_options opt{};
   cudaStream_t stream = nullptr;
   std::string err;

@@ -953,7 +953,6 @@ int arrowhead_lp_create(const ahlp_desc *descs, int32_t batch, const ahlp_option
       voff += a;
       d0 += m;
       cd += k;
-      p->amax = std::max(p->amax, a);
       p->maxT = std::max(p->maxT, bi.T);
       p->maxTp = std::max(p->maxTp, bi.Tp);
       SchurBlk sb{};

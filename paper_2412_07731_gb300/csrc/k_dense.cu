@@ -415,9 +415,9 @@ __device__ __forceinline__ void dz_stage_rows(F x, int row0, int nrow, int nri, 
 constexpr int kTrsmThreads = 128;
 constexpr size_t kTrsmSmem = NB * (NB + 1) * sizeof(double);
 template <int G>
-__global__ void __launch_bounds__(kTrsmThreads, G == 2 ? 3 : 4) pchol_trsm_kernel(double *buf, const BlkInfo *blk,
-                                                                  int k, __half *stage, int *dexp,
-                                                                  long long slots) {
+__global__ void __launch_bounds__(kTrsmThreads, G == 2 ? 3 : 4)
+    pchol_trsm_kernel(double *buf, const BlkInfo *blk, int k, __half *stage, int *dexp,
+                      long long slots) {
   pdl_begin();
   constexpr int R = 32 / G, kRows = kTrsmThreads / G, kC = NB / G;
   const BlkInfo bi = blk[blockIdx.y];
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kTrsmThreads, G == 2 ? 3 : 4) pchol_trsm_kerne
 // lane groups per row: as many as keep every warp of the step's tiles (2 G per
 // tile) on a partition of its own.  One tile: 70 us with a column's updates spread
 // over a CTA between two barriers.
-constexpr int kSMs = 152;
+constexpr int kSMs = 152;   // chooses layouts of the same arithmetic, nothing else
 inline int trsm_lanes(long long tiles) {
   return tiles * 16 <= 4 * kSMs ? 8 : tiles * 8 <= 4 * kSMs ? 4 : 2;
 }
@@ -1181,7 +1181,8 @@ __global__ void __launch_bounds__(kThreads) pchol_update_kernel(T *buf, const Bl
 #pragma unroll
     for (int i = 0; i < A; ++i) {
       const int r = tx + 16 * i;
-      if (r < nrI && c < nrJ && (I != J || sI != sJ || r >= c)) gc[(long long)c * bi.lda + r] -= acc[i][j];
+      if (r < nrI && c < nrJ && (I != J || sI != sJ || r >= c))
+        gc[(long long)c * bi.lda + r] -= acc[i][j];
     }
   }
 }
@@ -1967,9 +1968,9 @@ cudaError_t launch_pchol_ff(float *hi, float *lo, double *out, long long elems,
     if (prof) kt_mark(prof, 1, s);
     if (maxPanel > 0)
       count_launch(), launch_pdl(pchol_trsm_ff_kernel,
-                                 dim3((unsigned)((maxPanel + kFFRowTiles - 1) /
-                                                             kFFRowTiles),
-                                                  nblk), kFFRowThreads, kTrsmFFSmem, s, hi, lo, info, k, oz ? oz->dstage : nullptr, oz ? oz->dexp : nullptr);
+                                 dim3((unsigned)((maxPanel + kFFRowTiles - 1) / kFFRowTiles), nblk),
+                                 kFFRowThreads, kTrsmFFSmem, s, hi, lo, info, k,
+                                 oz ? oz->dstage : nullptr, oz ? oz->dexp : nullptr);
     if (prof) kt_mark(prof, 2, s);
     if (maxTrail > 0) {
       if (oz) {
@@ -2026,8 +2027,7 @@ cudaError_t launch_trsv(ahlp_problem *p, bool forward, const double *rhs, double
     if (forward)
       count_launch(), launch_pdl(trsv_fwd_kernel<float>, njobs, TrsvCfg<float, false>::threads, 0,
                                  s, p->aug32, p->tinv32, p->blk, sched, ticket, p->trsv_err,
-                                 p->vec, p->vec32, rhs,
-          p->yoff_d);
+                                 p->vec, p->vec32, rhs, p->yoff_d);
     else
       count_launch(), launch_pdl(trsv_bwd_kernel<float>, njobs, TrsvCfg<float, true>::threads, 0,
                                  s, p->aug32, p->tinv32, p->blk, sched, ticket, p->trsv_err,

@@ -15,11 +15,20 @@
 //     sum_k x_rk y_ck = 2^(E_r+E_c-14) sum_q 2^(-8q) D_q.
 // Over 64 pivot columns |D_q| <= (q + 1) 2^20 < 2^24, so the tensor core's
 // FP32 accumulation of FP16 products is exact.  The 36 digit products with
-// s + t <= 7 are kept; the dropped ones are near 2^-61 of the row scales'
-// product, well below the roundings of 64 chained FP64 multiply-adds.  The
-// epilogue adds the eight D_q in 64-bit integers, turns the sum into an FP64
-// number by shifts (one rounding) and subtracts it from C with one FP64
-// operation per entry (a second rounding).
+// s + t <= 7 are kept.  The dropped ones sum to about 7 2^20 2^-78 = 2^-55 of
+// 2^(E_r + E_c) at most, which is 2^-51 of the product of the rows' largest
+// entries at worst (E is up to two above an entry's binary magnitude); digits of
+// mixed signs leave about 2^-61 of the scales, below the roundings of 64 chained
+// FP64 multiply-adds.  The epilogue adds the eight D_q in 64-bit integers, rounded
+// to units of 2^-58 of the scales (12 bits less than the sum holds), turns the sum
+// into an FP64 number by shifts (a second rounding) and subtracts it from C with
+// one FP64 operation per entry (a third).
+// All of it is relative to the rows' scales, where FP64 arithmetic rounds each
+// product relative to itself.  The block factors meet the same normwise backward
+// error bound, and as preconditioners they take the same Krylov steps up to 16
+// decades of D.  Behind clamped pivots, whose rows grow by orders of magnitude,
+// they are worse; solves that fail then move to the FP64 pipe (solve_on_pipe,
+// ipm_solve's safeguards).
 //
 // One persistent CTA per SM walks the step's jobs (128 x 64 tiles of C, job
 // blockIdx.x + j * gridDim.x):
@@ -103,7 +112,7 @@ __device__ __forceinline__ void tmem_ld2(uint32_t taddr, float (&v)[2]) {
   v[1] = __uint_as_float(r1);
 }
 
-// sum_q D_q 2^(44-8q) as a 64-bit integer (the last 14 bits of the eight-digit
+// sum_q D_q 2^(44-8q) as a 64-bit integer (the last 12 bits of the eight-digit
 // sum rounded away).  |D_q| <= (q + 1) 2^20, |D_0| <= 2^18, so the pairs fit 32 bits.
 __device__ __forceinline__ long long dz_combine(const float (&D)[kDzQ]) {
   const int a = (__float2int_rn(D[0]) << 8) + __float2int_rn(D[1]);

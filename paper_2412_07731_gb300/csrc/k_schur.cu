@@ -918,16 +918,17 @@ cudaError_t launch_schur_assemble(ahlp_problem *p, double delta, double rho) {
     count_launch(), launch_pdl(assemble_T_kernel, dim3(nb((long long)lmax * lmax, 256), p->N - 1),
                                256, 0, s, A);
     if (p->N > 2)
-      count_launch(), launch_pdl(assemble_H_kernel, dim3(nb((long long)lmax * lmax, 256),
-                                 p->N - 2), 256, 0, s, A);
+      count_launch(), launch_pdl(assemble_H_kernel,
+                                 dim3(nb((long long)lmax * lmax, 256), p->N - 2), 256, 0, s, A);
     if (p->B > 0)
-      count_launch(), launch_pdl(assemble_E_kernel, dim3(nb((long long)lmax * p->B, 256),
-                                 p->N - 1), 256, 0, s, A);
+      count_launch(), launch_pdl(assemble_E_kernel,
+                                 dim3(nb((long long)lmax * p->B, 256), p->N - 1), 256, 0, s, A);
   }
-  if (p->B > 0) count_launch(), launch_pdl(assemble_SB_kernel, nb((long long)p->B * p->B, 256),
-                                        256, 0, s, A);
-  if (p->nf0 > 0) count_launch(), launch_pdl(scatter_add_kernel, nb(p->nf0, 256), 256, 0, s, p->Et,
-                                        p->f0_idx, p->f0_val, p->nf0);
+  if (p->B > 0)
+    count_launch(), launch_pdl(assemble_SB_kernel, nb((long long)p->B * p->B, 256), 256, 0, s, A);
+  if (p->nf0 > 0)
+    count_launch(), launch_pdl(scatter_add_kernel, nb(p->nf0, 256), 256, 0, s, p->Et, p->f0_idx,
+                               p->f0_val, p->nf0);
   if (p->nfg0 > 0)
     count_launch(), launch_pdl(scatter_add_kernel, nb(p->nfg0, 256), 256, 0, s, p->SB, p->fg0_idx,
                                p->fg0_val, p->nfg0);
@@ -959,8 +960,7 @@ cudaError_t launch_schur_factor(ahlp_problem *p) {
                                  A);
       if (p->B > 0)
         count_launch(), launch_pdl(chain_z_kernel, (unsigned)((p->B + 7) / 8), 256, 0, s, A,
-                                   p->zlo,
-                                                                                   p->zhi);
+                                   p->zlo, p->zhi);
     } else if (p->nchain_seg > 0) {
       count_launch(), launch_pdl(chain_factor_kernel, p->nchain_seg, 512, (size_t)lmax * lmax * 8,
                                  s, cargs(p));

@@ -546,8 +546,7 @@ cudaError_t launch_reduce_set(ahlp_problem *p, const RedOne *ops, int n) {
       nb = std::max(nb, S.nb[i]);
     }
     count_launch(), launch_pdl(reduce_set_kernel, dim3(nb, c), kRedThreads, 0, p->stream, S,
-                               p->red_part,
-                                                                                p->red_cnt);
+                               p->red_part, p->red_cnt);
   }
   return cudaGetLastError();
 }
@@ -618,8 +617,7 @@ cudaError_t launch_residual(ahlp_problem *p, const double *r_d, const double *r_
   T.e_c = e_c;
   T.adjoint = adjoint ? 1 : 0;
   count_launch(), launch_pdl(spmv_kernel<SP_RESID>, sp_ctas(a) + sp_ctas(b), kSpThreads, 0,
-                             p->stream, a, b,
-                                                                                              T);
+                             p->stream, a, b, T);
   return cudaGetLastError();
 }
 
@@ -656,8 +654,7 @@ cudaError_t launch_centrality_rc(double *rc2, const double *rc, const double *x,
                                  double ad, double lo, double hi, long long n, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   count_launch(), launch_pdl(centrality_rc_k, blocks_for(n, 256), 256, 0, s, rc2, rc, x, dx, ap, z,
-                             dz, ad,
-                                                                     lo, hi, n);
+                             dz, ad, lo, hi, n);
   return cudaGetLastError();
 }
 

@@ -6,14 +6,6 @@
 
 namespace ahlp {
 
-constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // 1 s
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
 // Solved entries are their own ready flags: the publication buffers are filled
 // with a bit pattern (all ones, a NaN no arithmetic produces) by the first
 // kernel of a solve, a writer stores an entry with a relaxed store, a reader

@@ -10,17 +10,8 @@
 
 namespace ahlp {
 
-constexpr unsigned long long kWaitNs = 1000000000ull;   // 1 s
-
-
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ unsigned long long globaltimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -51,9 +42,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 #pragma unroll 1
   for (int i = 0; i < 16; ++i)
     if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer();
+  const unsigned long long t0 = global_ns();
   while (!mbar_try(bar, parity))
-    if (globaltimer() - t0 > kWaitNs) return false;
+    if (global_ns() - t0 > kWaitLimitNs) return false;
   return true;
 }
 
