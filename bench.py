@@ -637,7 +637,15 @@ UPDATE_KERNEL = {("FP32", 1): "pchol_update_f32_kernel (FP32 pipe)",
                  ("float-float", 1): "pchol_update_ff8_kernel (double-float, FP32 pipe)",
                  ("float-float", 2): "pchol_update_oz_kernel (tcgen05 digits, one CTA per tile)",
                  ("float-float", 3): "pchol_update_oz2_kernel (tcgen05 digits, persistent)",
+                 ("FP64", 1): "pchol_update_kernel (FP64 pipe)",
                  ("FP64", 2): "pchol_update_dz_kernel (tcgen05 digits, persistent)"}
+
+
+def fp64_variant(flop, ms):
+    """2: updates on the tensor cores; 1: on the FP64 pipe, to which a factor moves when the
+    digits break down.  A time the pipe could not do the flops in tells them apart (the
+    digit updates are ten times faster than that)."""
+    return 2 if flop > FP64_PEAK_TFLOPS * 1e12 * ms / 1e3 else 1
 
 
 def kernel_roofline(P, prob, lp, x, z, prec_name, peaks):
@@ -671,7 +679,7 @@ def kernel_roofline(P, prob, lp, x, z, prec_name, peaks):
     upd_ms, launches = med("update_ms"), med("update_launches")
     jobs = P.kkt_update_jobs(prob)
     # option 0 picks the persistent kernels on a workload of this size
-    variant = 2 if prec_name == "FP64" else (
+    variant = fp64_variant(update_geometry(lp)[1], upd_ms) if prec_name == "FP64" else (
         saved.fp32_update if prec_name == "FP32" else saved.ff_update) or 3
     tensor_upd = variant in (2, 3)
     elems, flops = update_geometry(lp, jobs=jobs if tensor_upd else None)
@@ -738,18 +746,19 @@ def roofline(lp, win, peaks, opts=None, jobs=None):
     variant = None
     if opts is not None:
         variant = (opts.fp32_update if name == "FP32" else
-                   opts.ff_update if name == "float-float" else 2)
+                   opts.ff_update if name == "float-float" else fp64_variant(flops, ms))
     if variant in (0, 2, 3):   # tensor-core trailing updates
         _, upd_flops = update_geometry(lp, jobs=jobs)
         per, ratio, op = ((3, TF32_PER_BF16, "TF32") if name == "FP32" else
                           (21 if name == "float-float" else 36, FP16_PER_BF16, "FP16"))
         tpeak = peaks["bf16_tflops_sustained"] * ratio
+        fell = "; factors that moved to the FP64 pipe count in the mean" if name == "FP64" else ""
         achieved = per * upd_flops / (ms / 1e3) / 1e12
         out = {"bound": "tensor", "achieved": achieved, "peak": tpeak, "unit": "TFLOP/s",
                "frac": achieved / tpeak, "traffic": None,
                "kernel": f"batched block partial Cholesky ({name}; diagonal tile, panel, "
                          f"trailing update on the tensor cores as {per} {op} MMAs per "
-                         f"product), {flops:.4g} flop per factor, {ms:.2f} ms",
+                         f"product{fell}), {flops:.4g} flop per factor, {ms:.2f} ms",
                "peak_source": f"{peaks['source']} sustained BF16 peak x {ratio:.3f} "
                               f"(nominal {op}:BF16 dense ratio)",
                "fp64_equivalent_tflops": flops / (ms / 1e3) / 1e12}

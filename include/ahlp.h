@@ -55,8 +55,20 @@ extern "C" {
 #define AHLP_ERR_TIMEOUT        -10  /* a bounded device wait ran out                          */
 #define AHLP_ERR_STOPPED        -11  /* ipm_solve: the iteration callback asked to stop        */
 
-#define AHLP_PREC_FP64   0   /* every stage in FP64                                    */
+#define AHLP_PREC_FP64   0   /* FP64 block factors, their trailing updates on the tensor cores (below); all else in FP64 */
 #define AHLP_PREC_MIXED  1   /* FP32 block factors (float-float near the optimum), FP64 Schur factor and refinement */
+
+/* FP64 block factors (of handles with an augmented block order above 64) take their
+ * trailing updates as exact products of FP16 integer digits: every panel entry to 2^-63 of its row's
+ * largest, each update rounded to about 2^-55 of the rows' scales.  The factors
+ * meet the normwise backward error bound of FP64 arithmetic.  Where rows are
+ * graded by orders of magnitude (clamped pivots near a degenerate optimum) they
+ * can be worse preconditioners than FP64 arithmetic's.  kkt_factor therefore
+ * factors on the FP64 pipe when such a factor meets a NaN pivot, kkt_solve and
+ * kkt_adjoint_solve when their refinement fails on one (the better direction is
+ * returned), and ipm_solve from its first stalled direction on.  The FP64 pipe is
+ * also used when the driver cannot encode tensor maps and when the device has no
+ * room for the digits (64 KB per 64 rows, taken by the first factor). */
 
 /* ---- problem description (host memory, copied at create) --------------- */
 
@@ -387,6 +399,11 @@ int kkt_factor(ahlp_problem *p, const double *x, const double *z, double delta, 
  *   r_d [n_total], r_p [m_total], r_c [n_total] : right-hand side
  *   dx [n_total], dy [m_total], dz [n_total]    : output (caller-allocated)
  *   info : optional (NULL allowed)
+ * When the refinement fails on an FP64 factor whose updates ran on the tensor
+ * cores (a NaN, a residual above 1e-6 and ten times refine_tol, or every step used
+ * with ten times refine_tol not reached), the handle factors again on the FP64 pipe
+ * at the same point and solves again; info and the output hold the better
+ * direction, and the factor stays until the next kkt_factor.
  * Returns AHLP_ERR_INVALID_ARG if no factor exists.  Missing the refinement
  * target is reported in info, not as an error.
  */
