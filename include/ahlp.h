@@ -401,7 +401,7 @@ int kkt_factor(ahlp_problem *p, const double *x, const double *z, double delta, 
  *   info : optional (NULL allowed)
  * When the refinement fails on an FP64 factor whose updates ran on the tensor
  * cores (a NaN, a residual above 1e-6 and ten times refine_tol, or every step used
- * with ten times refine_tol not reached), the handle factors again on the FP64 pipe
+ * without reaching ten times refine_tol or 1e-12), the handle factors again on the FP64 pipe
  * at the same point and solves again; info and the output hold the better
  * direction, and the factor stays until the next kkt_factor.
  * Returns AHLP_ERR_INVALID_ARG if no factor exists.  Missing the refinement

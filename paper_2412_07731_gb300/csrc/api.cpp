@@ -1737,13 +1737,14 @@ int kkt_factor(ahlp_problem *p, const double *x, const double *z, double delta, 
 
 // Whether the Krylov refinement failed on a direction: a NaN that the right-hand side
 // does not explain, or steps taken that leave the residual far above the target
-// (1e-6 is where ipm_solve and the gradients stop trusting one).  No steps allowed
-// is not a failure: the residual is then that of the regularised system.
+// (1e-6 is where ipm_solve and the gradients stop trusting one; below 1e-12 no factor
+// gets much further).  No steps allowed is not a failure: the residual is then that of
+// the regularised system.
 static bool refinement_failed(const ahlp_problem *p, int status, const ahlp_solve_info &i) {
   if (status == AHLP_ERR_NOT_SPD)
     return std::isfinite(p->h_scal[10] + p->h_scal[11] + p->h_scal[12]);
   if (status != AHLP_OK || i.refine_steps == 0) return false;
-  const double above = 10.0 * p->opt.refine_tol;
+  const double above = std::max(10.0 * p->opt.refine_tol, 1e-12);
   return !(i.rel_residual <= std::max(1e-6, above)) ||
          (i.refine_steps >= std::min(p->opt.refine_max, kMaxKrylov) && i.rel_residual > above);
 }
